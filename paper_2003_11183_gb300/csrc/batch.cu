@@ -151,9 +151,11 @@ __global__ void __launch_bounds__(BATCH_T) k_batch(const BatchProblem* __restric
           const float bt = (bv * rs - sum) * iv;
           float w, wc;
           lattice_wf(xv, P.periodize, w, wc);
-          float f, la, y;
-          sov_step_f32_prod(at, bt, w, wc, f, la, y);
-          lsum += la;
+          float f, y;
+          if (at == -INFINITY)  // (the same for the whole block of samples)
+            sov_step_f32_upper(bt, w, wc, f, lsum, y);
+          else
+            sov_step_f32_prod(at, bt, w, wc, f, lsum, y);
           prod *= f;
           const int pb = __float_as_int(prod);
           pe += (pb >> 23) - 127;
@@ -197,12 +199,12 @@ struct BatchTcProblem {
   const int64_t* kcol_off;
   const int32_t* vmap16;    // W row of each column rank
   const float* BT;
-  const float* inv;
-  const float* band;
+  const float* rec;
   const uint64_t* Q;
   const uint64_t* D;
   const float* a;
   const float* b;
+  const int* two;           // nonzero: some lower limit of the problem is finite
 };
 
 template <int FLAGS>
@@ -213,54 +215,48 @@ __global__ void __launch_bounds__(STC_NS, 6)
                unsigned short* Wbase, int64_t kwmax, unsigned short* Ybase, int my, double* logP, int* err) {
   constexpr bool PER = FLAGS & SWEEP_PERIODIZE;
   extern __shared__ __align__(1024) unsigned char stc_smem[];
-  __shared__ uint32_t phases;
-  __shared__ int abort_flag;
-  __shared__ int cur;
-  const StcCta k = stc_cta_setup<1>(stc_smem, &phases, &abort_flag);
+  const StcCta k = stc_cta_setup(stc_smem);
   const int tid = threadIdx.x;
   StcPlace pl;
   pl.wx = 0;
   pl.wy = (int)(blockIdx.x * kwmax);
   pl.yrow = blockIdx.x * STC_NS;
-  pl.ysrow[0] = Ybase + ((int64_t)blockIdx.x * STC_NS + tid) * (2 * my);  // (hi at 0, lo at my)
-  pl.wcol[0] = Wbase + (int64_t)blockIdx.x * kwmax * STC_NS + tid;
+  pl.ysrow = Ybase + ((int64_t)blockIdx.x * STC_NS + tid) * (2 * my);  // (hi at 0, lo at my)
+  pl.wcol = Wbase + (int64_t)blockIdx.x * kwmax * STC_NS + tid;
   for (;;) {
     __syncthreads();  // every thread is done with the previous item
-    if (tid == 0) cur = atomicAdd(next, 1);
+    if (tid == 0) *k.item = atomicAdd(next, 1);
     __syncthreads();
-    const int it = cur;
-    if (it >= n_items || *(volatile int*)&abort_flag) break;
+    const int it = *(volatile int*)k.item;
+    if (it >= n_items || *(volatile int*)k.abort_flag) break;
     const BatchItem item = items[it];
     const BatchTcProblem& P = probs[item.prob];
-    const bool act[1] = {tid < item.count};
-    const int64_t g = item.sample0 + (act[0] ? tid : item.count - 1);  // inactive lanes shadow a valid sample
+    const bool act = tid < item.count;
+    const int64_t g = item.sample0 + (act ? tid : item.count - 1);  // inactive lanes shadow a valid sample
     const int64_t sh = g / P.n_points;
-    const uint32_t ks[1] = {(uint32_t)(g - sh * P.n_points) + 1u};
+    const uint32_t ks = (uint32_t)(g - sh * P.n_points) + 1u;
     const uint64_t* Drow = P.D + sh * (int64_t)(P.n + 1);
-    float rs[1] = {1.0f};
+    float rs = 1.0f;
     if (isfinite(P.nu)) {
       double w, wc;
-      lattice_w((uint64_t)ks[0] * P.Q[P.n] + Drow[P.n], PER ? 1 : 0, w, wc);
-      rs[0] = (float)sqrt(2.0 * gamma_p_inv(0.5 * P.nu, w, wc) / P.nu);
+      lattice_w((uint64_t)ks * P.Q[P.n] + Drow[P.n], PER ? 1 : 0, w, wc);
+      rs = (float)sqrt(2.0 * gamma_p_inv(0.5 * P.nu, w, wc) / P.nu);
     }
     const CUtensorMap* mp = pmaps + (int64_t)BATCH_TC_MAPS * item.prob;
-    float prod[1] = {1.0f}, lsum[1] = {0.0f};
-    int pe[1] = {0};
+    const bool two = *P.two != 0;
+    float prod = 1.0f, lsum = 0.0f;
+    int pe = 0;
     bool ok = true;
     for (int i = 0; i < P.r && ok; i++) {
       const int64_t t0 = P.tile_off[i];
       SweepTcArgs p;
-      DiagArgs32& d = p.d;
-      d.BT = P.BT + (int64_t)i * P.m * P.ldbt;
-      d.inv = P.inv + (int64_t)i * P.m;
-      d.band = P.band + (int64_t)i * P.m * 16;
-      d.mt = (int)(P.tile_off[i + 1] - t0);
-      d.ldbt = P.ldbt;
-      d.a = P.a + t0;
-      d.b = P.b + t0;
-      d.Q = P.Q;
-      d.coord0 = t0;
-      d.ys_lo = my;
+      p.rec = P.rec + (int64_t)i * P.m * STC_REC;
+      p.BT = P.BT + (int64_t)i * P.m * P.ldbt;
+      p.ldbt = P.ldbt;
+      p.mt = (int)(P.tile_off[i + 1] - t0);
+      p.a = P.a + t0;
+      p.b = P.b + t0;
+      p.ys_lo = my;
       p.brow0 = i * P.m;
       p.alo = my;
       p.blo = P.my;
@@ -269,33 +265,36 @@ __global__ void __launch_bounds__(STC_NS, 6)
       p.kr = (int)(P.krow_off[i + 1] - P.krow_off[i]);
       p.kcol0 = (int)P.kcol_off[i];
       p.kc = (int)(P.kcol_off[i + 1] - P.kcol_off[i]);
-      p.W = Wbase;
       p.ldw = STC_NS;
       p.vmap = P.vmap16 ? P.vmap16 + P.kcol_off[i] : nullptr;
       p.wscale = nullptr;
       p.tscale = 1.0f;
       p.err = err;
-      const uint64_t* const Ds[1] = {Drow + t0};
-      ok = stc_tile<FLAGS, false, 1>(&mapY, mp, &mapW, mp + 1, &mapY64, mp + 2, p, k, pl, act, Ds, ks, rs, prod,
-                                     lsum, pe);
+      if (two)
+        ok = stc_tile<FLAGS, false>(&mapY, mp, &mapW, mp + 1, &mapY64, mp + 2, p, k, pl, act, Drow + t0, ks, rs, prod,
+                                    lsum, pe);
+      else
+        ok = stc_tile<FLAGS | SWEEP_ONE_SIDED, false>(&mapY, mp, &mapW, mp + 1, &mapY64, mp + 2, p, k, pl, act,
+                                                      Drow + t0, ks, rs, prod, lsum, pe);
     }
-    if (ok && act[0])
-      logP[P.logp_off + g] = (double)(logf(prod[0]) + lsum[0]) + (double)pe[0] * 0.69314718055994530942;
+    if (ok && act) logP[P.logp_off + g] = (double)(logf(prod) + lsum) + (double)pe * 0.69314718055994530942;
   }
-  stc_cta_release<1>(k);
+  stc_cta_release(k);
 }
 static const void* batch_tc_kernel(int periodize) {
   return periodize ? (const void*)k_batch_tc<SWEEP_PERIODIZE> : (const void*)k_batch_tc<0>;
 }
 
 // limits of all problems: original order (staged) -> factor order, float; validation
-__global__ void k_permute_batch(const double* a, const double* b, const int64_t* perm_g, int64_t total, float* a32,
-                                float* b32, int* bad) {
+// (and, per problem, whether a lower limit is finite: prob_of maps a position to its problem)
+__global__ void k_permute_batch(const double* a, const double* b, const int64_t* perm_g, const int32_t* prob_of,
+                                int64_t total, float* a32, float* b32, int* bad, int* two) {
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= total) return;
   const int64_t src = perm_g[t];  // global index into the staged limits
   const double av = a[src], bv = b[src];
   if (isnan(av) || isnan(bv) || av > bv || av == INFINITY || bv == -INFINITY) atomicExch(bad, 1);
+  if (av != -INFINITY) two[prob_of[t]] = 1;
   a32[t] = (float)av;
   b32[t] = (float)bv;
 }
@@ -424,6 +423,8 @@ struct Batch {
   double *logP = nullptr, *ell = nullptr, *out = nullptr, *a_st = nullptr, *b_st = nullptr;
   float *a32 = nullptr, *b32 = nullptr;
   int64_t* perm_g = nullptr;
+  int32_t* prob_of = nullptr;  // problem of each position
+  int* dtwo = nullptr;         // per problem: a finite lower limit (set by the limits' permutation)
   uint64_t* D = nullptr;
   double* h_ab = nullptr;   // pinned staging of the limits
   double* h_out = nullptr;  // pinned results
@@ -448,6 +449,8 @@ struct Batch {
     dfree(a32);
     dfree(b32);
     dfree(perm_g);
+    dfree(prob_of);
+    dfree(dtwo);
     dfree(D);
     if (h_ab) cudaFreeHost(h_ab);
     if (h_out) cudaFreeHost(h_out);
@@ -490,15 +493,17 @@ static int batch_capture(Batch& B, int per_sm) {
   TLR_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   cudaMemsetAsync(B.dbad, 0, sizeof(int), st);
   cudaMemsetAsync(B.dnext, 0, sizeof(int), st);
+  cudaMemsetAsync(B.dtwo, 0, B.count * sizeof(int), st);
   if (B.tc) cudaMemsetAsync(B.derr, 0, sizeof(int), st);
-  k_permute_batch<<<nblk(B.total_n, 256), 256, 0, st>>>(B.a_st, B.b_st, B.perm_g, B.total_n, B.a32, B.b32, B.dbad);
+  k_permute_batch<<<nblk(B.total_n, 256), 256, 0, st>>>(B.a_st, B.b_st, B.perm_g, B.prob_of, B.total_n, B.a32, B.b32,
+                                                        B.dbad, B.dtwo);
   if (B.tc) {
     if (B.periodize)
-      k_batch_tc<SWEEP_PERIODIZE><<<grid, STC_NS, sweep_tc_smem_bytes<1>(), st>>>(
+      k_batch_tc<SWEEP_PERIODIZE><<<grid, STC_NS, sweep_tc_smem_bytes(), st>>>(
           B.dtprobs, B.dmaps, B.ditems, B.n_items, B.dnext, B.mapW, B.mapY, B.mapY64, B.W16, B.kwmax, B.Y16, B.my,
           B.logP, B.derr);
     else
-      k_batch_tc<0><<<grid, STC_NS, sweep_tc_smem_bytes<1>(), st>>>(B.dtprobs, B.dmaps, B.ditems, B.n_items, B.dnext,
+      k_batch_tc<0><<<grid, STC_NS, sweep_tc_smem_bytes(), st>>>(B.dtprobs, B.dmaps, B.ditems, B.n_items, B.dnext,
                                                                  B.mapW, B.mapY, B.mapY64, B.W16, B.kwmax, B.Y16,
                                                                  B.my, B.logP, B.derr);
   } else {
@@ -555,7 +560,9 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
   std::vector<int64_t> perm_g(B.total_n);
   std::vector<int64_t> d_off(count + 1, 0);
   for (int p = 0; p < count; p++) d_off[p + 1] = d_off[p] + (int64_t)B.M * (B.F[p]->n + 1);
-  TLR_CHECK(dalloc(&B.D, (size_t)d_off[count]));
+  TLR_CHECK(dalloc(&B.dtwo, (size_t)count));
+  TLR_CHECK(dalloc(&B.D, (size_t)d_off[count] + STC_DPAD));  // (the sweep reads a few shifts past a problem's last)
+  TLR_CUDA(cudaMemsetAsync(B.D + d_off[count], 0, STC_DPAD * 8, st));
   TLR_CHECK(dalloc(&B.a32, (size_t)B.total_n));
   TLR_CHECK(dalloc(&B.b32, (size_t)B.total_n));
   {
@@ -606,6 +613,10 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
   TLR_CHECK(dalloc(&B.dprobs, count));
   TLR_CHECK(dalloc(&B.ditems, items.size()));
   TLR_CHECK(dalloc(&B.perm_g, (size_t)B.total_n));
+  TLR_CHECK(dalloc(&B.prob_of, (size_t)B.total_n));
+  std::vector<int32_t> prob_of(B.total_n);
+  for (int p = 0; p < count; p++) std::fill(prob_of.begin() + B.n_off[p], prob_of.begin() + B.n_off[p + 1], p);
+  TLR_CUDA(cudaMemcpyAsync(B.prob_of, prob_of.data(), prob_of.size() * 4, cudaMemcpyHostToDevice, st));
   TLR_CUDA(cudaMemcpyAsync(B.dprobs, probs.data(), probs.size() * sizeof(BatchProblem), cudaMemcpyHostToDevice, st));
   TLR_CUDA(cudaMemcpyAsync(B.ditems, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, st));
   TLR_CUDA(cudaMemcpyAsync(B.perm_g, perm_g.data(), perm_g.size() * 8, cudaMemcpyHostToDevice, st));
@@ -618,7 +629,7 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
     // resident CTAs from the kernel's registers and shared memory (the occupancy query
     // reported one CTA per SM for this kernel where the launches fit six), and at most
     // 512 / 64 per SM: each holds its 64 TMEM columns until the end
-    TLR_CHECK(resident_ctas(kt, STC_NS, sweep_tc_smem_bytes<1>(), B.device, &B.per_sm_max));
+    TLR_CHECK(resident_ctas(kt, STC_NS, sweep_tc_smem_bytes(), B.device, &B.per_sm_max));
     B.per_sm_max = std::min(B.per_sm_max, 512 / STC_SUB);
   } else {
     const size_t smem = batch_smem();
@@ -677,8 +688,8 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
       T.kcol_off = P.kcol_off;
       T.vmap16 = F.vmap16;
       T.BT = P.BT;
-      T.inv = P.inv;
-      T.band = P.band;
+      T.rec = F.rec32;
+      T.two = B.dtwo + p;
       T.Q = P.Q;
       T.D = P.D;
       T.a = P.a;

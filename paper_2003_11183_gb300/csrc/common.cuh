@@ -102,6 +102,8 @@ struct Factor {
   //   band32 r x m x 16: band32[(i*m + v)*16 + k] = B_i[v+1+k][v] for k < 15 and
   //         v+1+k < m, else 0 (each variable's window column, contiguous)
   float* band32 = nullptr;
+  //   rec32 r x m x 24: the whole-tile sweep's record of each variable (sweep_tc.cuh)
+  float* rec32 = nullptr;
   int64_t ldbt = 0;
   float* B32 = nullptr;
   float* U32 = nullptr;  // row tile i at u32_off[i]: (Krow_i rounded up to 8) x m, U_i transposed, zero rows
@@ -261,19 +263,43 @@ __device__ __forceinline__ double ndtri_lower(double p, double lp) {
   }
   return x;
 }
+// Approximate float32 functions of the hardware, subnormals flushed (their callers keep every argument and
+// result normal or treat the flush as zero); without .ftz each takes three more instructions.
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float lg2_ftz(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float mul_ftz(float x, float y) {
+  float z;
+  asm("mul.ftz.f32 %0, %1, %2;" : "=f"(z) : "f"(x), "f"(y));
+  return z;
+}
+__device__ __forceinline__ float rcp_ftz(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // float32 normal quantile, lower half.  Two regions:
-//  * p > 0.0017 (w = -log(4 p (1 - p)) < 5; all but about 1 in 300 calls):
-//    Phi^-1(p) = -sqrt(2) (1 - 2p) R(w), R(w) = erfinv(1 - 2p) / (1 - 2p) as a
-//    degree-8 polynomial in w - 2.5 (the variable of M. Giles, Approximating the
-//    erfinv function, GPU Computing Gems, 2011; coefficients from the library's
-//    own fit, csrc/fit_ndtri.py, relative error about 2.2e-7 in float32);
+//  * p > 8.4e-5 (L = log2(4 p (1 - p)) > -11.54; all but about 1 in 6,000 calls):
+//    Phi^-1(p) = (1 - 2p) S(L), S = -sqrt(2) erfinv(1 - 2p) / (1 - 2p) as a degree-11
+//    polynomial in L + 3 (the variable of M. Giles, Approximating the erfinv
+//    function, GPU Computing Gems, 2011, in the base of the hardware logarithm;
+//    coefficients from the library's own fit, csrc/fit_ndtri.py, relative error at most
+//    1.4e-7 and 4e-8 rms in float32), its even and odd halves evaluated side by side:
+//    half the dependent steps of Horner's rule;
 //  * below: Wichura's tail forms in t = sqrt(-log p) (M. J. Wichura, Algorithm AS
 //    241, Applied Statistics 37 (1988) 477-484, PPND7, coefficients as
 //    published: t <= 5 and t > 5), from log p, so that the quantile stays finite
 //    when p underflows (to log p = -700: relative error about 4e-7 in float32).
 // lp_tiny = log p is read only when p < 1e-30 (p may then be 0); above that the
-// log is taken here.  A warp takes the tail branch only when one of its lanes
-// falls there.
+// log is taken here.
 __device__ __forceinline__ float ndtri_tail_f32(float lp) {
   const float nl = fminf(fmaxf(-lp, 0.0f), 3.0e38f);
   const float t = nl * rsqrtf(fmaxf(nl, 1e-30f));  // sqrt(-log p)
@@ -290,22 +316,26 @@ __device__ __forceinline__ float ndtri_tail_f32(float lp) {
   const float den = fmaf(fmaf(1.2258202635e-02f, s, 2.4197894225e-01f), s, 1.0f);
   return -num / den;
 }
+constexpr float NDTRI_LMIN = -11.54f;  // the central region's lower end in L
+// S(L) from z = L + 3
+__device__ __forceinline__ float ndtri_poly_f32(float z) {
+  const float z2 = z * z;
+  float e = -3.801838705e-11f, o = -8.133700961e-13f;
+  e = fmaf(e, z2, -3.658852776e-09f);
+  o = fmaf(o, z2, -6.615116233e-10f);
+  e = fmaf(e, z2, 7.295904538e-07f);
+  o = fmaf(o, z2, 4.085940475e-08f);
+  e = fmaf(e, z2, -7.131514576e-05f);
+  o = fmaf(o, z2, 1.178657385e-06f);
+  e = fmaf(e, z2, 1.605706289e-03f);
+  o = fmaf(o, z2, -7.643549470e-04f);
+  e = fmaf(e, z2, -1.975718498e+00f);
+  o = fmaf(o, z2, 2.444996089e-01f);
+  return fmaf(o, z, e);
+}
 __device__ __forceinline__ float ndtri_f32(float p, float lp_tiny) {
-  const float w = -__logf(p * fmaf(-4.0f, p, 4.0f));  // -log(4 p (1 - p))
-  if (w < 5.0f) {
-    // -sqrt(2) R(w) (the fitted coefficients times -sqrt(2)), times x = 1 - 2p
-    const float z = w - 2.5f;
-    float r = -3.958320960e-08f;
-    r = fmaf(r, z, -4.851791005e-07f);
-    r = fmaf(r, z, 4.981194706e-06f);
-    r = fmaf(r, z, 6.207880233e-06f);
-    r = fmaf(r, z, -3.091151011e-04f);
-    r = fmaf(r, z, 1.773041789e-03f);
-    r = fmaf(r, z, 5.908129737e-03f);
-    r = fmaf(r, z, -3.488026857e-01f);
-    r = fmaf(r, z, -2.123313665e+00f);
-    return r * fmaf(-2.0f, p, 1.0f);
-  }
+  const float L = lg2_ftz(p * fmaf(-4.0f, p, 4.0f));
+  if (L > NDTRI_LMIN) return ndtri_poly_f32(L + 3.0f) * fmaf(-2.0f, p, 1.0f);
   return ndtri_tail_f32(p >= 1e-30f ? __logf(p) : lp_tiny);
 }
 // (the float overload used by the general step: lp = log p)

@@ -323,12 +323,33 @@ __global__ void k_make_band(const double* B, int m, int64_t count, float* band) 
   band[t] = (k < 15 && u < m) ? (float)B[(i * m + u) * m + v] : 0.0f;
 }
 
+// rec32[(i*m + v)*24 + k]: the whole-tile sweep's record of variable v of tile i (sweep_tc.cuh)
+__global__ void k_make_rec(const double* B, const uint64_t* Q, const int64_t* tile_off, int m, int64_t count, float* rec) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= count) return;
+  const int64_t row = t / STC_REC, i = row / m, v = row % m;
+  const int k = (int)(t % STC_REC);
+  const int mt = (int)(tile_off[i + 1] - tile_off[i]);
+  float x = 0.0f;
+  if (k < 16) {
+    const int64_t u = (v & 1) ? v + 1 + k : (k < 14 ? v + 2 + k : v + 1);
+    if (k < 15 && u < m) x = (float)B[(i * m + u) * m + v];
+  } else if (k == 18) {
+    x = (float)(1.0 / B[(i * m + v) * m + v]);
+  } else if (k == 20 || k == 21) {
+    const uint64_t q = v < mt ? Q[tile_off[i] + v] : 0;
+    x = __uint_as_float((uint32_t)(k == 20 ? q : q >> 32));
+  }
+  rec[t] = x;
+}
+
 int ensure_float_tiles(Factor& F, cudaStream_t st) {
-  if (F.B32 && F.BT32 && F.inv32 && F.band32) return TLRMVN_OK;
+  if (F.B32 && F.BT32 && F.inv32 && F.band32 && F.rec32) return TLRMVN_OK;
   dfree(F.B32);  // a failed earlier attempt may have left some of these behind
   dfree(F.BT32);
   dfree(F.inv32);
   dfree(F.band32);
+  dfree(F.rec32);
   const int64_t nb = (int64_t)F.r * F.m * F.m;
   TLR_CHECK(dalloc(&F.B32, nb));
   k_convert<double, float><<<blocks_for(nb, 256), 256, 0, st>>>(F.B, F.B32, nb);
@@ -341,6 +362,21 @@ int ensure_float_tiles(Factor& F, cudaStream_t st) {
   const int64_t nw = (int64_t)F.r * F.m * 16;
   TLR_CHECK(dalloc(&F.band32, nw));
   k_make_band<<<blocks_for(nw, 256), 256, 0, st>>>(F.B, F.m, nw, F.band32);
+  int64_t* dto = nullptr;
+  TLR_CHECK(dalloc(&dto, (size_t)F.r + 1));
+  const int64_t nr = (int64_t)F.r * F.m * STC_REC;
+  int s = dalloc(&F.rec32, nr);
+  cudaError_t e = cudaSuccess;
+  if (s == TLRMVN_OK) {
+    e = cudaMemcpyAsync(dto, F.tile_off.data(), (F.r + 1) * 8, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) {
+      k_make_rec<<<blocks_for(nr, 256), 256, 0, st>>>(F.B, F.Q, dto, F.m, nr, F.rec32);
+      e = cudaStreamSynchronize(st);
+    }
+  }
+  dfree(dto);
+  TLR_CHECK(s);
+  TLR_CUDA(e);
   TLR_CUDA(cudaGetLastError());
   return TLRMVN_OK;
 }
@@ -373,7 +409,7 @@ static bool fp16_ready(const Factor& F) {
 }
 static bool copies_ready(const Factor& F, int precision) {
   if (precision == TLRMVN_FP64) return true;
-  if (!F.B32 || !F.BT32 || !F.inv32 || !F.band32) return false;
+  if (!F.B32 || !F.BT32 || !F.inv32 || !F.band32 || !F.rec32) return false;
   if (precision == TLRMVN_FP32) return (F.U32 && F.V32) || F.ktot == 0;
   if (precision == TLRMVN_FP16_SHIFT) return fp16_ready(F);
   return bf16_ready(F);
@@ -793,28 +829,21 @@ static SweepShape sweep_shape(int64_t C, int mt, int forced) {
 // The whole-tile sweep of the BF16- and FP16-shift paths, by (periodisation,
 // one-sided) flags and operand type.
 typedef void (*SweepTcKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
-                              const CUtensorMap, const CUtensorMap, SweepTcArgs);
-static SweepTcKernel sweep_tc_kernel(int flags, bool f16, int spt) {
-  static const SweepTcKernel table[16] = {
-      k_sweep_tc<0, false, 1>, k_sweep_tc<SWEEP_PERIODIZE, false, 1>, k_sweep_tc<SWEEP_ONE_SIDED, false, 1>,
-      k_sweep_tc<SWEEP_PERIODIZE | SWEEP_ONE_SIDED, false, 1>, k_sweep_tc<0, true, 1>,
-      k_sweep_tc<SWEEP_PERIODIZE, true, 1>, k_sweep_tc<SWEEP_ONE_SIDED, true, 1>,
-      k_sweep_tc<SWEEP_PERIODIZE | SWEEP_ONE_SIDED, true, 1>, k_sweep_tc<0, false, 2>,
-      k_sweep_tc<SWEEP_PERIODIZE, false, 2>, k_sweep_tc<SWEEP_ONE_SIDED, false, 2>,
-      k_sweep_tc<SWEEP_PERIODIZE | SWEEP_ONE_SIDED, false, 2>, k_sweep_tc<0, true, 2>,
-      k_sweep_tc<SWEEP_PERIODIZE, true, 2>, k_sweep_tc<SWEEP_ONE_SIDED, true, 2>,
-      k_sweep_tc<SWEEP_PERIODIZE | SWEEP_ONE_SIDED, true, 2>};
-  return table[((flags & SWEEP_PERIODIZE) ? 1 : 0) | ((flags & SWEEP_ONE_SIDED) ? 2 : 0) | (f16 ? 4 : 0) |
-               (spt == 2 ? 8 : 0)];
+                              const CUtensorMap, const CUtensorMap, const SweepTcArgs, const SweepTcLaunch);
+static SweepTcKernel sweep_tc_kernel(int flags, bool f16) {
+  static const SweepTcKernel table[8] = {
+      k_sweep_tc<0, false>, k_sweep_tc<SWEEP_PERIODIZE, false>, k_sweep_tc<SWEEP_ONE_SIDED, false>,
+      k_sweep_tc<SWEEP_PERIODIZE | SWEEP_ONE_SIDED, false>, k_sweep_tc<0, true>,
+      k_sweep_tc<SWEEP_PERIODIZE, true>, k_sweep_tc<SWEEP_ONE_SIDED, true>,
+      k_sweep_tc<SWEEP_PERIODIZE | SWEEP_ONE_SIDED, true>};
+  return table[((flags & SWEEP_PERIODIZE) ? 1 : 0) | ((flags & SWEEP_ONE_SIDED) ? 2 : 0) | (f16 ? 4 : 0)];
 }
 // Dynamic shared memory of a whole-tile sweep launch with `ctas` CTAs per SM: the
-// kernel's own need, or more so that no more than `ctas` fit (tuning; with two
-// samples per thread at most four fit by TMEM, so the shared memory keeps it there).
-static size_t sweep_tc_launch_smem(int ctas, int spt) {
-  size_t need = spt == 2 ? sweep_tc_smem_bytes<2>() : sweep_tc_smem_bytes<1>();
-  const int cap_ctas = spt == 2 ? 4 : 6;
-  ctas = std::min(std::max(ctas, 1), cap_ctas);
-  if (ctas < cap_ctas || spt == 2) {
+// kernel's own need, or more so that no more than `ctas` fit (tuning).
+static size_t sweep_tc_launch_smem(int ctas) {
+  size_t need = sweep_tc_smem_bytes();
+  ctas = std::min(std::max(ctas, 1), 6);
+  if (ctas < 6) {
     int dev = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
@@ -827,12 +856,10 @@ static size_t sweep_tc_launch_smem(int ctas, int spt) {
 static int set_sweep_smem(int sub) {
   for (int flags = 0; flags < 8; flags++)
     TLR_CHECK(raise_smem_limit((const void*)sweep_kernel(flags), sweep_smem_bytes(sub, 256)));
-  for (int t = 0; t < 16; t++) {  // every (periodisation, one-sided, operand type, samples per thread) variant
-    const int spt = (t & 8) ? 2 : 1;
-    const void* kf = (const void*)sweep_tc_kernel(((t & 1) ? SWEEP_PERIODIZE : 0) | ((t & 2) ? SWEEP_ONE_SIDED : 0),
-                                                  (t & 4) != 0, spt);
-    TLR_CHECK(raise_smem_limit(kf, sweep_tc_launch_smem(1, spt)));
-  }
+  for (int t = 0; t < 8; t++)  // every (periodisation, one-sided, operand type) variant
+    TLR_CHECK(raise_smem_limit((const void*)sweep_tc_kernel(((t & 1) ? SWEEP_PERIODIZE : 0) |
+                                                                ((t & 2) ? SWEEP_ONE_SIDED : 0), (t & 4) != 0),
+                               sweep_tc_launch_smem(1)));
   return TLRMVN_OK;
 }
 
@@ -853,37 +880,18 @@ struct TcOperands {
 
 // Whole diagonal tile i on the BF16-shift path: one launch of k_sweep_tc
 // (low-rank shifts, in-tile coupling, sweep and projections).
-static void sweep_tile_tc(const Factor& F, int i, int64_t C, const Lims& L, const float* rs32, const uint64_t* dD,
+static void sweep_tile_tc(const Factor& F, int i, const Lims& L, const float* rs32, const uint64_t* dD,
                           int64_t c0, int64_t N, int64_t Cc, int periodize, unsigned short* Ys, int64_t ldys,
                           double* logP, const TcOperands& tco, const Tuning& tu, cudaStream_t st, Prof& pf) {
   const int m = F.m, mt = (int)F.tsize(i);
   SweepTcArgs t;
-  DiagArgs32& a = t.d;
-  a.BT = F.BT32 + (size_t)i * m * F.ldbt;
-  a.inv = F.inv32 + (size_t)i * m;
-  a.band = F.band32 + (size_t)i * m * 16;
-  a.mt = mt;
-  a.ldbt = F.ldbt;
-  a.Delta = nullptr;  // (the shifts are products of the kernel)
-  a.ldd = C;
-  a.a = L.a32 + F.tile_off[i];
-  a.b = L.b32 + F.tile_off[i];
-  a.rs = rs32;
-  a.Q = F.Q;
-  a.D = dD;
-  a.ldD = F.n + 1;
-  a.coord0 = F.tile_off[i];
-  a.sample0 = c0;
-  a.N = N;
-  a.C = Cc;
-  a.periodize = periodize;
-  a.first = (i == 0);
-  a.Yv = nullptr;
-  a.ldyv = 0;
-  a.Ys = reinterpret_cast<__nv_bfloat16*>(Ys);  // (16-bit words of the operand type)
-  a.ldys = ldys;
-  a.ys_lo = tco.my;
-  a.logP = logP;
+  t.rec = F.rec32 + (size_t)i * m * STC_REC;
+  t.BT = F.BT32 + (size_t)i * m * F.ldbt;
+  t.ldbt = F.ldbt;
+  t.mt = mt;
+  t.a = L.a32 + F.tile_off[i];
+  t.b = L.b32 + F.tile_off[i];
+  t.ys_lo = tco.my;
   t.brow0 = i * m;
   t.alo = (int)tco.my;
   t.blo = (int)tco.my;
@@ -892,18 +900,29 @@ static void sweep_tile_tc(const Factor& F, int i, int64_t C, const Lims& L, cons
   t.kr = (int)F.krow(i);
   t.kcol0 = (int)F.kcol_off[i];
   t.kc = (int)F.kcol(i);
-  t.W = tco.W;
   t.ldw = tco.ldw;
   t.vmap = F.vmap16 ? F.vmap16 + F.kcol_off[i] : nullptr;
   t.wscale = (tco.f16 && F.wscale16) ? F.wscale16 + F.kcol_off[i] : nullptr;
   t.tscale = tco.f16 ? F.inv_g16 : 1.0f;
   t.err = tco.err;
+  SweepTcLaunch d;
+  d.D = dD;
+  d.ldD = F.n + 1;
+  d.coord0 = F.tile_off[i];
+  d.sample0 = c0;
+  d.N = N;
+  d.C = Cc;
+  d.rs = rs32;
+  d.Ys = Ys;
+  d.ldys = ldys;
+  d.W = tco.W;
+  d.logP = logP;
+  d.first = (i == 0);
   const int flags = (periodize ? SWEEP_PERIODIZE : 0) | (L.one_sided ? SWEEP_ONE_SIDED : 0);
   pf.begin(TLRMVN_KC_DIAG);
-  const int spt = tu.spt == 2 ? 2 : 1;
-  launch_pdl(sweep_tc_kernel(flags, tco.f16, spt), dim3((unsigned)((Cc + STC_NS * spt - 1) / (STC_NS * spt))),
-             dim3(STC_NS), sweep_tc_launch_smem(tu.tc_ctas, spt), st, tco.mapY32, tco.mapB32, tco.mapW, tco.mapU64, tco.mapY64,
-             tco.mapV64, t);
+  launch_pdl(sweep_tc_kernel(flags, tco.f16), dim3((unsigned)((Cc + STC_NS - 1) / STC_NS)), dim3(STC_NS),
+             sweep_tc_launch_smem(tu.tc_ctas), st, tco.mapY32, tco.mapB32, tco.mapW, tco.mapU64, tco.mapY64, tco.mapV64, t,
+             d);
   pf.end();
 }
 
@@ -1137,7 +1156,7 @@ static int run_chunks_bf16(Factor& F, const Lims& L, double nu, const tlrmvn_opt
       pf.end();
     }
     for (int i = 0; i < F.r; i++)
-      sweep_tile_tc(F, i, C, L, rs32, dD, c0, N, Cc, o.periodize, Y, ly, logP, tco, tu, st, pf);
+      sweep_tile_tc(F, i, L, rs32, dD, c0, N, Cc, o.periodize, Y, ly, logP, tco, tu, st, pf);
     TLR_CUDA(cudaGetLastError());
   }
   int herr = 0;
@@ -1152,7 +1171,7 @@ static int run_chunks_bf16(Factor& F, const Lims& L, double nu, const tlrmvn_opt
 int64_t prob_scratch_bytes(const Factor& F, const tlrmvn_opts& o) {
   const int64_t M = o.n_shifts, N = o.n_points, S = M * N, n = F.n, m = F.m;
   const Tuning tu = F.tuning(o.precision);
-  int64_t bytes = n * (8 * 2 + 4 * 2) + M * (n + 1) * 8 + M * 8 + S * 8 + 256;
+  int64_t bytes = n * (8 * 2 + 4 * 2) + (M * (n + 1) + STC_DPAD) * 8 + M * 8 + S * 8 + 256;
   if (o.precision == TLRMVN_BF16_SHIFT || o.precision == TLRMVN_FP16_SHIFT) {
     int64_t kw = 0;
     for (int i = 0; i < F.r; i++) kw += (F.krow(i) + 63) / 64 * 64;
@@ -1183,7 +1202,7 @@ int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, co
     TLR_CHECK(sc.get(&bp32, n));
   }
   TLR_CHECK(sc.get(&bad, 2));  // invalid limits; a finite lower limit
-  TLR_CHECK(sc.get(&dD, (size_t)M * (n + 1)));
+  TLR_CHECK(sc.get(&dD, (size_t)M * (n + 1) + STC_DPAD));
   TLR_CHECK(sc.get(&ell, M));
   if (per_sample_dev) logP = per_sample_dev;
   else TLR_CHECK(sc.get(&logP, S));

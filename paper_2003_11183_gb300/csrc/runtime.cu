@@ -107,6 +107,7 @@ Factor::~Factor() {
   dfree(BT32);
   dfree(inv32);
   dfree(band32);
+  dfree(rec32);
   dfree(U32);
   dfree(V32);
   dfree(U16);

@@ -77,8 +77,8 @@ __device__ inline double gamma_p_inv(double a, double p, double q) {
 // ---- float32 integrand helpers ------------------------------------------------------
 // Lattice value as floats for the float32 integrands: the cell midpoint of the
 // point's top 32 bits, (h + 1/2) / 2^32 with h = x >> 32, through the tent map
-// when periodised, |2 (h + 1/2) / 2^32 - 1| = (2a + 1) / 2^32 with a = d ^ (d >> 31)
-// and d = h - 2^31 as a signed 32-bit integer (|2d + 1| = 2a + 1).  Integer
+// when periodised, w = |2 (h + 1/2) / 2^32 - 1| = |2 d + 1| / 2^32 with d = h - 2^31, and
+// 1 - w = |2 h' + 1| / 2^32 with h' = h read as a signed integer.  Integer
 // arithmetic and two 32-bit conversions only (the float path issues no float64
 // instruction).  It differs from the exact value of the 53-bit definition
 // (lattice_w) by at most 2^-32 (2^-33 without the tent map): within half a
@@ -86,10 +86,8 @@ __device__ inline double gamma_p_inv(double a, double p, double q) {
 __device__ __forceinline__ void lattice_wf(uint64_t x, int periodize, float& w, float& wc) {
   const uint32_t h = (uint32_t)(x >> 32);
   if (periodize) {
-    const int32_t d = (int32_t)(h ^ 0x80000000u);
-    const uint32_t a = (uint32_t)(d ^ (d >> 31));  // in [0, 2^31)
-    w = fmaf((float)a, 4.656612873077393e-10f, 2.3283064365386963e-10f);                   // (2a + 1) / 2^32
-    wc = fmaf((float)(0x7FFFFFFFu - a), 4.656612873077393e-10f, 2.3283064365386963e-10f);  // 1 - w
+    w = fabsf(fmaf((float)(int32_t)(h ^ 0x80000000u), 4.656612873077393e-10f, 2.3283064365386963e-10f));
+    wc = fabsf(fmaf((float)(int32_t)h, 4.656612873077393e-10f, 2.3283064365386963e-10f));
   } else {
     w = fmaf((float)h, 2.3283064365386963e-10f, 1.1641532182693481e-10f);                  // (h + 1/2) / 2^32
     wc = fmaf((float)(0xFFFFFFFFu - h), 2.3283064365386963e-10f, 1.1641532182693481e-10f);
@@ -136,73 +134,97 @@ __device__ __forceinline__ void sov_step_f32(float at, float bt, float w, float 
   sov_step<float>(at, bt, w, wc, ld, y);
 }
 
-// Phi(-x) for x >= 0 in float32 (relative error about 1e-7 on [0, 12]; beyond
-// 12 the value is below 2e-33 and only needs to be small): phi(x) R(x), with R
-// the Mills ratio fitted as a degree-10 polynomial in t = 3 / (3 + x)
-// (coefficients from csrc/fit_mills.py), and exp(-x^2/2) taken from
-// x = xh + xl, xh the leading 12 significant bits of x, so that xh^2 is exact:
-// exp(-xh^2/2) exp(-xl (x + xh)/2).  Cheaper than 0.5 erfcf(x / sqrt 2).
+// Phi(-x) in float32 for x >= 0 (zero beyond 13, where it falls below the normal floats), straight-line:
+// exp(-x^2/2) R(x), with R half the scaled complementary error function as a degree-9 polynomial in
+// 1 / (2.5 + x) (coefficients from csrc/fit_mills.py; its even and odd halves side by side), and the
+// exponential from x^2 in two parts, x^2 + er exactly: -(x^2 + er) log2(e)/2 = n + f with n the nearest
+// integer, 2^f by the hardware and 2^n added to the exponent.  Relative error about 3e-7 at most.
 __device__ __forceinline__ float phi_neg_f32(float x) {
-  const float xh = __int_as_float(__float_as_int(x) & 0xFFFFF000);
-  const float xl = x - xh;
-  const float e1 = expf(-0.5f * (xh * xh));
-  const float e2 = __expf(-0.5f * (xl * (x + xh)));
-  const float t = __fdividef(3.0f, 3.0f + fminf(x, 12.5f));
-  float r = 2.330137213e-04f;
-  r = fmaf(r, t, -7.265756279e-02f);
-  r = fmaf(r, t, 3.999014199e-01f);
-  r = fmaf(r, t, -8.397881985e-01f);
-  r = fmaf(r, t, 7.416802049e-01f);
-  r = fmaf(r, t, -2.781317532e-01f);
-  r = fmaf(r, t, 3.698102236e-01f);
-  r = fmaf(r, t, 2.605797350e-01f);
-  r = fmaf(r, t, 3.388197124e-01f);
-  r = fmaf(r, t, 3.328486085e-01f);
-  r = fmaf(r, t, 1.874211193e-05f);
-  return (e1 * e2) * (0.3989422804014327f * r);
+  x = fminf(x, 13.0f);
+  const float x2 = x * x, er = fmaf(x, x, -x2);
+  const float kf = fmaf(x2, -7.213475108e-01f, 12582912.0f);  // the integer n in the low bits
+  float f = fmaf(x2, -7.213475108e-01f, 12582912.0f - kf);
+  f = fmaf(x2, -9.629815168e-09f, f);
+  f = fmaf(er, -7.213475108e-01f, f);
+  const float e = __int_as_float(__float_as_int(ex2_ftz(f)) + (__float_as_int(kf) << 23));
+  const float t = rcp_ftz(x + 2.5f), t2 = t * t;
+  float p = -6.734211731e+01f, q = 3.024349689e+00f;
+  p = fmaf(p, t2, -9.483559418e+01f);
+  q = fmaf(q, t2, 1.291362152e+02f);
+  p = fmaf(p, t2, -7.301989794e-01f);
+  q = fmaf(q, t2, 2.569419479e+01f);
+  p = fmaf(p, t2, 9.710934162e-01f);
+  q = fmaf(q, t2, 2.507573128e+00f);
+  p = fmaf(p, t2, -1.405569856e-05f);
+  q = fmaf(q, t2, 3.998731673e-01f);
+  return mul_ftz(e, fmaf(q, t, p));
 }
 
 // The same step for a caller that keeps the sample's probability as a running
-// product: returns y, a factor f to multiply into the product and a log la to
-// add to a separate sum (the step's probability is f exp(la)).  The one-sided
-// fast path returns f = Phi(bt), except when 1 - Phi(bt) = c < 2^-12, where
-// fl(1 - c) would lose c's digits and the step returns la = log1p(-c) taken as
-// -c - c^2/2 (the next term is below 2^-24 c); the deep tail and two-sided
-// intervals return their log.  No log is evaluated on the fast path.
-// sov_step_f32_upper is the one-sided (at = -inf) case on its own.
-__device__ __forceinline__ void sov_step_f32_upper(float bt, float w, float wc, float& f, float& la, float& y) {
-  if (bt != INFINITY && bt >= -12.0f) {
-    const float h = phi_neg_f32(fabsf(bt));  // Phi(-|bt|)
-    const bool neg = bt < 0.0f;
-    const float ph = neg ? h : 1.0f - h;  // Phi(bt)
-    const float pc = neg ? 1.0f - h : h;  // 1 - Phi(bt)
-    const bool near1 = !neg && pc < 0x1p-12f;
-    f = near1 ? 1.0f : ph;
-    la = near1 ? -pc * fmaf(0.5f, pc, 1.0f) : 0.0f;
-    const float u = w * ph, uc = pc + wc * ph;  // u + uc = 1
-    const bool lower = u <= uc;
-    const float pp = lower ? u : uc;
-    float lpp = 0.0f;
-    if (pp < 1e-30f) lpp = logf(w) + logf(ph);  // (u underflows; here ph < 1/2, so log Phi(bt) = log ph)
-    const float z = ndtri_f32(pp, lpp);
-    y = lower ? z : -z;
-    return;
-  }
-  float ld;
-  sov_step_f32(-INFINITY, bt, w, wc, ld, y);
-  f = 1.0f;
-  la = ld;
-}
-__device__ __forceinline__ void sov_step_f32_prod(float at, float bt, float w, float wc, float& f, float& la,
-                                                  float& y) {
-  if (at == -INFINITY) {
-    sov_step_f32_upper(bt, w, wc, f, la, y);
-    return;
-  }
-  float ld;
+// product: returns y, a factor f to multiply into the product and a log added to
+// the separate sum lsum.  The fast path's factor is the probability, except when its
+// complement c is below 3e-4, where fl(1 - c) would lose c's digits: then f = 1 and
+// log1p(-c) is added as -c - c^2/2 (the next term is below 4e-8 c).  f is at least
+// 2.5e-19, so that a caller may multiply two into a product in [1, 2).
+//
+// The fast path is straight-line code for every lane, and one branch follows for
+// the lanes it does not serve (limits in the deep tail; a quantile below 8.4e-5, a
+// lane in 6,000): the chain from a variable's sum to its y is what bounds the
+// sweeps, and branches cut it (the one-sided case, the quantile's tail when that
+// started at 0.0017 and one warp in ten took it, the underflow test) and keep the compiler from
+// filling its waits.  With u = Phi(at) + w (Phi(bt) - Phi(at)) and uc = 1 - u both accurate, the
+// quantile takes 4 p (1 - p) = 4 u uc and 1 - 2p = +-(uc - u) from them directly: no
+// minimum, comparison or select on the way to y.
+
+// (y, the step's log) of a lane off the fast path
+static __device__ __noinline__ float2 sov_step_rare_f32(float at, float bt, float w, float wc, float pp, bool deep) {
+  if (!deep) return make_float2(ndtri_tail_f32(__logf(pp)), 0.0f);
+  float ld, y;
   sov_step_f32(at, bt, w, wc, ld, y);
-  f = 1.0f;
-  la = ld;
+  return make_float2(y, ld);
+}
+
+// The one-sided (at = -inf) case.
+__device__ __forceinline__ void sov_step_f32_upper(float bt, float w, float wc, float& f, float& lsum, float& y) {
+  const float h = phi_neg_f32(fabsf(bt)), m = 1.0f - h;  // Phi(-|bt|), Phi(|bt|)
+  const bool neg = bt < 0.0f, near1 = bt > 3.5f;
+  const float ph = neg ? h : m, pc = neg ? m : h;  // Phi(bt), 1 - Phi(bt)
+  const float c = near1 ? h : 0.0f;
+  f = near1 ? 1.0f : ph;
+  lsum = fmaf(-c, fmaf(0.5f, c, 1.0f), lsum);
+  const float u = w * ph, uc = fmaf(wc, ph, pc);
+  const float L = lg2_ftz(u * uc);  // log2(4 u uc) - 2
+  y = ndtri_poly_f32(L + 5.0f) * (uc - u);
+  if (L < NDTRI_LMIN - 2.0f) {
+    // (a deep limit always comes here: u < Phi(-8.9) = 2.8e-19; above it pp > 3e-29)
+    const bool deep = bt < -8.9f;
+    const float2 r = sov_step_rare_f32(-INFINITY, bt, w, wc, fminf(u, uc), deep);
+    y = (deep || u <= uc) ? r.x : -r.x;
+    f = deep ? 1.0f : f;
+    lsum += r.y;
+  }
+}
+
+// Any interval.  With both limits on one side of 0 the probability is the difference of the two smaller tails.
+__device__ __forceinline__ void sov_step_f32_prod(float at, float bt, float w, float wc, float& f, float& lsum,
+                                                  float& y) {
+  const float ha = phi_neg_f32(fabsf(at)), hb = phi_neg_f32(fabsf(bt)), ma = 1.0f - ha;
+  const bool na = at < 0.0f, nb = bt < 0.0f, near1 = fminf(-at, bt) > 3.6f;
+  const float d = na ? ha : ma, ec = nb ? 1.0f - hb : hb;  // Phi(at), 1 - Phi(bt)
+  const float diff = nb ? hb - ha : (na ? ma - hb : ha - hb);
+  const float c = near1 ? ha + hb : 0.0f;
+  f = near1 ? 1.0f : diff;
+  lsum = fmaf(-c, fmaf(0.5f, c, 1.0f), lsum);
+  const float u = fmaf(w, diff, d), uc = fmaf(wc, diff, ec);
+  const float L = lg2_ftz(u * uc);
+  y = ndtri_poly_f32(L + 5.0f) * (uc - u);
+  const bool deep = !(diff >= 2.5e-19f);  // (also a zero-width interval and, through the comparison, a NaN)
+  if (deep || L < NDTRI_LMIN - 2.0f) {
+    const float2 r = sov_step_rare_f32(at, bt, w, wc, fminf(u, uc), deep);
+    y = (deep || u <= uc) ? r.x : -r.x;
+    f = deep ? 1.0f : f;
+    lsum += r.y;
+  }
 }
 
 }  // namespace tlrmvn

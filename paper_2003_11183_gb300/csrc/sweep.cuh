@@ -181,14 +181,13 @@ __global__ void k_diag_f32(DiagArgs32 p) {
         const float bt = (bv * rs[s] - sum[s]) * iv;
         float w, wc;
         lattice_wf((uint64_t)ks[s] * qv + dv, PER ? 1 : 0, w, wc);
-        float f, la;
+        float f;
         if (ONE) {
-          sov_step_f32_upper(bt, w, wc, f, la, y[s]);
+          sov_step_f32_upper(bt, w, wc, f, lsum[s], y[s]);
         } else {
           const float at = (av * rs[s] - sum[s]) * iv;
-          sov_step_f32_prod(at, bt, w, wc, f, la, y[s]);
+          sov_step_f32_prod(at, bt, w, wc, f, lsum[s], y[s]);
         }
-        lsum[s] += la;
         prod[s] *= f;  // prod in [1, 2) and f >= Phi(-12): a normal float
         const int pb = __float_as_int(prod[s]);
         pe[s] += (pb >> 23) - 127;

@@ -44,16 +44,12 @@ static std::string tune_key(const Factor& F, int precision, int64_t S, bool mvt)
 static std::vector<Tuning> candidates(const Factor& F, int precision, int64_t S) {
   std::vector<Tuning> c;
   if (precision == TLRMVN_BF16_SHIFT || precision == TLRMVN_FP16_SHIFT) {
-    for (int spt : {1, 2})
-      for (int ctas : {6, 4}) {
-        if (spt == 2 && ctas > 4) continue;  // (two samples per thread: at most four CTAs per SM)
-        for (int64_t chunk : {(int64_t)0, (S / 2 + 255) / 256 * 256}) {
-          Tuning t;
-          t.tc_ctas = ctas;
-          t.chunk = chunk;
-          t.spt = spt;
-          c.push_back(t);
-        }
+    for (int ctas : {6, 4})
+      for (int64_t chunk : {(int64_t)0, (S / 2 + 255) / 256 * 256}) {
+        Tuning t;
+        t.tc_ctas = ctas;
+        t.chunk = chunk;
+        c.push_back(t);
       }
   } else if (precision == TLRMVN_FP32) {
     for (int sub : {64, 128})
