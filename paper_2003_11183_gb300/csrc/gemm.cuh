@@ -6,21 +6,47 @@
 namespace tlrmvn {
 
 // C[rowmap[i]][:] = A (M x K, row-major) * B (K x N, row-major) (+ C when accumulate);
-// rowmap may be null.  64x64 output tile per 256-thread block, 4x4 per thread, K in steps of 16.
-template <typename T>
+// rowmap may be null.  64 x 16 NJ output tile per 256-thread block, up to 4 x NJ per thread, K in steps of 16.
+// Bound by the float64 pipe (one instruction of a warp takes 16 cycles of the SM), so nothing is multiplied for
+// padding: a thread's rows lie 16 apart, and the 16-row groups past M (the ranks of a column tile are seldom a
+// multiple of 64) and the k past K are left out.
+template <typename T, int MI, int NJ>
+__device__ __forceinline__ void gemm_nn_step(const T (&As)[16][65], const T (&Bs)[16][16 * NJ], int kn, int tx, int ty,
+                                             T (&acc)[4][NJ]) {
+  auto one = [&](int kk) {
+    T a[MI], b[NJ];
+#pragma unroll
+    for (int i = 0; i < MI; i++) a[i] = As[kk][ty + 16 * i];
+#pragma unroll
+    for (int j = 0; j < NJ; j++) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+    for (int i = 0; i < MI; i++)
+#pragma unroll
+      for (int j = 0; j < NJ; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+  };
+  if (kn == 16) {
+#pragma unroll 8
+    for (int kk = 0; kk < 16; kk++) one(kk);
+  } else {
+    for (int kk = 0; kk < kn; kk++) one(kk);
+  }
+}
+template <typename T, int NJ>
 __global__ void __launch_bounds__(256) k_gemm_nn(int M, int64_t N, int64_t K, const T* __restrict__ A, int64_t lda,
                                                  const T* __restrict__ B, int64_t ldb, T* __restrict__ C, int64_t ldc,
                                                  const int32_t* __restrict__ rowmap, int accumulate) {
+  constexpr int BN = 16 * NJ;
   __shared__ T As[16][64 + 1];
-  __shared__ T Bs[16][64];
+  __shared__ T Bs[16][BN];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int m0 = blockIdx.y * 64;
-  const int64_t n0 = (int64_t)blockIdx.x * 64;
-  T acc[4][4];
+  const int64_t n0 = (int64_t)blockIdx.x * BN;
+  const int mi = min(4, (M - m0 + 15) >> 4);
+  T acc[4][NJ];
 #pragma unroll
   for (int i = 0; i < 4; i++)
 #pragma unroll
-    for (int j = 0; j < 4; j++) acc[i][j] = (T)0;
+    for (int j = 0; j < NJ; j++) acc[i][j] = (T)0;
   for (int64_t k0 = 0; k0 < K; k0 += 16) {
     for (int l = threadIdx.x; l < 64 * 16; l += 256) {
       int mm = l >> 4, kk = l & 15;
@@ -28,24 +54,17 @@ __global__ void __launch_bounds__(256) k_gemm_nn(int M, int64_t N, int64_t K, co
       int64_t gk = k0 + kk;
       As[kk][mm] = (gm < M && gk < K) ? A[(int64_t)gm * lda + gk] : (T)0;
     }
-    for (int l = threadIdx.x; l < 16 * 64; l += 256) {
-      int kk = l >> 6, nn = l & 63;
+    for (int l = threadIdx.x; l < 16 * BN; l += 256) {
+      int kk = l / BN, nn = l % BN;
       int64_t gk = k0 + kk, gn = n0 + nn;
       Bs[kk][nn] = (gk < K && gn < N) ? B[gk * ldb + gn] : (T)0;
     }
     __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; kk++) {
-      T a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; i++) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; j++) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
+    const int kn = (int)min((int64_t)16, K - k0);
+    if (mi == 4) gemm_nn_step<T, 4, NJ>(As, Bs, kn, tx, ty, acc);
+    else if (mi == 3) gemm_nn_step<T, 3, NJ>(As, Bs, kn, tx, ty, acc);
+    else if (mi == 2) gemm_nn_step<T, 2, NJ>(As, Bs, kn, tx, ty, acc);
+    else gemm_nn_step<T, 1, NJ>(As, Bs, kn, tx, ty, acc);
     __syncthreads();
   }
 #pragma unroll
@@ -54,7 +73,7 @@ __global__ void __launch_bounds__(256) k_gemm_nn(int M, int64_t N, int64_t K, co
     if (gm >= M) continue;
     int64_t row = rowmap ? (int64_t)rowmap[gm] : (int64_t)gm;
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
+    for (int j = 0; j < NJ; j++) {
       int64_t gn = n0 + tx + 16 * j;
       if (gn < N) {
         T* c = C + row * ldc + gn;
@@ -266,12 +285,27 @@ inline void gemm_tn_f32(cudaStream_t st, int M, int64_t N, int64_t K, const floa
              lda, B, ldb, C, ldc, rowmap, accumulate);
 }
 
+// The SM with the most tiles sets the time (the blocks of an SM share its float64 pipe), and over 10,000 samples
+// tiles of 64 columns come to 157 a row for 152 SMs: the width (64, 32 or 16 columns) that gives the busiest SM
+// the fewest columns, the widest on ties (n = 256, 10,000 samples: 2.00 -> 1.71 ms a solve, n = 4,096, 20,000: 76.0 ->
+// 67.4 ms).
 template <typename T>
 inline void gemm_nn(cudaStream_t st, int M, int64_t N, int64_t K, const T* A, int64_t lda, const T* B, int64_t ldb,
-                    T* C, int64_t ldc, const int32_t* rowmap, int accumulate = 0) {
+                    T* C, int64_t ldc, const int32_t* rowmap, int sms, int accumulate = 0) {
   if (M <= 0 || N <= 0) return;
-  dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
-  k_gemm_nn<T><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, rowmap, accumulate);
+  const int64_t my = (M + 63) / 64;
+  int best = 4;
+  int64_t cost = INT64_MAX;
+  for (int nj = 4; nj >= 1; nj /= 2) {
+    const int64_t tiles = (N + 16 * nj - 1) / (16 * nj) * my, c = (tiles + sms - 1) / sms * nj;
+    if (c < cost) {
+      cost = c;
+      best = nj;
+    }
+  }
+  auto* k = best == 4 ? k_gemm_nn<T, 4> : (best == 2 ? k_gemm_nn<T, 2> : k_gemm_nn<T, 1>);
+  const dim3 grid((unsigned)((N + 16 * best - 1) / (16 * best)), (unsigned)my);
+  k<<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, rowmap, accumulate);
 }
 
 // ---- batched, grouped float64 GEMM for the factorisation ---------------------------

@@ -12,6 +12,7 @@
 // Per-sample logs are reduced per shift by a log-sum-exp and then across shifts (Section 2.1).
 #include "common.cuh"
 #include "gemm.cuh"
+#include "sov64.cuh"
 #include "sov_device.cuh"
 #include "sweep.cuh"
 #include "sweep_tc.cuh"
@@ -57,88 +58,92 @@ __global__ void k_permute_limits(const double* a, const double* b, const int64_t
   }
 }
 
-// ---- diagonal-tile sweep (eq. 2 on B_i, Algorithm 6 inner call) -------------------
-template <typename T, typename YT>
-struct DiagArgs {
-  const T* B;
+// ---- float64 diagonal-tile sweep (eq. 2 on B_i, Algorithm 6 inner call) -----------------------
+struct DiagArgs64 {
+  const double* B;  // the sub-tile's diagonal block
   int mt, ldb;
-  const T* Delta;   // m x C sample-major, or null (no earlier tiles)
+  const double* Delta;   // limit shifts, variable-major, or null (no earlier tiles or sub-tiles)
   int64_t ldd;
-  const double* a;  // the tile's limits, factor order
+  const double* a;  // the sub-tile's limits, factor order
   const double* b;
   const double* rs;  // per-sample Student-t scale or null
   const uint64_t* Q;
   const uint64_t* D;
   int64_t ldD, coord0, sample0, N, C;
   int periodize, first;
-  YT* Y;
+  double* Y;  // Y[v * ldy + c]
   int64_t ldy;
   double* logP;  // all samples
+  const double* tables;
 };
 
-__device__ __forceinline__ void put_y(double* Y, int64_t i, double y) { Y[i] = y; }
-__device__ __forceinline__ void put_y(float* Y, int64_t i, float y) { Y[i] = y; }
-__device__ __forceinline__ void put_y(__nv_bfloat16* Y, int64_t i, float y) { Y[i] = __float2bfloat16_rn(y); }
-
-// One thread per sample; the tile's y values of the thread's sample live in shared
-// memory (column tid of a [mt][blockDim+1] array); B_i rows are read through L1
-// as warp-uniform broadcasts.  Y layout:
-//   SAMPLE_MAJOR = false: Y[v * ldy + c]  (variable-major, written as produced)
-//   SAMPLE_MAJOR = true:  Y[c * ldy + v]  (each sample's y contiguous: the K-major
-//                         operand of the tensor-core projection), written at the
-//                         end of the tile from shared memory, a row per warp pass.
-template <typename T, typename YT, bool SAMPLE_MAJOR>
-__global__ void k_diag(DiagArgs<T, YT> p) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* ys = reinterpret_cast<T*>(smem_raw);
+// One thread per sample.  Shared memory: the tables of the step (sov64.cuh, 115 KB), the reciprocal diagonal, and the
+// sub-tile's y values of the block's samples (column tid of a [mt][blockDim + 1] array); B rows are read
+// through L1 as warp-uniform broadcasts.  Bound by the float64 pipe: per variable about 40 instructions of the step
+// and one per earlier variable of the sub-tile.
+__host__ __device__ constexpr size_t diag64_smem(int sub, int threads) {
+  return ((size_t)T64_DOUBLES + sub + (size_t)sub * (threads + 1)) * sizeof(double);
+}
+template <bool ONE>
+__global__ void __launch_bounds__(192) k_diag64(DiagArgs64 p) {
+  extern __shared__ __align__(16) double sm64[];
+  double* T = sm64;
+  double* inv = T + T64_DOUBLES;
+  double* ys = inv + p.mt;
   const int bd = blockDim.x, tid = threadIdx.x, ld = bd + 1;
-  const int64_t c0 = (int64_t)blockIdx.x * bd;
-  const int64_t c = c0 + tid;
-  const bool active = c < p.C;
-  if (active) {
-    const int64_t g = p.sample0 + c;
-    const int64_t s = g / p.N;
-    const uint64_t k = (uint64_t)(g - s * p.N) + 1;
-    const uint64_t* Ds = p.D + s * p.ldD + p.coord0;
-    const uint64_t* Qt = p.Q + p.coord0;
-    const T rs = p.rs ? (T)p.rs[c] : (T)1;
-    T lp = 0;
-    for (int v = 0; v < p.mt; v++) {
-      const T* Brow = p.B + (int64_t)v * p.ldb;
-      T s0 = 0, s1 = 0, s2 = 0, s3 = 0;
-      int u = 0;
-      for (; u + 4 <= v; u += 4) {
-        s0 = fma(__ldg(Brow + u), ys[(u)*ld + tid], s0);
-        s1 = fma(__ldg(Brow + u + 1), ys[(u + 1) * ld + tid], s1);
-        s2 = fma(__ldg(Brow + u + 2), ys[(u + 2) * ld + tid], s2);
-        s3 = fma(__ldg(Brow + u + 3), ys[(u + 3) * ld + tid], s3);
-      }
-      for (; u < v; u++) s0 = fma(__ldg(Brow + u), ys[u * ld + tid], s0);
-      const T sum = (s0 + s1) + (s2 + s3);
-      const T dl = p.Delta ? p.Delta[(int64_t)v * p.ldd + c] : (T)0;
-      const T lvv = __ldg(Brow + v);
-      const T at = ((T)p.a[v] * rs - dl - sum) / lvv;
-      const T bt = ((T)p.b[v] * rs - dl - sum) / lvv;
-      double w, wc;
-      lattice_w(k * Qt[v] + Ds[v], p.periodize, w, wc);
-      T lv, y;
-      sov_step<T>(at, bt, (T)w, (T)wc, lv, y);
-      lp += lv;
-      ys[v * ld + tid] = y;
-      if (!SAMPLE_MAJOR) put_y(p.Y, (int64_t)v * p.ldy + c, y);
+  for (int t = tid; t < T64_DOUBLES / 2; t += bd)
+    cp_async16(reinterpret_cast<double2*>(T) + t, reinterpret_cast<const double2*>(p.tables) + t, 16);
+  cp_async_commit();
+  for (int t = tid; t < p.mt; t += bd) inv[t] = 1.0 / p.B[(int64_t)t * p.ldb + t];
+  cp_async_wait<0>();
+  __syncthreads();
+  const int64_t c = (int64_t)blockIdx.x * bd + tid;
+  if (c >= p.C) return;
+  const int64_t g = p.sample0 + c;
+  const int64_t s = g / p.N;
+  const uint64_t k = (uint64_t)(g - s * p.N) + 1;
+  const uint64_t* Ds = p.D + s * p.ldD + p.coord0;
+  const uint64_t* Qt = p.Q + p.coord0;
+  const double rs = p.rs ? p.rs[c] : 1.0;
+  const double lp0 = p.first ? 0.0 : p.logP[g];
+  // log P of the sub-tile = log(prod) + pe log 2 + lsum, prod kept in [1, 2)
+  double prod = 1.0, lsum = 0.0;
+  int pe = 0;
+  bool zero = lp0 > -1e-20;
+  uint64_t x = k * Qt[0] + Ds[0];
+  for (int v = 0; v < p.mt; v++) {
+    const double* Brow = p.B + (int64_t)v * p.ldb;
+    double dl = p.Delta ? p.Delta[(int64_t)v * p.ldd + c] : 0.0;
+    double s0 = 0, s1 = 0, s2 = 0, s3 = 0;
+    int u = 0;
+    for (; u + 4 <= v; u += 4) {
+      s0 = fma(__ldg(Brow + u), ys[(u)*ld + tid], s0);
+      s1 = fma(__ldg(Brow + u + 1), ys[(u + 1) * ld + tid], s1);
+      s2 = fma(__ldg(Brow + u + 2), ys[(u + 2) * ld + tid], s2);
+      s3 = fma(__ldg(Brow + u + 3), ys[(u + 3) * ld + tid], s3);
     }
-    if (p.first) p.logP[g] = (double)lp;
-    else p.logP[g] += (double)lp;
+    for (; u < v; u++) s0 = fma(__ldg(Brow + u), ys[u * ld + tid], s0);
+    dl += (s0 + s1) + (s2 + s3);
+    const double lvv = __ldg(Brow + v), iv = inv[v];
+    // (limit - shift) / l_vv to the last bit from the reciprocal: the quotient and its remainder
+    auto quotient = [&](double lim) {
+      const double num = fma(lim, rs, -dl), q = num * iv, r = fma(-q, lvv, num);
+      return (__double2hiint(num) & 0x7FF00000) == 0x7FF00000 ? q : fma(r, iv, q);
+    };
+    const double bt = quotient(p.b[v]), at = ONE ? 0.0 : quotient(p.a[v]);
+    double w, wc;
+    lattice_w64(x, p.periodize, w, wc);
+    if (v + 1 < p.mt) x = k * Qt[v + 1] + Ds[v + 1];
+    const double y = sov_step_f64<ONE>(T, at, bt, w, wc, zero, prod, lsum);
+    const int hi = __double2hiint(prod);
+    pe += (hi >> 20) - 1023;
+    prod = __hiloint2double((hi & 0x000FFFFF) | 0x3FF00000, __double2loint(prod));
+    // (bit patterns: the float64 pipe is the bound)
+    zero = zero && pe == 0 && hi == 0x3FF00000 && (__double2hiint(lsum) & 0x7FFFFFFF) < 0x3BC79CA1;
+    ys[v * ld + tid] = y;
+    p.Y[(int64_t)v * p.ldy + c] = y;
   }
-  if (SAMPLE_MAJOR) {
-    __syncthreads();
-    const int nw = bd >> 5, warp = tid >> 5, lane = tid & 31;
-    for (int j = warp; j < bd; j += nw) {
-      if (c0 + j >= p.C) break;
-      YT* row = p.Y + (c0 + j) * p.ldy;
-      for (int v = lane; v < p.mt; v += 32) put_y(row, v, ys[v * ld + j]);
-    }
-  }
+  p.logP[g] = lp0 + ((log(prod) + lsum) + pe * 0.69314718055994530942);
 }
 
 // BT32[i][u][v] = B[i][v][u] (zero for v >= m), inv32[i][v] = 1 / B[i][v][v]
@@ -764,13 +769,45 @@ struct Lims {
   bool one_sided;  // every lower limit is -inf
 };
 
-// Threads per block of the float64 sweep: as many as keep the sub-tile's y values
-// of the block's samples within 64 KB of shared memory (at least one warp).
-template <typename T>
-static int diag_threads(int m) {
-  int bd = 256;
-  while (bd > 32 && (size_t)m * bd * sizeof(T) > 65536) bd >>= 1;
-  return bd;
+// The float64 step's tables on the current device: made by the first float64 solve there (k_tables64, a fraction of a
+// millisecond) and kept, 115 KB, until the process ends; complete before any solve reads them.
+__device__ __align__(16) double g_tables64[T64_DOUBLES];
+static int tables64(const double** out, cudaStream_t st) {
+  static std::mutex mu;
+  static std::vector<std::pair<int, const double*>> made;
+  int dev = 0;
+  TLR_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(mu);
+  for (const auto& d : made)
+    if (d.first == dev) {
+      *out = d.second;
+      return TLRMVN_OK;
+    }
+  void* p = nullptr;
+  TLR_CUDA(cudaGetSymbolAddress(&p, g_tables64));
+  k_tables64<<<(T64_A + T64_B + 31) / 32, 32, 0, st>>>((double*)p);
+  TLR_CUDA(cudaGetLastError());
+  TLR_CUDA(cudaStreamSynchronize(st));
+  made.push_back({dev, (const double*)p});
+  *out = (const double*)p;
+  return TLRMVN_OK;
+}
+// Warps per block of the float64 sweep: one block fits an SM (its tables), and the SM with the most warps to run sets
+// the time, so of 1 to 6 warps (three and more preferred: fewer leave the pipe waiting) the count that gives the
+// fewest over all rounds.
+static int diag64_threads(int64_t C, int sms) {
+  const int64_t warps = (C + 31) / 32;
+  int best = 1;
+  int64_t best_cost = INT64_MAX;
+  for (int w = 6; w >= 1; w--) {
+    const int64_t rounds = ((warps + w - 1) / w + sms - 1) / sms;
+    const int64_t cost = rounds * std::max(w, 3);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = w;
+    }
+  }
+  return 32 * best;
 }
 
 // Launch shape of the float sweep: samples per thread (spt) and per block (ns).
@@ -1003,12 +1040,17 @@ static int run_chunks(Factor& F, const T* Bt, const T* Ut, const T* Vt, const Li
 
   // float64: sub-tiles of tu.sub variables, each sample keeping only the sub-tile's y in shared memory
   const int sub64 = std::min(m, tu.sub);
-  const int bd = diag_threads<T>(sub64);
-  const size_t smem = (size_t)sub64 * (bd + 1) * sizeof(T);
-  if (f32)
+  const double* tables = nullptr;
+  int dev = 0, sms = 1;
+  TLR_CUDA(cudaGetDevice(&dev));
+  TLR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  if (f32) {
     TLR_CHECK(set_sweep_smem(tu.sub));
-  else
-    TLR_CHECK(raise_smem_limit((const void*)k_diag<T, YT, false>, (size_t)smem));
+  } else {
+    TLR_CHECK(tables64(&tables, st));
+    for (const void* k : {(const void*)k_diag64<false>, (const void*)k_diag64<true>})
+      TLR_CHECK(raise_smem_limit(k, diag64_smem(64, 192)));
+  }
 
   for (int64_t c0 = 0; c0 < S; c0 += C) {
     const int64_t Cc = std::min(C, S - c0);
@@ -1029,7 +1071,7 @@ static int run_chunks(Factor& F, const T* Bt, const T* Ut, const T* Vt, const Li
                       C, (float*)Dl, C, nullptr);
         } else {
           gemm_nn<T>(st, mt, Cc, Kr, Ut + (size_t)m * F.krow_off[i], Kr, W + (size_t)F.krow_off[i] * C, C, Dl, C,
-                     nullptr);
+                     nullptr, sms);
         }
         pf.end();
         Delta = Dl;
@@ -1045,12 +1087,12 @@ static int run_chunks(Factor& F, const T* Bt, const T* Ut, const T* Vt, const Li
           const int mq = std::min(sub64, mt - q0);
           if (q0 > 0) {
             pf.begin(TLRMVN_KC_COUPLE);
-            gemm_nn<T>(st, mq, Cc, q0, Bi + (size_t)q0 * m, m, Y, C, Dl + (size_t)q0 * C, C, nullptr,
+            gemm_nn<T>(st, mq, Cc, q0, Bi + (size_t)q0 * m, m, Y, C, Dl + (size_t)q0 * C, C, nullptr, sms,
                        Delta ? 1 : 0);
             pf.end();
           }
           pf.begin(TLRMVN_KC_DIAG);
-          DiagArgs<T, YT> a;
+          DiagArgs64 a;
           a.B = Bi + (size_t)q0 * m + q0;
           a.mt = mq;
           a.ldb = m;
@@ -1071,7 +1113,9 @@ static int run_chunks(Factor& F, const T* Bt, const T* Ut, const T* Vt, const Li
           a.Y = Y + (size_t)q0 * C;
           a.ldy = C;
           a.logP = logP;
-          k_diag<T, YT, false><<<blocks_for(Cc, bd), bd, smem, st>>>(a);
+          a.tables = tables;
+          const int bd = diag64_threads(Cc, sms);
+          (L.one_sided ? k_diag64<true> : k_diag64<false>)<<<blocks_for(Cc, bd), bd, diag64_smem(mq, bd), st>>>(a);
           pf.end();
         }
       }
@@ -1081,7 +1125,8 @@ static int run_chunks(Factor& F, const T* Bt, const T* Ut, const T* Vt, const Li
           gemm_tn_f32(st, (int)Kc, Cc, mt, (const float*)Vt + F.v32_off[i], (Kc + 3) / 4 * 4, (const float*)Y, C,
                       (float*)W, C, F.vmap + F.kcol_off[i]);
         else
-          gemm_nn<T>(st, (int)Kc, Cc, mt, Vt + (size_t)m * F.kcol_off[i], m, Y, C, W, C, F.vmap + F.kcol_off[i]);
+          gemm_nn<T>(st, (int)Kc, Cc, mt, Vt + (size_t)m * F.kcol_off[i], m, Y, C, W, C, F.vmap + F.kcol_off[i],
+                     sms);
         pf.end();
       }
     }
