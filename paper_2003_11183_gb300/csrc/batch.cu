@@ -10,13 +10,14 @@
 // captures the launch sequence (limit permutation, persistent kernel,
 // estimator) in a CUDA graph, replayed for every new set of limits.
 //
-// Two persistent kernels: k_batch (TLRMVN_FP32: the shifts and projections as
-// float SIMT loops, W float) and k_batch_tc (TLRMVN_BF16_SHIFT: every tile runs
-// the whole-tile sweep of the single-problem path, stc_tile, with the shifts,
-// in-tile coupling and projections on tcgen05; W and the sample-major y in
-// CTA-private bf16 regions read back by TMA through one tensor map each, the
-// per-problem factor operands through three tensor maps per problem kept in
-// global memory).
+// The persistent kernel k_batch_tc runs every tile through the whole-tile sweep of
+// the single-problem path, stc_tile (TLRMVN_BF16_SHIFT: 16-bit shifts; TLRMVN_FP32: every
+// operand split): shifts, in-tile coupling and projections on tcgen05; W and the
+// sample-major y in CTA-private 16-bit regions read back by TMA through one tensor map
+// each, the per-problem factor operands through three tensor maps per problem kept in
+// global memory.  Should a y of a TLRMVN_FP32 run leave fp16's range (limits tens of
+// thousands of standard deviations out), the run is repeated by k_batch, the shifts and
+// projections as float loops, whose operands are made then.
 #include "common.cuh"
 #include "sov_device.cuh"
 #include "sweep_tc.cuh"
@@ -200,6 +201,9 @@ struct BatchTcProblem {
   const int32_t* vmap16;    // W row of each column rank
   const float* BT;
   const float* rec;
+  const float* rscale;      // (float32)
+  const float* wscale;      // (float32)
+  int kmax;                 // ranks of the widest row tile, padded: the lo parts' offset in the U map (float32)
   const uint64_t* Q;
   const uint64_t* D;
   const float* a;
@@ -207,22 +211,23 @@ struct BatchTcProblem {
   const int* two;           // nonzero: some lower limit of the problem is finite
 };
 
-template <int FLAGS>
-__global__ void __launch_bounds__(STC_NS, 6)
+template <int FLAGS, int MODE, int NST>
+__global__ void __launch_bounds__(STC_NS, stc_ctas(NST))
     k_batch_tc(const BatchTcProblem* __restrict__ probs, const CUtensorMap* __restrict__ pmaps,
                const BatchItem* __restrict__ items, int n_items, int* next, const __grid_constant__ CUtensorMap mapW,
                const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapY64,
                unsigned short* Wbase, int64_t kwmax, unsigned short* Ybase, int my, double* logP, int* err) {
   constexpr bool PER = FLAGS & SWEEP_PERIODIZE;
   extern __shared__ __align__(1024) unsigned char stc_smem[];
-  const StcCta k = stc_cta_setup(stc_smem);
+  constexpr int64_t WROWS = MODE == STC_FP32 ? 2 : 1;  // (float32: hi rows, then lo rows)
+  const StcCta k = stc_cta_setup<MODE, NST>(stc_smem);
   const int tid = threadIdx.x;
   StcPlace pl;
   pl.wx = 0;
-  pl.wy = (int)(blockIdx.x * kwmax);
+  pl.wy = (int)(blockIdx.x * kwmax * WROWS);
   pl.yrow = blockIdx.x * STC_NS;
   pl.ysrow = Ybase + ((int64_t)blockIdx.x * STC_NS + tid) * (2 * my);  // (hi at 0, lo at my)
-  pl.wcol = Wbase + (int64_t)blockIdx.x * kwmax * STC_NS + tid;
+  pl.wcol = Wbase + (int64_t)blockIdx.x * kwmax * WROWS * STC_NS + tid;
   for (;;) {
     __syncthreads();  // every thread is done with the previous item
     if (tid == 0) *k.item = atomicAdd(next, 1);
@@ -267,23 +272,33 @@ __global__ void __launch_bounds__(STC_NS, 6)
       p.kc = (int)(P.kcol_off[i + 1] - P.kcol_off[i]);
       p.ldw = STC_NS;
       p.vmap = P.vmap16 ? P.vmap16 + P.kcol_off[i] : nullptr;
-      p.wscale = nullptr;
+      p.wscale = P.wscale ? P.wscale + P.kcol_off[i] : nullptr;
       p.tscale = 1.0f;
+      p.rscale = P.rscale ? P.rscale + (int64_t)i * P.m : nullptr;
+      p.wlo = (int)kwmax;
+      p.ulo = P.kmax;
+      p.vlo = P.my;
       p.err = err;
       if (two)
-        ok = stc_tile<FLAGS, false>(&mapY, mp, &mapW, mp + 1, &mapY64, mp + 2, p, k, pl, act, Drow + t0, ks, rs, prod,
-                                    lsum, pe);
+        ok = stc_tile<FLAGS, MODE, NST>(&mapY, mp, &mapW, mp + 1, &mapY64, mp + 2, p, k, pl, act, Drow + t0, ks, rs,
+                                        prod, lsum, pe);
       else
-        ok = stc_tile<FLAGS | SWEEP_ONE_SIDED, false>(&mapY, mp, &mapW, mp + 1, &mapY64, mp + 2, p, k, pl, act,
-                                                      Drow + t0, ks, rs, prod, lsum, pe);
+        ok = stc_tile<FLAGS | SWEEP_ONE_SIDED, MODE, NST>(&mapY, mp, &mapW, mp + 1, &mapY64, mp + 2, p, k, pl, act,
+                                                          Drow + t0, ks, rs, prod, lsum, pe);
     }
     if (ok && act) logP[P.logp_off + g] = (double)(logf(prod) + lsum) + (double)pe * 0.69314718055994530942;
   }
-  stc_cta_release(k);
+  stc_cta_release<MODE>(k);
 }
-static const void* batch_tc_kernel(int periodize) {
-  return periodize ? (const void*)k_batch_tc<SWEEP_PERIODIZE> : (const void*)k_batch_tc<0>;
+// float32: two stages, three CTAs per SM; bf16: one stage, six
+typedef void (*BatchTcKernel)(const BatchTcProblem*, const CUtensorMap*, const BatchItem*, int, int*, const CUtensorMap,
+                              const CUtensorMap, const CUtensorMap, unsigned short*, int64_t, unsigned short*, int,
+                              double*, int*);
+static BatchTcKernel batch_tc_kernel(bool f32, int periodize) {
+  if (f32) return periodize ? k_batch_tc<SWEEP_PERIODIZE, STC_FP32, 2> : k_batch_tc<0, STC_FP32, 2>;
+  return periodize ? k_batch_tc<SWEEP_PERIODIZE, STC_BF16, 1> : k_batch_tc<0, STC_BF16, 1>;
 }
+static size_t batch_tc_smem(bool f32) { return f32 ? sweep_tc_smem_bytes(STC_FP32, 2) : sweep_tc_smem_bytes(STC_BF16, 1); }
 
 // limits of all problems: original order (staged) -> factor order, float; validation
 // (and, per problem, whether a lower limit is finite: prob_of maps a position to its problem)
@@ -345,12 +360,12 @@ int make_tensor_map_16(CUtensorMap* map, const void* base, uint64_t inner, uint6
 
 int ensure_float_tiles(Factor& F, cudaStream_t st);  // prob.cu: BT32 / inv32
 
-// tc: the tensor-core kernel's operands (the factor's bf16 copies and the padded
+// tc: the tensor-core kernel's operands (the factor's copies for the precision and the padded
 // rank offsets) instead of the float SIMT copies UT / VT.
-static int make_batch_copies(Factor& F, BatchCopies& C, bool tc, cudaStream_t st) {
+static int make_batch_copies(Factor& F, BatchCopies& C, bool tc, int precision, cudaStream_t st) {
   const int r = F.r, m = F.m;
   if (tc) {
-    TLR_CHECK(ensure_precision_copies(F, TLRMVN_BF16_SHIFT, st));
+    TLR_CHECK(ensure_precision_copies(F, precision, st));
     TLR_CHECK(dalloc(&C.kpad_off, r + 1));
     TLR_CUDA(cudaMemcpyAsync(C.kpad_off, F.kpad_off.data(), (r + 1) * 8, cudaMemcpyHostToDevice, st));
   } else {
@@ -405,14 +420,16 @@ struct Batch {
   std::vector<Factor*> F;
   std::vector<int64_t> n_off;  // limits offsets of each problem (host)
   std::vector<BatchCopies> copies;
+  std::vector<BatchProblem> probs;  // (host table; its float copies are filled in by simt_prepare)
+  std::vector<BatchCopies> simt;    // float32, made when a run first needs them
+  cudaGraphExec_t exec_simt = nullptr;
   BatchProblem* dprobs = nullptr;
   BatchItem* ditems = nullptr;
   int n_items = 0, grid = 0, grid_max = 0, per_sm = 0, per_sm_max = 0, sms = 0;
   int* dnext = nullptr;
   int* dbad = nullptr;
   float* W = nullptr;
-  // tensor-core kernel (TLRMVN_BF16_SHIFT)
-  bool tc = false;
+  bool f32 = false;
   int64_t kwmax = 0;          // W rows of one CTA's region (the largest padded rank space)
   int my = 64;                // y hi columns of one sample's row in the CTA-private y (lo at + my)
   BatchTcProblem* dtprobs = nullptr;
@@ -431,6 +448,7 @@ struct Batch {
   cudaGraphExec_t exec = nullptr;
   ~Batch() {
     if (exec) cudaGraphExecDestroy(exec);
+    if (exec_simt) cudaGraphExecDestroy(exec_simt);
     dfree(dprobs);
     dfree(dtprobs);
     dfree(dmaps);
@@ -494,22 +512,12 @@ static int batch_capture(Batch& B, int per_sm) {
   cudaMemsetAsync(B.dbad, 0, sizeof(int), st);
   cudaMemsetAsync(B.dnext, 0, sizeof(int), st);
   cudaMemsetAsync(B.dtwo, 0, B.count * sizeof(int), st);
-  if (B.tc) cudaMemsetAsync(B.derr, 0, sizeof(int), st);
+  cudaMemsetAsync(B.derr, 0, 2 * sizeof(int), st);
   k_permute_batch<<<nblk(B.total_n, 256), 256, 0, st>>>(B.a_st, B.b_st, B.perm_g, B.prob_of, B.total_n, B.a32, B.b32,
                                                         B.dbad, B.dtwo);
-  if (B.tc) {
-    if (B.periodize)
-      k_batch_tc<SWEEP_PERIODIZE><<<grid, STC_NS, sweep_tc_smem_bytes(), st>>>(
-          B.dtprobs, B.dmaps, B.ditems, B.n_items, B.dnext, B.mapW, B.mapY, B.mapY64, B.W16, B.kwmax, B.Y16, B.my,
-          B.logP, B.derr);
-    else
-      k_batch_tc<0><<<grid, STC_NS, sweep_tc_smem_bytes(), st>>>(B.dtprobs, B.dmaps, B.ditems, B.n_items, B.dnext,
-                                                                 B.mapW, B.mapY, B.mapY64, B.W16, B.kwmax, B.Y16,
-                                                                 B.my, B.logP, B.derr);
-  } else {
-    k_batch<<<grid, BATCH_T, batch_smem(), st>>>(B.dprobs, B.ditems, B.n_items, B.dnext, B.W,
-                                                std::max<int64_t>(B.ktot_max, 1) * BATCH_T, B.logP);
-  }
+  batch_tc_kernel(B.f32, B.periodize)<<<grid, STC_NS, batch_tc_smem(B.f32), st>>>(
+      B.dtprobs, B.dmaps, B.ditems, B.n_items, B.dnext, B.mapW, B.mapY, B.mapY64, B.W16, B.kwmax, B.Y16, B.my, B.logP,
+      B.derr);
   k_shift_reduce<<<(unsigned)(B.count * B.M), 256, 0, st>>>(B.logP, B.N, B.ell);
   k_final_batch<<<B.count, 256, 0, st>>>(B.ell, B.M, B.out);
   cudaError_t ec = cudaStreamEndCapture(st, &graph);
@@ -525,13 +533,55 @@ static int batch_capture(Batch& B, int per_sm) {
   return TLRMVN_OK;
 }
 
+// The general float32 integrand of a plan (k_batch, then the estimator, on the limits as already permuted): its
+// operands and graph, made the first time that a run needs it.
+static int simt_prepare(Batch& B) {
+  if (B.exec_simt) return TLRMVN_OK;
+  cudaStream_t st = B.st;
+  if (B.simt.empty()) B.simt.resize(B.count);
+  for (int p = 0; p < B.count; p++) {
+    BatchCopies& C = B.simt[p];
+    if (!C.tile_off) TLR_CHECK(make_batch_copies(*B.F[p], C, false, TLRMVN_FP32, st));
+    BatchProblem& P = B.probs[p];
+    P.vt_off = C.vt_off;
+    P.kcpad = C.kcpad;
+    P.UT = C.UT;
+    P.VT = C.VT;
+  }
+  const size_t smem = batch_smem();
+  TLR_CHECK(raise_smem_limit((const void*)k_batch, smem));
+  int per_sm = 1;
+  TLR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch, BATCH_T, smem));
+  const int grid = std::max(1, std::min(std::max(per_sm, 1) * B.sms, B.n_items));
+  if (!B.dprobs) TLR_CHECK(dalloc(&B.dprobs, B.count));
+  if (!B.W) TLR_CHECK(dalloc(&B.W, (size_t)grid * std::max<int64_t>(B.ktot_max, 1) * BATCH_T));
+  TLR_CUDA(cudaMemcpyAsync(B.dprobs, B.probs.data(), B.probs.size() * sizeof(BatchProblem), cudaMemcpyHostToDevice, st));
+  TLR_CUDA(cudaStreamSynchronize(st));
+  cudaGraph_t graph;
+  TLR_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+  cudaMemsetAsync(B.dnext, 0, sizeof(int), st);
+  k_batch<<<grid, BATCH_T, smem, st>>>(B.dprobs, B.ditems, B.n_items, B.dnext, B.W,
+                                       std::max<int64_t>(B.ktot_max, 1) * BATCH_T, B.logP);
+  k_shift_reduce<<<(unsigned)(B.count * B.M), 256, 0, st>>>(B.logP, B.N, B.ell);
+  k_final_batch<<<B.count, 256, 0, st>>>(B.ell, B.M, B.out);
+  cudaError_t ec = cudaStreamEndCapture(st, &graph);
+  if (ec != cudaSuccess) return cuda_fail(ec, "capture of the general batched integrand");
+  ec = cudaGraphInstantiate(&B.exec_simt, graph, 0);
+  cudaGraphDestroy(graph);
+  if (ec != cudaSuccess) {
+    B.exec_simt = nullptr;
+    return cuda_fail(ec, "instantiate the general batched integrand graph");
+  }
+  return TLRMVN_OK;
+}
+
 static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, const double* nu,
                        const tlrmvn_opts& o) {
   B.count = count;
   B.M = o.n_shifts;
   B.N = o.n_points;
   B.periodize = o.periodize;
-  B.tc = o.precision == TLRMVN_BF16_SHIFT;
+  B.f32 = o.precision == TLRMVN_FP32;
   TLR_CUDA(cudaGetDevice(&B.device));
   TLR_CUDA(cudaStreamCreateWithFlags(&B.st, cudaStreamNonBlocking));
   cudaStream_t st = B.st;
@@ -541,22 +591,21 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
   for (int p = 0; p < count; p++) {
     Factor* F = reinterpret_cast<Factor*>(factors[p]);
     if (!F) return fail(TLRMVN_E_INVAL, "null factor in batch");
-    if (!B.tc && F->m > BATCH_MMAX) return fail(TLRMVN_E_NOTSUP, "FP32 batched problems need tile size <= 128");
+    if (B.f32 && F->m > BATCH_MMAX) return fail(TLRMVN_E_NOTSUP, "FP32 batched problems need tile size <= 128");
     if (!(nu[p] > 0.0)) return fail(TLRMVN_E_INVAL, "nu must be > 0");
     B.F[p] = F;
     B.n_off[p + 1] = B.n_off[p] + F->n;
     B.ktot_max = std::max(B.ktot_max, F->ktot);
-    TLR_CHECK(make_batch_copies(*F, B.copies[p], B.tc, st));
-    if (B.tc) {
-      B.kwmax = std::max(B.kwmax, F->kw16);
-      B.my = std::max<int>(B.my, (int)F->my16);
-    }
+    TLR_CHECK(make_batch_copies(*F, B.copies[p], true, o.precision, st));
+    B.kwmax = std::max(B.kwmax, F->kw16);
+    B.my = std::max<int>(B.my, (int)F->my16);
   }
   B.total_n = B.n_off[count];
   const int64_t S = (int64_t)B.M * B.N;
   B.total_samples = S * count;
   // device tables
-  std::vector<BatchProblem> probs(count);
+  std::vector<BatchProblem>& probs = B.probs;
+  probs.resize(count);
   std::vector<int64_t> perm_g(B.total_n);
   std::vector<int64_t> d_off(count + 1, 0);
   for (int p = 0; p < count; p++) d_off[p + 1] = d_off[p] + (int64_t)B.M * (B.F[p]->n + 1);
@@ -610,64 +659,64 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
   for (int p : order)
     for (int64_t c0 = 0; c0 < S; c0 += BATCH_T) items.push_back(BatchItem{p, (int)std::min<int64_t>(BATCH_T, S - c0), c0});
   B.n_items = (int)items.size();
-  TLR_CHECK(dalloc(&B.dprobs, count));
   TLR_CHECK(dalloc(&B.ditems, items.size()));
   TLR_CHECK(dalloc(&B.perm_g, (size_t)B.total_n));
   TLR_CHECK(dalloc(&B.prob_of, (size_t)B.total_n));
   std::vector<int32_t> prob_of(B.total_n);
   for (int p = 0; p < count; p++) std::fill(prob_of.begin() + B.n_off[p], prob_of.begin() + B.n_off[p + 1], p);
   TLR_CUDA(cudaMemcpyAsync(B.prob_of, prob_of.data(), prob_of.size() * 4, cudaMemcpyHostToDevice, st));
-  TLR_CUDA(cudaMemcpyAsync(B.dprobs, probs.data(), probs.size() * sizeof(BatchProblem), cudaMemcpyHostToDevice, st));
   TLR_CUDA(cudaMemcpyAsync(B.ditems, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, st));
   TLR_CUDA(cudaMemcpyAsync(B.perm_g, perm_g.data(), perm_g.size() * 8, cudaMemcpyHostToDevice, st));
   // persistent grid (all the CTAs that fit, until tuned) and its private projection buffers
   TLR_CUDA(cudaDeviceGetAttribute(&B.sms, cudaDevAttrMultiProcessorCount, B.device));
-  if (B.tc) {
-    const void* kt = batch_tc_kernel(B.periodize);
+  {
+    const void* kt = (const void*)batch_tc_kernel(B.f32, B.periodize);
     TLR_CUDA(cudaFuncSetAttribute(kt, cudaFuncAttributePreferredSharedMemoryCarveout,
                                   (int)cudaSharedmemCarveoutMaxShared));
+    TLR_CHECK(raise_smem_limit(kt, batch_tc_smem(B.f32)));
     // resident CTAs from the kernel's registers and shared memory (the occupancy query
     // reported one CTA per SM for this kernel where the launches fit six), and at most
-    // 512 / 64 per SM: each holds its 64 TMEM columns until the end
-    TLR_CHECK(resident_ctas(kt, STC_NS, sweep_tc_smem_bytes(), B.device, &B.per_sm_max));
-    B.per_sm_max = std::min(B.per_sm_max, 512 / STC_SUB);
-  } else {
-    const size_t smem = batch_smem();
-    TLR_CHECK(raise_smem_limit((const void*)k_batch, (size_t)smem));
-    TLR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&B.per_sm_max, k_batch, BATCH_T, smem));
+    // as many as their TMEM columns, held until the end, leave room for
+    TLR_CHECK(resident_ctas(kt, STC_NS, batch_tc_smem(B.f32), B.device, &B.per_sm_max));
+    B.per_sm_max = std::min<int>(B.per_sm_max, 512 / (int)stc_cols(B.f32 ? STC_FP32 : STC_BF16));
   }
   B.per_sm_max = std::max(B.per_sm_max, 1);
   B.grid_max = std::max(1, std::min(B.per_sm_max * B.sms, B.n_items));
-  if (B.tc) {
-    // CTA-private W (kwmax rank rows x 128 samples) and sample-major y (128 rows of
-    // 2 x 128 hi / lo columns), zeroed once: padding rows and columns meet zero
+  {
+    // CTA-private W (kwmax rank rows x 128 samples; float32: twice, hi and lo) and sample-major y (128 rows of
+    // hi / lo columns), zeroed once: padding rows and columns meet zero
     // operand entries and must stay finite
     B.kwmax = std::max<int64_t>(B.kwmax, 64);
-    if ((int64_t)B.grid_max * B.kwmax >= ((int64_t)1 << 31))
+    const int64_t wrows = B.kwmax * (B.f32 ? 2 : 1);
+    if ((int64_t)B.grid_max * wrows >= ((int64_t)1 << 31))
       return fail(TLRMVN_E_NOTSUP, "batched projections exceed the tensor map's coordinate range");
-    const size_t nw = (size_t)B.grid_max * B.kwmax * STC_NS, ny = (size_t)B.grid_max * STC_NS * 2 * B.my;
+    const size_t nw = (size_t)B.grid_max * wrows * STC_NS, ny = (size_t)B.grid_max * STC_NS * 2 * B.my;
     TLR_CHECK(dalloc(&B.W16, nw));
     TLR_CHECK(dalloc(&B.Y16, ny));
-    TLR_CHECK(dalloc(&B.derr, 1));
+    TLR_CHECK(dalloc(&B.derr, 2));
     TLR_CUDA(cudaMemsetAsync(B.W16, 0, nw * 2, st));
     TLR_CUDA(cudaMemsetAsync(B.Y16, 0, ny * 2, st));
-    TLR_CUDA(cudaMemsetAsync(B.derr, 0, sizeof(int), st));
-    TLR_CHECK(make_tensor_map_16(&B.mapW, B.W16, STC_NS, (uint64_t)B.grid_max * B.kwmax, STC_NS * 2, 64, 64, false));
+    TLR_CUDA(cudaMemsetAsync(B.derr, 0, 2 * sizeof(int), st));
+    const uint32_t deep = B.f32 ? 32 : 64;
+    TLR_CHECK(make_tensor_map_16(&B.mapW, B.W16, STC_NS, (uint64_t)B.grid_max * wrows, STC_NS * 2, deep, 64, B.f32));
     TLR_CHECK(make_tensor_map_16(&B.mapY, B.Y16, 2 * B.my, (uint64_t)B.grid_max * STC_NS, 2 * B.my * 2,
-                                 STC_NS, 32, false));
+                                 STC_NS, 32, B.f32));
     TLR_CHECK(make_tensor_map_16(&B.mapY64, B.Y16, 2 * B.my, (uint64_t)B.grid_max * STC_NS, 2 * B.my * 2, STC_NS,
-                                 64, false));
+                                 64, B.f32));
     // per problem: the split B, U and V maps, and its table entry
     std::vector<CUtensorMap> maps((size_t)BATCH_TC_MAPS * count);
     std::vector<BatchTcProblem> tp(count);
     for (int p = 0; p < count; p++) {
       const Factor& F = *B.F[p];
-      const int64_t ly = 2 * F.my16;
+      const int64_t ly = (B.f32 ? 3 : 2) * F.my16;
       CUtensorMap* mp = &maps[(size_t)BATCH_TC_MAPS * p];
-      TLR_CHECK(make_tensor_map_16(&mp[0], F.B16x2, ly, (uint64_t)F.r * F.m, ly * 2, 64, 32, false));
+      const void* B2 = B.f32 ? (const void*)F.Bs16 : (const void*)F.B16x2;
+      TLR_CHECK(make_tensor_map_16(&mp[0], B2, ly, (uint64_t)F.r * F.m, ly * 2, 64, 32, B.f32));
       if (F.ktot) {
-        TLR_CHECK(make_tensor_map_16(&mp[1], F.U16, F.kmax16, (uint64_t)F.r * F.m, F.kmax16 * 2, 64, 64, false));
-        TLR_CHECK(make_tensor_map_16(&mp[2], F.V16, F.my16, F.ktot, F.my16 * 2, 64, 64, false));
+        const void *U = B.f32 ? (const void*)F.Us16 : (const void*)F.U16, *V = B.f32 ? (const void*)F.Vs16 : (const void*)F.V16;
+        const int64_t lu = (B.f32 ? 3 : 1) * F.kmax16, lv = (B.f32 ? 3 : 1) * F.my16;
+        TLR_CHECK(make_tensor_map_16(&mp[1], U, lu, (uint64_t)F.r * F.m, lu * 2, 64, deep, B.f32));
+        TLR_CHECK(make_tensor_map_16(&mp[2], V, lv, F.ktot, lv * 2, 64, deep, B.f32));
       } else {
         mp[1] = B.mapW;  // (never read: no tile has ranks)
         mp[2] = B.mapW;
@@ -689,6 +738,9 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
       T.vmap16 = F.vmap16;
       T.BT = P.BT;
       T.rec = F.rec32;
+      T.rscale = B.f32 ? F.rscale32 : nullptr;
+      T.wscale = B.f32 ? F.wscale32 : nullptr;
+      T.kmax = (int)F.kmax16;
       T.two = B.dtwo + p;
       T.Q = P.Q;
       T.D = P.D;
@@ -699,8 +751,7 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
     TLR_CHECK(dalloc(&B.dtprobs, count));
     TLR_CUDA(cudaMemcpyAsync(B.dmaps, maps.data(), maps.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, st));
     TLR_CUDA(cudaMemcpyAsync(B.dtprobs, tp.data(), tp.size() * sizeof(BatchTcProblem), cudaMemcpyHostToDevice, st));
-  } else {
-    TLR_CHECK(dalloc(&B.W, (size_t)B.grid_max * std::max<int64_t>(B.ktot_max, 1) * BATCH_T));
+    TLR_CUDA(cudaStreamSynchronize(st));  // (the host tables go out of scope)
   }
   TLR_CHECK(dalloc(&B.dnext, 1));
   TLR_CHECK(dalloc(&B.dbad, 1));
@@ -730,15 +781,25 @@ static int batch_run(Batch& B, const double* const* a, const double* const* b, d
   TLR_CUDA(cudaGraphLaunch(B.exec, st));
   TLR_CUDA(cudaMemcpyAsync(B.h_out, B.out, (size_t)B.count * 2 * 8, cudaMemcpyDeviceToHost, st));
   TLR_CUDA(cudaMemcpyAsync(B.h_out + 2 * B.count, B.dbad, sizeof(int), cudaMemcpyDeviceToHost, st));
-  if (B.tc) TLR_CUDA(cudaMemcpyAsync(B.h_out + 2 * B.count + 1, B.derr, sizeof(int), cudaMemcpyDeviceToHost, st));
+  TLR_CUDA(cudaMemcpyAsync(B.h_out + 2 * B.count + 1, B.derr, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
   TLR_CUDA(cudaStreamSynchronize(st));
-  int bad = 0, terr = 0;
+  int bad = 0, terr[2] = {0, 0};
   memcpy(&bad, B.h_out + 2 * B.count, sizeof(int));
-  if (B.tc) memcpy(&terr, B.h_out + 2 * B.count + 1, sizeof(int));
+  memcpy(terr, B.h_out + 2 * B.count + 1, 2 * sizeof(int));
+  if (!bad && !terr[0] && terr[1]) {  // (float32) a y left fp16's range
+    const int s = simt_prepare(B);
+    if (s != TLRMVN_OK) {
+      cudaSetDevice(cur);
+      return s;
+    }
+    TLR_CUDA(cudaGraphLaunch(B.exec_simt, st));
+    TLR_CUDA(cudaMemcpyAsync(B.h_out, B.out, (size_t)B.count * 2 * 8, cudaMemcpyDeviceToHost, st));
+    TLR_CUDA(cudaStreamSynchronize(st));
+  }
   cudaSetDevice(cur);
   if (bad) return fail(TLRMVN_E_INVAL, "limits must satisfy a_i <= b_i, a_i < +inf, b_i > -inf, no NaN");
-  if (terr)
-    return fail(TLRMVN_E_TIMEOUT, "tensor-core batched kernel gave up waiting (code " + std::to_string(terr) + ")");
+  if (terr[0])
+    return fail(TLRMVN_E_TIMEOUT, "tensor-core batched kernel gave up waiting (code " + std::to_string(terr[0]) + ")");
   for (int p = 0; p < B.count; p++) {
     logp[p] = B.h_out[2 * p];
     err[p] = B.h_out[2 * p + 1];
@@ -793,7 +854,7 @@ extern "C" int tlrmvn_batch_tune(tlrmvn_batch_t plan, const double* const* a, co
       if (c == ' ') c = '_';
     int64_t ksum = 0;
     for (Factor* F : B.F) ksum += F->ktot;
-    key = dev + (B.tc ? " batch-bf16 c" : " batch c") + std::to_string(B.count) + " n" + std::to_string(B.total_n) + " k" +
+    key = dev + (B.f32 ? " batch-split c" : " batch-bf16 c") + std::to_string(B.count) + " n" + std::to_string(B.total_n) + " k" +
           std::to_string(ksum) + " s" + std::to_string((int64_t)B.M * B.N);
   }
   int best = -1;

@@ -105,7 +105,7 @@ struct Factor {
   //   rec32 r x m x 24: the whole-tile sweep's record of each variable (sweep_tc.cuh)
   float* rec32 = nullptr;
   int64_t ldbt = 0;
-  float* B32 = nullptr;
+  // (the general float32 path, taken when a y leaves fp16's range)
   float* U32 = nullptr;  // row tile i at u32_off[i]: (Krow_i rounded up to 8) x m, U_i transposed, zero rows
   std::vector<int64_t> u32_off;
   float* V32 = nullptr;  // column tile i at v32_off[i]: m x (Kcol_i rounded up to 4), V_i, zero columns
@@ -136,6 +136,16 @@ struct Factor {
   // (1/2, 1], so that badly scaled covariances keep fp16's range); the sweep multiplies
   // what it reads from the products by inv_g16 = 1 / g
   float inv_g16 = 1.0f;
+  // split fp16 operands of the float32 path (STC_FP32, sweep_tc.cuh), in each row hi, then lo, then third parts:
+  // Bs16 = B g, Us16 = U g / s (rows (r*m) x 3 my16 and 3 kmax16), Vs16 = V t (ktot x 3 my16), with powers of two
+  // g per row of B and U (max |B g|, |U g / s| in (1/2, 1], of B the part left of the row's 64-variable sub-tile: the
+  // coupling's; the rest is zero), t per Vcat row (max |V t| in (1/2, 1]) and s per rank
+  // (|V s|_2 in (1/2, 1]: the stored projections s V^T y are of order 1); rscale32 = 1 / g, wscale32 = s / t
+  __half* Us16 = nullptr;
+  __half* Vs16 = nullptr;
+  __half* Bs16 = nullptr;
+  float* rscale32 = nullptr;
+  float* wscale32 = nullptr;
   // lattice generators for n + 1 coordinates (device), and the permutation (device)
   uint64_t* Q = nullptr;
   int64_t* dperm = nullptr;

@@ -319,7 +319,8 @@ __global__ void k_split_b16h(const double* B, double g, int m, int64_t my, int64
   out[t] = h ? __double2half(b - (double)__half2float(hi)) : hi;
 }
 
-// float32 diagonal tiles: row-major B32, transposed BT32 (ld ldbt), reciprocal diagonal inv32
+// The general float32 path's copies and the batched kernel's: transposed tiles BT32 (ld ldbt), reciprocal diagonal
+// inv32 and window columns,
 // band32[(i*m + v)*16 + k] = B_i[v+1+k][v] (k < 15, v+1+k < m), else 0
 __global__ void k_make_band(const double* B, int m, int64_t count, float* band) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -349,15 +350,11 @@ __global__ void k_make_rec(const double* B, const uint64_t* Q, const int64_t* ti
 }
 
 int ensure_float_tiles(Factor& F, cudaStream_t st) {
-  if (F.B32 && F.BT32 && F.inv32 && F.band32 && F.rec32) return TLRMVN_OK;
-  dfree(F.B32);  // a failed earlier attempt may have left some of these behind
-  dfree(F.BT32);
+  if (F.BT32 && F.inv32 && F.band32 && F.rec32) return TLRMVN_OK;
+  dfree(F.BT32);  // a failed earlier attempt may have left some of these behind
   dfree(F.inv32);
   dfree(F.band32);
   dfree(F.rec32);
-  const int64_t nb = (int64_t)F.r * F.m * F.m;
-  TLR_CHECK(dalloc(&F.B32, nb));
-  k_convert<double, float><<<blocks_for(nb, 256), 256, 0, st>>>(F.B, F.B32, nb);
   F.ldbt = ((int64_t)F.m + DIAG_VB - 1) / DIAG_VB * DIAG_VB;
   const int64_t nt = (int64_t)F.r * F.m * F.ldbt;
   TLR_CHECK(dalloc(&F.BT32, nt + DIAG_PAD));
@@ -386,6 +383,85 @@ int ensure_float_tiles(Factor& F, cudaStream_t st) {
   return TLRMVN_OK;
 }
 
+// ---- split operands of the float32 path (STC_FP32): see Factor ------------------------------------------
+// the power of two that takes x > 0 into (1/2, 1] (1 for 0), within float's exponents
+__device__ __forceinline__ double pow2_scale(double x) {
+  if (!(x > 0.0)) return 1.0;
+  int e;
+  const double f = frexp(x, &e);  // f in [1/2, 1)
+  if (f == 0.5) e--;              // (1/2 2^e: into 1)
+  return scalbn(1.0, max(-126, min(126, -e)));
+}
+// per Vcat row (a warp each): t, and s for its rank
+__global__ void __launch_bounds__(256) k_scale_v(const double* Vcat, const int32_t* vmap, int m, int64_t ktot, double* tv,
+                                                 double* su, float* wscale) {
+  const int64_t g = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (g >= ktot) return;
+  double mx = 0.0;
+  for (int u = lane; u < m; u += 32) mx = fmax(mx, fabs(Vcat[g * m + u]));
+  for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  const double t = pow2_scale(mx);
+  double ss = 0.0;
+  for (int u = lane; u < m; u += 32) {
+    const double x = Vcat[g * m + u] * t;
+    ss += x * x;
+  }
+  for (int o = 16; o; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if (lane == 0) {
+    const double n = pow2_scale(sqrt(ss));  // |V t n|_2 in (1/2, 1]: s = t n
+    tv[g] = t;
+    su[vmap[g]] = t * n;
+    wscale[g] = (float)n;
+  }
+}
+// per row of B and U (a warp each): g
+__global__ void __launch_bounds__(256) k_scale_rows(const double* B, const double* Ucat, const int64_t* krow_off,
+                                                    const double* su, int m, int64_t rows, double* g, float* rscale) {
+  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (row >= rows) return;
+  const int64_t i = row / m, v = row % m, k0 = krow_off[i], Kr = krow_off[i + 1] - k0;
+  double mx = 0.0;
+  for (int u = lane; u < (int)(v & ~(int64_t)63); u += 32) mx = fmax(mx, fabs(B[row * m + u]));
+  const double* U = Ucat + (int64_t)m * k0 + v * Kr;
+  for (int64_t k = lane; k < Kr; k += 32) mx = fmax(mx, fabs(U[k] / su[k0 + k]));
+  for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) {
+    const double s = pow2_scale(mx);
+    g[row] = s;
+    rscale[row] = (float)(1.0 / s);
+  }
+}
+// hi (a multiple of 2^-10), lo or third fp16 part of x, |x| <= 1
+__device__ __forceinline__ __half split_part(double x, int h) {
+  const __half hi = __double2half(rint(x * 1024.0) * 0.0009765625);
+  if (h == 0) return hi;
+  const double r = x - (double)__half2float(hi);
+  const __half lo = __double2half(r);
+  return h == 1 ? lo : __double2half(r - (double)__half2float(lo));
+}
+__global__ void k_split_b32(const double* B, const double* g, int m, int64_t my, int64_t count, __half* out) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= count) return;
+  const int64_t row = t / (3 * my), c = t % (3 * my), u = c % my, v = row % m;
+  out[t] = split_part(u < (v & ~(int64_t)63) ? B[row * m + u] * g[row] : 0.0, (int)(c / my));
+}
+__global__ void k_split_u32(const double* Ucat, const int64_t* krow_off, const double* g, const double* su, int m,
+                            int64_t kmax, int64_t count, __half* out) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= count) return;
+  const int64_t row = t / (3 * kmax), c = t % (3 * kmax), k = c % kmax, i = row / m, v = row % m;
+  const int64_t k0 = krow_off[i], Kr = krow_off[i + 1] - k0;
+  out[t] = split_part(k < Kr ? Ucat[(int64_t)m * k0 + v * Kr + k] * (g[row] / su[k0 + k]) : 0.0, (int)(c / kmax));
+}
+__global__ void k_split_v32(const double* Vcat, const double* tv, int m, int64_t my, int64_t count, __half* out) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= count) return;
+  const int64_t row = t / (3 * my), c = t % (3 * my), u = c % my;
+  out[t] = split_part(u < m ? Vcat[row * m + u] * tv[row] : 0.0, (int)(c / my));
+}
+
 // out[k * m + v] = U[v * kr + k] for k < kr, else 0 (one row tile's U, float, k-major,
 // its ranks padded to a multiple of 8: ld8 rows)
 __global__ void k_pad_u32t(const double* U, int64_t kr, int64_t m, int64_t cnt, float* out) {
@@ -406,16 +482,23 @@ __global__ void k_pad_v32(const double* Vt, int64_t kc, int64_t kc4, int64_t m, 
 // Makes the copies a precision needs; the first caller makes them (and waits for
 // them) under the factor's lock, so concurrent streams never see a partial copy.
 static int ensure_copies_locked(Factor& F, int precision, cudaStream_t st);
+static bool layout_ready(const Factor& F) { return !F.kpad_off.empty() && (F.ktot == 0 || F.vmap16); }
 static bool bf16_ready(const Factor& F) {
-  return !F.kpad_off.empty() && (F.ktot == 0 || (F.U16 && F.V16 && F.vmap16)) && F.B16x2;
+  return layout_ready(F) && (F.ktot == 0 || (F.U16 && F.V16)) && F.B16x2;
 }
 static bool fp16_ready(const Factor& F) {
-  return bf16_ready(F) && (F.ktot == 0 || (F.U16h && F.V16h && F.wscale16)) && F.B16x2h;
+  return layout_ready(F) && (F.ktot == 0 || (F.U16h && F.V16h && F.wscale16)) && F.B16x2h;
 }
+static bool fp32_ready(const Factor& F) {
+  return layout_ready(F) && (F.ktot == 0 || (F.Us16 && F.Vs16 && F.wscale32)) && F.Bs16 && F.rscale32;
+}
+// (copies of the general float32 path: precision TLRMVN_FP32 with this added)
+constexpr int SIMT_COPIES = 16;
 static bool copies_ready(const Factor& F, int precision) {
   if (precision == TLRMVN_FP64) return true;
-  if (!F.B32 || !F.BT32 || !F.inv32 || !F.band32 || !F.rec32) return false;
-  if (precision == TLRMVN_FP32) return (F.U32 && F.V32) || F.ktot == 0;
+  if (!F.BT32 || !F.inv32 || !F.band32 || !F.rec32) return false;
+  if (precision == TLRMVN_FP32 + SIMT_COPIES) return (F.U32 && F.V32) || F.ktot == 0;
+  if (precision == TLRMVN_FP32) return fp32_ready(F);
   if (precision == TLRMVN_FP16_SHIFT) return fp16_ready(F);
   return bf16_ready(F);
 }
@@ -426,7 +509,7 @@ static int ensure_copies(Factor& F, int precision, cudaStream_t st) {
   TLR_CUDA(cudaStreamSynchronize(st));
   return TLRMVN_OK;
 }
-// FP16-shift operands with per-tile scaling (the factor's bf16 layout must exist).
+// FP16-shift operands with per-tile scaling (the padded rank layout must exist).
 // All products are of the factor scaled by one power of two g with max |B g| in
 // (1/2, 1] (the probability and every y are unchanged by scaling the factor and
 // the limits alike, and the sweep undoes g where it reads the products), so a
@@ -554,10 +637,82 @@ static int make_fp16_copies(Factor& F, cudaStream_t st) {
   return TLRMVN_OK;
 }
 
+// The padded rank space (row tile i starts at a multiple of 64) and vmap16: for each Vcat row, its row of it.
+static int make_layout(Factor& F, cudaStream_t st) {
+  dfree(F.vmap16);
+  const int r = F.r, m = F.m;
+  std::vector<int64_t> off(r + 1, 0);
+  int64_t kmax = 0;
+  for (int i = 0; i < r; i++) {
+    off[i + 1] = off[i] + (F.krow(i) + 63) / 64 * 64;
+    kmax = std::max(kmax, F.krow(i));
+  }
+  F.kw16 = std::max<int64_t>(off[r], 64);
+  F.kmax16 = std::max<int64_t>((kmax + 63) / 64 * 64, 64);
+  F.my16 = ((int64_t)m + 63) / 64 * 64;
+  if (F.ktot) {
+    std::vector<int32_t> v16(F.ktot);
+    for (int j = 0; j < r; j++) {
+      int64_t row = F.kcol_off[j];
+      for (int i = j + 1; i < r; i++) {
+        int64_t local = 0;
+        for (int t = 0; t < j; t++) local += F.rank[(size_t)i * r + t];
+        for (int c = 0; c < F.rank[(size_t)i * r + j]; c++) v16[row++] = (int32_t)(off[i] + local + c);
+      }
+    }
+    TLR_CHECK(dalloc(&F.vmap16, (size_t)F.ktot));
+    TLR_CUDA(cudaMemcpyAsync(F.vmap16, v16.data(), v16.size() * 4, cudaMemcpyHostToDevice, st));
+    TLR_CUDA(cudaStreamSynchronize(st));
+  }
+  F.kpad_off = off;
+  return TLRMVN_OK;
+}
+static int make_fp32_copies(Factor& F, cudaStream_t st) {
+  dfree(F.Us16);
+  dfree(F.Vs16);
+  dfree(F.Bs16);
+  dfree(F.rscale32);
+  dfree(F.wscale32);
+  const int m = F.m;
+  const int64_t rows = (int64_t)F.r * m, nb = rows * 3 * F.my16, nu = rows * 3 * F.kmax16, nv = F.ktot * 3 * F.my16;
+  double *tv = nullptr, *su = nullptr, *g = nullptr;
+  int64_t* kro = nullptr;
+  auto build = [&]() -> int {
+    TLR_CHECK(dalloc(&F.rscale32, (size_t)rows));
+    TLR_CHECK(dalloc(&F.Bs16, (size_t)nb));
+    TLR_CHECK(dalloc(&g, (size_t)rows));
+    TLR_CHECK(dalloc(&kro, (size_t)F.r + 1));
+    TLR_CUDA(cudaMemcpyAsync(kro, F.krow_off.data(), (F.r + 1) * 8, cudaMemcpyHostToDevice, st));
+    if (F.ktot) {
+      TLR_CHECK(dalloc(&F.wscale32, (size_t)F.ktot));
+      TLR_CHECK(dalloc(&F.Us16, (size_t)nu));
+      TLR_CHECK(dalloc(&F.Vs16, (size_t)nv));
+      TLR_CHECK(dalloc(&tv, (size_t)F.ktot));
+      TLR_CHECK(dalloc(&su, (size_t)F.ktot));
+      k_scale_v<<<blocks_for(F.ktot, 8), 256, 0, st>>>(F.Vcat, F.vmap, m, F.ktot, tv, su, F.wscale32);
+    }
+    k_scale_rows<<<blocks_for(rows, 8), 256, 0, st>>>(F.B, F.Ucat, kro, su, m, rows, g, F.rscale32);
+    k_split_b32<<<blocks_for(nb, 256), 256, 0, st>>>(F.B, g, m, F.my16, nb, F.Bs16);
+    if (F.ktot) {
+      k_split_u32<<<blocks_for(nu, 256), 256, 0, st>>>(F.Ucat, kro, g, su, m, F.kmax16, nu, F.Us16);
+      k_split_v32<<<blocks_for(nv, 256), 256, 0, st>>>(F.Vcat, tv, m, F.my16, nv, F.Vs16);
+    }
+    TLR_CUDA(cudaGetLastError());
+    TLR_CUDA(cudaStreamSynchronize(st));
+    return TLRMVN_OK;
+  };
+  const int s = build();
+  dfree(tv);
+  dfree(su);
+  dfree(g);
+  dfree(kro);
+  return s;
+}
+
 static int ensure_copies_locked(Factor& F, int precision, cudaStream_t st) {
   const int64_t nu = (int64_t)F.m * F.ktot;
   if (precision != TLRMVN_FP64) TLR_CHECK(ensure_float_tiles(F, st));
-  if (precision == TLRMVN_FP32 && !(F.U32 && F.V32) && nu) {
+  if (precision == TLRMVN_FP32 + SIMT_COPIES && !(F.U32 && F.V32) && nu) {
     dfree(F.U32);
     dfree(F.V32);
     // the first factors of the float products, k-major (a k-step of them is one plain
@@ -582,41 +737,22 @@ static int ensure_copies_locked(Factor& F, int precision, cudaStream_t st) {
                                                          F.m, cntv, F.V32 + F.v32_off[i]);
     }
   }
-  if ((precision == TLRMVN_BF16_SHIFT || precision == TLRMVN_FP16_SHIFT) && !bf16_ready(F)) {
+  if ((precision == TLRMVN_FP32 || precision == TLRMVN_BF16_SHIFT || precision == TLRMVN_FP16_SHIFT) &&
+      !layout_ready(F))
+    TLR_CHECK(make_layout(F, st));
+  if (precision == TLRMVN_FP32 && !fp32_ready(F)) TLR_CHECK(make_fp32_copies(F, st));
+  if (precision == TLRMVN_BF16_SHIFT && !bf16_ready(F)) {
     // (a failed earlier attempt may have left some of these behind)
     dfree(F.U16);
     dfree(F.V16);
-    dfree(F.vmap16);
     dfree(F.B16x2);
-    // padded rank space: row tile i starts at a multiple of 64
     const int r = F.r, m = F.m;
-    F.kpad_off.assign(r + 1, 0);
-    int64_t kmax = 0;
-    for (int i = 0; i < r; i++) {
-      F.kpad_off[i + 1] = F.kpad_off[i] + (F.krow(i) + 63) / 64 * 64;
-      kmax = std::max(kmax, F.krow(i));
-    }
-    F.kw16 = std::max<int64_t>(F.kpad_off[r], 64);
-    F.kmax16 = std::max<int64_t>((kmax + 63) / 64 * 64, 64);
-    F.my16 = ((int64_t)m + 63) / 64 * 64;
     {
       const int64_t nb2 = (int64_t)r * m * 2 * F.my16;
       TLR_CHECK(dalloc(&F.B16x2, nb2));
       k_split_b16<<<blocks_for(nb2, 256), 256, 0, st>>>(F.B, m, F.my16, nb2, F.B16x2);
     }
     if (F.ktot) {
-      // vmap16: for each Vcat row, its column in the padded rank space
-      std::vector<int32_t> v16(F.ktot);
-      for (int j = 0; j < r; j++) {
-        int64_t row = F.kcol_off[j];
-        for (int i = j + 1; i < r; i++) {
-          int64_t local = 0;
-          for (int t = 0; t < j; t++) local += F.rank[(size_t)i * r + t];
-          for (int c = 0; c < F.rank[(size_t)i * r + j]; c++) v16[row++] = (int32_t)(F.kpad_off[i] + local + c);
-        }
-      }
-      TLR_CHECK(dalloc(&F.vmap16, (size_t)F.ktot));
-      TLR_CUDA(cudaMemcpyAsync(F.vmap16, v16.data(), v16.size() * 4, cudaMemcpyHostToDevice, st));
       std::vector<int64_t> kro(F.krow_off);
       int64_t* dkro = nullptr;
       TLR_CHECK(dalloc(&dkro, kro.size()));
@@ -752,12 +888,20 @@ static int64_t chunk_simt(const tlrmvn_opts& o, const Tuning& tu, int64_t S, int
   const double per = (double)(ktot + 2 * m) * es + 16.0;
   return round_chunk((int64_t)std::max(256.0, std::min((double)S, budget / per)), S);
 }
-static int64_t chunk_bf16(const tlrmvn_opts& o, const Tuning& tu, int64_t S, int64_t kw, int64_t ly) {
+// (float32 path: within 8 GiB, and passes of equal size that fit the three CTAs an SM holds -- a launch over one CTA
+// more than that would run twice as long)
+static int64_t chunk_tc(const tlrmvn_opts& o, const Tuning& tu, int64_t S, int64_t wrows, int64_t ly, bool f32, int sms) {
   if (o.sample_chunk > 0) return round_chunk(o.sample_chunk, S);
   if (tu.chunk > 0) return round_chunk(tu.chunk, S);
-  const double budget = 32.0 * (1ull << 30);
-  const double per = (double)kw * 2 + (double)ly * 2 + 16.0;
-  return round_chunk((int64_t)std::max(256.0, std::min((double)S, budget / per)), S);
+  const double budget = (f32 ? 8.0 : 32.0) * (1ull << 30);
+  const double per = (double)wrows * 2 + (double)ly * 2 + 16.0;
+  int64_t C = (int64_t)std::max(256.0, std::min((double)S, budget / per));
+  if (f32) {
+    C = std::min(C, (int64_t)3 * sms * STC_NS);
+    const int64_t passes = (S + C - 1) / C;
+    C = (S + passes - 1) / passes;
+  }
+  return round_chunk(C, S);
 }
 
 // Limits in factor order, in float64 and (for the float paths) float32.
@@ -863,24 +1007,35 @@ static SweepShape sweep_shape(int64_t C, int mt, int forced) {
   memo = best;
   return best;
 }
-// The whole-tile sweep of the BF16- and FP16-shift paths, by (periodisation,
-// one-sided) flags and operand type.
+// The whole-tile sweep by its arithmetic, stages and (periodisation, one-sided) flags.  Stages: a launch that leaves
+// at most two CTAs to an SM takes four (float32: three; its products wait for copies, and shared memory is idle);
+// else the 16-bit paths take one, so that six CTAs share an SM, and the float32 path two (three CTAs, by its TMEM
+// columns four at most).
 typedef void (*SweepTcKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                               const CUtensorMap, const CUtensorMap, const SweepTcArgs, const SweepTcLaunch);
-static SweepTcKernel sweep_tc_kernel(int flags, bool f16) {
-  static const SweepTcKernel table[8] = {
-      k_sweep_tc<0, false>, k_sweep_tc<SWEEP_PERIODIZE, false>, k_sweep_tc<SWEEP_ONE_SIDED, false>,
-      k_sweep_tc<SWEEP_PERIODIZE | SWEEP_ONE_SIDED, false>, k_sweep_tc<0, true>,
-      k_sweep_tc<SWEEP_PERIODIZE, true>, k_sweep_tc<SWEEP_ONE_SIDED, true>,
-      k_sweep_tc<SWEEP_PERIODIZE | SWEEP_ONE_SIDED, true>};
-  return table[((flags & SWEEP_PERIODIZE) ? 1 : 0) | ((flags & SWEEP_ONE_SIDED) ? 2 : 0) | (f16 ? 4 : 0)];
+template <int MODE, int NST>
+static SweepTcKernel sweep_tc_variant(int f) {
+  static const SweepTcKernel t[4] = {k_sweep_tc<0, MODE, NST>, k_sweep_tc<SWEEP_PERIODIZE, MODE, NST>,
+                                     k_sweep_tc<SWEEP_ONE_SIDED, MODE, NST>,
+                                     k_sweep_tc<SWEEP_PERIODIZE | SWEEP_ONE_SIDED, MODE, NST>};
+  return t[f];
 }
-// Dynamic shared memory of a whole-tile sweep launch with `ctas` CTAs per SM: the
-// kernel's own need, or more so that no more than `ctas` fit (tuning).
-static size_t sweep_tc_launch_smem(int ctas) {
-  size_t need = sweep_tc_smem_bytes();
+static SweepTcKernel sweep_tc_kernel(int flags, int mode, int nst) {
+  const int f = ((flags & SWEEP_PERIODIZE) ? 1 : 0) | ((flags & SWEEP_ONE_SIDED) ? 2 : 0);
+  if (mode == STC_FP32) return nst == 3 ? sweep_tc_variant<STC_FP32, 3>(f) : sweep_tc_variant<STC_FP32, 2>(f);
+  if (mode == STC_FP16) return nst == 4 ? sweep_tc_variant<STC_FP16, 4>(f) : sweep_tc_variant<STC_FP16, 1>(f);
+  return nst == 4 ? sweep_tc_variant<STC_BF16, 4>(f) : sweep_tc_variant<STC_BF16, 1>(f);
+}
+static int sweep_tc_stages(int mode, int64_t ctas, int sms) {
+  const bool few = ctas <= 2 * (int64_t)sms;
+  return mode == STC_FP32 ? (few ? 3 : 2) : (few ? 4 : 1);
+}
+// Dynamic shared memory of a whole-tile sweep launch: the kernel's own need, or (tuning, one-stage launches) more, so
+// that no more than `ctas` fit an SM.
+static size_t sweep_tc_launch_smem(int ctas, int mode, int nst) {
+  size_t need = sweep_tc_smem_bytes(mode, nst);
   ctas = std::min(std::max(ctas, 1), 6);
-  if (ctas < 6) {
+  if (nst == 1 && ctas < 6) {
     int dev = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
@@ -893,10 +1048,6 @@ static size_t sweep_tc_launch_smem(int ctas) {
 static int set_sweep_smem(int sub) {
   for (int flags = 0; flags < 8; flags++)
     TLR_CHECK(raise_smem_limit((const void*)sweep_kernel(flags), sweep_smem_bytes(sub, 256)));
-  for (int t = 0; t < 8; t++)  // every (periodisation, one-sided, operand type) variant
-    TLR_CHECK(raise_smem_limit((const void*)sweep_tc_kernel(((t & 1) ? SWEEP_PERIODIZE : 0) |
-                                                                ((t & 2) ? SWEEP_ONE_SIDED : 0), (t & 4) != 0),
-                               sweep_tc_launch_smem(1)));
   return TLRMVN_OK;
 }
 
@@ -912,10 +1063,11 @@ struct TcOperands {
   int64_t ldw = 0;
   int64_t my;
   int* err;
-  bool f16 = false;  // fp16 operands (FP16-shift path), else bf16
+  int mode = STC_BF16;
+  int sms = 1;
 };
 
-// Whole diagonal tile i on the BF16-shift path: one launch of k_sweep_tc
+// Whole diagonal tile i: one launch of k_sweep_tc
 // (low-rank shifts, in-tile coupling, sweep and projections).
 static void sweep_tile_tc(const Factor& F, int i, const Lims& L, const float* rs32, const uint64_t* dD,
                           int64_t c0, int64_t N, int64_t Cc, int periodize, unsigned short* Ys, int64_t ldys,
@@ -939,8 +1091,14 @@ static void sweep_tile_tc(const Factor& F, int i, const Lims& L, const float* rs
   t.kc = (int)F.kcol(i);
   t.ldw = tco.ldw;
   t.vmap = F.vmap16 ? F.vmap16 + F.kcol_off[i] : nullptr;
-  t.wscale = (tco.f16 && F.wscale16) ? F.wscale16 + F.kcol_off[i] : nullptr;
-  t.tscale = tco.f16 ? F.inv_g16 : 1.0f;
+  t.wscale = nullptr;
+  if (tco.mode == STC_FP16 && F.wscale16) t.wscale = F.wscale16 + F.kcol_off[i];
+  if (tco.mode == STC_FP32 && F.wscale32) t.wscale = F.wscale32 + F.kcol_off[i];
+  t.tscale = tco.mode == STC_FP16 ? F.inv_g16 : 1.0f;
+  t.rscale = tco.mode == STC_FP32 ? F.rscale32 + (size_t)i * m : nullptr;
+  t.wlo = (int)F.kw16;
+  t.ulo = (int)F.kmax16;
+  t.vlo = (int)F.my16;
   t.err = tco.err;
   SweepTcLaunch d;
   d.D = dD;
@@ -957,13 +1115,15 @@ static void sweep_tile_tc(const Factor& F, int i, const Lims& L, const float* rs
   d.first = (i == 0);
   const int flags = (periodize ? SWEEP_PERIODIZE : 0) | (L.one_sided ? SWEEP_ONE_SIDED : 0);
   pf.begin(TLRMVN_KC_DIAG);
-  launch_pdl(sweep_tc_kernel(flags, tco.f16), dim3((unsigned)((Cc + STC_NS - 1) / STC_NS)), dim3(STC_NS),
-             sweep_tc_launch_smem(tu.tc_ctas), st, tco.mapY32, tco.mapB32, tco.mapW, tco.mapU64, tco.mapY64, tco.mapV64, t,
-             d);
+  const int64_t ctas = (Cc + STC_NS - 1) / STC_NS;
+  const int nst = sweep_tc_stages(tco.mode, ctas, tco.sms);
+  launch_pdl(sweep_tc_kernel(flags, tco.mode, nst), dim3((unsigned)ctas), dim3(STC_NS),
+             sweep_tc_launch_smem(tu.tc_ctas, tco.mode, nst), st, tco.mapY32, tco.mapB32, tco.mapW, tco.mapU64, tco.mapY64,
+             tco.mapV64, t, d);
   pf.end();
 }
 
-// Float sweep of diagonal tile i (FP32 path), `sub` variables at a time.  Before
+// Float sweep of diagonal tile i (general float32 path), `sub` variables at a time.  Before
 // each sub-tile q > 0, the coupling to the tile's earlier sub-tiles,
 // B_i[q, <q] y_i[<q], is added to the limit shifts Dl (variable-major, ld C) by
 // a dense SIMT product; y goes to Yv (float, variable-major, ld C).  has_shift:
@@ -1135,53 +1295,62 @@ static int run_chunks(Factor& F, const T* Bt, const T* Ut, const T* Vt, const Li
   return TLRMVN_OK;
 }
 
-// BF16-shift integrand: one whole-tile sweep per diagonal tile (k_sweep_tc): the
-// low-rank shifts, the in-tile coupling between 64-variable sub-tiles (split
-// bf16 operands: x = hi + lo, hi*hi + hi*lo + lo*hi, relative error ~1e-5) and
-// the projections on tcgen05 with fp32 accumulation in TMEM, the sweep itself in
-// float32.  Layouts (C = samples in the chunk):
-//   W16  kw16 x ldw bf16, rank-major (ldw = C rounded up to 64): row k holds
+// The integrand of the float32, BF16- and FP16-shift paths: one whole-tile sweep per diagonal tile (k_sweep_tc): the
+// low-rank shifts, the in-tile coupling between 64-variable sub-tiles and the projections on tcgen05 with fp32
+// accumulation in TMEM, the sweep itself in float32.  Layouts (C = samples in the chunk):
+//   W16  kw16 x ldw 16-bit, rank-major (ldw = C rounded up to 64): row k holds
 //        projection k of every sample (written as whole rows by the tile that
-//        owns the rank, read as an MN-major operand by the later tiles' shifts)
-//   Y16  C x 2 my16 bf16, sample-major: the tile's y (hi) in columns [0, my16) and
-//        bf16(y - hi) in [my16, 2 my16)
-static int run_chunks_bf16(Factor& F, const Lims& L, double nu, const tlrmvn_opts& o, const Tuning& tu,
-                           const uint64_t* dD, double* logP, Scratch& sc, cudaStream_t st, Prof& pf) {
+//        owns the rank, read as an MN-major operand by the later tiles' shifts);
+//        float32 path: hi parts, then as many rows of lo parts
+//   Y16  C x 2 my16 16-bit, sample-major: the tile's y (hi) in columns [0, my16) and
+//        its lo part in [my16, 2 my16)
+// out_of_range (float32 path): set when a y or a projection left fp16's range, and the results are not to be used.
+static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts& o, const Tuning& tu,
+                         const uint64_t* dD, double* logP, Scratch& sc, cudaStream_t st, Prof& pf, bool* out_of_range) {
   const int64_t M = o.n_shifts, N = o.n_points, S = M * N;
   const int m = F.m;
-  const bool f16 = o.precision == TLRMVN_FP16_SHIFT;
+  TcOperands tco;
+  const int mode = o.precision == TLRMVN_FP32 ? STC_FP32 : (o.precision == TLRMVN_FP16_SHIFT ? STC_FP16 : STC_BF16);
+  const bool f16 = mode != STC_BF16;
+  const int64_t wrows = mode == STC_FP32 ? 2 * F.kw16 : F.kw16;
+  int dev = 0;
+  TLR_CUDA(cudaGetDevice(&dev));
+  TLR_CUDA(cudaDeviceGetAttribute(&tco.sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t ly = 2 * F.my16;  // Y16 row: hi halves, then lo halves
-  const int64_t C = chunk_bf16(o, tu, S, F.kw16, ly);
+  const int64_t C = chunk_tc(o, tu, S, wrows, ly, mode == STC_FP32, tco.sms);
   unsigned short *W = nullptr, *Y = nullptr;
   float* rs32 = nullptr;
   int* err = nullptr;
   const int64_t ldw = (C + 63) / 64 * 64;
-  TLR_CHECK(sc.get(&W, (size_t)F.kw16 * ldw));
+  TLR_CHECK(sc.get(&W, (size_t)wrows * ldw));
   TLR_CHECK(sc.get(&Y, (size_t)ly * C));
-  TLR_CHECK(sc.get(&err, 1));
+  TLR_CHECK(sc.get(&err, 2));
   const bool mvt = std::isfinite(nu);
   if (mvt) TLR_CHECK(sc.get(&rs32, (size_t)C));
   // padding columns of W and Y must hold finite values: they meet zero operand columns
-  TLR_CUDA(cudaMemsetAsync(W, 0, (size_t)F.kw16 * ldw * 2, st));
+  TLR_CUDA(cudaMemsetAsync(W, 0, (size_t)wrows * ldw * 2, st));
   TLR_CUDA(cudaMemsetAsync(Y, 0, (size_t)ly * C * 2, st));
-  TLR_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
+  TLR_CUDA(cudaMemsetAsync(err, 0, 2 * sizeof(int), st));
 
   // tensor maps: A operands (samples) take 128-row boxes, B operands 64-row boxes
   //   shift      T = W16^T (A, MN-major) x U16 rows (B)
   //   coupling   T += Y16 rows (A, hi/lo) x B16x2 rows (B, hi/lo)
   //   projection T = Y16 rows (A, hi) x V16 rows (B)
-  TcOperands tco;
-  tco.f16 = f16;
-  const void* B2 = f16 ? (const void*)F.B16x2h : (const void*)F.B16x2;
-  TLR_CHECK(make_map(&tco.mapB32, B2, ly, (uint64_t)F.r * m, ly * 2, 64, 32, f16));
+  //   (float32 path: W16 as hi/lo, U, V and B in three parts, in boxes 32 ranks or variables deep)
+  tco.mode = mode;
+  const void* B2 = mode == STC_FP32 ? (const void*)F.Bs16 : (f16 ? (const void*)F.B16x2h : (const void*)F.B16x2);
+  const uint32_t deep = mode == STC_FP32 ? 32 : 64;
+  const int64_t lb = (mode == STC_FP32 ? 3 : 2) * F.my16;
+  TLR_CHECK(make_map(&tco.mapB32, B2, lb, (uint64_t)F.r * m, lb * 2, 64, 32, f16));
   TLR_CHECK(make_map(&tco.mapY32, Y, ly, C, ly * 2, STC_NS, 32, f16));
   TLR_CHECK(make_map(&tco.mapY64, Y, ly, C, ly * 2, STC_NS, 64, f16));
-  TLR_CHECK(make_map(&tco.mapW, W, ldw, F.kw16, ldw * 2, 64, 64, f16));
+  TLR_CHECK(make_map(&tco.mapW, W, ldw, wrows, ldw * 2, deep, 64, f16));
   if (F.ktot) {
-    const void* U = f16 ? (const void*)F.U16h : (const void*)F.U16;
-    const void* V = f16 ? (const void*)F.V16h : (const void*)F.V16;
-    TLR_CHECK(make_map(&tco.mapU64, U, F.kmax16, (uint64_t)F.r * m, F.kmax16 * 2, 64, 64, f16));
-    TLR_CHECK(make_map(&tco.mapV64, V, F.my16, F.ktot, F.my16 * 2, 64, 64, f16));
+    const void* U = mode == STC_FP32 ? (const void*)F.Us16 : (f16 ? (const void*)F.U16h : (const void*)F.U16);
+    const void* V = mode == STC_FP32 ? (const void*)F.Vs16 : (f16 ? (const void*)F.V16h : (const void*)F.V16);
+    const int64_t lu = (mode == STC_FP32 ? 3 : 1) * F.kmax16, lv = (mode == STC_FP32 ? 3 : 1) * F.my16;
+    TLR_CHECK(make_map(&tco.mapU64, U, lu, (uint64_t)F.r * m, lu * 2, 64, deep, f16));
+    TLR_CHECK(make_map(&tco.mapV64, V, lv, F.ktot, lv * 2, 64, deep, f16));
   } else {
     tco.mapU64 = tco.mapW;  // (never read: no tile has ranks)
     tco.mapV64 = tco.mapW;
@@ -1190,7 +1359,12 @@ static int run_chunks_bf16(Factor& F, const Lims& L, double nu, const tlrmvn_opt
   tco.ldw = ldw;
   tco.my = F.my16;
   tco.err = err;
-  TLR_CHECK(set_sweep_smem(64));
+  for (int f = 0; f < 4; f++)
+    for (int few = 0; few < 2; few++) {
+      const int nst = sweep_tc_stages(mode, few ? 1 : INT64_MAX, 1);
+      const int flags = ((f & 1) ? SWEEP_PERIODIZE : 0) | ((f & 2) ? SWEEP_ONE_SIDED : 0);
+      TLR_CHECK(raise_smem_limit((const void*)sweep_tc_kernel(flags, mode, nst), sweep_tc_launch_smem(1, mode, nst)));
+    }
 
   for (int64_t c0 = 0; c0 < S; c0 += C) {
     const int64_t Cc = std::min(C, S - c0);
@@ -1204,10 +1378,12 @@ static int run_chunks_bf16(Factor& F, const Lims& L, double nu, const tlrmvn_opt
       sweep_tile_tc(F, i, L, rs32, dD, c0, N, Cc, o.periodize, Y, ly, logP, tco, tu, st, pf);
     TLR_CUDA(cudaGetLastError());
   }
-  int herr = 0;
-  TLR_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  int herr[2] = {0, 0};
+  TLR_CUDA(cudaMemcpyAsync(herr, err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
   TLR_CUDA(cudaStreamSynchronize(st));
-  if (herr) return fail(TLRMVN_E_TIMEOUT, "tensor-core kernel gave up waiting (code " + std::to_string(herr) + ")");
+  if (herr[0])
+    return fail(TLRMVN_E_TIMEOUT, "tensor-core kernel gave up waiting (code " + std::to_string(herr[0]) + ")");
+  *out_of_range = herr[1] != 0;
   return TLRMVN_OK;
 }
 
@@ -1217,19 +1393,25 @@ int64_t prob_scratch_bytes(const Factor& F, const tlrmvn_opts& o) {
   const int64_t M = o.n_shifts, N = o.n_points, S = M * N, n = F.n, m = F.m;
   const Tuning tu = F.tuning(o.precision);
   int64_t bytes = n * (8 * 2 + 4 * 2) + (M * (n + 1) + STC_DPAD) * 8 + M * 8 + S * 8 + 256;
-  if (o.precision == TLRMVN_BF16_SHIFT || o.precision == TLRMVN_FP16_SHIFT) {
+  int64_t simt = 0, tc = 0;
+  if (o.precision != TLRMVN_FP64) {
+    const bool f32 = o.precision == TLRMVN_FP32;
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int64_t kw = 0;
     for (int i = 0; i < F.r; i++) kw += (F.krow(i) + 63) / 64 * 64;
-    kw = std::max<int64_t>(kw, 64);
+    kw = std::max<int64_t>(kw, 64) * (f32 ? 2 : 1);
     const int64_t my = (m + 63) / 64 * 64, ly = 2 * my;
-    const int64_t C = chunk_bf16(o, tu, S, kw, ly);
-    bytes += C * (kw * 2 + ly * 2 + 4);
-  } else {
+    const int64_t C = chunk_tc(o, tu, S, kw, ly, f32, sms);
+    tc = C * (kw * 2 + ly * 2 + 4);
+  }
+  if (o.precision == TLRMVN_FP64 || o.precision == TLRMVN_FP32) {  // (float32: should a y leave fp16's range)
     const int64_t es = o.precision == TLRMVN_FP64 ? 8 : 4;
     const int64_t C = chunk_simt(o, tu, S, F.ktot, m, es);
-    bytes += C * ((F.ktot + 2 * m) * es + 8);
+    simt = C * ((F.ktot + 2 * m) * es + 8);
   }
-  return bytes;
+  return bytes + std::max(simt, tc);
 }
 
 int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, const tlrmvn_opts& o,
@@ -1281,10 +1463,17 @@ int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, co
   const Tuning tu = F.tuning(o.precision);
   if (o.precision == TLRMVN_FP64)
     s = run_chunks<double, double>(F, F.B, F.Ucat, F.Vcat, L, nu, o, tu, dD, logP, sc, st, pf);
-  else if (o.precision == TLRMVN_FP32)
-    s = run_chunks<float, float>(F, F.B32, F.U32, F.V32, L, nu, o, tu, dD, logP, sc, st, pf);
-  else
-    s = run_chunks_bf16(F, L, nu, o, tu, dD, logP, sc, st, pf);
+  else {
+    bool out_of_range = false;
+    {
+      Scratch own(st);
+      s = run_chunks_tc(F, L, nu, o, tu, dD, logP, own, st, pf, &out_of_range);
+    }
+    if (s == TLRMVN_OK && out_of_range) {  // limits tens of thousands of standard deviations out
+      TLR_CHECK(ensure_copies(F, TLRMVN_FP32 + SIMT_COPIES, st));
+      s = run_chunks<float, float>(F, (const float*)nullptr, F.U32, F.V32, L, nu, o, tu, dD, logP, sc, st, pf);
+    }
+  }
   TLR_CHECK(s);
   pf.begin(TLRMVN_KC_REDUCE);
   k_shift_reduce<<<(unsigned)M, 256, 0, st>>>(logP, N, ell);

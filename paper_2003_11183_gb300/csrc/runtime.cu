@@ -103,7 +103,6 @@ Factor::~Factor() {
   dfree(Ucat);
   dfree(Vcat);
   dfree(vmap);
-  dfree(B32);
   dfree(BT32);
   dfree(inv32);
   dfree(band32);
@@ -118,6 +117,11 @@ Factor::~Factor() {
   dfree(V16h);
   dfree(B16x2h);
   dfree(wscale16);
+  dfree(Us16);
+  dfree(Vs16);
+  dfree(Bs16);
+  dfree(rscale32);
+  dfree(wscale32);
   dfree(Q);
   dfree(dperm);
 }

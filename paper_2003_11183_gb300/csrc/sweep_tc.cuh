@@ -50,6 +50,23 @@
 
 namespace tlrmvn {
 
+// Arithmetic of the products:
+//   STC_BF16, STC_FP16  16-bit operands, the coupling's split into hi and lo parts (the BF16- and FP16-shift paths)
+//   STC_FP32            every operand split into fp16 parts: the FP32 path's.  The tensor cores accumulate float32
+//                       sums by truncation, which in one accumulator shifts a sum of 512 terms by about 1e-6 of
+//                       itself, always towards zero (ten times the error of float32 FMAs).  So the factor's operands
+//                       are scaled by powers of two into [-1, 1] (each row of U and of the tile's part left of the
+//                       sub-tile, each row of V) and the projections to order 1, and hi parts are rounded to multiples
+//                       of 2^-10: the products hi*hi are multiples of 2^-20 and their sums, below 16, exact; the
+//                       other products (hi*lo, lo*hi, lo*lo), 2^-10 of those, have an accumulator of their own (128
+//                       TMEM columns).  The factor's operands have a third part, and hi*third is added there: their
+//                       rounding to two parts, the same for all samples, was the largest error left.  Errors of
+//                       the samples' logs against 64 bits (rms; float32 FMAs before in brackets): n = 8,192, tiles
+//                       of 256: 1.9e-5 (2.7e-5); n = 1,024, tiles of 128, nu = 7: 4.5e-6 (6.3e-6); n = 2,048, tiles
+//                       of 512: 1.0e-5 (1.3e-5).  Times against the float32 FMA products and sweeps: n = 16,384, 20
+//                       x 5,000 samples: 55.0 -> 25.9 ms a solve; n = 4,096, nu = 7, 10 x 1,000: 4.41 -> 2.35 ms; 64
+//                       batched problems, 10 x 2,000: 87.9 -> 18.8 ms.
+enum StcMode { STC_BF16 = 0, STC_FP16 = 1, STC_FP32 = 2 };
 constexpr int STC_SUB = 64;   // variables per sub-tile
 constexpr int STC_NS = 128;   // samples per CTA (TMEM lanes)
 constexpr int STC_KB = 32;    // K depth of a coupling k-block
@@ -82,9 +99,16 @@ struct Op16<true> {
   static __device__ __forceinline__ unsigned short one(float a) { return __half_as_ushort(__float2half_rn(a)); }
 };
 
+// hi and lo fp16 parts of two floats for STC_FP32, packed low word first: hi a multiple of 2^-10 (of more above 2)
+__device__ __forceinline__ void split_f32(float a, float b, uint32_t& hi, uint32_t& lo) {
+  float ha, hb, la, lb;
+  hi = Op16<true>::pack((a + 12288.0f) - 12288.0f, (b + 12288.0f) - 12288.0f, ha, hb);
+  lo = Op16<true>::pack(a - ha, b - hb, la, lb);
+}
+
 // Per variable: [0, 16) the window column (for an even variable v B[v+2+k][v] at k < 14 and B[v+1][v] at 14,
 // so that the pair update of the sweep reads aligned pairs; for an odd one B[v+1+k][v] at k < 15),
-// then a, b, 1 / B_vv and one spare, the lattice generator (8 bytes) and 8 spare bytes.
+// then a, b, 1 / B_vv and (STC_FP32) the inverse of its row's scale, the lattice generator (8 bytes) and 8 spare bytes.
 constexpr int STC_REC = 24;  // floats
 // Entries after the lattice shifts' table: a sample's row is read up to three entries past a tile's last variable.
 constexpr int STC_DPAD = 4;
@@ -107,7 +131,9 @@ struct SweepTcArgs {
   const float* wscale;    // FP16 path: per column rank, the factor applied to a projection before it is
                           // stored (the inverse of the per-tile scales of U and V); null on the BF16 path
   float tscale;           // FP16 path: 1 / g, undoing the products' global scale g where the sweep reads them
-  int* err;
+  const float* rscale;    // STC_FP32: per variable of the tile, the inverse of its row's scale
+  int wlo, ulo, vlo;      // STC_FP32: the lo parts' row offset in W, x offsets in the U and V maps (third parts: twice)
+  int* err;               // [0] a bounded wait's code; [1] (STC_FP32) a y or a projection beyond fp16's range
 };
 using StcProjCfg = tc::Cfg<64, false, false, 64, 1>;  // projection k-block: y rows x V rows, 64 deep
 static_assert(StcProjCfg::SB == StcCfg::SB, "a projection k-block fills the same stage");
@@ -115,11 +141,16 @@ using StcShiftCfg = tc::Cfg<64, false, true, 64, 1>;  // shift k-block: W (MN-ma
 static_assert(StcShiftCfg::SB == StcCfg::SB, "a shift k-block fills the same stage");
 
 constexpr int STC_TRI = 6 * 256;  // floats: the 16 x 16 blocks (ub, vb), ub < vb, at vb (vb - 1) / 2 + ub
-// [stage][records][triangle blocks][barriers, TMEM slot] (the dynamic shared memory starts 1 KB-aligned: the
+// [NST stages][records][triangle blocks][barriers, TMEM slot] (the dynamic shared memory starts 1 KB-aligned: the
 // kernels have no static shared memory, and the system's own part is 1 KB)
-__host__ __device__ constexpr size_t sweep_tc_smem_bytes() {
-  return (size_t)StcCfg::SB + (STC_SUB * STC_REC + STC_TRI) * sizeof(float) + 64;
+__host__ __device__ constexpr uint32_t stc_stage_bytes(int mode) {
+  return StcCfg::SB + (mode == STC_FP32 ? StcCfg::B_BYTES : 0);  // (the third part of the factor's operand)
 }
+__host__ __device__ constexpr size_t sweep_tc_smem_bytes(int mode, int nst) {
+  return (size_t)nst * stc_stage_bytes(mode) + (STC_SUB * STC_REC + STC_TRI) * sizeof(float) + 128;
+}
+// TMEM columns of a CTA: the sums (and y) of a sub-tile, and STC_FP32's second accumulator
+__host__ __device__ constexpr uint32_t stc_cols(int mode) { return mode == STC_FP32 ? 2 * STC_SUB : STC_SUB; }
 
 // Shared-memory layout and per-CTA state of the whole-tile sweep (set up once per
 // kernel: a persistent kernel runs many tiles through the same stage, barriers
@@ -128,10 +159,10 @@ struct StcCta {
   unsigned char* stage;
   float* rec;            // the sub-tile's records
   float* tri;            // its triangle blocks
-  uint64_t* full;        // the stage's copies landed
-  uint64_t* freeb;       // the products reading the stage are done
+  uint64_t* full;        // [NST] the stage's copies landed
+  uint64_t* freeb;       // [NST] the products reading the stage are done
   uint32_t tmem;         // first of the CTA's TMEM columns
-  uint32_t* phases;      // thread 0's barrier parities (bit 0: full, bit 1: freeb)
+  uint32_t* count;       // k-blocks gone through the stages so far (block i uses stage i mod NST)
   int* abort_flag;
   int* item;             // (persistent kernel) the work item
 };
@@ -155,43 +186,113 @@ __device__ __forceinline__ void tmem_ld16(uint32_t (&r)[16], uint32_t addr) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// Thread 0's ring of NST stages.  load(i, st) starts the copies of k-block i into a stage, mma(i, st) issues its
+// products.  Runs blocks [0, nk), of which the first `pre` were loaded before, and waits for all products; `count`
+// numbers the blocks over the CTA's life.  Returns false (every copy and product in flight waited for, bounded) when
+// a wait expired.
+template <int NST, typename Load, typename Mma>
+__device__ __forceinline__ bool stc_ring(const StcCta& k, uint32_t& count, int nk, int pre, int* err, Load load,
+                                         Mma mma) {
+  int issued = pre, kb = 0;
+  bool ok = true;
+  for (; kb < nk; kb++) {
+    for (; issued < nk && issued < kb + NST; issued++) {
+      const uint32_t i = count + (uint32_t)issued;
+      if (i >= NST && !tc::mbar_wait(k.freeb + i % NST, (i / NST - 1) & 1, err, 9)) {
+        ok = false;
+        break;
+      }
+      load(issued, i % NST);
+    }
+    const uint32_t i = count + (uint32_t)kb;
+    if (!ok || !tc::mbar_wait(k.full + i % NST, (i / NST) & 1, err, 8)) {
+      ok = false;
+      break;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    mma(kb, i % NST);
+    tc::mma_commit(k.freeb + i % NST);
+  }
+  if (kb > 0) {  // (products complete in order)
+    const uint32_t i = count + (uint32_t)kb - 1;
+    if (!tc::mbar_wait(k.freeb + i % NST, (i / NST) & 1, err, 9)) ok = false;
+  }
+  if (!ok)
+    for (; kb < issued; kb++) {
+      const uint32_t i = count + (uint32_t)kb;
+      tc::mbar_wait(k.full + i % NST, (i / NST) & 1, err, 5);
+    }
+  count += (uint32_t)nk;
+  return ok;
+}
+
 // One diagonal tile for the CTA's samples: the low-rank shifts and in-tile
 // coupling on tcgen05, the float sweep of eq. 2, the projections.  act: the thread's
 // sample exists (else it shadows one and writes nothing); Ds: its row of lattice shifts
 // at the tile's first variable (read up to three entries past the tile); ks: its point
 // index; rs: its MVT scale (1 for MVN).  The tile's log P is added to (prod, pe, lsum).
 // Returns false when a bounded wait expired.
-template <int FLAGS, bool F16>
+template <int FLAGS, int MODE, int NST>
 __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensorMap* mapB, const CUtensorMap* mapW,
                                          const CUtensorMap* mapU, const CUtensorMap* mapY64, const CUtensorMap* mapV,
                                          const SweepTcArgs& p, const StcCta& k, const StcPlace& pl, const bool act,
                                          const uint64_t* Ds, const uint32_t ks, const float rs, float& prod,
                                          float& lsum, int& pe) {
   constexpr bool PER = FLAGS & SWEEP_PERIODIZE, ONE = FLAGS & SWEEP_ONE_SIDED;
+  constexpr bool F16 = MODE != STC_BF16, SPLIT = MODE == STC_FP32;
   using Op = Op16<F16>;
   constexpr uint32_t ID_C = F16 ? StcCfg::IDESC_F16 : StcCfg::IDESC;
   constexpr uint32_t ID_S = F16 ? StcShiftCfg::IDESC_F16 : StcShiftCfg::IDESC;
   constexpr uint32_t ID_P = F16 ? StcProjCfg::IDESC_F16 : StcProjCfg::IDESC;
   constexpr uint32_t CA = StcCfg::A_BYTES, CHALF = StcCfg::HALF, SA = StcShiftCfg::A_BYTES, PA = StcProjCfg::A_BYTES;
-  constexpr uint32_t SB = StcCfg::SB;
+  constexpr uint32_t SB = stc_stage_bytes(MODE), CB3 = StcCfg::SB;  // (a stage; its third B part)
+  constexpr int KS = SPLIT ? STC_KB : 64;  // depth of a shift or projection k-block
   unsigned char* stage = k.stage;
-  uint64_t* full = k.full;
-  uint64_t* freeb = k.freeb;
   volatile int* abort_flag = k.abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int mt = p.mt;
   const uint32_t tmem = k.tmem;
   const uint32_t tl = tmem + ((uint32_t)(32 * warp) << 16);  // this warp's 32 lanes
-  const int nks = (p.kr + 63) / 64;
-  // the copies of shift k-block kb: two 64-sample MN-major boxes of W, one box of U rows
-  auto load_shift = [&](int kb, int q0) {
-    tc::mbar_expect_tx(full, SB);
-    const int y = pl.wy + p.krow0 + kb * 64;
-    tc::tma_load_2d(stage, mapW, full, pl.wx, y);
-    tc::tma_load_2d(stage + SA / 2, mapW, full, pl.wx + 64, y);
-    tc::tma_load_2d(stage + SA, mapU, full, kb * 64, p.urow0 + q0);
+  const int nks = (p.kr + KS - 1) / KS;
+  // the copies of shift k-block kb.  16-bit: two 64-sample MN-major boxes of W (64 ranks), one box of U rows.  Split:
+  // [W hi: two 64-sample boxes of 32 ranks][U hi][W lo][U lo][U third]
+  auto load_shift = [&](int kb, int q0, uint32_t st) {
+    unsigned char* d = stage + st * SB;
+    uint64_t* bar = k.full + st;
+    tc::mbar_expect_tx(bar, SB);
+    const int y = pl.wy + p.krow0 + kb * KS;
+    if constexpr (SPLIT) {
+#pragma unroll
+      for (int h = 0; h < 2; h++) {
+        tc::tma_load_2d(d + h * CHALF, mapW, bar, pl.wx, y + h * p.wlo);
+        tc::tma_load_2d(d + h * CHALF + CA / 2, mapW, bar, pl.wx + 64, y + h * p.wlo);
+        tc::tma_load_2d(d + h * CHALF + CA, mapU, bar, kb * KS + h * p.ulo, p.urow0 + q0);
+      }
+      tc::tma_load_2d(d + CB3, mapU, bar, kb * KS + 2 * p.ulo, p.urow0 + q0);
+    } else {
+      tc::tma_load_2d(d, mapW, bar, pl.wx, y);
+      tc::tma_load_2d(d + SA / 2, mapW, bar, pl.wx + 64, y);
+      tc::tma_load_2d(d + SA, mapU, bar, kb * 64, p.urow0 + q0);
+    }
+  };
+  // the products of a split stage [A hi][B hi][A lo][B lo]([B third]), 32 deep: A's descriptors and their advance per 16-deep step
+  auto mma_split = [&](uint64_t ah, uint64_t al, uint64_t astep, uint32_t sa, uint32_t idesc, bool first) {
+    const uint64_t bh = tc::sdesc<STC_KB>(sa + CA), bl = tc::sdesc<STC_KB>(sa + CHALF + CA);
+#pragma unroll
+    for (int kk = 0; kk < STC_KB / 16; kk++) {
+      const uint64_t oa = astep * (uint64_t)kk, ob = (uint64_t)(2 * kk);  // 32 bytes per 16-deep step of B
+      const uint32_t acc = (!first || kk > 0) ? 1u : 0u;
+      tc::mma_f16(tmem, ah + oa, bh + ob, idesc, acc);
+      tc::mma_f16(SPLIT ? tmem + STC_SUB : tmem, ah + oa, bl + ob, idesc, SPLIT ? acc : 1u);
+      tc::mma_f16(SPLIT ? tmem + STC_SUB : tmem, al + oa, bh + ob, idesc, 1u);
+      if constexpr (SPLIT) {
+        tc::mma_f16(tmem + STC_SUB, al + oa, bl + ob, idesc, 1u);
+        tc::mma_f16(tmem + STC_SUB, ah + oa, tc::sdesc<STC_KB>(sa + CB3) + ob, idesc, 1u);
+      }
+    }
   };
 
+  int pre = 0;  // (thread 0) shift k-blocks of the coming sub-tile already under way
   for (int q0 = 0; q0 < mt; q0 += STC_SUB) {
     const int mq = min(STC_SUB, mt - q0);
     // every thread is past the previous sub-tile's reads of the records and its TMEM accesses
@@ -202,7 +303,8 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
         const int v = t / 6, c = t - v * 6;
         const float* src = p.rec + (int64_t)(q0 + v) * STC_REC + 4 * c;
         if (c == 4)
-          reinterpret_cast<float4*>(k.rec)[t] = make_float4(p.a[q0 + v], p.b[q0 + v], __ldg(src + 2), 0.0f);
+          reinterpret_cast<float4*>(k.rec)[t] =
+              make_float4(p.a[q0 + v], p.b[q0 + v], __ldg(src + 2), SPLIT ? __ldg(p.rscale + q0 + v) : 0.0f);
         else
           cp_async16(reinterpret_cast<float4*>(k.rec) + t, src, 16);
       }
@@ -217,62 +319,50 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
       cp_async_wait<0>();
     }
     if ((q0 > 0 || p.kr > 0) && tid == 0) {
-      // T = W[ranks of row tile i, samples]^T U_i[q0 + v, ranks]^T     (the low-rank shifts, 64-deep stages)
+      // T = W[ranks of row tile i, samples]^T U_i[q0 + v, ranks]^T     (the low-rank shifts)
       //   + y[:, <q0] B_i[q0 + v, <q0]^T                              (the coupling, 32-deep split stages)
-      const uint32_t sa = tc::smem_u32(stage);
-      const uint64_t dbh = tc::sdesc<STC_KB>(sa + CA), dbl = tc::sdesc<STC_KB>(sa + CHALF + CA);
-      const uint64_t dah = tc::sdesc<STC_KB>(sa), dal = tc::sdesc<STC_KB>(sa + CHALF);
-      const uint64_t du = tc::sdesc<64>(sa + SA), dw = tc::sdesc_mn(sa);
-      const int nk = nks + q0 / STC_KB;
-      uint32_t ph = *k.phases;
-      int bad = 0;  // 1: copies left in flight, 2: products left in flight
-      for (int kb = 0; kb < nk; kb++) {
-        if (kb < nks) {
-          if (kb > 0 || q0 == 0) load_shift(kb, q0);  // (the first one was copied during the sweep before)
-        } else {
-          tc::mbar_expect_tx(full, SB);
-          const int x = (kb - nks) * STC_KB;
-          tc::tma_load_2d(stage, mapY, full, x, pl.yrow);
-          tc::tma_load_2d(stage + CHALF, mapY, full, p.alo + x, pl.yrow);
-          tc::tma_load_2d(stage + CA, mapB, full, x, p.brow0 + q0);
-          tc::tma_load_2d(stage + CHALF + CA, mapB, full, p.blo + x, p.brow0 + q0);
-        }
-        if (!tc::mbar_wait(full, ph & 1, p.err, 8)) {
-          bad = 1;
-          break;
-        }
-        ph ^= 1;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (kb < nks) {
-          // per 16-deep step: MN-major W two 1 KB K groups on (+128), U rows 32 bytes on (+2)
+      const uint32_t sa0 = tc::smem_u32(stage);
+      uint32_t count = *k.count;
+      const bool ok = stc_ring<NST>(
+          k, count, nks + q0 / STC_KB, pre, p.err,
+          [&](int kb, uint32_t st) {
+            if (kb < nks) {
+              load_shift(kb, q0, st);
+              return;
+            }
+            unsigned char* d = stage + st * SB;
+            uint64_t* bar = k.full + st;
+            tc::mbar_expect_tx(bar, SB);
+            const int x = (kb - nks) * STC_KB;
+            tc::tma_load_2d(d, mapY, bar, x, pl.yrow);
+            tc::tma_load_2d(d + CHALF, mapY, bar, p.alo + x, pl.yrow);
+            tc::tma_load_2d(d + CA, mapB, bar, x, p.brow0 + q0);
+            tc::tma_load_2d(d + CHALF + CA, mapB, bar, p.blo + x, p.brow0 + q0);
+            if constexpr (SPLIT) tc::tma_load_2d(d + CB3, mapB, bar, 2 * p.blo + x, p.brow0 + q0);
+          },
+          [&](int kb, uint32_t st) {
+            const uint32_t sa = sa0 + st * SB;
+            if (kb >= nks) {
+              mma_split(tc::sdesc<STC_KB>(sa), tc::sdesc<STC_KB>(sa + CHALF), 2, sa, ID_C, kb == 0);
+            } else if constexpr (SPLIT) {
+              // per 16-deep step MN-major W is two 1 KB K groups on (+128)
+              mma_split(tc::sdesc_mn(sa, CA / 2), tc::sdesc_mn(sa + CHALF, CA / 2), 128, sa, ID_S, kb == 0);
+            } else {
+              const uint64_t dw = tc::sdesc_mn(sa, SA / 2), du = tc::sdesc<64>(sa + SA);
 #pragma unroll
-          for (int kk = 0; kk < 4; kk++)
-            tc::mma_f16(tmem, dw + (uint64_t)(128 * kk), du + (uint64_t)(2 * kk), ID_S, (kb > 0 || kk > 0) ? 1u : 0u);
-        } else {
-#pragma unroll
-          for (int kk = 0; kk < STC_KB / 16; kk++) {
-            const uint64_t o = (uint64_t)(kk * 2);  // 32 bytes per 16-deep step, in 16-byte units
-            tc::mma_f16(tmem, dah + o, dbh + o, ID_C, (kb > 0 || kk > 0) ? 1u : 0u);
-            tc::mma_f16(tmem, dah + o, dbl + o, ID_C, 1u);
-            tc::mma_f16(tmem, dal + o, dbh + o, ID_C, 1u);
-          }
-        }
-        tc::mma_commit(freeb);
-        if (!tc::mbar_wait(freeb, (ph >> 1) & 1, p.err, 9)) {
-          bad = 2;
-          break;
-        }
-        ph ^= 2;
-      }
-      if (bad) {
-        // wait (bounded) for the copies or products still in flight
-        if (bad == 1) tc::mbar_wait(full, ph & 1, p.err, 5);
-        else tc::mbar_wait(freeb, (ph >> 1) & 1, p.err, 5);
+              for (int kk = 0; kk < 4; kk++)
+                tc::mma_f16(tmem, dw + (uint64_t)(128 * kk), du + (uint64_t)(2 * kk), ID_S,
+                            (kb > 0 || kk > 0) ? 1u : 0u);
+            }
+          });
+      pre = 0;
+      if (!ok) {
         *abort_flag = 1;
-      } else if (nks > 0 && q0 + STC_SUB < mt) {
-        load_shift(0, q0 + STC_SUB);  // lands during the sweep (W and U are complete)
+      } else if (q0 + STC_SUB < mt) {
+        // these land during the sweep (W and U are complete; all products have read their stages)
+        for (; pre < NST && pre < nks; pre++) load_shift(pre, q0 + STC_SUB, (count + (uint32_t)pre) % NST);
       }
-      *k.phases = ph;
+      *k.count = count;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();  // records and triangle staged; shifts and coupling are in TMEM
@@ -289,10 +379,21 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
       if (q0 > 0 || p.kr > 0) {
         uint32_t r[DIAG_VB];
         tmem_ld16(r, tl + (uint32_t)v0);
+        if constexpr (SPLIT) {
+          uint32_t l[DIAG_VB];
+          tmem_ld16(l, tl + (uint32_t)(STC_SUB + v0));
+          const float* sc = k.rec + v0 * STC_REC + 19;  // (rows past a ragged tile: stale, unused)
 #pragma unroll
-        for (int j = 0; j < DIAG_VB / 2; j++)
-          acc[j] = F16 ? make_float2(__uint_as_float(r[2 * j]) * p.tscale, __uint_as_float(r[2 * j + 1]) * p.tscale)
-                       : make_float2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+          for (int j = 0; j < DIAG_VB / 2; j++)
+            acc[j] = make_float2(
+                (__uint_as_float(r[2 * j]) + __uint_as_float(l[2 * j])) * sc[2 * j * STC_REC],
+                (__uint_as_float(r[2 * j + 1]) + __uint_as_float(l[2 * j + 1])) * sc[(2 * j + 1) * STC_REC]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < DIAG_VB / 2; j++)
+            acc[j] = F16 ? make_float2(__uint_as_float(r[2 * j]) * p.tscale, __uint_as_float(r[2 * j + 1]) * p.tscale)
+                         : make_float2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+        }
       } else {
 #pragma unroll
         for (int j = 0; j < DIAG_VB / 2; j++) acc[j] = make_float2(0.0f, 0.0f);
@@ -390,13 +491,20 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
         if (act) {
           unsigned short* row = pl.ysrow + q0 + v0;
           uint32_t hi2[DIAG_VB / 2], lo2[DIAG_VB / 2];
+          float top = 0.0f;
 #pragma unroll
           for (int j = 0; j < DIAG_VB; j += 2) {
             const float y0 = __uint_as_float(r[j]), y1 = __uint_as_float(r[j + 1]);
-            float h0, h1, l0, l1;
-            hi2[j / 2] = Op::pack(y0, y1, h0, h1);
-            lo2[j / 2] = Op::pack(y0 - h0, y1 - h1, l0, l1);
+            if constexpr (SPLIT) {
+              split_f32(y0, y1, hi2[j / 2], lo2[j / 2]);
+              top = fmaxf(top, j < nb ? fmaxf(fabsf(y0), fabsf(y1)) : 0.0f);
+            } else {
+              float h0, h1, l0, l1;
+              hi2[j / 2] = Op::pack(y0, y1, h0, h1);
+              lo2[j / 2] = Op::pack(y0 - h0, y1 - h1, l0, l1);
+            }
           }
+          if (SPLIT && top > 32768.0f) p.err[1] = 1;
           if (nb == DIAG_VB) {
             uint4* dh = reinterpret_cast<uint4*>(row);
             uint4* dlo = reinterpret_cast<uint4*>(row + p.ys_lo);
@@ -428,36 +536,38 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
   // stages of the CTA's y rows and of V rows)
   for (int r0 = 0; r0 < p.kc; r0 += 64) {
     if (tid == 0) {
-      const uint32_t sa = tc::smem_u32(stage);
-      const uint64_t da = tc::sdesc<64>(sa), db = tc::sdesc<64>(sa + PA);
-      uint32_t ph = *k.phases;
-      int bad = 0;
-      for (int kb = 0; kb < (mt + 63) / 64; kb++) {
-        tc::mbar_expect_tx(full, SB);
-        tc::tma_load_2d(stage, mapY64, full, kb * 64, pl.yrow);
-        tc::tma_load_2d(stage + PA, mapV, full, kb * 64, p.kcol0 + r0);
-        if (!tc::mbar_wait(full, ph & 1, p.err, 8)) {
-          bad = 1;
-          break;
-        }
-        ph ^= 1;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t sa0 = tc::smem_u32(stage);
+      uint32_t count = *k.count;
+      const bool ok = stc_ring<NST>(
+          k, count, (mt + KS - 1) / KS, 0, p.err,
+          [&](int kb, uint32_t st) {
+            unsigned char* d = stage + st * SB;
+            uint64_t* bar = k.full + st;
+            tc::mbar_expect_tx(bar, SB);
+            if constexpr (SPLIT) {
+              tc::tma_load_2d(d, mapY, bar, kb * KS, pl.yrow);
+              tc::tma_load_2d(d + CHALF, mapY, bar, p.alo + kb * KS, pl.yrow);
+              tc::tma_load_2d(d + CA, mapV, bar, kb * KS, p.kcol0 + r0);
+              tc::tma_load_2d(d + CHALF + CA, mapV, bar, p.vlo + kb * KS, p.kcol0 + r0);
+              tc::tma_load_2d(d + CB3, mapV, bar, 2 * p.vlo + kb * KS, p.kcol0 + r0);
+            } else {
+              tc::tma_load_2d(d, mapY64, bar, kb * 64, pl.yrow);
+              tc::tma_load_2d(d + PA, mapV, bar, kb * 64, p.kcol0 + r0);
+            }
+          },
+          [&](int kb, uint32_t st) {
+            const uint32_t sa = sa0 + st * SB;
+            if constexpr (SPLIT) {
+              mma_split(tc::sdesc<STC_KB>(sa), tc::sdesc<STC_KB>(sa + CHALF), 2, sa, ID_C, kb == 0);
+            } else {
+              const uint64_t da = tc::sdesc<64>(sa), db = tc::sdesc<64>(sa + PA);
 #pragma unroll
-        for (int kk = 0; kk < 4; kk++)
-          tc::mma_f16(tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), ID_P, (kb > 0 || kk > 0) ? 1u : 0u);
-        tc::mma_commit(freeb);
-        if (!tc::mbar_wait(freeb, (ph >> 1) & 1, p.err, 9)) {
-          bad = 2;
-          break;
-        }
-        ph ^= 2;
-      }
-      if (bad) {
-        if (bad == 1) tc::mbar_wait(full, ph & 1, p.err, 5);
-        else tc::mbar_wait(freeb, (ph >> 1) & 1, p.err, 5);
-        *abort_flag = 1;
-      }
-      *k.phases = ph;
+              for (int kk = 0; kk < 4; kk++)
+                tc::mma_f16(tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), ID_P, (kb > 0 || kk > 0) ? 1u : 0u);
+            }
+          });
+      if (!ok) *abort_flag = 1;
+      *k.count = count;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -467,7 +577,33 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
     for (int h = 0; h < 64; h += 16) {
       uint32_t r[16];
       tmem_ld16(r, tl + (uint32_t)h);
-      if (act) {
+      if constexpr (SPLIT) {
+        uint32_t l[16];
+        tmem_ld16(l, tl + (uint32_t)(STC_SUB + h));
+        if (act) {
+          float top = 0.0f;
+#pragma unroll
+          for (int j = 0; j < 16; j += 2)
+            if (r0 + h + j < p.kc) {
+              const bool two = r0 + h + j + 1 < p.kc;
+              const int rr = r0 + h + j, r1 = two ? rr + 1 : rr;
+              const float w0 = (__uint_as_float(r[j]) + __uint_as_float(l[j])) * p.wscale[rr];
+              const float w1 = (__uint_as_float(r[j + 1]) + __uint_as_float(l[j + 1])) * p.wscale[r1];
+              uint32_t hi, lo;
+              split_f32(w0, w1, hi, lo);
+              top = fmaxf(top, fmaxf(fabsf(w0), two ? fabsf(w1) : 0.0f));
+              unsigned short* d0 = pl.wcol + (int64_t)p.vmap[rr] * p.ldw;
+              d0[0] = (unsigned short)hi;
+              d0[(int64_t)p.wlo * p.ldw] = (unsigned short)lo;
+              if (two) {
+                unsigned short* d1 = pl.wcol + (int64_t)p.vmap[r1] * p.ldw;
+                d1[0] = (unsigned short)(hi >> 16);
+                d1[(int64_t)p.wlo * p.ldw] = (unsigned short)(lo >> 16);
+              }
+            }
+          if (top > 32768.0f) p.err[1] = 1;
+        }
+      } else if (act) {
 #pragma unroll
         for (int j = 0; j < 16; j++)
           if (r0 + h + j < p.kc)
@@ -483,30 +619,34 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
   return true;
 }
 
-// The CTA's stage, records, barriers and TMEM columns (dynamic shared memory of
-// sweep_tc_smem_bytes()); the barriers initialised and the columns allocated.
+// The CTA's stages, records, barriers and TMEM columns (dynamic shared memory of
+// sweep_tc_smem_bytes(MODE, NST)); the barriers initialised and the columns allocated.
 // Ends with every thread past the allocation.
+template <int MODE, int NST>
 __device__ __forceinline__ StcCta stc_cta_setup(unsigned char* smem) {
   StcCta k;
   k.stage = smem;
-  k.rec = reinterpret_cast<float*>(smem + StcCfg::SB);
+  k.rec = reinterpret_cast<float*>(smem + NST * stc_stage_bytes(MODE));
   k.tri = k.rec + STC_SUB * STC_REC;
   k.full = reinterpret_cast<uint64_t*>(k.tri + STC_TRI);
-  k.freeb = k.full + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(k.freeb + 1);
-  k.phases = tmem_slot + 1;
+  k.freeb = k.full + NST;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(k.freeb + NST);
+  k.count = tmem_slot + 1;
   k.abort_flag = reinterpret_cast<int*>(tmem_slot + 2);
   k.item = k.abort_flag + 1;
   if (threadIdx.x == 0) {
     *k.abort_flag = 0;
-    *k.phases = 0;
-    tc::mbar_init(k.full, 1);
-    tc::mbar_init(k.freeb, 1);
+    *k.count = 0;
+#pragma unroll
+    for (int s = 0; s < NST; s++) {
+      tc::mbar_init(k.full + s, 1);
+      tc::mbar_init(k.freeb + s, 1);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if ((threadIdx.x >> 5) == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(tmem_slot)),
-                 "r"(STC_SUB)
+                 "r"(stc_cols(MODE))
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -518,16 +658,19 @@ __device__ __forceinline__ StcCta stc_cta_setup(unsigned char* smem) {
 }
 
 // Frees the CTA's TMEM columns once every thread is done with them.
+template <int MODE>
 __device__ __forceinline__ void stc_cta_release(const StcCta& k) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if ((threadIdx.x >> 5) == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(k.tmem), "r"(STC_SUB) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(k.tmem), "r"(stc_cols(MODE))
+                 : "memory");
 }
 
 // One launch per diagonal tile of one problem: CTA x owns samples [128 x, 128 (x + 1)) of the
-// chunk.  Six CTAs per SM, 80 registers each.
+// chunk.  CTAs per SM: six with one stage (80 registers each), three with two, two with three or four.
+__host__ __device__ constexpr int stc_ctas(int nst) { return nst == 1 ? 6 : (nst == 2 ? 3 : 2); }
 struct SweepTcLaunch {
   const uint64_t* D;
   int64_t ldD, coord0, sample0, N, C;
@@ -538,14 +681,14 @@ struct SweepTcLaunch {
   double* logP;
   int first;
 };
-template <int FLAGS, bool F16>
-__global__ void __launch_bounds__(STC_NS, 6)
+template <int FLAGS, int MODE, int NST>
+__global__ void __launch_bounds__(STC_NS, stc_ctas(NST))
     k_sweep_tc(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapB,
                const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapU,
                const __grid_constant__ CUtensorMap mapY64, const __grid_constant__ CUtensorMap mapV,
                const __grid_constant__ SweepTcArgs p, const __grid_constant__ SweepTcLaunch d) {
   extern __shared__ __align__(1024) unsigned char stc_smem[];
-  const StcCta k = stc_cta_setup(stc_smem);
+  const StcCta k = stc_cta_setup<MODE, NST>(stc_smem);
   pdl_trigger();  // (after the allocation: a successor's CTAs never hold TMEM this grid still needs)
   pdl_wait();  // limit shifts, y and log P of the preceding kernels
 
@@ -565,14 +708,14 @@ __global__ void __launch_bounds__(STC_NS, 6)
   pl.yrow = c0;
   pl.ysrow = d.Ys + (int64_t)cs * d.ldys;
   pl.wcol = d.W + cs;
-  const bool ok = stc_tile<FLAGS, F16>(&mapY, &mapB, &mapW, &mapU, &mapY64, &mapV, p, k, pl, act,
-                                       d.D + sh * d.ldD + d.coord0, ks, rs, prod, lsum, pe);
+  const bool ok = stc_tile<FLAGS, MODE, NST>(&mapY, &mapB, &mapW, &mapU, &mapY64, &mapV, p, k, pl, act,
+                                             d.D + sh * d.ldD + d.coord0, ks, rs, prod, lsum, pe);
   if (ok && act) {
     const double lp = (double)(logf(prod) + lsum) + (double)pe * 0.69314718055994530942;
     if (d.first) d.logP[g] = lp;
     else d.logP[g] += lp;
   }
-  stc_cta_release(k);
+  stc_cta_release<MODE>(k);
 }
 
 }  // namespace tlrmvn

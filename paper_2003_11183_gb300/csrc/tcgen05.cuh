@@ -64,13 +64,13 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr) {
 }
 
 // MN-major operand (A_MN): TMA writes each 64-element-wide MN slice of the tile
-// as 64 K-rows of 128 bytes (128-byte swizzle); the two slices of a 128-row tile
-// sit 8 KB apart (leading byte offset, between MN atoms) and the 8-row K groups
+// as K-rows of 128 bytes (128-byte swizzle); the two slices of a 128-row tile
+// sit `slice` bytes apart (leading byte offset, between MN atoms) and the 8-row K groups
 // 1 KB apart (stride byte offset).  One 16-deep K step spans two K groups (2 KB).
-__device__ __forceinline__ uint64_t sdesc_mn(uint32_t saddr) {
+__device__ __forceinline__ uint64_t sdesc_mn(uint32_t saddr, uint32_t slice) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)(8192 >> 4) << 16;  // leading byte offset: next 64-element MN slice
+  d |= (uint64_t)(slice >> 4) << 16;  // leading byte offset: next 64-element MN slice
   d |= (uint64_t)(1024 >> 4) << 32;  // stride byte offset: next 8-row K group
   d |= (uint64_t)1 << 46;            // version
   d |= (uint64_t)2 << 61;            // 128-byte swizzle
