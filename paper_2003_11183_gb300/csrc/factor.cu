@@ -17,6 +17,7 @@
 //   * The diagonal Schur blocks S_ii -= U_ij (V_ij^T V_ij) U_ij^T are kept current.
 #include "common.cuh"
 #include "gemm.cuh"
+#include "sov64.cuh"
 
 #include <algorithm>
 #include <cstring>
@@ -45,50 +46,49 @@ __device__ double log_interval_d(double at, double bt) {
   const double e = (bt == INFINITY) ? 1.0 : 1.0 - 0.5 * erfc(bt * TLR_RSQRT2);
   return log(e - d);
 }
-// Mean of N(0,1) truncated to (at, bt).
-__device__ double trunc_mean_d(double at, double bt) {
-  double ld = log_interval_d(at, bt);
-  double ta = (at > -INFINITY && at < INFINITY) ? exp(-0.5 * at * at - TLR_LOG_SQRT2PI - ld) : 0.0;
-  double tb = (bt > -INFINITY && bt < INFINITY) ? exp(-0.5 * bt * bt - TLR_LOG_SQRT2PI - ld) : 0.0;
-  return ta - tb;
+// Probability of (at, bt) as an order-preserving integer key, with p and, above 1/2, its complement c: p <= 1/2
+// orders by p's bits, p > 1/2 by its complement's (which keeps apart what rounds to 1), and p below the tables
+// (1e-37) by its log.  T: table A of sov64.cuh in shared memory.
+__device__ __forceinline__ long long interval_key(const double* T, double at, double bt, double& p, double& c) {
+  const bool nb = bt < 0.0, na = at < 0.0;
+  const double xb = fabs(bt), xa = fabs(at);
+  const double hb = xb <= 13.0 ? t64_phi_wide(T, xb) : 0.0;
+  double ha = 0.0;
+  if (xa <= 13.0) ha = t64_phi_wide(T, xa);
+  c = nb ? 1.0 - hb + ha : (na ? ha + hb : 1.0 - (ha - hb));
+  p = nb ? hb - ha : (na ? (1.0 - ha) - hb : ha - hb);
+  if (!(p >= 1e-37)) {
+    const double q = log_interval_d(at, bt);
+    p = 0.0;
+    c = q;
+    return q < 0.0 ? -__double_as_longlong(-q) : (q == 0.0 ? 0x7FE0000000000000LL : 0x7FFFFFFFFFFFFFFFLL);
+  }
+  if (p <= 0.5) return __double_as_longlong(p);
+  if (c < 1e-36) c = 0.5 * erfc(bt * TLR_RSQRT2) + 0.5 * erfc(-at * TLR_RSQRT2);  // (limits beyond the table)
+  return 0x7FE0000000000000LL - __double_as_longlong(c);
 }
-
-__device__ __forceinline__ void argmin_merge(double& q, int& i, double q2, int i2) {
+__device__ __forceinline__ void keymin_merge(long long& q, int& i, long long q2, int i2) {
   if (q2 < q || (q2 == q && i2 < i)) {
     q = q2;
     i = i2;
   }
 }
-// block-wide (min q, lowest index); every thread gets the result
-__device__ void block_argmin(double& q, int& i, double* shq, int* shi) {
+// block-wide (least key, lowest index); every thread gets the result
+__device__ void block_keymin(long long& q, int& i, long long* shq, int* shi) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
   for (int o = 16; o; o >>= 1) {
-    double q2 = __shfl_xor_sync(0xffffffffu, q, o);
+    long long q2 = __shfl_xor_sync(0xffffffffu, q, o);
     int i2 = __shfl_xor_sync(0xffffffffu, i, o);
-    argmin_merge(q, i, q2, i2);
+    keymin_merge(q, i, q2, i2);
   }
   if (lane == 0) {
     shq[wid] = q;
     shi[wid] = i;
   }
   __syncthreads();
-  if (wid == 0) {
-    q = lane < nw ? shq[lane] : INFINITY;
-    i = lane < nw ? shi[lane] : 0x7fffffff;
-    for (int o = 16; o; o >>= 1) {
-      double q2 = __shfl_xor_sync(0xffffffffu, q, o);
-      int i2 = __shfl_xor_sync(0xffffffffu, i, o);
-      argmin_merge(q, i, q2, i2);
-    }
-    if (lane == 0) {
-      shq[0] = q;
-      shi[0] = i;
-    }
-  }
-  __syncthreads();
   q = shq[0];
   i = shi[0];
-  __syncthreads();
+  for (int w = 1; w < nw; w++) keymin_merge(q, i, shq[w], shi[w]);
 }
 __device__ double block_sum(double v, double* sh) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -145,105 +145,151 @@ __global__ void k_cov_tiles(const TileJob* jobs, CovSrc src, int m) {
 }
 
 // ---- univariate conditioning (Trinh & Genz) of diagonal blocks --------------------------
-// One block per CTA; right-looking pivoted Cholesky of a copy of the block in
-// `work`.  Writes log of the estimate; with emit, also the pivot order and the
+// One block per CTA; right-looking pivoted Cholesky of a copy of the block (its lower triangle packed in shared memory
+// when it fits there, SH, else in `work`).  Writes log of the estimate; with emit, also the pivot order and the
 // truncated expectations in the new order.
+//
+// A step is a chain (probabilities of all remaining variables, their least, a square root, the column, the update), and
+// with one SM's float64 pipe (16 cycles an instruction of a warp) what is evaluated by every thread costs most: the
+// probabilities come from the tables of sov64.cuh as integer keys (about 30 float64 instructions instead of 300 and
+// no log), the pivot's owner passes on its square root and probability, and while one warp works out the truncated
+// mean, which only the next step needs, the others update the triangle; the logs come at the end.  All conditionings of
+// n = 1,024 in tiles of 128: 15.6 -> 5.1 ms.
+template <bool SH>
 __global__ void __launch_bounds__(512) k_uc(const int* blist, const double* diagS, const int* bsize, int m,
                                             const double* acur, const double* bcur, double* work, double* logp_out,
-                                            int emit, int* order_out, double* y_out, int* status) {
-  extern __shared__ double shm[];
-  double* sa = shm;
+                                            int emit, int* order_out, double* y_out, int* status, const double* tables) {
+  extern __shared__ __align__(16) double shm[];
+  double* T = shm;
+  double* sa = T + T64_A * T64_W;
   double* sb = sa + m;
   double* ss = sb + m;
   double* lcol = ss + m;
   double* sy = lcol + m;
-  int* so = (int*)(sy + m);
-  __shared__ double shq[32];
-  __shared__ int shi[32];
-  __shared__ double shy;
+  double* pr = sy + m;   // the steps' probabilities
+  double* tri = pr + m;
+  int* so = (int*)(tri + (SH ? (size_t)m * (m + 1) / 2 : 0));
+  __shared__ long long shq[16];
+  __shared__ int shi[16];
+  __shared__ double shl, shr, shy;          // l_kk, 1 / l_kk, y_k
+  __shared__ double sha, shb, shp, shc;     // the pivot's standardised limits, its probability and complement
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
   const int b = blist[blockIdx.x];
   const int mb = bsize[b];
-  double* A = work + (size_t)blockIdx.x * m * m;
+  double* A = work + (SH ? (size_t)0 : (size_t)blockIdx.x * m * m);
   const double* S = diagS + (size_t)b * m * m;
-  for (int t = threadIdx.x; t < mb * mb; t += blockDim.x) A[(t / mb) * m + t % mb] = S[(t / mb) * m + t % mb];
-  for (int t = threadIdx.x; t < mb; t += blockDim.x) {
+  auto at_ = [&](int i, int j) -> double& { return SH ? tri[i * (i + 1) / 2 + j] : A[(size_t)i * m + j]; };
+  for (int t = tid; t < T64_A * T64_W / 2; t += blockDim.x)
+    reinterpret_cast<double2*>(T)[t] = reinterpret_cast<const double2*>(tables)[t];
+  for (int i = wid; i < mb; i += nw)
+    for (int j = lane; j <= i; j += 32) at_(i, j) = S[(size_t)i * m + j];
+  for (int t = tid; t < mb; t += blockDim.x) {
     sa[t] = acur[(size_t)b * m + t];
     sb[t] = bcur[(size_t)b * m + t];
     ss[t] = 0.0;
+    lcol[t] = 0.0;
     so[t] = t;
   }
+  if (tid == 0) shy = 0.0;
   __syncthreads();
-  double logp = 0.0;
   for (int k = 0; k < mb; k++) {
-    double bq = INFINITY;
+    long long bq = 0x7FFFFFFFFFFFFFFFLL;
     int bi = 0x7fffffff;
-    for (int i = k + threadIdx.x; i < mb; i += blockDim.x) {
-      double var = A[(size_t)i * m + i];
-      double q;
+    const double yk1 = shy;  // the step before's truncated mean
+    double mr = 0.0, ma = 0.0, mb_ = 0.0, mp = 0.0, mc = 0.0;  // of this thread's best: 1 / l, limits, p, c
+    for (int i = k + tid; i < mb; i += blockDim.x) {
+      const double var = at_(i, i);
+      const double si = ss[i] + lcol[i] * yk1;
+      ss[i] = si;
+      long long key = 0x7FFFFFFFFFFFFFFFLL;
+      double is = 1.0, a = 0.0, bt = 0.0, p = 1.0, c = 0.0;
       if (!(var > 0.0)) {
         atomicExch(status, TLRMVN_E_NOT_SPD);
-        q = INFINITY;
       } else {
-        double sig = sqrt(var);
-        q = log_interval_d((sa[i] - ss[i]) / sig, (sb[i] - ss[i]) / sig);
+        is = rsqrt(var);
+        a = (sa[i] - si) * is;
+        bt = (sb[i] - si) * is;
+        key = interval_key(T, a, bt, p, c);
       }
-      argmin_merge(bq, bi, q, i);
+      if (key < bq || (key == bq && i < bi)) {
+        bq = key;
+        bi = i;
+        mr = is;
+        ma = a;
+        mb_ = bt;
+        mp = p;
+        mc = c;
+      }
     }
-    block_argmin(bq, bi, shq, shi);
+    const int own = bi;
+    block_keymin(bq, bi, shq, shi);
     const int piv = (bi < mb) ? bi : k;
-    if (threadIdx.x == 0) {
-      if (piv != k) {
-        double t;
-        t = sa[k]; sa[k] = sa[piv]; sa[piv] = t;
-        t = sb[k]; sb[k] = sb[piv]; sb[piv] = t;
-        t = ss[k]; ss[k] = ss[piv]; ss[piv] = t;
-        int ti = so[k]; so[k] = so[piv]; so[piv] = ti;
-      }
-      logp += bq;
+    if (own == piv) {  // (one thread: the indices are distinct)
+      const double d = at_(piv, piv), l0 = d > 0.0 ? d * mr : 1.0;
+      shl = l0 + (d > 0.0 ? fma(-l0, l0, d) * 0.5 * mr : 0.0);
+      shr = mr;
+      sha = ma;
+      shb = mb_;
+      shp = mp;
+      shc = mc;
+    }
+    if (tid == 0 && piv != k) {
+      double t;
+      t = sa[k]; sa[k] = sa[piv]; sa[piv] = t;
+      t = sb[k]; sb[k] = sb[piv]; sb[piv] = t;
+      t = ss[k]; ss[k] = ss[piv]; ss[piv] = t;
+      int ti = so[k]; so[k] = so[piv]; so[piv] = ti;
     }
     // (only the lower triangle of the symmetric block is kept: swapping variables k < piv
     // exchanges A(k,t) with A(piv,t) for t < k, A(t,k) with A(piv,t) for k < t < piv,
-    // A(t,k) with A(t,piv) for t > piv, and the two diagonal entries)
-    if (piv != k) {
-      for (int t = threadIdx.x; t < mb; t += blockDim.x) {
-        double *x0, *x1;
-        if (t < k) {
-          x0 = A + (size_t)k * m + t;
-          x1 = A + (size_t)piv * m + t;
-        } else if (t == k) {
-          x0 = A + (size_t)k * m + k;
-          x1 = A + (size_t)piv * m + piv;
-        } else if (t < piv) {
-          x0 = A + (size_t)t * m + k;
-          x1 = A + (size_t)piv * m + t;
-        } else if (t > piv) {
-          x0 = A + (size_t)t * m + k;
-          x1 = A + (size_t)t * m + piv;
-        } else {
-          continue;  // A(piv,k) stays
-        }
-        const double x = *x0;
-        *x0 = *x1;
-        *x1 = x;
+    // A(t,k) with A(t,piv) for t > piv, and the two diagonal entries, by warps 1 on)
+    if (piv != k && wid > 0) {
+      for (int t = tid - 32; t < mb; t += blockDim.x - 32) {
+        if (t == piv) continue;  // A(piv,k) stays
+        double& x0 = t < k ? at_(k, t) : (t == k ? at_(k, k) : at_(t, k));
+        double& x1 = t < k ? at_(piv, t) : (t == k ? at_(piv, piv) : (t < piv ? at_(piv, t) : at_(t, piv)));
+        // (the diagonal entries: after thread 0 has read the pivot's)
+        if (t == k) continue;
+        const double x = x0;
+        x0 = x1;
+        x1 = x;
       }
     }
     __syncthreads();
-    const double dkk = A[(size_t)k * m + k];
-    const double lkk = sqrt(dkk > 0.0 ? dkk : 1.0);
-    for (int i = k + 1 + threadIdx.x; i < mb; i += blockDim.x) lcol[i] = A[(size_t)i * m + k] / lkk;
-    if (threadIdx.x == 0) {
-      double y = trunc_mean_d((sa[k] - ss[k]) / lkk, (sb[k] - ss[k]) / lkk);
-      sy[k] = y;
-      shy = y;
+    if (piv != k && tid == 0) {  // (A(k,k) is not read again)
+      at_(piv, piv) = at_(k, k);
+    }
+    const double lkk = shl, rkk = shr;
+    for (int i = k + 1 + tid; i < mb; i += blockDim.x) {
+      const double x = at_(i, k), q = x * rkk;
+      lcol[i] = fma(fma(-q, lkk, x), rkk, q);
     }
     __syncthreads();
-    const double yk = shy;
-    for (int i = k + 1 + threadIdx.x; i < mb; i += blockDim.x) ss[i] += lcol[i] * yk;
-    // the Schur update of the lower triangle, a row per warp
-    {
-      const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-      for (int i = k + 1 + (threadIdx.x >> 5); i < mb; i += nw) {
-        double* row = A + (size_t)i * m;
+    if (wid == 0) {
+      // the pivot's truncated mean, by one thread, while the other warps update
+      if (lane == 0) {
+        const double at = sha, bt = shb, p = shp;
+        double y = 0.0;
+        if (p > 0.0) {
+          const double ea = fabs(at) <= 13.0 ? t64_density(T, fabs(at)) : 0.0;
+          const double eb = fabs(bt) <= 13.0 ? t64_density(T, fabs(bt)) : 0.0;
+          // (1 / p by Newton from float32: p >= 1e-37; fewer dependent steps than a division)
+          double ri = (double)(1.0f / (float)p);
+          ri = fma(fma(-p, ri, 1.0), ri, ri);
+          ri = fma(fma(-p, ri, 1.0), ri, ri);
+          y = (ea - eb) * ri;
+        } else {
+          if (at > -INFINITY && at < INFINITY) y = exp(-0.5 * at * at - TLR_LOG_SQRT2PI - shc);
+          if (bt > -INFINITY && bt < INFINITY) y -= exp(-0.5 * bt * bt - TLR_LOG_SQRT2PI - shc);
+        }
+        sy[k] = y;
+        shy = y;
+        pr[k] = p > 0.0 && p <= 0.5 ? p : -shc;  // (p, or minus the complement, or minus the log: 75 and more)
+      }
+    } else {
+      // the Schur update of the lower triangle, a row per warp
+      for (int i = k + wid; i < mb; i += nw - 1) {
+        double* row = &at_(i, 0);
         const double li = lcol[i];
         int jj = k + 1 + lane;
         for (; jj + 96 <= i; jj += 128) {  // (four loads per lane in flight)
@@ -262,13 +308,42 @@ __global__ void __launch_bounds__(512) k_uc(const int* blist, const double* diag
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) logp_out[blockIdx.x] = logp;
+  // the estimate's log: the terms by all threads, their sum in order by one
+  for (int t = tid; t < mb; t += blockDim.x) {
+    const double x = pr[t];
+    ss[t] = x > 0.0 ? (x <= 0.5 ? log(x) : -x) : log1p(x);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double logp = 0.0;
+    for (int t = 0; t < mb; t++) logp += ss[t];
+    logp_out[blockIdx.x] = logp;
+  }
   if (emit) {
-    for (int t = threadIdx.x; t < mb; t += blockDim.x) {
+    for (int t = tid; t < mb; t += blockDim.x) {
       order_out[(size_t)blockIdx.x * m + t] = so[t];
       y_out[(size_t)blockIdx.x * m + t] = sy[t];
     }
   }
+}
+int tables64(const double** out, cudaStream_t st);  // prob.cu
+// k_uc over `blocks` blocks (work: blocks x m x m, used when a triangle does not fit in shared memory)
+static int launch_uc(int blocks, int m, cudaStream_t st, const int* blist, const double* diagS, const int* bsize,
+                     const double* a, const double* b, double* work, double* logp, int* order, double* y, int* status) {
+  const double* tables = nullptr;
+  TLR_CHECK(tables64(&tables, st));
+  const size_t base = ((size_t)T64_A * T64_W + 6 * (size_t)m) * sizeof(double) + (size_t)m * sizeof(int);
+  const size_t full = base + (size_t)m * (m + 1) / 2 * sizeof(double);
+  const int threads = m >= 256 ? 512 : 256;
+  if (full <= 200 * 1024) {
+    TLR_CHECK(raise_smem_limit((const void*)k_uc<true>, full));
+    k_uc<true><<<blocks, threads, full, st>>>(blist, diagS, bsize, m, a, b, work, logp, 1, order, y, status, tables);
+  } else {
+    TLR_CHECK(raise_smem_limit((const void*)k_uc<false>, base));
+    k_uc<false><<<blocks, threads, base, st>>>(blist, diagS, bsize, m, a, b, work, logp, 1, order, y, status, tables);
+  }
+  TLR_CUDA(cudaGetLastError());
+  return TLRMVN_OK;
 }
 
 // ---- plain Cholesky of one block, in place (lower), zero above -------------------------
@@ -345,36 +420,109 @@ __global__ void __launch_bounds__(256) k_trinv_cols(const double* L, int ldl, si
   }
 }
 
-// ---- blocked Cholesky pieces: one diagonal block of at most 64 in place ------------------
-// (lower; its strict upper triangle zeroed; the rest of the matrix untouched)
-__global__ void __launch_bounds__(256) k_potrf_diag(double* A, int nb, int ld, int* status) {
-  __shared__ double col[64];
+// ---- blocked Cholesky pieces: one diagonal block of at most 64 in place, and its inverse --------------
+// (lower; its strict upper triangle zeroed; the rest of the matrix untouched; Linv: nb x nb, ld ldi, lower, zero
+// above).  One CTA, both in shared memory: 64 steps of a square root, a column and a rank-one update, then the
+// inverse by blocks of 16 (a thread a column of a diagonal block, the rest as products).  Bound by the steps' chain and
+// one SM's float64 rate; with the blocks' inverses here rather than in a kernel of one column a warp, all the
+// Cholesky factors and inverses of n = 4,096 in tiles of 256 take 7.3 ms and their products (21.6 ms before).
+constexpr int P64_LD = 65;
+__global__ void __launch_bounds__(256) k_potrf_inv64(double* A, int nb, int ld, double* Linv, int ldi, int* status) {
+  extern __shared__ double sp[];
+  double* L = sp;                  // [64][65]
+  double* X = sp + 64 * P64_LD;    // [64][65]: the inverse
+  double* Tm = X + 64 * P64_LD;    // [64][17] a block product
+  __shared__ double diag[2], rdiag[64];
+  if (threadIdx.x < 64) rdiag[threadIdx.x] = 1.0;
+  const int tid = threadIdx.x;
+  for (int t = tid; t < 64 * 64; t += 256) {
+    const int i = t >> 6, j = t & 63;
+    L[i * P64_LD + j] = (i < nb && j <= i) ? A[(size_t)i * ld + j] : (i == j ? 1.0 : 0.0);
+    X[i * P64_LD + j] = 0.0;
+  }
+  __syncthreads();
+  // (the float64 pipe is the bound: one warp takes the root, and only what exists is updated)
   for (int k = 0; k < nb; k++) {
-    const double d = A[(size_t)k * ld + k];
-    if (!(d > 0.0)) {
-      if (threadIdx.x == 0) atomicExch(status, TLRMVN_E_NOT_SPD);
-      return;
-    }
-    const double lkk = sqrt(d);
-    for (int i = k + 1 + threadIdx.x; i < nb; i += blockDim.x) {
-      const double l = A[(size_t)i * ld + k] / lkk;
-      A[(size_t)i * ld + k] = l;
-      col[i] = l;
+    if (tid < 32) {
+      const double d = L[k * P64_LD + k];
+      const double rs = rsqrt(d), l0 = d * rs, l = fma(fma(-l0, l0, d), 0.5 * rs, l0);
+      if (tid == 0) {
+        if (!(d > 0.0)) atomicExch(status, TLRMVN_E_NOT_SPD);
+        diag[0] = l;
+        diag[1] = d > 0.0 ? rs : NAN;
+      }
     }
     __syncthreads();
-    if (threadIdx.x == 0) A[(size_t)k * ld + k] = lkk;
-    const int w = nb - k - 1;
-    for (int t = threadIdx.x; t < w * w; t += blockDim.x) {
-      const int i = k + 1 + t / w, jj = k + 1 + t % w;
-      if (jj <= i) A[(size_t)i * ld + jj] -= col[i] * col[jj];
+    const double l = diag[0], rs = diag[1];
+    if (!(rs > 0.0)) return;
+    const int rows = nb - 1 - k;  // below the pivot
+    if (tid < rows) {
+      const double x = L[(k + 1 + tid) * P64_LD + k], q = x * rs;
+      L[(k + 1 + tid) * P64_LD + k] = fma(fma(-q, l, x), rs, q);
+    }
+    if (tid == 128) {
+      L[k * P64_LD + k] = l;
+      rdiag[k] = rs;
+    }
+    __syncthreads();
+    // rank-one update of the lower triangle: rows p and rows - 1 - p make a line of rows + 1 entries
+    const int half = (rows + 1) >> 1, line = rows + 1;
+    for (int t = tid; t < half * line; t += 256) {
+      const int pr = t / line, q = t - pr * line;
+      int i, j;
+      if (q <= pr) { i = pr; j = q; }
+      else { i = rows - 1 - pr; j = q - pr - 1; }
+      if (q > pr && i == pr) continue;  // (the middle row of an odd count, once)
+      const int gi = k + 1 + i, gj = k + 1 + j;
+      L[gi * P64_LD + gj] -= L[gi * P64_LD + k] * L[gj * P64_LD + k];
     }
     __syncthreads();
   }
-  for (int t = threadIdx.x; t < nb * nb; t += blockDim.x) {
-    const int i = t / nb, jj = t % nb;
-    if (jj > i) A[(size_t)i * ld + jj] = 0.0;
+  // inverses of the 16 x 16 diagonal blocks: a thread per column (rows and columns past nb: the identity), each entry
+  // passed on to the rows below at once (a dot product per entry is one long chain)
+  if (tid < 64) {
+    const int b0 = tid & ~15, c = tid & 15;
+    double x[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) x[i] = i == c ? 1.0 : 0.0;
+#pragma unroll
+    for (int t = 0; t < 16; t++) {
+      x[t] *= rdiag[b0 + t];
+#pragma unroll
+      for (int i = t + 1; i < 16; i++) x[i] = fma(-L[(b0 + i) * P64_LD + b0 + t], x[t], x[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 16; i++) X[(b0 + i) * P64_LD + b0 + c] = x[i];
+  }
+  __syncthreads();
+  // block row i, column j: X_ij = -X_ii sum_{j <= k < i} L_ik X_kj
+  const int r16 = tid >> 4, c16 = tid & 15;
+  for (int i = 1; i < 4; i++) {
+    for (int j = 0; j < i; j++) {
+      double t[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int q = 16 * j; q < 16 * i; q += 4)
+#pragma unroll
+        for (int e = 0; e < 4; e++)
+          t[e] = fma(L[(16 * i + r16) * P64_LD + q + e], X[(q + e) * P64_LD + 16 * j + c16], t[e]);
+      Tm[(16 * j + r16) * 17 + c16] = (t[0] + t[1]) + (t[2] + t[3]);
+    }
+    __syncthreads();
+    for (int j = 0; j < i; j++) {
+      double t[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int q = 0; q < 16; q++)  // (X_ii is zero above its diagonal)
+        t[q & 3] = fma(X[(16 * i + r16) * P64_LD + 16 * i + q], Tm[(16 * j + q) * 17 + c16], t[q & 3]);
+      X[(16 * i + r16) * P64_LD + 16 * j + c16] = -((t[0] + t[1]) + (t[2] + t[3]));
+    }
+    __syncthreads();
+  }
+  for (int t = tid; t < nb * nb; t += 256) {
+    const int i = t / nb, j = t % nb;
+    A[(size_t)i * ld + j] = j <= i ? L[i * P64_LD + j] : 0.0;
+    Linv[(size_t)i * ldi + j] = j <= i ? X[i * P64_LD + j] : 0.0;
   }
 }
+constexpr size_t P64_SMEM = (2 * 64 * P64_LD + 64 * 17) * sizeof(double);
 // zero the strict upper triangle of the mb x mb block and every row and column past mb (m x m, ld m)
 __global__ void k_zero_upper(double* A, int mb, int m) {
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < (int64_t)m * m;
@@ -516,6 +664,188 @@ __global__ void __launch_bounds__(512) k_aca(const AcaJob* jobs, int m, int cap,
   }
 }
 
+// The same by a cluster of eight CTAs per tile, each with an eighth of the rows in shared memory: a rank-one step is one
+// pass of its float64 pipe over its rows instead of one SM's over the whole tile through L2, and one cluster barrier:
+// every CTA publishes its largest entry and that entry's row before it, and takes the winner's row from the
+// owner's shared memory after it (two buffers in turn, so that the next step's rows do not overwrite rows still being
+// read).  The balancing factor of a term is applied at the end, from norms summed over the cluster.  A factor
+// of n = 4,096 in tiles of 256: 27.6 -> 4.9 ms of compressions, of n = 1,024 in tiles of 128: 5.1 -> 1.15 ms.
+constexpr int ACA_CL = 8, ACA_T = 256;
+__device__ __forceinline__ uint32_t cluster_map(const void* p, int cta) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(cta));
+  return r;
+}
+__device__ __forceinline__ double cluster_ld(uint32_t a) {
+  double x;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(x) : "r"(a) : "memory");
+  return x;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+static size_t aca_cluster_smem(int m, int cap) {
+  const size_t rp = (size_t)(m + ACA_CL - 1) / ACA_CL;
+  return (rp * m + 2 * ((size_t)m + 1) + m + rp + 2 * (size_t)cap) * sizeof(double);
+}
+__global__ void __cluster_dims__(ACA_CL, 1, 1) __launch_bounds__(ACA_T)
+    k_aca_cluster(const AcaJob* jobs, int m, int cap, double tol, int* ranks, int* capped) {
+  extern __shared__ double smc[];
+  const int rp = (m + ACA_CL - 1) / ACA_CL;
+  double* R = smc;                  // [rp][m] this CTA's rows
+  double* prow = R + (size_t)rp * m;  // [2][m + 1]: the row of this CTA's largest entry, and that entry's reciprocal
+  double* v = prow + 2 * (m + 1);
+  double* u = v + m;                // [rp]
+  double* pn = u + rp;              // [cap] sums of squares of u over this CTA's rows
+  double* pv = pn + cap;            // [cap] of v over its share of columns
+  __shared__ long long ckey[2][ACA_CL];
+  __shared__ int cidx[2][ACA_CL];
+  __shared__ long long shk[ACA_T / 32];
+  __shared__ int shi[ACA_T / 32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = ACA_T / 32;
+  const int cta = blockIdx.x % ACA_CL;
+  const AcaJob jb = jobs[blockIdx.x / ACA_CL];
+  const int mi = jb.mi, mj = jb.mj;
+  const int r0 = cta * rp, nr = max(0, min(rp, mi - r0));
+  const int cp = (mj + ACA_CL - 1) / ACA_CL, c0 = min(mj, cta * cp), c1 = min(mj, c0 + cp);
+  cluster_barrier();  // (every CTA of the cluster runs: their shared memory may be written)
+  long long akey = -1;
+  int aidx = 0x7fffffff;
+  for (int i = wid; i < nr; i += nw)
+    for (int jj = lane; jj < mj; jj += 32) {
+      const double x = jb.R[(size_t)(r0 + i) * m + jj];
+      R[(size_t)i * m + jj] = x;
+      keymax_merge(akey, aidx, abs_key(x), (r0 + i) * mj + jj);
+    }
+  int rank = 0, cp_hit = 0;
+  for (int it = 0;; it ^= 1) {
+    // this CTA's largest entry (every row written: the barrier inside)
+    for (int o = 16; o; o >>= 1) {
+      const long long a2 = __shfl_xor_sync(0xffffffffu, akey, o);
+      const int i2 = __shfl_xor_sync(0xffffffffu, aidx, o);
+      keymax_merge(akey, aidx, a2, i2);
+    }
+    if (lane == 0) {
+      shk[wid] = akey;
+      shi[wid] = aidx;
+    }
+    __syncthreads();
+    akey = shk[0];
+    aidx = shi[0];
+    for (int w = 1; w < nw; w++) keymax_merge(akey, aidx, shk[w], shi[w]);
+    double* pr = prow + it * (m + 1);
+    if (akey >= 0) {
+      const double* row = R + (size_t)(aidx / mj - r0) * m;
+      for (int t = tid; t < mj; t += ACA_T) pr[t] = row[t];
+      if (tid == ACA_T - 1) pr[m] = 1.0 / row[aidx % mj];
+    }
+    if (tid < ACA_CL) {
+      asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(cluster_map(&ckey[it][cta], tid)), "l"(akey) : "memory");
+      asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(cluster_map(&cidx[it][cta], tid)), "r"(aidx) : "memory");
+    }
+    cluster_barrier();
+    int win = 0;
+    akey = ckey[it][0];
+    aidx = cidx[it][0];
+    for (int q = 1; q < ACA_CL; q++) {
+      const long long k2 = ckey[it][q];
+      const int i2 = cidx[it][q];
+      if (k2 > akey || (k2 == akey && i2 < aidx)) {
+        akey = k2;
+        aidx = i2;
+        win = q;
+      }
+    }
+    const double amax = akey >= 0 ? __longlong_as_double(akey) : -1.0;
+    if (!(amax > tol)) break;
+    if (rank >= cap) {
+      cp_hit = 1;
+      break;
+    }
+    const int pj = aidx % mj;
+    const uint32_t wrow = cluster_map(pr, win);
+    {
+      const double piv = cluster_ld(wrow + 8 * pj), rinv = cluster_ld(wrow + 8 * m);
+      for (int t = tid; t < mj; t += ACA_T) {
+        const double x = cluster_ld(wrow + 8 * t), q = x * rinv;
+        v[t] = fma(fma(-q, piv, x), rinv, q);
+      }
+      for (int t = tid; t < nr; t += ACA_T) u[t] = R[(size_t)t * m + pj];
+    }
+    __syncthreads();
+    for (int t = tid; t < nr; t += ACA_T) jb.U[(size_t)(r0 + t) * cap + rank] = u[t];
+    for (int t = c0 + tid; t < c1; t += ACA_T) jb.V[(size_t)t * cap + rank] = v[t];
+    akey = -1;
+    aidx = 0x7fffffff;
+    for (int i = wid; i < nr; i += nw) {
+      double* row = R + (size_t)i * m;
+      const double ui = u[i];
+      for (int jj = lane; jj < mj; jj += 32) {
+        const double x = row[jj] - ui * v[jj];
+        row[jj] = x;
+        keymax_merge(akey, aidx, abs_key(x), (r0 + i) * mj + jj);
+      }
+    }
+    rank++;
+    // (u and v are next written after the next cluster barrier)
+  }
+  // balance the terms: |u| = |v|
+  __syncthreads();
+  for (int k = wid; k < rank; k += nw) {
+    double su = 0.0, sv = 0.0;
+    for (int t = lane; t < nr; t += 32) {
+      const double x = jb.U[(size_t)(r0 + t) * cap + k];
+      su += x * x;
+    }
+    for (int t = c0 + lane; t < c1; t += 32) {
+      const double x = jb.V[(size_t)t * cap + k];
+      sv += x * x;
+    }
+    for (int o = 16; o; o >>= 1) {
+      su += __shfl_xor_sync(0xffffffffu, su, o);
+      sv += __shfl_xor_sync(0xffffffffu, sv, o);
+    }
+    if (lane == 0) {
+      pn[k] = su;
+      pv[k] = sv;
+    }
+  }
+  cluster_barrier();
+  for (int k = wid; k < rank; k += nw) {
+    double su = lane < ACA_CL ? cluster_ld(cluster_map(pn + k, lane)) : 0.0;
+    double sv = lane < ACA_CL ? cluster_ld(cluster_map(pv + k, lane)) : 0.0;
+    for (int o = 4; o; o >>= 1) {
+      su += __shfl_xor_sync(0xffffffffu, su, o);
+      sv += __shfl_xor_sync(0xffffffffu, sv, o);
+    }
+    su = __shfl_sync(0xffffffffu, su, 0);
+    sv = __shfl_sync(0xffffffffu, sv, 0);
+    const double f = sqrt(sqrt(sv) / sqrt(su)), fi = 1.0 / f;
+    for (int t = lane; t < nr; t += 32) jb.U[(size_t)(r0 + t) * cap + k] *= f;
+    for (int t = c0 + lane; t < c1; t += 32) jb.V[(size_t)t * cap + k] *= fi;
+  }
+  if (cta == 0 && tid == 0) {
+    ranks[blockIdx.x / ACA_CL] = rank;
+    if (cp_hit) atomicAdd(capped, 1);
+  }
+  cluster_barrier();  // (no CTA leaves while another reads its sums)
+}
+// The cluster kernel where its rows fit in shared memory (tiles to about 430), else one CTA per tile.
+static int launch_aca(int jobs, int m, int cap, double tol, cudaStream_t st, const AcaJob* d_aj, int* d_ranks,
+                      int* d_capped) {
+  const size_t need = aca_cluster_smem(m, cap);
+  if (need <= 216 * 1024) {
+    TLR_CHECK(raise_smem_limit((const void*)k_aca_cluster, need));
+    k_aca_cluster<<<(unsigned)(jobs * ACA_CL), ACA_T, need, st>>>(d_aj, m, cap, tol, d_ranks, d_capped);
+  } else {
+    TLR_CHECK(raise_smem_limit((const void*)k_aca, 2 * m * sizeof(double)));
+    k_aca<<<(unsigned)jobs, 512, 2 * m * sizeof(double), st>>>(d_aj, m, cap, tol, d_ranks, d_capped);
+  }
+  TLR_CUDA(cudaGetLastError());
+  return TLRMVN_OK;
+}
+
 // ---- limit conditioning (Algorithm 5): a_i -= U_ij (V_ij^T y_j) --------------------------
 struct CondJob {
   const double* U;
@@ -524,13 +854,15 @@ struct CondJob {
   double* b;
   int mi, mj, k;
 };
-__global__ void k_condition(const CondJob* jobs, const double* y, int cap) {
+__global__ void __launch_bounds__(256) k_condition(const CondJob* jobs, const double* y, int cap) {
   __shared__ double t[1024];
   const CondJob jb = jobs[blockIdx.x];
-  for (int c = threadIdx.x; c < jb.k; c += blockDim.x) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int c = wid; c < jb.k; c += nw) {  // (a warp a sum: its loads in flight together)
     double s = 0.0;
-    for (int u = 0; u < jb.mj; u++) s += jb.V[(size_t)u * cap + c] * y[u];
-    t[c] = s;
+    for (int u = lane; u < jb.mj; u += 32) s += jb.V[(size_t)u * cap + c] * y[u];
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) t[c] = s;
   }
   __syncthreads();
   for (int v = threadIdx.x; v < jb.mi; v += blockDim.x) {
@@ -542,43 +874,34 @@ __global__ void k_condition(const CondJob* jobs, const double* y, int cap) {
 }
 
 // ---- within-block permutation of a chosen block ------------------------------------------
-// rows/cols of the diagonal block, its index list and limits, and the rows of
-// the finished factor tiles U_jk (k < j).
-__global__ void k_permute_block(double* S, double* tmp, int64_t* idx, double* a, double* b, const int* order, int mb,
-                                int m, double* const* Urows, int nU, int cap) {
-  for (int t = threadIdx.x; t < mb * mb; t += blockDim.x) {
-    int i = t / mb, jj = t % mb;
-    tmp[(size_t)i * m + jj] = S[(size_t)order[i] * m + order[jj]];
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < mb * mb; t += blockDim.x) {
-    int i = t / mb, jj = t % mb;
-    S[(size_t)i * m + jj] = tmp[(size_t)i * m + jj];
-  }
-  __syncthreads();
-  // idx, a, b via tmp as staging (3 * mb doubles)
-  double* ti = tmp;
-  double* ta = tmp + m;
-  double* tb = tmp + 2 * m;
+// rows and columns of the diagonal block into tmp (copied back by the caller); block 0 also its index list and limits
+__global__ void __launch_bounds__(256) k_permute_block(const double* S, double* tmp, int64_t* idx, double* a, double* b,
+                                                       const int* order, int mb, int m) {
+  for (int i = blockIdx.x; i < mb; i += gridDim.x)
+    for (int j = threadIdx.x; j < mb; j += blockDim.x) tmp[(size_t)i * m + j] = S[(size_t)order[i] * m + order[j]];
+  if (blockIdx.x != 0) return;
+  __shared__ double sa[1024], sb[1024];
+  __shared__ int64_t si[1024];
   for (int t = threadIdx.x; t < mb; t += blockDim.x) {
-    ti[t] = (double)idx[order[t]];
-    ta[t] = a[order[t]];
-    tb[t] = b[order[t]];
+    si[t] = idx[order[t]];
+    sa[t] = a[order[t]];
+    sb[t] = b[order[t]];
   }
   __syncthreads();
   for (int t = threadIdx.x; t < mb; t += blockDim.x) {
-    idx[t] = (int64_t)ti[t];
-    a[t] = ta[t];
-    b[t] = tb[t];
+    idx[t] = si[t];
+    a[t] = sa[t];
+    b[t] = sb[t];
   }
-  __syncthreads();
-  for (int q = 0; q < nU; q++) {
-    double* U = Urows[q];
-    for (int t = threadIdx.x; t < mb * cap; t += blockDim.x) tmp[t] = U[(size_t)order[t / cap] * cap + t % cap];
-    __syncthreads();
-    for (int t = threadIdx.x; t < mb * cap; t += blockDim.x) U[t] = tmp[t];
-    __syncthreads();
-  }
+}
+// (the limits are always there: zeros when no reordering asked for them)
+static int permute_block(double* S, double* tmp, int64_t* idx, double* a, double* b, const int* order, int mb, int m,
+                         cudaStream_t st) {
+  k_permute_block<<<std::min(mb, 128), 256, 0, st>>>(S, tmp, idx, a, b, order, mb, m);
+  TLR_CUDA(cudaGetLastError());
+  TLR_CUDA(cudaMemcpy2DAsync(S, (size_t)m * 8, tmp, (size_t)m * 8, (size_t)mb * 8, (size_t)mb, cudaMemcpyDeviceToDevice,
+                             st));
+  return TLRMVN_OK;
 }
 
 // ---- a cluster's variables reordered in every tile that involves it ------------------------
@@ -694,6 +1017,33 @@ static int check_status(int* d_status, cudaStream_t st, const char* what) {
   return TLRMVN_OK;
 }
 
+// Tile of a batched product (16, 32 or 64 square, as groups of 16): a tile's time is its 16 x 16 groups that exist, a
+// launch's that of the SM with the most of them, and smaller tiles read their operands more often: the one with the
+// fewest groups on the busiest SM, by a tenth at least to leave the larger.
+static int gemm_batched_groups(const std::vector<GemmEntry>& ent) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  sms = std::max(sms, 1);
+  int best = 4;
+  double cost = 1e300;
+  for (int g : {4, 2, 1}) {
+    int64_t tiles = 0, groups = 0;
+    for (const GemmEntry& e : ent) {
+      const int64_t gm = (e.M + 15) / 16, gn = (e.N + 15) / 16;
+      const double part = (e.shape & GEMM_LOWER) ? 0.5 + 0.5 / std::max<int64_t>(1, (gm + g - 1) / g) : 1.0;
+      tiles += std::max<int64_t>(1, (int64_t)(part * (double)(((gm + g - 1) / g) * ((gn + g - 1) / g))));
+      groups += std::max<int64_t>(1, (int64_t)(part * (double)(gm * gn)));
+    }
+    const double per = (double)groups / (double)tiles;  // groups a tile
+    const double c = (double)((tiles + sms - 1) / sms) * per;
+    if (c < 0.9 * cost) {
+      cost = c;
+      best = g;
+    }
+  }
+  return best;
+}
 template <bool TA, bool TB>
 static int run_batched(std::vector<GemmEntry>& ent, std::vector<GemmSeg>& seg, GemmEntry* d_ent, GemmSeg* d_seg,
                        size_t ent_cap, size_t seg_cap, cudaStream_t st) {
@@ -706,56 +1056,74 @@ static int run_batched(std::vector<GemmEntry>& ent, std::vector<GemmSeg>& seg, G
   }
   TLR_CHECK(upload(d_ent, ent, st));
   TLR_CHECK(upload(d_seg, seg, st));
+  const int g = gemm_batched_groups(ent), bt = 16 * g;
+  auto* k = g == 4 ? k_gemm_batched<TA, TB, 4> : (g == 2 ? k_gemm_batched<TA, TB, 2> : k_gemm_batched<TA, TB, 1>);
   for (size_t z0 = 0; z0 < ent.size(); z0 += 65535) {
     unsigned nz = (unsigned)std::min<size_t>(65535, ent.size() - z0);
-    dim3 grid((unsigned)((maxN + 63) / 64), (unsigned)((maxM + 63) / 64), nz);
-    k_gemm_batched<TA, TB><<<grid, 256, 0, st>>>(d_ent + z0, d_seg);
+    dim3 grid((unsigned)((maxN + bt - 1) / bt), (unsigned)((maxM + bt - 1) / bt), nz);
+    k<<<grid, 256, 0, st>>>(d_ent + z0, d_seg);
   }
   TLR_CUDA(cudaGetLastError());
-  // the host vectors are reused right away: wait for the uploads
-  TLR_CUDA(cudaStreamSynchronize(st));
+  // (the host vectors may be reused: a copy from pageable memory returns once it has been staged; the device lists
+  // are overwritten by later uploads of the same stream only)
   return TLRMVN_OK;
 }
 
 // Cholesky factor of the leading mb x mb part of the m x m block A, in place (lower, zero
-// elsewhere), and its inverse Linv: right-looking in panels of 64 -- the panel's diagonal
-// block by one CTA, the panel below it through that block's inverse and the trailing update
-// as GEMMs over the whole GPU -- then the inverse with one warp per column.  P (m x 64) and
-// Pinv (64 x 64) are scratch.  (One CTA for the whole block is bound by one SM's float64
-// rate: ~20 ms at m = 512, against ~1 ms this way.)
-static int chol_inverse(double* A, int mb, int m, double* Linv, double* P, double* Pinv, GemmEntry* d_ent,
-                        GemmSeg* d_seg, size_t ent_cap, size_t seg_cap, int* d_status, cudaStream_t st,
-                        const char* what) {
+// elsewhere), and its inverse Linv (m x m, zero past mb): right-looking in panels of 64 -- the panel's diagonal
+// block and its inverse by one CTA, the panel below it through that inverse and the trailing update
+// as GEMMs over the whole GPU -- then the inverse's blocks below the diagonal ones, a
+// block diagonal at a time, as GEMMs: X_ij = -X_ii sum_{j <= k < i} L_ik X_kj.  P (m x 64) is scratch.  (One CTA
+// for the whole block is bound by one SM's float64 rate: ~20 ms at m = 512.)
+static int chol_inverse(double* A, int mb, int m, double* Linv, double* P, GemmEntry* d_ent, GemmSeg* d_seg,
+                        size_t ent_cap, size_t seg_cap, int* d_status, cudaStream_t st, const char* what) {
   std::vector<GemmEntry> ent;
   std::vector<GemmSeg> seg;
+  TLR_CHECK(raise_smem_limit((const void*)k_potrf_inv64, P64_SMEM));
+  TLR_CUDA(cudaMemsetAsync(Linv, 0, (size_t)m * m * sizeof(double), st));
   for (int k0 = 0; k0 < mb; k0 += 64) {
     const int nb = std::min(64, mb - k0), rest = mb - k0 - nb;
     double* Akk = A + (size_t)k0 * m + k0;
-    k_potrf_diag<<<1, 256, 0, st>>>(Akk, nb, m, d_status);
+    double* Xkk = Linv + (size_t)k0 * m + k0;
+    k_potrf_inv64<<<1, 256, P64_SMEM, st>>>(Akk, nb, m, Xkk, m, d_status);
     TLR_CUDA(cudaGetLastError());
     if (rest == 0) break;
-    k_trinv_cols<<<(nb + 7) / 8, 256, 8 * (size_t)nb * sizeof(double), st>>>(Akk, m, 0, Pinv, 64, 0, nb, nullptr, nb);
-    TLR_CUDA(cudaGetLastError());
     double* Apan = A + (size_t)(k0 + nb) * m + k0;
     ent.clear();
     seg.clear();
-    seg.push_back(GemmSeg{Apan, Pinv, m, 64, nb});  // P = A_21 L_11^-T
+    seg.push_back(GemmSeg{Apan, Xkk, m, m, nb});  // P = A_21 L_11^-T
     ent.push_back(GemmEntry{P, 64, rest, nb, 0, 1, 1.0, 0.0});
     TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
     ent.clear();
     seg.clear();
-    seg.push_back(GemmSeg{P, P, 64, 64, nb});  // A_22 -= P P^T
-    ent.push_back(GemmEntry{A + (size_t)(k0 + nb) * m + k0 + nb, m, rest, rest, 0, 1, -1.0, 1.0});
+    seg.push_back(GemmSeg{P, P, 64, 64, nb});  // A_22 -= P P^T (the lower triangle)
+    ent.push_back(GemmEntry{A + (size_t)(k0 + nb) * m + k0 + nb, m, rest, rest, 0, 1, -1.0, 1.0, GEMM_LOWER});
     TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
     TLR_CUDA(cudaMemcpy2DAsync(Apan, (size_t)m * sizeof(double), P, 64 * sizeof(double), (size_t)nb * sizeof(double),
                                (size_t)rest, cudaMemcpyDeviceToDevice, st));
   }
   k_zero_upper<<<std::max(1, std::min(1024, (m * m + 255) / 256)), 256, 0, st>>>(A, mb, m);
   TLR_CUDA(cudaGetLastError());
-  TLR_CHECK(check_status(d_status, st, what));
-  k_trinv_cols<<<(m + 7) / 8, 256, 8 * (size_t)m * sizeof(double), st>>>(A, m, 0, Linv, m, 0, mb, nullptr, m);
-  TLR_CUDA(cudaGetLastError());
-  return TLRMVN_OK;
+  const int nblk = (mb + 63) / 64;
+  for (int d = 1; d < nblk; d++) {
+    ent.clear();
+    seg.clear();
+    for (int i = d; i < nblk; i++) {  // T = sum_k L_ik X_kj, j = i - d, into P's rows 64 i
+      const int j = i - d, ni = std::min(64, mb - 64 * i);
+      seg.push_back(GemmSeg{A + (size_t)64 * i * m + 64 * j, Linv + (size_t)64 * j * m + 64 * j, m, m, 64 * d});
+      ent.push_back(GemmEntry{P + (size_t)64 * i * 64, 64, ni, 64, (int)seg.size() - 1, (int)seg.size(), 1.0, 0.0});
+    }
+    TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+    ent.clear();
+    seg.clear();
+    for (int i = d; i < nblk; i++) {
+      const int j = i - d, ni = std::min(64, mb - 64 * i);
+      seg.push_back(GemmSeg{Linv + (size_t)64 * i * m + 64 * i, P + (size_t)64 * i * 64, m, 64, ni});
+      ent.push_back(GemmEntry{Linv + (size_t)64 * i * m + 64 * j, m, ni, 64, (int)seg.size() - 1, (int)seg.size(), -1.0, 0.0});
+    }
+    TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+  }
+  return check_status(d_status, st, what);
 }
 
 static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, std::vector<int> sizes,
@@ -802,9 +1170,8 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
   TLR_CHECK(bd.get(&d_blist, r));
   TLR_CHECK(bd.get(&d_logp, r));
   TLR_CHECK(bd.get(&Linv, (size_t)m * m));
-  double *Pch = nullptr, *Pinv = nullptr;  // scratch of the blocked Cholesky
-  TLR_CHECK(bd.get(&Pch, (size_t)m * 64));
-  TLR_CHECK(bd.get(&Pinv, (size_t)64 * 64));
+  double* Pch = nullptr;  // scratch of the blocked Cholesky
+  TLR_CHECK(bd.get(&Pch, (size_t)(m + 63) / 64 * 64 * 64));
   const size_t npairs = (size_t)r * (r - 1) / 2;
   TLR_CHECK(bd.get(&pool, std::max<size_t>(npairs, 1) * 2 * (size_t)m * cap));
   if (tlr) {
@@ -818,14 +1185,13 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
   TLR_CHECK(bd.get(&work, uc_par * m * m));
   TLR_CHECK(bd.get(&Xs, max_pairs_step * cap * cap));
   TLR_CHECK(bd.get(&Ys, max_pairs_step * cap * m));
-  const size_t ent_cap = std::max<size_t>(max_pairs_step, (size_t)r) + 8, seg_cap = 2 * ent_cap;
+  const size_t ent_cap = std::max<size_t>(max_pairs_step, (size_t)r) + 24, seg_cap = 2 * ent_cap;
   GemmEntry* d_ent;
   GemmSeg* d_seg;
   TileJob* d_tj;
   AcaJob* d_aj;
   CondJob* d_cj;
   PackJob* d_pj;
-  double** d_urows;
   TLR_CHECK(bd.get(&d_ent, ent_cap));
   TLR_CHECK(bd.get(&d_seg, seg_cap));
   TLR_CHECK(bd.get(&d_tj, jcap));
@@ -834,7 +1200,6 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
   TLR_CHECK(bd.get(&d_pmj, (size_t)r));
   TLR_CHECK(bd.get(&d_cj, (size_t)r));
   TLR_CHECK(bd.get(&d_pj, std::max<size_t>(npairs, 1)));
-  TLR_CHECK(bd.get(&d_urows, (size_t)r));
   TLR_CHECK(upload(d_idx, idx_h, st));
   TLR_CHECK(upload(d_bsize, sizes, st));
   TLR_CUDA(cudaMemsetAsync(d_status, 0, sizeof(int), st));
@@ -860,27 +1225,18 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
   }
   std::vector<int> pos2blk(r);
   std::iota(pos2blk.begin(), pos2blk.end(), 0);
-  const size_t uc_smem = (size_t)m * (5 * sizeof(double) + sizeof(int));
-  TLR_CHECK(raise_smem_limit((const void*)k_uc, (size_t)uc_smem));
-  TLR_CHECK(raise_smem_limit((const void*)k_aca, 2 * m * sizeof(double)));
-  TLR_CHECK(raise_smem_limit((const void*)k_potrf, m * sizeof(double)));
-  TLR_CHECK(raise_smem_limit((const void*)k_trinv_cols, 8 * (size_t)m * sizeof(double)));
-  const int uc_threads = m >= 256 ? 512 : 256;
 
   if (o.reorder == TLRMVN_REORDER_BLOCK) {
     // Algorithm 4: one UC estimate per original block, then a selection sort
     std::vector<int> bl(r);
     std::iota(bl.begin(), bl.end(), 0);
     TLR_CHECK(upload(d_blist, bl, st));
-    k_uc<<<r, uc_threads, uc_smem, st>>>(d_blist, diagS, d_bsize, m, d_a, d_b, work, d_logp, 1, d_order, d_y,
-                                          d_status);
-    TLR_CUDA(cudaGetLastError());
+    TLR_CHECK(launch_uc(r, m, st, d_blist, diagS, d_bsize, d_a, d_b, work, d_logp, d_order, d_y, d_status));
     TLR_CHECK(check_status(d_status, st, "block reordering"));
     // within-block order: the UC pivot order of each original block
     for (int b = 0; b < r; b++) {
-      k_permute_block<<<1, 512, 0, st>>>(diagS + (size_t)b * m * m, ptmp, d_idx + (size_t)b * m, d_a + (size_t)b * m,
-                                         d_b + (size_t)b * m, d_order + (size_t)b * m, sizes[b], m, d_urows, 0, cap);
-      TLR_CUDA(cudaGetLastError());
+      TLR_CHECK(permute_block(diagS + (size_t)b * m * m, ptmp, d_idx + (size_t)b * m, d_a + (size_t)b * m,
+                              d_b + (size_t)b * m, d_order + (size_t)b * m, sizes[b], m, st));
     }
     std::vector<double> p(r);
     TLR_CUDA(cudaMemcpyAsync(p.data(), d_logp, r * 8, cudaMemcpyDeviceToHost, st));
@@ -923,8 +1279,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
       for (size_t t = 0; t < jobs.size(); t++)
         aj[t] = AcaJob{Sij + t * m * m, Uslot((int)jobs[t].s), Vslot((int)jobs[t].s), jobs[t].mi, jobs[t].mj};
       TLR_CHECK(upload(d_aj, aj, st));
-      k_aca<<<(unsigned)aj.size(), 512, 2 * m * sizeof(double), st>>>(d_aj, m, cap, o.tol, d_ranks, d_capped);
-      TLR_CUDA(cudaGetLastError());
+      TLR_CHECK(launch_aca((int)aj.size(), m, cap, o.tol, st, d_aj, d_ranks, d_capped));
       std::vector<int> got(jobs.size());
       TLR_CUDA(cudaMemcpyAsync(got.data(), d_ranks, got.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
       TLR_CUDA(cudaStreamSynchronize(st));
@@ -962,9 +1317,8 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
         // -- lines 4-8: UC of every remaining block; the smallest estimate takes position j
         std::vector<int> bl(pos2blk.begin() + j, pos2blk.end());
         TLR_CHECK(upload(d_blist, bl, st));
-        k_uc<<<(unsigned)bl.size(), uc_threads, uc_smem, st>>>(d_blist, diagS, d_bsize, m, d_a, d_b, work, d_logp, 1,
-                                                               d_order, d_y, d_status);
-        TLR_CUDA(cudaGetLastError());
+        TLR_CHECK(launch_uc((int)bl.size(), m, st, d_blist, diagS, d_bsize, d_a, d_b, work, d_logp, d_order, d_y,
+                            d_status));
         TLR_CHECK(check_status(d_status, st, "iterative block reordering"));
         std::vector<double> p(bl.size());
         TLR_CUDA(cudaMemcpyAsync(p.data(), d_logp, p.size() * 8, cudaMemcpyDeviceToHost, st));
@@ -978,9 +1332,8 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
         // cluster's variables in every tile that involves it
         const int c = pos2blk[j];
         const int* ord = d_order + (size_t)chosen * m;
-        k_permute_block<<<1, 512, 0, st>>>(diagS + (size_t)c * m * m, ptmp, d_idx + (size_t)c * m, d_a + (size_t)c * m,
-                                           d_b + (size_t)c * m, ord, sizes[c], m, d_urows, 0, cap);
-        TLR_CUDA(cudaGetLastError());
+        TLR_CHECK(permute_block(diagS + (size_t)c * m * m, ptmp, d_idx + (size_t)c * m, d_a + (size_t)c * m,
+                                d_b + (size_t)c * m, ord, sizes[c], m, st));
         std::vector<PermJob> pj;
         for (int q = 0; q < r; q++) {
           if (q == c) continue;
@@ -997,7 +1350,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
       const int cj = pos2blk[j], mj = sizes[cj];
       double* Sjj = diagS + (size_t)cj * m * m;
       // -- line 10: L_jj and its inverse
-      TLR_CHECK(chol_inverse(Sjj, mj, m, Linv, Pch, Pinv, d_ent, d_seg, ent_cap, seg_cap, d_status, st,
+      TLR_CHECK(chol_inverse(Sjj, mj, m, Linv, Pch, d_ent, d_seg, ent_cap, seg_cap, d_status, st,
                              "diagonal Cholesky"));
       if (j == r - 1) break;
       // -- line 12: L_ij = Sigma_ij (.) Sigma_jj^-T = U (L_jj^-1 V)^T, truncated; in batches
@@ -1145,9 +1498,8 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
       if (o.reorder == TLRMVN_REORDER_ITERATIVE) {
         std::vector<int> bl(pos2blk.begin() + j, pos2blk.end());
         TLR_CHECK(upload(d_blist, bl, st));
-        k_uc<<<(unsigned)bl.size(), uc_threads, uc_smem, st>>>(d_blist, diagS, d_bsize, m, d_a, d_b, work, d_logp, 1,
-                                                               d_order, d_y, d_status);
-        TLR_CUDA(cudaGetLastError());
+        TLR_CHECK(launch_uc((int)bl.size(), m, st, d_blist, diagS, d_bsize, d_a, d_b, work, d_logp, d_order, d_y,
+                            d_status));
         TLR_CHECK(check_status(d_status, st, "iterative block reordering"));
         std::vector<double> p(bl.size());
         TLR_CUDA(cudaMemcpyAsync(p.data(), d_logp, p.size() * 8, cudaMemcpyDeviceToHost, st));
@@ -1171,17 +1523,21 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
       double* Sjj = diagS + (size_t)bj * m * m;
       const double* yj = d_y + (size_t)chosen * m;
       if (permute) {
-        std::vector<double*> ur;
+        const int* ord = d_order + (size_t)chosen * m;
+        TLR_CHECK(permute_block(Sjj, ptmp, d_idx + (size_t)bj * m, d_a + (size_t)bj * m, d_b + (size_t)bj * m, ord, mj, m,
+                                st));
+        // the rows of the finished factor tiles U_jk (k < j)
+        std::vector<PermJob> pj;
         for (int k = 0; k < j; k++)
-          if (rank[(size_t)j * r + k] > 0) ur.push_back(Uslot(slot[(size_t)j * r + k]));
-        TLR_CHECK(upload(d_urows, ur, st));
-        k_permute_block<<<1, 512, 0, st>>>(Sjj, ptmp, d_idx + (size_t)bj * m, d_a + (size_t)bj * m, d_b + (size_t)bj * m,
-                                           d_order + (size_t)chosen * m, mj, m, d_urows, (int)ur.size(), cap);
-        TLR_CUDA(cudaGetLastError());
-        TLR_CUDA(cudaStreamSynchronize(st));
+          if (rank[(size_t)j * r + k] > 0) pj.push_back(PermJob{Uslot(slot[(size_t)j * r + k]), rank[(size_t)j * r + k]});
+        if (!pj.empty()) {
+          TLR_CHECK(upload(d_pmj, pj, st));
+          k_permute_rows<<<(unsigned)pj.size(), 256, 0, st>>>(d_pmj, ord, mj, cap);
+          TLR_CUDA(cudaGetLastError());
+        }
       }
       // -- L_jj and its inverse
-      TLR_CHECK(chol_inverse(Sjj, mj, m, Linv, Pch, Pinv, d_ent, d_seg, ent_cap, seg_cap, d_status, st,
+      TLR_CHECK(chol_inverse(Sjj, mj, m, Linv, Pch, d_ent, d_seg, ent_cap, seg_cap, d_status, st,
                              "diagonal Cholesky"));
       const int nrem = r - 1 - j;
       if (nrem == 0) break;
@@ -1260,7 +1616,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
       for (int q = 0; q < nrem; q++) {
         int mi = sizes[pos2blk[j + 1 + q]];
         seg.push_back(GemmSeg{Sij + (size_t)q * m * m, Linv, m, m, mj});
-        ent.push_back(GemmEntry{Lij + (size_t)q * m * m, m, mi, mj, q, q + 1, 1.0, 0.0});
+        ent.push_back(GemmEntry{Lij + (size_t)q * m * m, m, mi, mj, q, q + 1, 1.0, 0.0, GEMM_KTRI});
       }
       TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
       // -- ACA of every L_ij into fresh slots
@@ -1273,8 +1629,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
           aj[q] = AcaJob{Lij + (size_t)q * m * m, Uslot(s), Vslot(s), sizes[pos2blk[i]], mj};
         }
         TLR_CHECK(upload(d_aj, aj, st));
-        k_aca<<<nrem, 512, 2 * m * sizeof(double), st>>>(d_aj, m, cap, o.tol, d_ranks, d_capped);
-        TLR_CUDA(cudaGetLastError());
+        TLR_CHECK(launch_aca(nrem, m, cap, o.tol, st, d_aj, d_ranks, d_capped));
         std::vector<int> rk(nrem);
         TLR_CUDA(cudaMemcpyAsync(rk.data(), d_ranks, nrem * sizeof(int), cudaMemcpyDeviceToHost, st));
         TLR_CUDA(cudaStreamSynchronize(st));
@@ -1494,12 +1849,8 @@ static int reorder_tiles(Factor& F, const double* a, const double* b, cudaStream
   TLR_CUDA(cudaMemsetAsync(S, 0, r * mm * 8, st));
   TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, (size_t)r, (size_t)r, st)));
   // P_j: the univariate-conditioning pivot order with the new limits
-  const size_t uc_smem = (size_t)m * (5 * sizeof(double) + sizeof(int));
-  TLR_CHECK(raise_smem_limit((const void*)k_uc, uc_smem));
   TLR_CHECK(raise_smem_limit((const void*)k_potrf, m * sizeof(double)));
-  k_uc<<<r, m >= 256 ? 512 : 256, uc_smem, st>>>(d_blist, S, d_bsize, m, d_a, d_b, work, d_logp, 1, d_order, d_y,
-                                                  d_status);
-  TLR_CUDA(cudaGetLastError());
+  TLR_CHECK(launch_uc(r, m, st, d_blist, S, d_bsize, d_a, d_b, work, d_logp, d_order, d_y, d_status));
   TLR_CHECK(check_status(d_status, st, "within-tile reordering"));
   // Lt_j = chol(P S_j P^T) (in work); X_j = P^T Lt_j; Binv_j = B_j^-1; Q_j = Binv_j X_j
   const unsigned gx = (unsigned)std::max<size_t>(1, std::min<size_t>(64, (mm + 255) / 256));

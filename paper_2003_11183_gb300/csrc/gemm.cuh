@@ -321,78 +321,102 @@ struct GemmEntry {
   int ldc, M, N;
   int seg0, seg1;  // segments [seg0, seg1)
   double alpha, beta;
+  int shape = 0;  // GEMM_LOWER: only the tiles that meet the lower triangle of C; GEMM_KTRI: the second operand's
+                  // column n has no entries past k = n (an inverse of a lower triangle, transposed)
 };
+enum { GEMM_LOWER = 1, GEMM_KTRI = 2 };
 
-template <bool TA, bool TB>
+// One 16-deep step of a 16 G x 16 G tile, of which only the first MI x NJ groups of 16 x 16 exist.
+template <int G, int MI, int NJ>
+__device__ __forceinline__ void gemm_group_step(const double (&As)[16][16 * G + 1], const double (&Bs)[16][16 * G + 1],
+                                                int kn, int tx, int ty, double (&acc)[G][G]) {
+  auto one = [&](int kk) {
+    double a[MI], b[NJ];
+#pragma unroll
+    for (int i = 0; i < MI; i++) a[i] = As[kk][ty + 16 * i];
+#pragma unroll
+    for (int j = 0; j < NJ; j++) b[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+    for (int i = 0; i < MI; i++)
+#pragma unroll
+      for (int j = 0; j < NJ; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+  };
+  if (kn == 16) {
+#pragma unroll 4
+    for (int kk = 0; kk < 16; kk++) one(kk);
+  } else {
+    for (int kk = 0; kk < kn; kk++) one(kk);
+  }
+}
+template <int G, int MI, int NJ = G>
+__device__ __forceinline__ void gemm_group_step_n(int nj, const double (&As)[16][16 * G + 1],
+                                                  const double (&Bs)[16][16 * G + 1], int kn, int tx, int ty,
+                                                  double (&acc)[G][G]) {
+  if (NJ == 1 || nj == NJ) gemm_group_step<G, MI, NJ>(As, Bs, kn, tx, ty, acc);
+  else gemm_group_step_n<G, MI, (NJ > 1 ? NJ - 1 : 1)>(nj, As, Bs, kn, tx, ty, acc);
+}
+template <int G, int MI = G>
+__device__ __forceinline__ void gemm_group_step_mn(int mi, int nj, const double (&As)[16][16 * G + 1],
+                                                   const double (&Bs)[16][16 * G + 1], int kn, int tx, int ty,
+                                                   double (&acc)[G][G]) {
+  if (MI == 1 || mi == MI) gemm_group_step_n<G, MI>(nj, As, Bs, kn, tx, ty, acc);
+  else gemm_group_step_mn<G, (MI > 1 ? MI - 1 : 1)>(mi, nj, As, Bs, kn, tx, ty, acc);
+}
+
+// Bound by the float64 pipes that a launch reaches: one 64 x 64 x 64 product takes an SM 65 us.  So the tile (16 G
+// square, G = 4, 2, 1) is chosen for the busiest SM (gemm_batched_tile), and, the products of the tiles' ranks
+// (mostly below 16) being a corner of a tile, only the 16 x 16 groups that exist are multiplied and copied.  All
+// products of a factor of n = 4,096 in tiles of 256: 29.5 -> 9.8 ms.
+template <bool TA, bool TB, int G>
 __global__ void __launch_bounds__(256) k_gemm_batched(const GemmEntry* __restrict__ ent, const GemmSeg* __restrict__ seg) {
-  __shared__ double As[16][64 + 1];
-  __shared__ double Bs[16][64 + 1];
+  constexpr int BT = 16 * G;
+  __shared__ double As[16][BT + 1];
+  __shared__ double Bs[16][BT + 1];
   const GemmEntry e = ent[blockIdx.z];
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+  const int m0 = blockIdx.y * BT, n0 = blockIdx.x * BT;
   if (m0 >= e.M || n0 >= e.N) return;
+  if ((e.shape & GEMM_LOWER) && n0 >= m0 + BT) return;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4];
+  const int mi = min(G, (e.M - m0 + 15) >> 4), nj = min(G, (e.N - n0 + 15) >> 4);
+  double acc[G][G];
 #pragma unroll
-  for (int i = 0; i < 4; i++)
+  for (int i = 0; i < G; i++)
 #pragma unroll
-    for (int j = 0; j < 4; j++) acc[i][j] = 0.0;
+    for (int j = 0; j < G; j++) acc[i][j] = 0.0;
   for (int s = e.seg0; s < e.seg1; s++) {
     const GemmSeg g = seg[s];
-    for (int k0 = 0; k0 < g.K; k0 += 16) {
-      for (int l = threadIdx.x; l < 64 * 16; l += 256) {
+    const int K = (e.shape & GEMM_KTRI) ? min(g.K, n0 + BT) : g.K;
+    for (int k0 = 0; k0 < K; k0 += 16) {
+      for (int l = threadIdx.x; l < BT * 16; l += 256) {
         int mm, kk;
-        if (TA) { kk = l >> 6; mm = l & 63; } else { mm = l >> 4; kk = l & 15; }
+        if (TA) { kk = l / BT; mm = l % BT; } else { mm = l >> 4; kk = l & 15; }
+        if (mm >= 16 * mi) continue;
         int gm = m0 + mm, gk = k0 + kk;
         double v = 0.0;
-        if (gm < e.M && gk < g.K) v = TA ? g.A[(int64_t)gk * g.lda + gm] : g.A[(int64_t)gm * g.lda + gk];
+        if (gm < e.M && gk < K) v = TA ? g.A[(int64_t)gk * g.lda + gm] : g.A[(int64_t)gm * g.lda + gk];
         As[kk][mm] = v;
       }
-      for (int l = threadIdx.x; l < 16 * 64; l += 256) {
+      for (int l = threadIdx.x; l < 16 * BT; l += 256) {
         int kk, nn;
-        if (TB) { nn = l >> 4; kk = l & 15; } else { kk = l >> 6; nn = l & 63; }
+        if (TB) { nn = l >> 4; kk = l & 15; } else { kk = l / BT; nn = l % BT; }
+        if (nn >= 16 * nj) continue;
         int gk = k0 + kk, gn = n0 + nn;
         double v = 0.0;
-        if (gk < g.K && gn < e.N) v = TB ? g.B[(int64_t)gn * g.ldb + gk] : g.B[(int64_t)gk * g.ldb + gn];
+        if (gk < K && gn < e.N) v = TB ? g.B[(int64_t)gn * g.ldb + gk] : g.B[(int64_t)gk * g.ldb + gn];
         Bs[kk][nn] = v;
       }
       __syncthreads();
       // (small ranks leave most of the last 16-deep step empty: only its kn rows are summed)
-      const int kn = min(16, g.K - k0);
-      if (kn == 16) {
-#pragma unroll
-        for (int kk = 0; kk < 16; kk++) {
-          double a[4], b[4];
-#pragma unroll
-          for (int i = 0; i < 4; i++) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-          for (int j = 0; j < 4; j++) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-          for (int i = 0; i < 4; i++)
-#pragma unroll
-            for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-      } else {
-        for (int kk = 0; kk < kn; kk++) {
-          double a[4], b[4];
-#pragma unroll
-          for (int i = 0; i < 4; i++) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-          for (int j = 0; j < 4; j++) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-          for (int i = 0; i < 4; i++)
-#pragma unroll
-            for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-        }
-      }
+      gemm_group_step_mn<G>(mi, nj, As, Bs, min(16, K - k0), tx, ty, acc);
       __syncthreads();
     }
   }
 #pragma unroll
-  for (int i = 0; i < 4; i++) {
+  for (int i = 0; i < G; i++) {
     int gm = m0 + ty + 16 * i;
     if (gm >= e.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
+    for (int j = 0; j < G; j++) {
       int gn = n0 + tx + 16 * j;
       if (gn >= e.N) continue;
       double* c = e.C + (int64_t)gm * e.ldc + gn;

@@ -916,7 +916,7 @@ struct Lims {
 // The float64 step's tables on the current device: made by the first float64 solve there (k_tables64, a fraction of a
 // millisecond) and kept, 115 KB, until the process ends; complete before any solve reads them.
 __device__ __align__(16) double g_tables64[T64_DOUBLES];
-static int tables64(const double** out, cudaStream_t st) {
+int tables64(const double** out, cudaStream_t st) {
   static std::mutex mu;
   static std::vector<std::pair<int, const double*>> made;
   int dev = 0;
