@@ -124,6 +124,7 @@ struct Factor {
   int32_t* vmap16 = nullptr;
   std::vector<int64_t> kpad_off;
   int64_t kmax16 = 0, kw16 = 0, my16 = 0;
+  void* stc_tiles = nullptr;  // r StcTile (sweep_tc.cuh)
   // fp16 operands of the FP16-shift path, same layouts: U16h = U g a_ij and V16h = V c_ij
   // with per-tile powers of two a_ij, c_ij (max |U g a| and max |V c| in (1/2, 1], a_ij
   // raised where the projections' range needs it), B16x2h the fp16 split of B g; wscale16

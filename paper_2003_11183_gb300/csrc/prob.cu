@@ -482,7 +482,7 @@ __global__ void k_pad_v32(const double* Vt, int64_t kc, int64_t kc4, int64_t m, 
 // Makes the copies a precision needs; the first caller makes them (and waits for
 // them) under the factor's lock, so concurrent streams never see a partial copy.
 static int ensure_copies_locked(Factor& F, int precision, cudaStream_t st);
-static bool layout_ready(const Factor& F) { return !F.kpad_off.empty() && (F.ktot == 0 || F.vmap16); }
+static bool layout_ready(const Factor& F) { return !F.kpad_off.empty() && F.stc_tiles && (F.ktot == 0 || F.vmap16); }
 static bool bf16_ready(const Factor& F) {
   return layout_ready(F) && (F.ktot == 0 || (F.U16 && F.V16)) && F.B16x2;
 }
@@ -640,6 +640,7 @@ static int make_fp16_copies(Factor& F, cudaStream_t st) {
 // The padded rank space (row tile i starts at a multiple of 64) and vmap16: for each Vcat row, its row of it.
 static int make_layout(Factor& F, cudaStream_t st) {
   dfree(F.vmap16);
+  dfree(F.stc_tiles);
   const int r = F.r, m = F.m;
   std::vector<int64_t> off(r + 1, 0);
   int64_t kmax = 0;
@@ -662,6 +663,17 @@ static int make_layout(Factor& F, cudaStream_t st) {
     }
     TLR_CHECK(dalloc(&F.vmap16, (size_t)F.ktot));
     TLR_CUDA(cudaMemcpyAsync(F.vmap16, v16.data(), v16.size() * 4, cudaMemcpyHostToDevice, st));
+    TLR_CUDA(cudaStreamSynchronize(st));
+  }
+  {
+    std::vector<StcTile> tiles(r);
+    for (int i = 0; i < r; i++)
+      tiles[i] = StcTile{(int)F.tile_off[i], (int)F.tsize(i),       (int)off[i], (int)F.krow(i),
+                         (int)F.kcol_off[i], (int)F.kcol(i), {0, 0}};
+    StcTile* d = nullptr;
+    TLR_CHECK(dalloc(&d, (size_t)r));
+    F.stc_tiles = d;
+    TLR_CUDA(cudaMemcpyAsync(d, tiles.data(), tiles.size() * sizeof(StcTile), cudaMemcpyHostToDevice, st));
     TLR_CUDA(cudaStreamSynchronize(st));
   }
   F.kpad_off = off;
@@ -888,19 +900,17 @@ static int64_t chunk_simt(const tlrmvn_opts& o, const Tuning& tu, int64_t S, int
   const double per = (double)(ktot + 2 * m) * es + 16.0;
   return round_chunk((int64_t)std::max(256.0, std::min((double)S, budget / per)), S);
 }
-// (float32 path: within 8 GiB, and passes of equal size that fit the three CTAs an SM holds -- a launch over one CTA
-// more than that would run twice as long)
+// (passes of equal size that fit the six CTAs, float32: three, that an SM holds -- one CTA more would run a whole
+// solve on its own -- and the float32 path within 8 GiB)
 static int64_t chunk_tc(const tlrmvn_opts& o, const Tuning& tu, int64_t S, int64_t wrows, int64_t ly, bool f32, int sms) {
   if (o.sample_chunk > 0) return round_chunk(o.sample_chunk, S);
   if (tu.chunk > 0) return round_chunk(tu.chunk, S);
   const double budget = (f32 ? 8.0 : 32.0) * (1ull << 30);
   const double per = (double)wrows * 2 + (double)ly * 2 + 16.0;
   int64_t C = (int64_t)std::max(256.0, std::min((double)S, budget / per));
-  if (f32) {
-    C = std::min(C, (int64_t)3 * sms * STC_NS);
-    const int64_t passes = (S + C - 1) / C;
-    C = (S + passes - 1) / passes;
-  }
+  C = std::min(C, (int64_t)(f32 ? 3 : 6) * sms * STC_NS);
+  const int64_t passes = (S + C - 1) / C;
+  C = (S + passes - 1) / passes;
   return round_chunk(C, S);
 }
 
@@ -1012,7 +1022,7 @@ static SweepShape sweep_shape(int64_t C, int mt, int forced) {
 // else the 16-bit paths take one, so that six CTAs share an SM, and the float32 path two (three CTAs, by its TMEM
 // columns four at most).
 typedef void (*SweepTcKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
-                              const CUtensorMap, const CUtensorMap, const SweepTcArgs, const SweepTcLaunch);
+                              const CUtensorMap, const CUtensorMap, const SweepTcLaunch);
 template <int MODE, int NST>
 static SweepTcKernel sweep_tc_variant(int f) {
   static const SweepTcKernel t[4] = {k_sweep_tc<0, MODE, NST>, k_sweep_tc<SWEEP_PERIODIZE, MODE, NST>,
@@ -1030,6 +1040,10 @@ static int sweep_tc_stages(int mode, int64_t ctas, int sms) {
   const bool few = ctas <= 2 * (int64_t)sms;
   return mode == STC_FP32 ? (few ? 3 : 2) : (few ? 4 : 1);
 }
+// Tiles of one launch: a launch of many blocks keeps its CTAs' places on the SMs until all its tiles are done, so a
+// solve of many variables goes in launches of about 16,384 (10 to 25 ms where every SM is full), between which
+// the kernels of other streams get their turn.
+static int sweep_tc_span(int m) { return std::max(1, 16384 / m); }
 // Dynamic shared memory of a whole-tile sweep launch: the kernel's own need, or (tuning, one-stage launches) more, so
 // that no more than `ctas` fit an SM.
 static size_t sweep_tc_launch_smem(int ctas, int mode, int nst) {
@@ -1064,46 +1078,54 @@ struct TcOperands {
   int64_t my;
   int* err;
   int mode = STC_BF16;
-  int sms = 1;
+  int nst = 1;
 };
 
-// Whole diagonal tile i: one launch of k_sweep_tc
-// (low-rank shifts, in-tile coupling, sweep and projections).
-static void sweep_tile_tc(const Factor& F, int i, const Lims& L, const float* rs32, const uint64_t* dD,
-                          int64_t c0, int64_t N, int64_t Cc, int periodize, unsigned short* Ys, int64_t ldys,
-                          double* logP, const TcOperands& tco, const Tuning& tu, cudaStream_t st, Prof& pf) {
-  const int m = F.m, mt = (int)F.tsize(i);
-  SweepTcArgs t;
-  t.rec = F.rec32 + (size_t)i * m * STC_REC;
-  t.BT = F.BT32 + (size_t)i * m * F.ldbt;
+// Zeroes what no sweep writes of W and its products read: the rows between a tile's ranks and the next multiple of 64,
+// and the columns [C, ldw) (finite values: they meet zeros, or are of samples that nobody reads).  parts: W's hi rows,
+// or these and as many lo rows.
+static __global__ void __launch_bounds__(256) k_w_padding(const StcTile* tiles, int parts, int64_t kw, int64_t C,
+                                                          int64_t ldw, unsigned short* W) {
+  const StcTile t = tiles[blockIdx.x];
+  const int end = (t.kr + 63) / 64 * 64, rest = (int)(ldw - C);
+  for (int h = 0; h < parts; h++) {
+    unsigned short* w = W + (h * kw + t.krow0) * ldw;
+    for (int64_t x = ((int64_t)blockIdx.y * blockDim.x + threadIdx.x) * 8; x < ldw;
+         x += (int64_t)gridDim.y * blockDim.x * 8)
+      for (int k = t.kr; k < end; k++) *reinterpret_cast<uint4*>(w + k * ldw + x) = make_uint4(0, 0, 0, 0);
+    for (int64_t e = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; e < (int64_t)t.kr * rest;
+         e += (int64_t)gridDim.y * blockDim.x)
+      w[e / rest * ldw + C + e % rest] = 0;
+  }
+}
+
+// The chunk's tiles in launches of k_sweep_tc (low-rank shifts, in-tile coupling, sweep and projections).
+static void sweep_tiles_tc(const Factor& F, const Lims& L, const float* rs32, const uint64_t* dD, int64_t c0, int64_t N,
+                           int64_t Cc, int periodize, unsigned short* Ys, int64_t ldys, double* logP, const TcOperands& tco,
+                           const Tuning& tu, cudaStream_t st, Prof& pf) {
+  SweepTcLaunch d{};
+  SweepTcArgs& t = d.base;
+  t.rec = F.rec32;
+  t.BT = F.BT32;
   t.ldbt = F.ldbt;
-  t.mt = mt;
-  t.a = L.a32 + F.tile_off[i];
-  t.b = L.b32 + F.tile_off[i];
+  t.a = L.a32;
+  t.b = L.b32;
   t.ys_lo = tco.my;
-  t.brow0 = i * m;
   t.alo = (int)tco.my;
   t.blo = (int)tco.my;
-  t.urow0 = i * m;
-  t.krow0 = (int)F.kpad_off[i];
-  t.kr = (int)F.krow(i);
-  t.kcol0 = (int)F.kcol_off[i];
-  t.kc = (int)F.kcol(i);
   t.ldw = tco.ldw;
-  t.vmap = F.vmap16 ? F.vmap16 + F.kcol_off[i] : nullptr;
-  t.wscale = nullptr;
-  if (tco.mode == STC_FP16 && F.wscale16) t.wscale = F.wscale16 + F.kcol_off[i];
-  if (tco.mode == STC_FP32 && F.wscale32) t.wscale = F.wscale32 + F.kcol_off[i];
+  t.vmap = F.vmap16;
+  t.wscale = tco.mode == STC_FP16 ? F.wscale16 : (tco.mode == STC_FP32 ? F.wscale32 : nullptr);
   t.tscale = tco.mode == STC_FP16 ? F.inv_g16 : 1.0f;
-  t.rscale = tco.mode == STC_FP32 ? F.rscale32 + (size_t)i * m : nullptr;
+  t.rscale = tco.mode == STC_FP32 ? F.rscale32 : nullptr;
   t.wlo = (int)F.kw16;
   t.ulo = (int)F.kmax16;
   t.vlo = (int)F.my16;
   t.err = tco.err;
-  SweepTcLaunch d;
+  d.tiles = (const StcTile*)F.stc_tiles;
+  d.m = F.m;
   d.D = dD;
   d.ldD = F.n + 1;
-  d.coord0 = F.tile_off[i];
   d.sample0 = c0;
   d.N = N;
   d.C = Cc;
@@ -1112,15 +1134,17 @@ static void sweep_tile_tc(const Factor& F, int i, const Lims& L, const float* rs
   d.ldys = ldys;
   d.W = tco.W;
   d.logP = logP;
-  d.first = (i == 0);
   const int flags = (periodize ? SWEEP_PERIODIZE : 0) | (L.one_sided ? SWEEP_ONE_SIDED : 0);
-  pf.begin(TLRMVN_KC_DIAG);
-  const int64_t ctas = (Cc + STC_NS - 1) / STC_NS;
-  const int nst = sweep_tc_stages(tco.mode, ctas, tco.sms);
-  launch_pdl(sweep_tc_kernel(flags, tco.mode, nst), dim3((unsigned)ctas), dim3(STC_NS),
-             sweep_tc_launch_smem(tu.tc_ctas, tco.mode, nst), st, tco.mapY32, tco.mapB32, tco.mapW, tco.mapU64, tco.mapY64,
-             tco.mapV64, t, d);
-  pf.end();
+  const int span = sweep_tc_span(F.m);
+  const unsigned ctas = (unsigned)((Cc + STC_NS - 1) / STC_NS);
+  const size_t smem = sweep_tc_launch_smem(tu.tc_ctas, tco.mode, tco.nst);
+  for (d.i0 = 0; d.i0 < F.r; d.i0 = d.i1) {
+    d.i1 = std::min(F.r, d.i0 + span);
+    pf.begin(TLRMVN_KC_DIAG);
+    sweep_tc_kernel(flags, tco.mode, tco.nst)<<<ctas, STC_NS, smem, st>>>(
+        tco.mapY32, tco.mapB32, tco.mapW, tco.mapU64, tco.mapY64, tco.mapV64, d);
+    pf.end();
+  }
 }
 
 // Float sweep of diagonal tile i (general float32 path), `sub` variables at a time.  Before
@@ -1313,11 +1337,12 @@ static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts&
   const int mode = o.precision == TLRMVN_FP32 ? STC_FP32 : (o.precision == TLRMVN_FP16_SHIFT ? STC_FP16 : STC_BF16);
   const bool f16 = mode != STC_BF16;
   const int64_t wrows = mode == STC_FP32 ? 2 * F.kw16 : F.kw16;
-  int dev = 0;
+  int dev = 0, sms = 1;
   TLR_CUDA(cudaGetDevice(&dev));
-  TLR_CUDA(cudaDeviceGetAttribute(&tco.sms, cudaDevAttrMultiProcessorCount, dev));
+  TLR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t ly = 2 * F.my16;  // Y16 row: hi halves, then lo halves
-  const int64_t C = chunk_tc(o, tu, S, wrows, ly, mode == STC_FP32, tco.sms);
+  const int64_t C = chunk_tc(o, tu, S, wrows, ly, mode == STC_FP32, sms);
+  tco.nst = sweep_tc_stages(mode, (C + STC_NS - 1) / STC_NS, sms);
   unsigned short *W = nullptr, *Y = nullptr;
   float* rs32 = nullptr;
   int* err = nullptr;
@@ -1328,7 +1353,8 @@ static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts&
   const bool mvt = std::isfinite(nu);
   if (mvt) TLR_CHECK(sc.get(&rs32, (size_t)C));
   // padding columns of W and Y must hold finite values: they meet zero operand columns
-  TLR_CUDA(cudaMemsetAsync(W, 0, (size_t)wrows * ldw * 2, st));
+  k_w_padding<<<dim3((unsigned)F.r, (unsigned)std::min<int64_t>(blocks_for(ldw, 8 * 256), 65535)), 256, 0, st>>>(
+      (const StcTile*)F.stc_tiles, mode == STC_FP32 ? 2 : 1, F.kw16, std::min(C, S), ldw, W);
   TLR_CUDA(cudaMemsetAsync(Y, 0, (size_t)ly * C * 2, st));
   TLR_CUDA(cudaMemsetAsync(err, 0, 2 * sizeof(int), st));
 
@@ -1359,12 +1385,8 @@ static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts&
   tco.ldw = ldw;
   tco.my = F.my16;
   tco.err = err;
-  for (int f = 0; f < 4; f++)
-    for (int few = 0; few < 2; few++) {
-      const int nst = sweep_tc_stages(mode, few ? 1 : INT64_MAX, 1);
-      const int flags = ((f & 1) ? SWEEP_PERIODIZE : 0) | ((f & 2) ? SWEEP_ONE_SIDED : 0);
-      TLR_CHECK(raise_smem_limit((const void*)sweep_tc_kernel(flags, mode, nst), sweep_tc_launch_smem(1, mode, nst)));
-    }
+  const int flags = (o.periodize ? SWEEP_PERIODIZE : 0) | (L.one_sided ? SWEEP_ONE_SIDED : 0);
+  TLR_CHECK(raise_smem_limit((const void*)sweep_tc_kernel(flags, mode, tco.nst), sweep_tc_launch_smem(1, mode, tco.nst)));
 
   for (int64_t c0 = 0; c0 < S; c0 += C) {
     const int64_t Cc = std::min(C, S - c0);
@@ -1374,8 +1396,7 @@ static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts&
                                                        o.periodize);
       pf.end();
     }
-    for (int i = 0; i < F.r; i++)
-      sweep_tile_tc(F, i, L, rs32, dD, c0, N, Cc, o.periodize, Y, ly, logP, tco, tu, st, pf);
+    sweep_tiles_tc(F, L, rs32, dD, c0, N, Cc, o.periodize, Y, ly, logP, tco, tu, st, pf);
     TLR_CUDA(cudaGetLastError());
   }
   int herr[2] = {0, 0};

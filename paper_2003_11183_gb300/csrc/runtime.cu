@@ -113,6 +113,7 @@ Factor::~Factor() {
   dfree(V16);
   dfree(B16x2);
   dfree(vmap16);
+  dfree(stc_tiles);
   dfree(U16h);
   dfree(V16h);
   dfree(B16x2h);

@@ -118,6 +118,7 @@ struct SweepTcArgs {
   const float* BT;   // transposed diagonal tile, BT[u * ldbt + v] = B[v][u]
   int64_t ldbt;
   int mt;            // variables in the tile
+  int t0;            // (k_sweep_tc) its first variable
   const float* a;    // limits at the tile's first variable
   const float* b;
   int64_t ys_lo;     // offset of the lo parts in a sample's row of y
@@ -135,19 +136,21 @@ struct SweepTcArgs {
   int wlo, ulo, vlo;      // STC_FP32: the lo parts' row offset in W, x offsets in the U and V maps (third parts: twice)
   int* err;               // [0] a bounded wait's code; [1] (STC_FP32) a y or a projection beyond fp16's range
 };
+constexpr int STC_ARGS = 256;  // shared memory of a tile's arguments
+static_assert(sizeof(SweepTcArgs) <= STC_ARGS, "the arguments' place");
 using StcProjCfg = tc::Cfg<64, false, false, 64, 1>;  // projection k-block: y rows x V rows, 64 deep
 static_assert(StcProjCfg::SB == StcCfg::SB, "a projection k-block fills the same stage");
 using StcShiftCfg = tc::Cfg<64, false, true, 64, 1>;  // shift k-block: W (MN-major) x U rows, 64 deep
 static_assert(StcShiftCfg::SB == StcCfg::SB, "a shift k-block fills the same stage");
 
 constexpr int STC_TRI = 6 * 256;  // floats: the 16 x 16 blocks (ub, vb), ub < vb, at vb (vb - 1) / 2 + ub
-// [NST stages][records][triangle blocks][barriers, TMEM slot] (the dynamic shared memory starts 1 KB-aligned: the
+// [NST stages][records][triangle blocks][barriers, TMEM slot][a tile's arguments] (the dynamic shared memory starts 1 KB-aligned: the
 // kernels have no static shared memory, and the system's own part is 1 KB)
 __host__ __device__ constexpr uint32_t stc_stage_bytes(int mode) {
   return StcCfg::SB + (mode == STC_FP32 ? StcCfg::B_BYTES : 0);  // (the third part of the factor's operand)
 }
 __host__ __device__ constexpr size_t sweep_tc_smem_bytes(int mode, int nst) {
-  return (size_t)nst * stc_stage_bytes(mode) + (STC_SUB * STC_REC + STC_TRI) * sizeof(float) + 128;
+  return (size_t)nst * stc_stage_bytes(mode) + (STC_SUB * STC_REC + STC_TRI) * sizeof(float) + 128 + STC_ARGS;
 }
 // TMEM columns of a CTA: the sums (and y) of a sub-tile, and STC_FP32's second accumulator
 __host__ __device__ constexpr uint32_t stc_cols(int mode) { return mode == STC_FP32 ? 2 * STC_SUB : STC_SUB; }
@@ -164,7 +167,8 @@ struct StcCta {
   uint32_t tmem;         // first of the CTA's TMEM columns
   uint32_t* count;       // k-blocks gone through the stages so far (block i uses stage i mod NST)
   int* abort_flag;
-  int* item;             // (persistent kernel) the work item
+  int* item;             // the work item
+  SweepTcArgs* args;     // (k_sweep_tc) the tile's arguments
 };
 
 // Where the CTA's samples sit in the operand maps and the result buffers.
@@ -634,6 +638,7 @@ __device__ __forceinline__ StcCta stc_cta_setup(unsigned char* smem) {
   k.count = tmem_slot + 1;
   k.abort_flag = reinterpret_cast<int*>(tmem_slot + 2);
   k.item = k.abort_flag + 1;
+  k.args = reinterpret_cast<SweepTcArgs*>(reinterpret_cast<unsigned char*>(k.full) + 128);
   if (threadIdx.x == 0) {
     *k.abort_flag = 0;
     *k.count = 0;
@@ -668,30 +673,40 @@ __device__ __forceinline__ void stc_cta_release(const StcCta& k) {
                  : "memory");
 }
 
-// One launch per diagonal tile of one problem: CTA x owns samples [128 x, 128 (x + 1)) of the
-// chunk.  CTAs per SM: six with one stage (80 registers each), three with two, two with three or four.
+// CTAs per SM: six with one stage (80 registers each), three with two, two with three or four.
 __host__ __device__ constexpr int stc_ctas(int nst) { return nst == 1 ? 6 : (nst == 2 ? 3 : 2); }
+
+// A diagonal tile: its first variable and size, its rank rows of W (first, count), its column ranks (first, count).
+struct StcTile {
+  int t0, mt, krow0, kr, kcol0, kc, pad[2];
+};
 struct SweepTcLaunch {
+  SweepTcArgs base;      // the arguments as of tile 0 at variable, rank row and column rank 0
+  const StcTile* tiles;
+  int i0, i1;            // the launch's tiles
+  int m;                 // largest tile
   const uint64_t* D;
-  int64_t ldD, coord0, sample0, N, C;
+  int64_t ldD, sample0, N, C;
   const float* rs;
   unsigned short* Ys;
   int64_t ldys;
   unsigned short* W;
   double* logP;
-  int first;
 };
+
+// All tiles [i0, i1) of a chunk's samples in one launch; CTA x owns samples [128 x, 128 (x + 1)), whose tiles need
+// nothing of the other CTAs.  (A launch for each tile has every tile end with its slowest CTA, and all CTAs
+// allocate and load anew: n = 65,536, 20 x 5,000 samples, tiles of 512, bf16: 60.8 -> 57.4 ms a solve; n = 16,384,
+// 10 x 1,000, tiles of 256: 7.22 -> 6.78; 20 requests of n = 512 to 4,096 on four streams: 11.0 -> 8.8.  A queue of (tile, block) items over fewer CTAs, the same number on each
+// SM, was slower: 63 ms with four or five CTAs on each, for the CTAs then run out of step and their y out of L2.)
 template <int FLAGS, int MODE, int NST>
 __global__ void __launch_bounds__(STC_NS, stc_ctas(NST))
     k_sweep_tc(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapB,
                const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapU,
                const __grid_constant__ CUtensorMap mapY64, const __grid_constant__ CUtensorMap mapV,
-               const __grid_constant__ SweepTcArgs p, const __grid_constant__ SweepTcLaunch d) {
+               const __grid_constant__ SweepTcLaunch d) {
   extern __shared__ __align__(1024) unsigned char stc_smem[];
   const StcCta k = stc_cta_setup<MODE, NST>(stc_smem);
-  pdl_trigger();  // (after the allocation: a successor's CTAs never hold TMEM this grid still needs)
-  pdl_wait();  // limit shifts, y and log P of the preceding kernels
-
   const int tid = threadIdx.x;
   const int c0 = blockIdx.x * STC_NS;  // (a chunk holds fewer than 2^31 samples)
   const bool act = c0 + tid < d.C;
@@ -699,21 +714,48 @@ __global__ void __launch_bounds__(STC_NS, stc_ctas(NST))
   const int64_t g = d.sample0 + cs, sh = g / d.N;
   const uint32_t ks = (uint32_t)(g - sh * d.N) + 1u;  // lattice point index k = 1..N (N < 2^31)
   const float rs = d.rs ? d.rs[cs] : 1.0f;
-  // log P of the tile = log(prod) + pe log 2 + lsum, prod kept in [1, 2)
-  float prod = 1.0f, lsum = 0.0f;
-  int pe = 0;
   StcPlace pl;
   pl.wx = c0;
   pl.wy = 0;
   pl.yrow = c0;
   pl.ysrow = d.Ys + (int64_t)cs * d.ldys;
   pl.wcol = d.W + cs;
-  const bool ok = stc_tile<FLAGS, MODE, NST>(&mapY, &mapB, &mapW, &mapU, &mapY64, &mapV, p, k, pl, act,
-                                             d.D + sh * d.ldD + d.coord0, ks, rs, prod, lsum, pe);
-  if (ok && act) {
-    const double lp = (double)(logf(prod) + lsum) + (double)pe * 0.69314718055994530942;
-    if (d.first) d.logP[g] = lp;
-    else d.logP[g] += lp;
+#pragma unroll 1
+  for (int i = d.i0; i < d.i1; i++) {
+    if (tid == 0) {
+      const int4 t = __ldg(reinterpret_cast<const int4*>(d.tiles + i));
+      const int2 c = __ldg(reinterpret_cast<const int2*>(d.tiles + i) + 2);
+      SweepTcArgs& p = *k.args;
+      p = d.base;
+      p.rec += (int64_t)i * d.m * STC_REC;
+      p.BT += (int64_t)i * d.m * p.ldbt;
+      p.mt = t.y;
+      p.t0 = t.x;
+      p.a += t.x;
+      p.b += t.x;
+      p.brow0 = i * d.m;
+      p.urow0 = i * d.m;
+      p.krow0 = t.z;
+      p.kr = t.w;
+      p.kcol0 = c.x;
+      p.kc = c.y;
+      p.vmap += c.x;
+      p.wscale += c.x;
+      p.rscale += (int64_t)i * d.m;
+    }
+    __syncthreads();
+    // log P of the tile = log(prod) + pe log 2 + lsum, prod kept in [1, 2)
+    float prod = 1.0f, lsum = 0.0f;
+    int pe = 0;
+    if (!stc_tile<FLAGS, MODE, NST>(&mapY, &mapB, &mapW, &mapU, &mapY64, &mapV, *k.args, k, pl, act,
+                                    d.D + sh * d.ldD + k.args->t0, ks, rs, prod, lsum, pe))
+      break;
+    if (act) {
+      const double lp = (double)(logf(prod) + lsum) + (double)pe * 0.69314718055994530942;
+      if (i == 0) d.logP[g] = lp;
+      else atomicAdd(d.logP + g, lp);  // (this thread's alone: an add that nothing waits for)
+    }
+    __syncthreads();  // the arguments read by all
   }
   stc_cta_release<MODE>(k);
 }
