@@ -188,16 +188,13 @@ __global__ void __launch_bounds__(BATCH_T) k_batch(const BatchProblem* __restric
 }
 
 // ---- tensor-core batched integrand (BF16-shift precision) ----------------------------------
-constexpr int BATCH_TC_MAPS = 3;  // per problem: split B (32-deep boxes), U rows, V rows (64 x 64 boxes)
+constexpr int BATCH_TC_MAPS = 3;  // per problem: split B, U rows, V rows
 
 struct BatchTcProblem {
   int n, r, m, my;  // my: the factor's split-B lo offset (m rounded up to 64)
   int64_t n_points, ldbt, logp_off;
   double nu;
-  const int64_t* tile_off;
-  const int64_t* kpad_off;  // first W row of each row tile's ranks (multiples of 64)
-  const int64_t* krow_off;
-  const int64_t* kcol_off;
+  const StcTile* tiles;
   const int32_t* vmap16;    // W row of each column rank
   const float* BT;
   const float* rec;
@@ -211,16 +208,17 @@ struct BatchTcProblem {
   const int* two;           // nonzero: some lower limit of the problem is finite
 };
 
-template <int FLAGS, int MODE, int NST>
-__global__ void __launch_bounds__(STC_NS, stc_ctas(NST))
+template <int FLAGS, int MODE>
+__global__ void __launch_bounds__(STC_NS, stc_ctas(MODE, false))
     k_batch_tc(const BatchTcProblem* __restrict__ probs, const CUtensorMap* __restrict__ pmaps,
                const BatchItem* __restrict__ items, int n_items, int* next, const __grid_constant__ CUtensorMap mapW,
-               const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapY64,
+               const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapYp,
                unsigned short* Wbase, int64_t kwmax, unsigned short* Ybase, int my, double* logP, int* err) {
   constexpr bool PER = FLAGS & SWEEP_PERIODIZE;
   extern __shared__ __align__(1024) unsigned char stc_smem[];
   constexpr int64_t WROWS = MODE == STC_FP32 ? 2 : 1;  // (float32: hi rows, then lo rows)
-  const StcCta k = stc_cta_setup<MODE, NST>(stc_smem);
+  constexpr int NST = stc_stages(MODE, false);
+  const StcCta k = stc_cta_setup<MODE, NST, false>(stc_smem);
   const int tid = threadIdx.x;
   StcPlace pl;
   pl.wx = 0;
@@ -228,6 +226,8 @@ __global__ void __launch_bounds__(STC_NS, stc_ctas(NST))
   pl.yrow = blockIdx.x * STC_NS;
   pl.ysrow = Ybase + ((int64_t)blockIdx.x * STC_NS + tid) * (2 * my);  // (hi at 0, lo at my)
   pl.wcol = Wbase + (int64_t)blockIdx.x * kwmax * WROWS * STC_NS + tid;
+  StcRun run{0, 0, 0, 0, 0};
+  uint32_t step = 0;
   for (;;) {
     __syncthreads();  // every thread is done with the previous item
     if (tid == 0) *k.item = atomicAdd(next, 1);
@@ -236,6 +236,8 @@ __global__ void __launch_bounds__(STC_NS, stc_ctas(NST))
     if (it >= n_items || *(volatile int*)k.abort_flag) break;
     const BatchItem item = items[it];
     const BatchTcProblem& P = probs[item.prob];
+    const CUtensorMap* mp = pmaps + (int64_t)BATCH_TC_MAPS * item.prob;
+    const StcOps o{&mapY, &mapYp, mp, &mapW, mp + 1, mp + 2, my, P.my, (int)kwmax, P.kmax, P.my, err};
     const bool act = tid < item.count;
     const int64_t g = item.sample0 + (act ? tid : item.count - 1);  // inactive lanes shadow a valid sample
     const int64_t sh = g / P.n_points;
@@ -247,58 +249,47 @@ __global__ void __launch_bounds__(STC_NS, stc_ctas(NST))
       lattice_w((uint64_t)ks * P.Q[P.n] + Drow[P.n], PER ? 1 : 0, w, wc);
       rs = (float)sqrt(2.0 * gamma_p_inv(0.5 * P.nu, w, wc) / P.nu);
     }
-    const CUtensorMap* mp = pmaps + (int64_t)BATCH_TC_MAPS * item.prob;
     const bool two = *P.two != 0;
     float prod = 1.0f, lsum = 0.0f;
     int pe = 0;
     bool ok = true;
     for (int i = 0; i < P.r && ok; i++) {
-      const int64_t t0 = P.tile_off[i];
       SweepTcArgs p;
-      p.rec = P.rec + (int64_t)i * P.m * STC_REC;
-      p.BT = P.BT + (int64_t)i * P.m * P.ldbt;
+      p.rec = P.rec;
+      p.BT = P.BT;
       p.ldbt = P.ldbt;
-      p.mt = (int)(P.tile_off[i + 1] - t0);
-      p.a = P.a + t0;
-      p.b = P.b + t0;
+      p.a = P.a;
+      p.b = P.b;
       p.ys_lo = my;
-      p.brow0 = i * P.m;
-      p.alo = my;
-      p.blo = P.my;
-      p.urow0 = i * P.m;
-      p.krow0 = (int)P.kpad_off[i];
-      p.kr = (int)(P.krow_off[i + 1] - P.krow_off[i]);
-      p.kcol0 = (int)P.kcol_off[i];
-      p.kc = (int)(P.kcol_off[i + 1] - P.kcol_off[i]);
       p.ldw = STC_NS;
-      p.vmap = P.vmap16 ? P.vmap16 + P.kcol_off[i] : nullptr;
-      p.wscale = P.wscale ? P.wscale + P.kcol_off[i] : nullptr;
+      p.vmap = P.vmap16;
+      p.wscale = P.wscale;
       p.tscale = 1.0f;
-      p.rscale = P.rscale ? P.rscale + (int64_t)i * P.m : nullptr;
+      p.rscale = P.rscale;
       p.wlo = (int)kwmax;
-      p.ulo = P.kmax;
-      p.vlo = P.my;
       p.err = err;
+      p.at(P.tiles[i], i, P.m);
       if (two)
-        ok = stc_tile<FLAGS, MODE, NST>(&mapY, mp, &mapW, mp + 1, &mapY64, mp + 2, p, k, pl, act, Drow + t0, ks, rs,
-                                        prod, lsum, pe);
+        ok = stc_tile<FLAGS, MODE, NST, false>(p, k, pl, step, o, run, i * P.m, act, Drow, ks, rs, prod, lsum, pe);
       else
-        ok = stc_tile<FLAGS | SWEEP_ONE_SIDED, MODE, NST>(&mapY, mp, &mapW, mp + 1, &mapY64, mp + 2, p, k, pl, act,
-                                                          Drow + t0, ks, rs, prod, lsum, pe);
+        ok = stc_tile<FLAGS | SWEEP_ONE_SIDED, MODE, NST, false>(p, k, pl, step, o, run, i * P.m, act, Drow, ks, rs,
+                                                               prod, lsum, pe);
     }
     if (ok && act) logP[P.logp_off + g] = (double)(logf(prod) + lsum) + (double)pe * 0.69314718055994530942;
   }
-  stc_cta_release<MODE>(k);
+  stc_cta_release<MODE, false>(k);
 }
-// float32: two stages, three CTAs per SM; bf16: one stage, six
 typedef void (*BatchTcKernel)(const BatchTcProblem*, const CUtensorMap*, const BatchItem*, int, int*, const CUtensorMap,
                               const CUtensorMap, const CUtensorMap, unsigned short*, int64_t, unsigned short*, int,
                               double*, int*);
 static BatchTcKernel batch_tc_kernel(bool f32, int periodize) {
-  if (f32) return periodize ? k_batch_tc<SWEEP_PERIODIZE, STC_FP32, 2> : k_batch_tc<0, STC_FP32, 2>;
-  return periodize ? k_batch_tc<SWEEP_PERIODIZE, STC_BF16, 1> : k_batch_tc<0, STC_BF16, 1>;
+  if (f32) return periodize ? k_batch_tc<SWEEP_PERIODIZE, STC_FP32> : k_batch_tc<0, STC_FP32>;
+  return periodize ? k_batch_tc<SWEEP_PERIODIZE, STC_BF16> : k_batch_tc<0, STC_BF16>;
 }
-static size_t batch_tc_smem(bool f32) { return f32 ? sweep_tc_smem_bytes(STC_FP32, 2) : sweep_tc_smem_bytes(STC_BF16, 1); }
+static size_t batch_tc_smem(bool f32) {
+  const int mode = f32 ? STC_FP32 : STC_BF16;
+  return sweep_tc_smem_bytes(mode, stc_stages(mode, false));
+}
 
 // limits of all problems: original order (staged) -> factor order, float; validation
 // (and, per problem, whether a lower limit is finite: prob_of maps a position to its problem)
@@ -341,7 +332,7 @@ static inline unsigned nblk(int64_t n, int t) { return (unsigned)((n + t - 1) / 
 struct BatchCopies {
   float* UT = nullptr;
   float* VT = nullptr;
-  int64_t *tile_off = nullptr, *krow_off = nullptr, *kcol_off = nullptr, *vt_off = nullptr, *kpad_off = nullptr;
+  int64_t *tile_off = nullptr, *krow_off = nullptr, *kcol_off = nullptr, *vt_off = nullptr;
   int32_t* kcpad = nullptr;
   ~BatchCopies() {
     dfree(UT);
@@ -350,7 +341,6 @@ struct BatchCopies {
     dfree(krow_off);
     dfree(kcol_off);
     dfree(vt_off);
-    dfree(kpad_off);
     dfree(kcpad);
   }
 };
@@ -366,8 +356,6 @@ static int make_batch_copies(Factor& F, BatchCopies& C, bool tc, int precision, 
   const int r = F.r, m = F.m;
   if (tc) {
     TLR_CHECK(ensure_precision_copies(F, precision, st));
-    TLR_CHECK(dalloc(&C.kpad_off, r + 1));
-    TLR_CUDA(cudaMemcpyAsync(C.kpad_off, F.kpad_off.data(), (r + 1) * 8, cudaMemcpyHostToDevice, st));
   } else {
     std::lock_guard<std::mutex> lk(F.copy_mu);
     TLR_CHECK(ensure_float_tiles(F, st));
@@ -435,7 +423,7 @@ struct Batch {
   BatchTcProblem* dtprobs = nullptr;
   CUtensorMap* dmaps = nullptr;
   unsigned short *W16 = nullptr, *Y16 = nullptr;
-  CUtensorMap mapW{}, mapY{}, mapY64{};
+  CUtensorMap mapW{}, mapY{}, mapYp{};
   int* derr = nullptr;
   double *logP = nullptr, *ell = nullptr, *out = nullptr, *a_st = nullptr, *b_st = nullptr;
   float *a32 = nullptr, *b32 = nullptr;
@@ -516,8 +504,7 @@ static int batch_capture(Batch& B, int per_sm) {
   k_permute_batch<<<nblk(B.total_n, 256), 256, 0, st>>>(B.a_st, B.b_st, B.perm_g, B.prob_of, B.total_n, B.a32, B.b32,
                                                         B.dbad, B.dtwo);
   batch_tc_kernel(B.f32, B.periodize)<<<grid, STC_NS, batch_tc_smem(B.f32), st>>>(
-      B.dtprobs, B.dmaps, B.ditems, B.n_items, B.dnext, B.mapW, B.mapY, B.mapY64, B.W16, B.kwmax, B.Y16, B.my, B.logP,
-      B.derr);
+      B.dtprobs, B.dmaps, B.ditems, B.n_items, B.dnext, B.mapW, B.mapY, B.mapYp, B.W16, B.kwmax, B.Y16, B.my, B.logP, B.derr);
   k_shift_reduce<<<(unsigned)(B.count * B.M), 256, 0, st>>>(B.logP, B.N, B.ell);
   k_final_batch<<<B.count, 256, 0, st>>>(B.ell, B.M, B.out);
   cudaError_t ec = cudaStreamEndCapture(st, &graph);
@@ -678,7 +665,7 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
     // reported one CTA per SM for this kernel where the launches fit six), and at most
     // as many as their TMEM columns, held until the end, leave room for
     TLR_CHECK(resident_ctas(kt, STC_NS, batch_tc_smem(B.f32), B.device, &B.per_sm_max));
-    B.per_sm_max = std::min<int>(B.per_sm_max, 512 / (int)stc_cols(B.f32 ? STC_FP32 : STC_BF16));
+    B.per_sm_max = std::min<int>(B.per_sm_max, stc_ctas(B.f32 ? STC_FP32 : STC_BF16, false));
   }
   B.per_sm_max = std::max(B.per_sm_max, 1);
   B.grid_max = std::max(1, std::min(B.per_sm_max * B.sms, B.n_items));
@@ -698,11 +685,11 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
     TLR_CUDA(cudaMemsetAsync(B.Y16, 0, ny * 2, st));
     TLR_CUDA(cudaMemsetAsync(B.derr, 0, 2 * sizeof(int), st));
     const uint32_t deep = B.f32 ? 32 : 64;
+    TLR_CHECK(make_tensor_map_16(&B.mapYp, B.Y16, 2 * B.my, (uint64_t)B.grid_max * STC_NS, 2 * B.my * 2, STC_NS,
+                                 deep, B.f32));
     TLR_CHECK(make_tensor_map_16(&B.mapW, B.W16, STC_NS, (uint64_t)B.grid_max * wrows, STC_NS * 2, deep, 64, B.f32));
     TLR_CHECK(make_tensor_map_16(&B.mapY, B.Y16, 2 * B.my, (uint64_t)B.grid_max * STC_NS, 2 * B.my * 2,
                                  STC_NS, 32, B.f32));
-    TLR_CHECK(make_tensor_map_16(&B.mapY64, B.Y16, 2 * B.my, (uint64_t)B.grid_max * STC_NS, 2 * B.my * 2, STC_NS,
-                                 64, B.f32));
     // per problem: the split B, U and V maps, and its table entry
     std::vector<CUtensorMap> maps((size_t)BATCH_TC_MAPS * count);
     std::vector<BatchTcProblem> tp(count);
@@ -731,10 +718,7 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
       T.ldbt = P.ldbt;
       T.logp_off = P.logp_off;
       T.nu = P.nu;
-      T.tile_off = P.tile_off;
-      T.kpad_off = B.copies[p].kpad_off;
-      T.krow_off = P.krow_off;
-      T.kcol_off = P.kcol_off;
+      T.tiles = (const StcTile*)F.stc_tiles;
       T.vmap16 = F.vmap16;
       T.BT = P.BT;
       T.rec = F.rec32;

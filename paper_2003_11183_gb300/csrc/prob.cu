@@ -668,8 +668,9 @@ static int make_layout(Factor& F, cudaStream_t st) {
   {
     std::vector<StcTile> tiles(r);
     for (int i = 0; i < r; i++)
-      tiles[i] = StcTile{(int)F.tile_off[i], (int)F.tsize(i),       (int)off[i], (int)F.krow(i),
-                         (int)F.kcol_off[i], (int)F.kcol(i), {0, 0}};
+      tiles[i] = StcTile{(int)F.tile_off[i],    (int)F.tsize(i), (int)off[i], (int)F.krow(i),
+                         (int)F.kcol_off[i],    (int)F.kcol(i),
+                         (int)F.krow(i) - (i > 0 ? F.rank[(size_t)i * r + i - 1] : 0), 0};
     StcTile* d = nullptr;
     TLR_CHECK(dalloc(&d, (size_t)r));
     F.stc_tiles = d;
@@ -900,7 +901,7 @@ static int64_t chunk_simt(const tlrmvn_opts& o, const Tuning& tu, int64_t S, int
   const double per = (double)(ktot + 2 * m) * es + 16.0;
   return round_chunk((int64_t)std::max(256.0, std::min((double)S, budget / per)), S);
 }
-// (passes of equal size that fit the six CTAs, float32: three, that an SM holds -- one CTA more would run a whole
+// (passes of equal size that fit the CTAs that an SM holds -- one CTA more would run a whole
 // solve on its own -- and the float32 path within 8 GiB)
 static int64_t chunk_tc(const tlrmvn_opts& o, const Tuning& tu, int64_t S, int64_t wrows, int64_t ly, bool f32, int sms) {
   if (o.sample_chunk > 0) return round_chunk(o.sample_chunk, S);
@@ -908,7 +909,7 @@ static int64_t chunk_tc(const tlrmvn_opts& o, const Tuning& tu, int64_t S, int64
   const double budget = (f32 ? 8.0 : 32.0) * (1ull << 30);
   const double per = (double)wrows * 2 + (double)ly * 2 + 16.0;
   int64_t C = (int64_t)std::max(256.0, std::min((double)S, budget / per));
-  C = std::min(C, (int64_t)(f32 ? 3 : 6) * sms * STC_NS);
+  C = std::min(C, (int64_t)stc_ctas(f32 ? STC_FP32 : STC_BF16, false) * sms * STC_NS);
   const int64_t passes = (S + C - 1) / C;
   C = (S + passes - 1) / passes;
   return round_chunk(C, S);
@@ -1017,39 +1018,33 @@ static SweepShape sweep_shape(int64_t C, int mt, int forced) {
   memo = best;
   return best;
 }
-// The whole-tile sweep by its arithmetic, stages and (periodisation, one-sided) flags.  Stages: a launch that leaves
-// at most two CTAs to an SM takes four (float32: three; its products wait for copies, and shared memory is idle);
-// else the 16-bit paths take one, so that six CTAs share an SM, and the float32 path two (three CTAs, by its TMEM
-// columns four at most).
+// The whole-tile sweep by its arithmetic, whether its products overlap the sweep (launches of at most two CTAs an SM)
+// and (periodisation, one-sided) flags.
 typedef void (*SweepTcKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
                               const CUtensorMap, const CUtensorMap, const SweepTcLaunch);
-template <int MODE, int NST>
+template <int MODE, bool OV>
 static SweepTcKernel sweep_tc_variant(int f) {
-  static const SweepTcKernel t[4] = {k_sweep_tc<0, MODE, NST>, k_sweep_tc<SWEEP_PERIODIZE, MODE, NST>,
-                                     k_sweep_tc<SWEEP_ONE_SIDED, MODE, NST>,
-                                     k_sweep_tc<SWEEP_PERIODIZE | SWEEP_ONE_SIDED, MODE, NST>};
+  static const SweepTcKernel t[4] = {k_sweep_tc<0, MODE, OV>, k_sweep_tc<SWEEP_PERIODIZE, MODE, OV>,
+                                     k_sweep_tc<SWEEP_ONE_SIDED, MODE, OV>,
+                                     k_sweep_tc<SWEEP_PERIODIZE | SWEEP_ONE_SIDED, MODE, OV>};
   return t[f];
 }
-static SweepTcKernel sweep_tc_kernel(int flags, int mode, int nst) {
+static SweepTcKernel sweep_tc_kernel(int flags, int mode, bool ov) {
   const int f = ((flags & SWEEP_PERIODIZE) ? 1 : 0) | ((flags & SWEEP_ONE_SIDED) ? 2 : 0);
-  if (mode == STC_FP32) return nst == 3 ? sweep_tc_variant<STC_FP32, 3>(f) : sweep_tc_variant<STC_FP32, 2>(f);
-  if (mode == STC_FP16) return nst == 4 ? sweep_tc_variant<STC_FP16, 4>(f) : sweep_tc_variant<STC_FP16, 1>(f);
-  return nst == 4 ? sweep_tc_variant<STC_BF16, 4>(f) : sweep_tc_variant<STC_BF16, 1>(f);
-}
-static int sweep_tc_stages(int mode, int64_t ctas, int sms) {
-  const bool few = ctas <= 2 * (int64_t)sms;
-  return mode == STC_FP32 ? (few ? 3 : 2) : (few ? 4 : 1);
+  if (mode == STC_FP32) return ov ? sweep_tc_variant<STC_FP32, true>(f) : sweep_tc_variant<STC_FP32, false>(f);
+  if (mode == STC_FP16) return ov ? sweep_tc_variant<STC_FP16, true>(f) : sweep_tc_variant<STC_FP16, false>(f);
+  return ov ? sweep_tc_variant<STC_BF16, true>(f) : sweep_tc_variant<STC_BF16, false>(f);
 }
 // Tiles of one launch: a launch of many blocks keeps its CTAs' places on the SMs until all its tiles are done, so a
 // solve of many variables goes in launches of about 16,384 (10 to 25 ms where every SM is full), between which
 // the kernels of other streams get their turn.
 static int sweep_tc_span(int m) { return std::max(1, 16384 / m); }
-// Dynamic shared memory of a whole-tile sweep launch: the kernel's own need, or (tuning, one-stage launches) more, so
-// that no more than `ctas` fit an SM.
-static size_t sweep_tc_launch_smem(int ctas, int mode, int nst) {
-  size_t need = sweep_tc_smem_bytes(mode, nst);
-  ctas = std::min(std::max(ctas, 1), 6);
-  if (nst == 1 && ctas < 6) {
+// Dynamic shared memory of a whole-tile sweep launch: the kernel's own need, or (tuning) more, so that no more than
+// `ctas` fit an SM.
+static size_t sweep_tc_launch_smem(int ctas, int mode, bool ov) {
+  size_t need = sweep_tc_smem_bytes(mode, stc_stages(mode, ov));
+  ctas = std::max(ctas, 1);
+  if (!ov && ctas < stc_ctas(mode, ov)) {
     int dev = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
@@ -1071,14 +1066,13 @@ static int set_sweep_smem(int sub) {
 // halves for the projection; the projections W, the offset of the lo halves and
 // the error flag.
 struct TcOperands {
-  CUtensorMap mapB32, mapY32, mapY64;
-  CUtensorMap mapW{}, mapU64{}, mapV64{};
+  CUtensorMap mapB, mapY, mapYp, mapW{}, mapU{}, mapV{};
   unsigned short* W = nullptr;
   int64_t ldw = 0;
   int64_t my;
   int* err;
   int mode = STC_BF16;
-  int nst = 1;
+  bool ov = false;  // products overlapped
 };
 
 // Zeroes what no sweep writes of W and its products read: the rows between a tile's ranks and the next multiple of 64,
@@ -1111,38 +1105,37 @@ static void sweep_tiles_tc(const Factor& F, const Lims& L, const float* rs32, co
   t.a = L.a32;
   t.b = L.b32;
   t.ys_lo = tco.my;
-  t.alo = (int)tco.my;
-  t.blo = (int)tco.my;
   t.ldw = tco.ldw;
   t.vmap = F.vmap16;
   t.wscale = tco.mode == STC_FP16 ? F.wscale16 : (tco.mode == STC_FP32 ? F.wscale32 : nullptr);
   t.tscale = tco.mode == STC_FP16 ? F.inv_g16 : 1.0f;
   t.rscale = tco.mode == STC_FP32 ? F.rscale32 : nullptr;
   t.wlo = (int)F.kw16;
-  t.ulo = (int)F.kmax16;
-  t.vlo = (int)F.my16;
   t.err = tco.err;
+  d.alo = d.blo = (int)tco.my;
+  d.ulo = (int)F.kmax16;
+  d.vlo = (int)F.my16;
   d.tiles = (const StcTile*)F.stc_tiles;
   d.m = F.m;
   d.D = dD;
   d.ldD = F.n + 1;
+  d.Ys = Ys;
+  d.ldys = ldys;
+  d.W = tco.W;
   d.sample0 = c0;
   d.N = N;
   d.C = Cc;
   d.rs = rs32;
-  d.Ys = Ys;
-  d.ldys = ldys;
-  d.W = tco.W;
   d.logP = logP;
   const int flags = (periodize ? SWEEP_PERIODIZE : 0) | (L.one_sided ? SWEEP_ONE_SIDED : 0);
   const int span = sweep_tc_span(F.m);
   const unsigned ctas = (unsigned)((Cc + STC_NS - 1) / STC_NS);
-  const size_t smem = sweep_tc_launch_smem(tu.tc_ctas, tco.mode, tco.nst);
+  const size_t smem = sweep_tc_launch_smem(tu.tc_ctas, tco.mode, tco.ov);
   for (d.i0 = 0; d.i0 < F.r; d.i0 = d.i1) {
     d.i1 = std::min(F.r, d.i0 + span);
     pf.begin(TLRMVN_KC_DIAG);
-    sweep_tc_kernel(flags, tco.mode, tco.nst)<<<ctas, STC_NS, smem, st>>>(
-        tco.mapY32, tco.mapB32, tco.mapW, tco.mapU64, tco.mapY64, tco.mapV64, d);
+    sweep_tc_kernel(flags, tco.mode, tco.ov)<<<ctas, tco.ov ? StcPlan<true>::THREADS : StcPlan<false>::THREADS, smem, st>>>(
+        tco.mapY, tco.mapYp, tco.mapB, tco.mapW, tco.mapU, tco.mapV, d);
     pf.end();
   }
 }
@@ -1342,7 +1335,7 @@ static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts&
   TLR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t ly = 2 * F.my16;  // Y16 row: hi halves, then lo halves
   const int64_t C = chunk_tc(o, tu, S, wrows, ly, mode == STC_FP32, sms);
-  tco.nst = sweep_tc_stages(mode, (C + STC_NS - 1) / STC_NS, sms);
+  tco.ov = (C + STC_NS - 1) / STC_NS <= 2 * (int64_t)sms;
   unsigned short *W = nullptr, *Y = nullptr;
   float* rs32 = nullptr;
   int* err = nullptr;
@@ -1365,28 +1358,28 @@ static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts&
   //   (float32 path: W16 as hi/lo, U, V and B in three parts, in boxes 32 ranks or variables deep)
   tco.mode = mode;
   const void* B2 = mode == STC_FP32 ? (const void*)F.Bs16 : (f16 ? (const void*)F.B16x2h : (const void*)F.B16x2);
-  const uint32_t deep = mode == STC_FP32 ? 32 : 64;
   const int64_t lb = (mode == STC_FP32 ? 3 : 2) * F.my16;
-  TLR_CHECK(make_map(&tco.mapB32, B2, lb, (uint64_t)F.r * m, lb * 2, 64, 32, f16));
-  TLR_CHECK(make_map(&tco.mapY32, Y, ly, C, ly * 2, STC_NS, 32, f16));
-  TLR_CHECK(make_map(&tco.mapY64, Y, ly, C, ly * 2, STC_NS, 64, f16));
+  TLR_CHECK(make_map(&tco.mapB, B2, lb, (uint64_t)F.r * m, lb * 2, 64, 32, f16));
+  TLR_CHECK(make_map(&tco.mapY, Y, ly, C, ly * 2, STC_NS, 32, f16));
+  const uint32_t deep = mode == STC_FP32 ? 32 : 64;
+  TLR_CHECK(make_map(&tco.mapYp, Y, ly, C, ly * 2, STC_NS, deep, f16));
   TLR_CHECK(make_map(&tco.mapW, W, ldw, wrows, ldw * 2, deep, 64, f16));
   if (F.ktot) {
     const void* U = mode == STC_FP32 ? (const void*)F.Us16 : (f16 ? (const void*)F.U16h : (const void*)F.U16);
     const void* V = mode == STC_FP32 ? (const void*)F.Vs16 : (f16 ? (const void*)F.V16h : (const void*)F.V16);
     const int64_t lu = (mode == STC_FP32 ? 3 : 1) * F.kmax16, lv = (mode == STC_FP32 ? 3 : 1) * F.my16;
-    TLR_CHECK(make_map(&tco.mapU64, U, lu, (uint64_t)F.r * m, lu * 2, 64, deep, f16));
-    TLR_CHECK(make_map(&tco.mapV64, V, lv, F.ktot, lv * 2, 64, deep, f16));
+    TLR_CHECK(make_map(&tco.mapU, U, lu, (uint64_t)F.r * m, lu * 2, 64, deep, f16));
+    TLR_CHECK(make_map(&tco.mapV, V, lv, F.ktot, lv * 2, 64, deep, f16));
   } else {
-    tco.mapU64 = tco.mapW;  // (never read: no tile has ranks)
-    tco.mapV64 = tco.mapW;
+    tco.mapU = tco.mapW;  // (never read: no tile has ranks)
+    tco.mapV = tco.mapW;
   }
   tco.W = W;
   tco.ldw = ldw;
   tco.my = F.my16;
   tco.err = err;
   const int flags = (o.periodize ? SWEEP_PERIODIZE : 0) | (L.one_sided ? SWEEP_ONE_SIDED : 0);
-  TLR_CHECK(raise_smem_limit((const void*)sweep_tc_kernel(flags, mode, tco.nst), sweep_tc_launch_smem(1, mode, tco.nst)));
+  TLR_CHECK(raise_smem_limit((const void*)sweep_tc_kernel(flags, mode, tco.ov), sweep_tc_launch_smem(1, mode, tco.ov)));
 
   for (int64_t c0 = 0; c0 < S; c0 += C) {
     const int64_t Cc = std::min(C, S - c0);

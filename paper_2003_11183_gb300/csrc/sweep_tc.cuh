@@ -2,9 +2,8 @@
 // tile): the tile's low-rank limit shifts, the sweep with its in-tile coupling, and the tile's projections
 // for the later tiles, the products on the tensor cores.
 //
-// One CTA of 128 threads owns 128 samples, one per thread and per TMEM lane, and
-// 64 TMEM columns.  The tile runs in sub-tiles of 64 variables.  Before sub-tile
-// q, one thread accumulates into the columns, by tcgen05 products,
+// Four warps of a CTA own 128 samples, one per thread and per TMEM lane. The tile runs in sub-tiles of 64 variables. The
+// sums that sub-tile q starts from are accumulated, by tcgen05 products issued by one thread, in 64 TMEM columns:
 //     T[c][v] = sum_k U_i[q0 + v][k] W[k][c]           (the low-rank shifts: W the
 //               rank-major projections of the earlier tiles, read MN-major; U
 //               the tile's rows of the row factors; 16-bit operands, fp32 accumulation)
@@ -19,30 +18,28 @@
 // products' sums come from the thread's TMEM lane (tcgen05.ld); the y of the
 // sub-tile go to the same lane, into the columns whose sums have been read
 // (tcgen05.st).  After each block its y are stored, sample-major 16-bit hi and
-// lo, for the later products.  After the last sub-tile the CTA computes the
-// tile's projections W[k][c] = sum_v V_i[k][v] y_v[c] in passes of 64 ranks through
-// the same columns and writes them as rows of W.  So neither the shifts nor the
+// lo, for the later products.  After the last sub-tile come the
+// tile's projections W[k][c] = sum_v V_i[k][v] y_v[c], in steps of 64 ranks through
+// the same columns, written as rows of W.  So neither the shifts nor the
 // coupling go through global memory, the per-variable loads of B are
 // shared-memory broadcasts, and the sample's log P is closed once per tile.
 //
-// Shared memory per CTA (36.1 KB, six CTAs per SM): one 24 KB stage of MMA operands,
-// staged by TMA (shift and projection k-blocks 64 deep, 128-byte swizzle; coupling
-// k-blocks 32 deep, 64-byte swizzle), and what the sweep reads: a 96-byte record per
+// Shared memory per CTA: stages of MMA operands (24 KB; float32 28), staged by TMA (128-byte swizzle where 64 deep, 64-byte
+// where 32 deep), and what the sweep reads: a 96-byte record per
 // variable (its window column of B, limits, reciprocal diagonal, lattice generator) and
-// the six 16 x 16 blocks of the sub-tile's triangle that lie left of the windows.
-// These have a place of their own, so that the idle threads load them while one
-// thread runs the products, and the first shift k-block of the next sub-tile is copied
-// during the sweep.  Every wait is bounded; on expiry the CTA records an error code,
-// skips the rest, waits (bounded) for its copies and products in flight, frees its
+// the six 16 x 16 blocks of the sub-tile's triangle that lie left of the windows.  Every wait is bounded; on expiry the
+// CTA records an error code, skips the rest, waits (bounded) for its copies and products in flight, frees its
 // TMEM and returns.
 //
 // What bounds it: the chain from a variable's sum to its y (about 110 instructions, most
-// of them dependent) and, with five CTAs per SM, the issue slots; the arithmetic pipe
+// of them dependent) and, with six CTAs per SM, the issue slots; the arithmetic pipe
 // (compares, selects, integer operations: half the rate of the FMA pipe) came first
 // with 64 of 176 instructions a variable, so the step avoids them: see
 // sov_step_f32_upper.  With that step, the constants' loads beside the products and the pairwise
 // renormalisation and TMEM stores: n = 65,536, 20 x 5,000 samples, tiles of 512: 73.5 -> 60.4 ms a solve; n =
-// 16,384, 10 x 1,000, tiles of 256: 10.0 -> 7.2 ms; two-sided limits (n = 3,900, 8 x 1,301): 4.43 -> 1.99 ms.
+// 16,384, 10 x 1,000, tiles of 256: 10.0 -> 7.2 ms; two-sided limits (n = 3,900, 8 x 1,301): 4.43 -> 1.99 ms.  With one
+// launch for all tiles (k_sweep_tc): 57.4, 6.77, 1.85; with the products beside the sweep (StcPlan) and the projections'
+// row numbers read into shared memory together: 56.8, 5.94, 1.60.
 #pragma once
 #include "gemm.cuh"
 #include "tcgen05.cuh"
@@ -71,6 +68,9 @@ constexpr int STC_SUB = 64;   // variables per sub-tile
 constexpr int STC_NS = 128;   // samples per CTA (TMEM lanes)
 constexpr int STC_KB = 32;    // K depth of a coupling k-block
 using StcCfg = tc::Cfg<64, true, false, STC_KB, 1>;
+using StcShiftCfg = tc::Cfg<64, false, true, 64, 1>;  // 16-bit shift k-block: W (MN-major) x U rows, 64 deep
+using StcProjCfg = tc::Cfg<64, false, false, 64, 1>;  // 16-bit projection k-block: y rows x V rows, 64 deep
+static_assert(StcProjCfg::SB == StcCfg::SB && StcShiftCfg::SB == StcCfg::SB, "they fill the same stage");
 
 // The 16-bit operand type of the products: bf16 (BF16-shift path) or fp16
 // (FP16-shift path), as raw 16-bit words.  pack rounds two floats to the type
@@ -113,62 +113,91 @@ constexpr int STC_REC = 24;  // floats
 // Entries after the lattice shifts' table: a sample's row is read up to three entries past a tile's last variable.
 constexpr int STC_DPAD = 4;
 
+// A diagonal tile: its first variable and size, its rank rows of W (first, count), its column ranks (first, count),
+// and how many of its first ranks come from tiles before the one before it.
+struct StcTile {
+  int t0, mt, krow0, kr, kcol0, kc, kearly, pad;
+};
+// A tile for the sweeping warps.
 struct SweepTcArgs {
   const float* rec;  // the factor's records at the tile's first variable (limits not filled in)
   const float* BT;   // transposed diagonal tile, BT[u * ldbt + v] = B[v][u]
   int64_t ldbt;
   int mt;            // variables in the tile
-  int t0;            // (k_sweep_tc) its first variable
   const float* a;    // limits at the tile's first variable
   const float* b;
   int64_t ys_lo;     // offset of the lo parts in a sample's row of y
-  int brow0;     // row of the tile's first variable in the split-B map
-  int alo, blo;  // x offsets of the lo halves in the y and split-B maps
-  int urow0;     // row of the tile's first variable in the U map
-  int krow0, kr; // the tile's rank rows in the W map (first, count; 0: no low-rank shift)
-  int kcol0, kc; // the tile's column ranks: first row in the V map, count (0: no projection)
-  int64_t ldw;   // projections, rank-major: row vmap[r], ldw samples a row
+  int kr, kc;        // the tile's ranks (0: no low-rank shift), its column ranks (0: no projection)
+  int64_t ldw;       // projections, rank-major: row vmap[r], ldw samples a row
   const int32_t* vmap;    // at the tile's first column rank
   const float* wscale;    // FP16 path: per column rank, the factor applied to a projection before it is
                           // stored (the inverse of the per-tile scales of U and V); null on the BF16 path
   float tscale;           // FP16 path: 1 / g, undoing the products' global scale g where the sweep reads them
   const float* rscale;    // STC_FP32: per variable of the tile, the inverse of its row's scale
-  int wlo, ulo, vlo;      // STC_FP32: the lo parts' row offset in W, x offsets in the U and V maps (third parts: twice)
+  StcTile t;              // the tile (for the products)
+  int wlo;                // STC_FP32: the lo parts' row offset in W
   int* err;               // [0] a bounded wait's code; [1] (STC_FP32) a y or a projection beyond fp16's range
+
+  // from the arguments as of tile 0, variable 0 and column rank 0 to those of tile i of at most m variables
+  __device__ void at(const StcTile& tile, int i, int m) {
+    t = tile;
+    rec += (int64_t)i * m * STC_REC;
+    BT += (int64_t)i * m * ldbt;
+    mt = t.mt;
+    a += t.t0;
+    b += t.t0;
+    kr = t.kr;
+    kc = t.kc;
+    vmap += t.kcol0;
+    wscale += t.kcol0;
+    rscale += (int64_t)i * m;
+  }
 };
 constexpr int STC_ARGS = 256;  // shared memory of a tile's arguments
 static_assert(sizeof(SweepTcArgs) <= STC_ARGS, "the arguments' place");
-using StcProjCfg = tc::Cfg<64, false, false, 64, 1>;  // projection k-block: y rows x V rows, 64 deep
-static_assert(StcProjCfg::SB == StcCfg::SB, "a projection k-block fills the same stage");
-using StcShiftCfg = tc::Cfg<64, false, true, 64, 1>;  // shift k-block: W (MN-major) x U rows, 64 deep
-static_assert(StcShiftCfg::SB == StcCfg::SB, "a shift k-block fills the same stage");
+// The operands for the producing thread: tensor maps (32-deep boxes; 16-bit W, U and V, and mapYp, 64-deep), x offsets of the lo halves in the y and split-B maps,
+// STC_FP32: of the lo parts in the W (rows), U and V maps (third parts: twice).
+struct StcOps {
+  const CUtensorMap *mapY, *mapYp, *mapB, *mapW, *mapU, *mapV;
+  int alo, blo, wlo, ulo, vlo;
+  int* err;
+};
 
 constexpr int STC_TRI = 6 * 256;  // floats: the 16 x 16 blocks (ub, vb), ub < vb, at vb (vb - 1) / 2 + ub
-// [NST stages][records][triangle blocks][barriers, TMEM slot][a tile's arguments] (the dynamic shared memory starts 1 KB-aligned: the
-// kernels have no static shared memory, and the system's own part is 1 KB)
+// A stage: [A hi][B hi][A lo][B lo] of a split k-block, 32 deep (STC_FP32: [B third] too), or [A][B] of a 16-bit shift
+// or projection k-block, 64 deep.
 __host__ __device__ constexpr uint32_t stc_stage_bytes(int mode) {
-  return StcCfg::SB + (mode == STC_FP32 ? StcCfg::B_BYTES : 0);  // (the third part of the factor's operand)
+  return StcCfg::SB + (mode == STC_FP32 ? StcCfg::B_BYTES : 0);
 }
+// [NST stages][records][triangle blocks][barriers, TMEM slot, a tile][a tile's arguments] (the dynamic shared memory starts
+// 1 KB-aligned: the kernels have no static shared memory, and the system's own part is 1 KB)
 __host__ __device__ constexpr size_t sweep_tc_smem_bytes(int mode, int nst) {
-  return (size_t)nst * stc_stage_bytes(mode) + (STC_SUB * STC_REC + STC_TRI) * sizeof(float) + 128 + STC_ARGS;
+  return (size_t)nst * stc_stage_bytes(mode) + (STC_SUB * STC_REC + STC_TRI) * sizeof(float) + 256 + STC_ARGS;
 }
-// TMEM columns of a CTA: the sums (and y) of a sub-tile, and STC_FP32's second accumulator
+// TMEM columns of one accumulator (the sums, then the y, of a sub-tile; STC_FP32: and the second sums).
 __host__ __device__ constexpr uint32_t stc_cols(int mode) { return mode == STC_FP32 ? 2 * STC_SUB : STC_SUB; }
 
-// Shared-memory layout and per-CTA state of the whole-tile sweep (set up once per
-// kernel: a persistent kernel runs many tiles through the same stage, barriers
-// and TMEM columns).
+// The producing thread's place: k-blocks gone through the stages, steps begun, steps whose first half and whole the
+// sweeping warps are known to have done (overlapped), k-blocks of the coming step under way (otherwise).
+struct StcRun {
+  uint32_t count, step, half, whole;
+  int pre;
+};
+
+// Shared-memory layout and per-CTA state of the whole-tile sweep (set up once per kernel).
 struct StcCta {
   unsigned char* stage;
   float* rec;            // the sub-tile's records
   float* tri;            // its triangle blocks
   uint64_t* full;        // [NST] the stage's copies landed
   uint64_t* freeb;       // [NST] the products reading the stage are done
+  uint64_t* acc;         // [2] the accumulator's products are done
+  uint64_t* ready;       // [2] a step's first half, its whole is done (one arrival per sweeping warp)
   uint32_t tmem;         // first of the CTA's TMEM columns
-  uint32_t* count;       // k-blocks gone through the stages so far (block i uses stage i mod NST)
   int* abort_flag;
-  int* item;             // the work item
+  int* item;             // (persistent kernel) the work item
   SweepTcArgs* args;     // (k_sweep_tc) the tile's arguments
+  StcTile* next;         // (k_sweep_tc) the coming tile
 };
 
 // Where the CTA's samples sit in the operand maps and the result buffers.
@@ -190,120 +219,309 @@ __device__ __forceinline__ void tmem_ld16(uint32_t (&r)[16], uint32_t addr) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// Thread 0's ring of NST stages.  load(i, st) starts the copies of k-block i into a stage, mma(i, st) issues its
-// products.  Runs blocks [0, nk), of which the first `pre` were loaded before, and waits for all products; `count`
-// numbers the blocks over the CTA's life.  Returns false (every copy and product in flight waited for, bounded) when
-// a wait expired.
-template <int NST, typename Load, typename Mma>
-__device__ __forceinline__ bool stc_ring(const StcCta& k, uint32_t& count, int nk, int pre, int* err, Load load,
-                                         Mma mma) {
-  int issued = pre, kb = 0;
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
+}
+// Bounded wait: false when the limit expires (the error code set) or the CTA has given up.
+__device__ __forceinline__ bool stc_wait(const StcCta& k, uint64_t* bar, uint32_t parity, int* err, int code) {
+  for (uint32_t i = 0; i < tc::WAIT_LIMIT; i++) {
+    if (tc::mbar_try_wait(bar, parity)) return true;
+    if ((i & 255) == 255 && *(volatile int*)k.abort_flag) return false;
+  }
+  atomicExch(err, code);
+  return false;
+}
+
+// Who issues the products.  Overlapped (a launch of at most two CTAs an SM): a fifth warp's first thread, into two
+// accumulators by turns, so that most of a step's products (a step: a sub-tile, or a projection pass) run while the
+// step before is swept.  Otherwise thread 0 of the four sweeping warps, between the steps, one accumulator: with six CTAs
+// an SM (float32: three) the others' sweeps fill that time.  A fifth warp's registers and a second accumulator
+// leave four (two), and those are slower as soon as there are samples for more than two: n = 65,536, 20 x 5,000: 74 against
+// 57 ms; two CTAs an SM, n = 8,192, 38,000 samples, tiles of 512: bf16 3.44 against 3.95 ms, float32 3.96
+// against 4.86; one: n = 16,384, 10 x 1,000: 5.94 against 6.77; float32, n = 1,024: 0.55 against 0.61.
+template <bool OV>
+struct StcPlan;
+template <>
+struct StcPlan<true> {
+  static constexpr int THREADS = 160, NBUF = 2;
+};
+template <>
+struct StcPlan<false> {
+  static constexpr int THREADS = 128, NBUF = 1;
+};
+__host__ __device__ constexpr int stc_stages(int mode, bool ov) {
+  return mode == STC_FP32 ? (ov ? 3 : 2) : (ov ? 4 : 1);
+}
+// CTAs per SM: six (80 registers a thread), STC_FP32 three; overlapped two.
+__host__ __device__ constexpr int stc_ctas(int mode, bool ov) { return ov ? 2 : (mode == STC_FP32 ? 3 : 6); }
+
+// Step u of a tile: its k-blocks are nsh of ranks, then those of y.
+template <int MODE>
+struct StcStep {
+  static constexpr bool SPLIT = MODE == STC_FP32;
+  static constexpr int KS = SPLIT ? STC_KB : 64;  // depth of a shift or projection k-block
+  int nsub, q0, r0, nsh, nk;
+  bool proj;
+  __device__ StcStep(const StcTile& t, int u) {
+    nsub = (t.mt + STC_SUB - 1) / STC_SUB;
+    proj = u >= nsub;
+    q0 = u * STC_SUB;
+    r0 = (u - nsub) * STC_SUB;
+    nsh = proj ? 0 : (t.kr + KS - 1) / KS;
+    nk = proj ? (t.mt + KS - 1) / KS : nsh + q0 / STC_KB;
+  }
+  // What k-block kb waits for, overlapped: nothing, the first half (32 variables) of the step before (1), all of it (2).
+  __device__ int gate(const StcTile& t, int u, int kb) const {
+    if (kb < nsh) return u == 0 && kb >= t.kearly / KS ? 2 : 0;
+    const int j = kb - nsh;
+    if (!proj) return j < nk - nsh - 2 ? 0 : (j == nk - nsh - 2 ? 1 : 2);
+    if (u > nsub) return 0;
+    if (!SPLIT) return j < nsub - 1 ? 0 : 2;
+    return j < 2 * (nsub - 1) ? 0 : (j == 2 * (nsub - 1) ? 1 : 2);
+  }
+  // Starts the copies of k-block kb into stage st.
+  __device__ void load(const StcOps& o, const StcTile& t, int row0, const StcCta& k, const StcPlace& pl, int kb,
+                       uint32_t st) const {
+    constexpr uint32_t A = StcCfg::A_BYTES, HALF = StcCfg::HALF, SB = stc_stage_bytes(MODE), B3 = 2 * HALF;
+    unsigned char* s = k.stage + st * SB;
+    uint64_t* bar = k.full + st;
+    tc::mbar_expect_tx(bar, SB);
+    if (kb < nsh) {  // two 64-sample MN-major boxes of W, a box of U rows
+      const int y = pl.wy + t.krow0 + kb * KS;
+      if constexpr (SPLIT) {
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          tc::tma_load_2d(s + h * HALF, o.mapW, bar, pl.wx, y + h * o.wlo);
+          tc::tma_load_2d(s + h * HALF + A / 2, o.mapW, bar, pl.wx + 64, y + h * o.wlo);
+          tc::tma_load_2d(s + h * HALF + A, o.mapU, bar, kb * KS + h * o.ulo, row0 + q0);
+        }
+        tc::tma_load_2d(s + B3, o.mapU, bar, kb * KS + 2 * o.ulo, row0 + q0);
+      } else {
+        tc::tma_load_2d(s, o.mapW, bar, pl.wx, y);
+        tc::tma_load_2d(s + StcShiftCfg::A_BYTES / 2, o.mapW, bar, pl.wx + 64, y);
+        tc::tma_load_2d(s + StcShiftCfg::A_BYTES, o.mapU, bar, kb * KS, row0 + q0);
+      }
+    } else if (!SPLIT && proj) {
+      tc::tma_load_2d(s, o.mapYp, bar, kb * KS, pl.yrow);
+      tc::tma_load_2d(s + StcProjCfg::A_BYTES, o.mapV, bar, kb * KS, t.kcol0 + r0);
+    } else {
+      const int x = (kb - nsh) * STC_KB;
+      const CUtensorMap* mb = proj ? o.mapV : o.mapB;
+      const int lo = proj ? o.vlo : o.blo, y = proj ? t.kcol0 + r0 : row0 + q0;
+      tc::tma_load_2d(s, o.mapY, bar, x, pl.yrow);
+      tc::tma_load_2d(s + HALF, o.mapY, bar, o.alo + x, pl.yrow);
+      tc::tma_load_2d(s + A, mb, bar, x, y);
+      tc::tma_load_2d(s + HALF + A, mb, bar, lo + x, y);
+      if constexpr (SPLIT) tc::tma_load_2d(s + B3, mb, bar, 2 * lo + x, y);
+    }
+  }
+  // Issues its products into the accumulator at d (STC_FP32: all but hi x hi at d + 64).
+  __device__ void mma(const StcCta& k, int kb, uint32_t st, uint32_t d) const {
+    constexpr bool F16 = MODE != STC_BF16;
+    constexpr uint32_t ID_K = F16 ? StcCfg::IDESC_F16 : StcCfg::IDESC;            // A K-major (y)
+    constexpr uint32_t ID_M = F16 ? StcShiftCfg::IDESC_F16 : StcShiftCfg::IDESC;  // A MN-major (W)
+    constexpr uint32_t A = StcCfg::A_BYTES, HALF = StcCfg::HALF;
+    const uint32_t sa = tc::smem_u32(k.stage) + st * stc_stage_bytes(MODE);
+    const bool sh = kb < nsh;
+    if (!SPLIT && (sh || proj)) {
+      // per 16-deep step MN-major W is two 1 KB K groups on (+128), K-major rows 32 bytes (+2)
+      const uint64_t da = sh ? tc::sdesc_mn(sa, StcShiftCfg::A_BYTES / 2) : tc::sdesc<64>(sa);
+      const uint64_t db = tc::sdesc<64>(sa + StcShiftCfg::A_BYTES), step = sh ? 128 : 2;
+#pragma unroll
+      for (int kk = 0; kk < 4; kk++)
+        tc::mma_f16(d, da + step * (uint64_t)kk, db + (uint64_t)(2 * kk), sh ? ID_M : ID_K, (kb > 0 || kk > 0) ? 1u : 0u);
+      return;
+    }
+    const uint64_t ah = SPLIT && sh ? tc::sdesc_mn(sa, A / 2) : tc::sdesc<STC_KB>(sa);
+    const uint64_t al = SPLIT && sh ? tc::sdesc_mn(sa + HALF, A / 2) : tc::sdesc<STC_KB>(sa + HALF);
+    const uint64_t bh = tc::sdesc<STC_KB>(sa + A), bl = tc::sdesc<STC_KB>(sa + HALF + A);
+    const uint64_t step = SPLIT && sh ? 128 : 2;
+    const uint32_t id = SPLIT && sh ? ID_M : ID_K, d2 = SPLIT ? d + STC_SUB : d;
+#pragma unroll
+    for (int kk = 0; kk < STC_KB / 16; kk++) {
+      const uint64_t oa = step * (uint64_t)kk, ob = (uint64_t)(2 * kk);
+      const uint32_t acc = (kb > 0 || kk > 0) ? 1u : 0u;
+      tc::mma_f16(d, ah + oa, bh + ob, id, acc);
+      tc::mma_f16(d2, ah + oa, bl + ob, id, SPLIT ? acc : 1u);
+      tc::mma_f16(d2, al + oa, bh + ob, id, 1u);
+      if constexpr (SPLIT) {
+        tc::mma_f16(d2, al + oa, bl + ob, id, 1u);
+        tc::mma_f16(d2, ah + oa, tc::sdesc<STC_KB>(sa + 2 * HALF) + ob, id, 1u);
+      }
+    }
+  }
+};
+
+// The products of step u of a tile, by one thread: its k-blocks through a ring of NST stages, then the accumulator's
+// barrier.  Overlapped, a step's accumulator is complete only after the step before it has been swept, but most of its
+// k-blocks need nothing of that step: all but the last two of a sub-tile's coupling and of the first projection pass
+// (the first of these waits for the step's first half), and all but the ranks of the tile before in a tile's first shift.
+// Returns false (its copies and products in flight waited for, bounded) when a wait expired or the CTA gave up.
+template <int MODE, int NST, bool OV>
+__device__ __forceinline__ bool stc_products(const StcOps& o, const StcTile& t, int row0, const StcCta& k,
+                                             const StcPlace& pl, int u, StcRun& r) {
+  const StcStep<MODE> s(t, u);
+  // the step before is swept: its first 32 variables, or all
+  auto swept = [&](bool whole) -> bool {
+    if (r.half < r.step) {
+      if (!stc_wait(k, k.ready, (r.step - 1) & 1, o.err, 6)) return false;
+      r.half = r.step;
+    }
+    if (whole && r.whole < r.step) {
+      if (!stc_wait(k, k.ready + 1, (r.step - 1) & 1, o.err, 7)) return false;
+      r.whole = r.step;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    return true;
+  };
+  const uint32_t buf = OV ? r.step & 1 : 0;
+  int issued = OV ? 0 : r.pre, kb = 0;
   bool ok = true;
-  for (; kb < nk; kb++) {
-    for (; issued < nk && issued < kb + NST; issued++) {
-      const uint32_t i = count + (uint32_t)issued;
-      if (i >= NST && !tc::mbar_wait(k.freeb + i % NST, (i / NST - 1) & 1, err, 9)) {
+  for (; kb < s.nk; kb++) {
+    for (; issued < s.nk && issued < kb + NST; issued++) {
+      if constexpr (OV) {
+        const int g = s.gate(t, u, issued);
+        if (g != 0 && (g == 1 ? r.half : r.whole) < r.step) {
+          if (issued > kb) break;  // (first the products of what has been loaded)
+          if (!swept(g == 2)) {
+            ok = false;
+            break;
+          }
+        }
+      }
+      const uint32_t i = r.count + (uint32_t)issued;
+      if (i >= NST && !stc_wait(k, k.freeb + i % NST, (i / NST - 1) & 1, o.err, 9)) {
         ok = false;
         break;
       }
-      load(issued, i % NST);
+      s.load(o, t, row0, k, pl, issued, i % NST);
     }
-    const uint32_t i = count + (uint32_t)kb;
-    if (!ok || !tc::mbar_wait(k.full + i % NST, (i / NST) & 1, err, 8)) {
+    const uint32_t i = r.count + (uint32_t)kb;
+    if (!ok || !stc_wait(k, k.full + i % NST, (i / NST) & 1, o.err, 8)) {
       ok = false;
       break;
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    mma(kb, i % NST);
+    s.mma(k, kb, i % NST, k.tmem + buf * stc_cols(MODE));
     tc::mma_commit(k.freeb + i % NST);
   }
-  if (kb > 0) {  // (products complete in order)
-    const uint32_t i = count + (uint32_t)kb - 1;
-    if (!tc::mbar_wait(k.freeb + i % NST, (i / NST) & 1, err, 9)) ok = false;
-  }
-  if (!ok)
-    for (; kb < issued; kb++) {
-      const uint32_t i = count + (uint32_t)kb;
-      tc::mbar_wait(k.full + i % NST, (i / NST) & 1, err, 5);
+  if (OV && ok) ok = swept(true);
+  if (!ok) {
+    *(volatile int*)k.abort_flag = 1;
+    for (int j = kb; j < issued; j++) {  // copies in flight
+      const uint32_t i = r.count + (uint32_t)j;
+      tc::mbar_wait(k.full + i % NST, (i / NST) & 1, o.err, 5);
     }
-  count += (uint32_t)nk;
-  return ok;
+    if (r.count + (uint32_t)kb > 0) {  // products in flight (they complete in order)
+      const uint32_t i = r.count + (uint32_t)kb - 1;
+      tc::mbar_wait(k.freeb + i % NST, (i / NST) & 1, o.err, 5);
+    }
+    return false;
+  }
+  r.count += (uint32_t)s.nk;
+  r.pre = 0;
+  if (s.nk > 0) tc::mma_commit(k.acc + buf);
+  else mbar_arrive(k.acc + buf);
+  r.step++;
+  return true;
+}
+// Not overlapped, after a step's products: the copies of the next sub-tile's first shift k-blocks, which land during
+// the sweep (W and U are complete, all products have read their stages).
+template <int MODE, int NST>
+__device__ __forceinline__ void stc_prefetch(const StcOps& o, const StcTile& t, int row0, const StcCta& k,
+                                             const StcPlace& pl, int u, StcRun& r) {
+  const StcStep<MODE> s(t, u);
+  if (s.proj) return;
+  for (; r.pre < NST && r.pre < s.nsh; r.pre++) s.load(o, t, row0, k, pl, r.pre, (r.count + (uint32_t)r.pre) % NST);
+}
+// Overlapped: all products of a tile.
+template <int MODE, int NST>
+__device__ __forceinline__ bool stc_produce(const StcOps& o, const StcTile& t, int row0, const StcCta& k,
+                                            const StcPlace& pl, StcRun& r) {
+  const int steps = (t.mt + STC_SUB - 1) / STC_SUB + (t.kc + STC_SUB - 1) / STC_SUB;
+  for (int u = 0; u < steps; u++)
+    if (!stc_products<MODE, NST, true>(o, t, row0, k, pl, u, r)) return false;
+  return true;
 }
 
-// One diagonal tile for the CTA's samples: the low-rank shifts and in-tile
-// coupling on tcgen05, the float sweep of eq. 2, the projections.  act: the thread's
+// A barrier of the sweeping warps; true (to all of them) when a wait before it failed.
+template <bool OV>
+__device__ __forceinline__ bool stc_bar(const StcCta& k, bool failed) {
+  if constexpr (OV) {
+    uint32_t any;
+    __syncwarp();
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, 128, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+        : "=r"(any)
+        : "r"(failed ? 1u : 0u)
+        : "memory");
+    if (any) *(volatile int*)k.abort_flag = 1;
+    return any != 0;
+  } else {  // (thread 0 alone waits, and sets the flag)
+    __syncthreads();
+    return *(volatile int*)k.abort_flag != 0;
+  }
+}
+// The arguments of tile i (of end, the largest of m variables) for the sweeping warps; base: those as of tile 0.  The
+// tile after it is copied during the sweep.
+template <bool OV>
+__device__ __forceinline__ void stc_args(const StcCta& k, const SweepTcArgs& base, const StcTile* tiles, int i, int end,
+                                         int m, bool first) {
+  stc_bar<OV>(k, false);  // those of the tile before read by all
+  if (threadIdx.x == 0) {
+    SweepTcArgs p = base;
+    p.at(first ? tiles[i] : *k.next, i, m);
+    *k.args = p;
+    if (i + 1 < end) {
+      cp_async16(reinterpret_cast<float4*>(k.next), reinterpret_cast<const float*>(tiles + i + 1), 16);
+      cp_async16(reinterpret_cast<float4*>(k.next) + 1, reinterpret_cast<const float*>(tiles + i + 1) + 4, 16);
+      cp_async_commit();
+    }
+  }
+  stc_bar<OV>(k, false);
+}
+
+// The warp's part of the step's first half (0) or whole (1) is done, its y or projections visible to copies, its TMEM
+// accesses complete.
+template <bool OV>
+__device__ __forceinline__ void stc_done(const StcCta& k, int which) {
+  asm volatile("fence.proxy.async;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  if constexpr (OV) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(k.ready + which);
+  }
+}
+
+// One diagonal tile for the CTA's samples, by the sweeping warps: the float sweep of eq. 2 and the projections, of the
+// products' sums.  step: steps so far.  o, run, row0: thread
+// 0's, to issue the products when no other warp does.  act: the thread's
 // sample exists (else it shadows one and writes nothing); Ds: its row of lattice shifts
-// at the tile's first variable (read up to three entries past the tile); ks: its point
+// (read up to three entries past the tile); ks: its point
 // index; rs: its MVT scale (1 for MVN).  The tile's log P is added to (prod, pe, lsum).
-// Returns false when a bounded wait expired.
-template <int FLAGS, int MODE, int NST>
-__device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensorMap* mapB, const CUtensorMap* mapW,
-                                         const CUtensorMap* mapU, const CUtensorMap* mapY64, const CUtensorMap* mapV,
-                                         const SweepTcArgs& p, const StcCta& k, const StcPlace& pl, const bool act,
-                                         const uint64_t* Ds, const uint32_t ks, const float rs, float& prod,
-                                         float& lsum, int& pe) {
+// Returns false (to all sweeping warps) when a bounded wait expired.
+template <int FLAGS, int MODE, int NST, bool OV>
+__device__ __forceinline__ bool stc_tile(const SweepTcArgs& p, const StcCta& k, const StcPlace& pl, uint32_t& step,
+                                         const StcOps& o, StcRun& run, int row0, const bool act, const uint64_t* Ds, const uint32_t ks,
+                                         const float rs,
+                                         float& prod, float& lsum, int& pe) {
   constexpr bool PER = FLAGS & SWEEP_PERIODIZE, ONE = FLAGS & SWEEP_ONE_SIDED;
   constexpr bool F16 = MODE != STC_BF16, SPLIT = MODE == STC_FP32;
   using Op = Op16<F16>;
-  constexpr uint32_t ID_C = F16 ? StcCfg::IDESC_F16 : StcCfg::IDESC;
-  constexpr uint32_t ID_S = F16 ? StcShiftCfg::IDESC_F16 : StcShiftCfg::IDESC;
-  constexpr uint32_t ID_P = F16 ? StcProjCfg::IDESC_F16 : StcProjCfg::IDESC;
-  constexpr uint32_t CA = StcCfg::A_BYTES, CHALF = StcCfg::HALF, SA = StcShiftCfg::A_BYTES, PA = StcProjCfg::A_BYTES;
-  constexpr uint32_t SB = stc_stage_bytes(MODE), CB3 = StcCfg::SB;  // (a stage; its third B part)
-  constexpr int KS = SPLIT ? STC_KB : 64;  // depth of a shift or projection k-block
-  unsigned char* stage = k.stage;
-  volatile int* abort_flag = k.abort_flag;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int mt = p.mt;
-  const uint32_t tmem = k.tmem;
-  const uint32_t tl = tmem + ((uint32_t)(32 * warp) << 16);  // this warp's 32 lanes
-  const int nks = (p.kr + KS - 1) / KS;
-  // the copies of shift k-block kb.  16-bit: two 64-sample MN-major boxes of W (64 ranks), one box of U rows.  Split:
-  // [W hi: two 64-sample boxes of 32 ranks][U hi][W lo][U lo][U third]
-  auto load_shift = [&](int kb, int q0, uint32_t st) {
-    unsigned char* d = stage + st * SB;
-    uint64_t* bar = k.full + st;
-    tc::mbar_expect_tx(bar, SB);
-    const int y = pl.wy + p.krow0 + kb * KS;
-    if constexpr (SPLIT) {
-#pragma unroll
-      for (int h = 0; h < 2; h++) {
-        tc::tma_load_2d(d + h * CHALF, mapW, bar, pl.wx, y + h * p.wlo);
-        tc::tma_load_2d(d + h * CHALF + CA / 2, mapW, bar, pl.wx + 64, y + h * p.wlo);
-        tc::tma_load_2d(d + h * CHALF + CA, mapU, bar, kb * KS + h * p.ulo, p.urow0 + q0);
-      }
-      tc::tma_load_2d(d + CB3, mapU, bar, kb * KS + 2 * p.ulo, p.urow0 + q0);
-    } else {
-      tc::tma_load_2d(d, mapW, bar, pl.wx, y);
-      tc::tma_load_2d(d + SA / 2, mapW, bar, pl.wx + 64, y);
-      tc::tma_load_2d(d + SA, mapU, bar, kb * 64, p.urow0 + q0);
-    }
-  };
-  // the products of a split stage [A hi][B hi][A lo][B lo]([B third]), 32 deep: A's descriptors and their advance per 16-deep step
-  auto mma_split = [&](uint64_t ah, uint64_t al, uint64_t astep, uint32_t sa, uint32_t idesc, bool first) {
-    const uint64_t bh = tc::sdesc<STC_KB>(sa + CA), bl = tc::sdesc<STC_KB>(sa + CHALF + CA);
-#pragma unroll
-    for (int kk = 0; kk < STC_KB / 16; kk++) {
-      const uint64_t oa = astep * (uint64_t)kk, ob = (uint64_t)(2 * kk);  // 32 bytes per 16-deep step of B
-      const uint32_t acc = (!first || kk > 0) ? 1u : 0u;
-      tc::mma_f16(tmem, ah + oa, bh + ob, idesc, acc);
-      tc::mma_f16(SPLIT ? tmem + STC_SUB : tmem, ah + oa, bl + ob, idesc, SPLIT ? acc : 1u);
-      tc::mma_f16(SPLIT ? tmem + STC_SUB : tmem, al + oa, bh + ob, idesc, 1u);
-      if constexpr (SPLIT) {
-        tc::mma_f16(tmem + STC_SUB, al + oa, bl + ob, idesc, 1u);
-        tc::mma_f16(tmem + STC_SUB, ah + oa, tc::sdesc<STC_KB>(sa + CB3) + ob, idesc, 1u);
-      }
-    }
-  };
-
-  int pre = 0;  // (thread 0) shift k-blocks of the coming sub-tile already under way
-  for (int q0 = 0; q0 < mt; q0 += STC_SUB) {
+  const uint32_t tmem = k.tmem + ((uint32_t)(32 * warp) << 16);  // this warp's 32 lanes
+  for (int q0 = 0; q0 < mt; q0 += STC_SUB, step++) {
     const int mq = min(STC_SUB, mt - q0);
-    // every thread is past the previous sub-tile's reads of the records and its TMEM accesses
-    if (tid >= 32) {
-      // the sub-tile's records, limits and triangle blocks, by the warps that do not run the products
-      const int t0 = tid - 32;
-      for (int t = t0; t < mq * 6; t += STC_NS - 32) {
+    const uint32_t buf = OV ? step & 1 : 0, tl = tmem + buf * stc_cols(MODE);
+    stc_bar<OV>(k, false);  // every sweeping thread is past the previous sub-tile's reads of the records and its accumulator
+    if (!OV && tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      stc_products<MODE, NST, OV>(o, p.t, row0, k, pl, q0 / STC_SUB, run);
+    }
+    if (OV || tid >= 32) {
+      constexpr int T0 = OV ? 0 : 32;  // (the warp that issues the products is late)
+      for (int t = tid - T0; t < mq * 6; t += STC_NS - T0) {
         const int v = t / 6, c = t - v * 6;
         const float* src = p.rec + (int64_t)(q0 + v) * STC_REC + 4 * c;
         if (c == 4)
@@ -312,7 +530,7 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
         else
           cp_async16(reinterpret_cast<float4*>(k.rec) + t, src, 16);
       }
-      for (int t = t0; t < STC_TRI / 4; t += STC_NS - 32) {
+      for (int t = tid - T0; t < STC_TRI / 4; t += STC_NS - T0) {
         const int blk = t >> 6, u = (t >> 2) & 15, c = t & 3;
         const int vb = blk < 1 ? 1 : (blk < 3 ? 2 : 3), ub = blk - vb * (vb - 1) / 2;
         if (16 * vb < mq)
@@ -320,60 +538,17 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
                      p.BT + (int64_t)(q0 + 16 * ub + u) * p.ldbt + q0 + 16 * vb + 4 * c, 16);
       }
       cp_async_commit();
-      cp_async_wait<0>();
     }
-    if ((q0 > 0 || p.kr > 0) && tid == 0) {
-      // T = W[ranks of row tile i, samples]^T U_i[q0 + v, ranks]^T     (the low-rank shifts)
-      //   + y[:, <q0] B_i[q0 + v, <q0]^T                              (the coupling, 32-deep split stages)
-      const uint32_t sa0 = tc::smem_u32(stage);
-      uint32_t count = *k.count;
-      const bool ok = stc_ring<NST>(
-          k, count, nks + q0 / STC_KB, pre, p.err,
-          [&](int kb, uint32_t st) {
-            if (kb < nks) {
-              load_shift(kb, q0, st);
-              return;
-            }
-            unsigned char* d = stage + st * SB;
-            uint64_t* bar = k.full + st;
-            tc::mbar_expect_tx(bar, SB);
-            const int x = (kb - nks) * STC_KB;
-            tc::tma_load_2d(d, mapY, bar, x, pl.yrow);
-            tc::tma_load_2d(d + CHALF, mapY, bar, p.alo + x, pl.yrow);
-            tc::tma_load_2d(d + CA, mapB, bar, x, p.brow0 + q0);
-            tc::tma_load_2d(d + CHALF + CA, mapB, bar, p.blo + x, p.brow0 + q0);
-            if constexpr (SPLIT) tc::tma_load_2d(d + CB3, mapB, bar, 2 * p.blo + x, p.brow0 + q0);
-          },
-          [&](int kb, uint32_t st) {
-            const uint32_t sa = sa0 + st * SB;
-            if (kb >= nks) {
-              mma_split(tc::sdesc<STC_KB>(sa), tc::sdesc<STC_KB>(sa + CHALF), 2, sa, ID_C, kb == 0);
-            } else if constexpr (SPLIT) {
-              // per 16-deep step MN-major W is two 1 KB K groups on (+128)
-              mma_split(tc::sdesc_mn(sa, CA / 2), tc::sdesc_mn(sa + CHALF, CA / 2), 128, sa, ID_S, kb == 0);
-            } else {
-              const uint64_t dw = tc::sdesc_mn(sa, SA / 2), du = tc::sdesc<64>(sa + SA);
-#pragma unroll
-              for (int kk = 0; kk < 4; kk++)
-                tc::mma_f16(tmem, dw + (uint64_t)(128 * kk), du + (uint64_t)(2 * kk), ID_S,
-                            (kb > 0 || kk > 0) ? 1u : 0u);
-            }
-          });
-      pre = 0;
-      if (!ok) {
-        *abort_flag = 1;
-      } else if (q0 + STC_SUB < mt) {
-        // these land during the sweep (W and U are complete; all products have read their stages)
-        for (; pre < NST && pre < nks; pre++) load_shift(pre, q0 + STC_SUB, (count + (uint32_t)pre) % NST);
-      }
-      *k.count = count;
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();  // records and triangle staged; shifts and coupling are in TMEM
+    bool ok = true;  // (not overlapped, the others wait at the barrier: their polls would take the other CTAs' issue slots)
+    if (OV || tid == 0) ok = stc_wait(k, k.acc + buf, (OV ? step >> 1 : step) & 1, p.err, 4);
+    if (!OV && !ok) *(volatile int*)k.abort_flag = 1;
+    if (!OV && tid == 0 && ok) stc_prefetch<MODE, NST>(o, p.t, row0, k, pl, q0 / STC_SUB + 1, run);
+    cp_async_wait<0>();
+    // records and triangle staged; shifts and coupling are in TMEM
+    if (stc_bar<OV>(k, !ok)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (*abort_flag) return false;
 
-    const uint64_t* Dp = Ds + q0;
+    const uint64_t* Dp = Ds + p.t.t0 + q0;
     uint64_t d0 = Dp[0], d1 = Dp[1];  // the lattice shifts of a pair of variables, loaded one pair ahead
     for (int v0 = 0; v0 < mq; v0 += DIAG_VB) {
       const int nb = min(DIAG_VB, mq - v0);
@@ -528,55 +703,37 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
           }
         }
       }
+      if (OV && v0 == STC_KB - DIAG_VB && mq > STC_KB) stc_done<OV>(k, 0);
     }
-    // y stored and visible to the copies (global), the records free for the next sub-tile's (shared), the TMEM
-    // columns free for the next products
-    asm volatile("fence.proxy.async;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    if (OV && mq <= STC_KB) stc_done<OV>(k, 0);
+    stc_done<OV>(k, 1);
   }
-  // the tile's projections for the later tiles, 64 ranks a pass through the same
-  // TMEM columns: W[vmap[r]][c] = sum_v V[kcol0 + r][v] y_v[c] (y hi parts, 64-deep
-  // stages of the CTA's y rows and of V rows)
-  for (int r0 = 0; r0 < p.kc; r0 += 64) {
-    if (tid == 0) {
-      const uint32_t sa0 = tc::smem_u32(stage);
-      uint32_t count = *k.count;
-      const bool ok = stc_ring<NST>(
-          k, count, (mt + KS - 1) / KS, 0, p.err,
-          [&](int kb, uint32_t st) {
-            unsigned char* d = stage + st * SB;
-            uint64_t* bar = k.full + st;
-            tc::mbar_expect_tx(bar, SB);
-            if constexpr (SPLIT) {
-              tc::tma_load_2d(d, mapY, bar, kb * KS, pl.yrow);
-              tc::tma_load_2d(d + CHALF, mapY, bar, p.alo + kb * KS, pl.yrow);
-              tc::tma_load_2d(d + CA, mapV, bar, kb * KS, p.kcol0 + r0);
-              tc::tma_load_2d(d + CHALF + CA, mapV, bar, p.vlo + kb * KS, p.kcol0 + r0);
-              tc::tma_load_2d(d + CB3, mapV, bar, 2 * p.vlo + kb * KS, p.kcol0 + r0);
-            } else {
-              tc::tma_load_2d(d, mapY64, bar, kb * 64, pl.yrow);
-              tc::tma_load_2d(d + PA, mapV, bar, kb * 64, p.kcol0 + r0);
-            }
-          },
-          [&](int kb, uint32_t st) {
-            const uint32_t sa = sa0 + st * SB;
-            if constexpr (SPLIT) {
-              mma_split(tc::sdesc<STC_KB>(sa), tc::sdesc<STC_KB>(sa + CHALF), 2, sa, ID_C, kb == 0);
-            } else {
-              const uint64_t da = tc::sdesc<64>(sa), db = tc::sdesc<64>(sa + PA);
-#pragma unroll
-              for (int kk = 0; kk < 4; kk++)
-                tc::mma_f16(tmem, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), ID_P, (kb > 0 || kk > 0) ? 1u : 0u);
-            }
-          });
-      if (!ok) *abort_flag = 1;
-      *k.count = count;
+  // the tile's projections for the later tiles, 64 ranks a step: W[vmap[r]][c] = sum_v V[kcol0 + r][v] y_v[c]; the
+  // rows' places and scales are in the records' and the triangle's, up to RANKS at a time
+  constexpr int RANKS = STC_SUB * STC_REC;
+  static_assert(RANKS <= STC_TRI && RANKS % STC_SUB == 0, "room for the scales");
+  int32_t* const vm = reinterpret_cast<int32_t*>(k.rec);
+  float* const ws = k.tri;
+#pragma unroll 1
+  for (int r0 = 0, rb = 0; r0 < p.kc; r0 += STC_SUB, step++) {
+    const uint32_t buf = OV ? step & 1 : 0, tl = tmem + buf * stc_cols(MODE);
+    if (!OV || r0 % RANKS == 0) stc_bar<OV>(k, false);  // every sweeping thread is done with those, and the accumulator
+    if (!OV && tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      stc_products<MODE, NST, OV>(o, p.t, row0, k, pl, (mt + STC_SUB - 1) / STC_SUB + r0 / STC_SUB, run);
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+    if (r0 % RANKS == 0) {
+      rb = r0;
+      for (int t = tid; t < RANKS && r0 + t < p.kc; t += STC_NS) {
+        vm[t] = __ldg(p.vmap + r0 + t);
+        if (F16) ws[t] = __ldg(p.wscale + r0 + t);
+      }
+    }
+    bool ok = true;
+    if (OV || tid == 0) ok = stc_wait(k, k.acc + buf, (OV ? step >> 1 : step) & 1, p.err, 4);
+    if (!OV && !ok) *(volatile int*)k.abort_flag = 1;
+    if (stc_bar<OV>(k, !ok)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (*abort_flag) return false;
 #pragma unroll 1
     for (int h = 0; h < 64; h += 16) {
       uint32_t r[16];
@@ -591,16 +748,16 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
             if (r0 + h + j < p.kc) {
               const bool two = r0 + h + j + 1 < p.kc;
               const int rr = r0 + h + j, r1 = two ? rr + 1 : rr;
-              const float w0 = (__uint_as_float(r[j]) + __uint_as_float(l[j])) * p.wscale[rr];
-              const float w1 = (__uint_as_float(r[j + 1]) + __uint_as_float(l[j + 1])) * p.wscale[r1];
+              const float w0 = (__uint_as_float(r[j]) + __uint_as_float(l[j])) * ws[rr - rb];
+              const float w1 = (__uint_as_float(r[j + 1]) + __uint_as_float(l[j + 1])) * ws[r1 - rb];
               uint32_t hi, lo;
               split_f32(w0, w1, hi, lo);
               top = fmaxf(top, fmaxf(fabsf(w0), two ? fabsf(w1) : 0.0f));
-              unsigned short* d0 = pl.wcol + (int64_t)p.vmap[rr] * p.ldw;
+              unsigned short* d0 = pl.wcol + (int64_t)vm[rr - rb] * p.ldw;
               d0[0] = (unsigned short)hi;
               d0[(int64_t)p.wlo * p.ldw] = (unsigned short)lo;
               if (two) {
-                unsigned short* d1 = pl.wcol + (int64_t)p.vmap[r1] * p.ldw;
+                unsigned short* d1 = pl.wcol + (int64_t)vm[r1 - rb] * p.ldw;
                 d1[0] = (unsigned short)(hi >> 16);
                 d1[(int64_t)p.wlo * p.ldw] = (unsigned short)(lo >> 16);
               }
@@ -611,14 +768,12 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
 #pragma unroll
         for (int j = 0; j < 16; j++)
           if (r0 + h + j < p.kc)
-            pl.wcol[(int64_t)p.vmap[r0 + h + j] * p.ldw] =
-                Op::one(F16 ? __uint_as_float(r[j]) * p.wscale[r0 + h + j] : __uint_as_float(r[j]));
+            pl.wcol[(int64_t)vm[r0 - rb + h + j] * p.ldw] =
+                Op::one(F16 ? __uint_as_float(r[j]) * ws[r0 - rb + h + j] : __uint_as_float(r[j]));
       }
     }
-    // W visible to the copies of the next tile's shifts, when the same CTA runs it
-    asm volatile("fence.proxy.async;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();  // the TMEM columns and the stage free for the next pass
+    if (OV) stc_done<OV>(k, 0);
+    stc_done<OV>(k, 1);
   }
   return true;
 }
@@ -626,7 +781,7 @@ __device__ __forceinline__ bool stc_tile(const CUtensorMap* mapY, const CUtensor
 // The CTA's stages, records, barriers and TMEM columns (dynamic shared memory of
 // sweep_tc_smem_bytes(MODE, NST)); the barriers initialised and the columns allocated.
 // Ends with every thread past the allocation.
-template <int MODE, int NST>
+template <int MODE, int NST, bool OV>
 __device__ __forceinline__ StcCta stc_cta_setup(unsigned char* smem) {
   StcCta k;
   k.stage = smem;
@@ -634,24 +789,31 @@ __device__ __forceinline__ StcCta stc_cta_setup(unsigned char* smem) {
   k.tri = k.rec + STC_SUB * STC_REC;
   k.full = reinterpret_cast<uint64_t*>(k.tri + STC_TRI);
   k.freeb = k.full + NST;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(k.freeb + NST);
-  k.count = tmem_slot + 1;
-  k.abort_flag = reinterpret_cast<int*>(tmem_slot + 2);
+  k.acc = k.freeb + NST;
+  k.ready = k.acc + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(k.ready + 2);
+  static_assert((2 * NST + 4) * 8 + 12 <= 192, "the barriers' place");
+  k.abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
   k.item = k.abort_flag + 1;
-  k.args = reinterpret_cast<SweepTcArgs*>(reinterpret_cast<unsigned char*>(k.full) + 128);
+  k.next = reinterpret_cast<StcTile*>(reinterpret_cast<unsigned char*>(k.full) + 192);
+  k.args = reinterpret_cast<SweepTcArgs*>(reinterpret_cast<unsigned char*>(k.full) + 256);
   if (threadIdx.x == 0) {
     *k.abort_flag = 0;
-    *k.count = 0;
 #pragma unroll
     for (int s = 0; s < NST; s++) {
       tc::mbar_init(k.full + s, 1);
       tc::mbar_init(k.freeb + s, 1);
     }
+#pragma unroll
+    for (int s = 0; s < 2; s++) {
+      tc::mbar_init(k.acc + s, 1);
+      tc::mbar_init(k.ready + s, STC_NS / 32);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if ((threadIdx.x >> 5) == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(tmem_slot)),
-                 "r"(stc_cols(MODE))
+                 "r"(StcPlan<OV>::NBUF * stc_cols(MODE))
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -663,28 +825,23 @@ __device__ __forceinline__ StcCta stc_cta_setup(unsigned char* smem) {
 }
 
 // Frees the CTA's TMEM columns once every thread is done with them.
-template <int MODE>
+template <int MODE, bool OV>
 __device__ __forceinline__ void stc_cta_release(const StcCta& k) {
+  __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if ((threadIdx.x >> 5) == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(k.tmem), "r"(stc_cols(MODE))
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(k.tmem), "r"(StcPlan<OV>::NBUF * stc_cols(MODE))
                  : "memory");
 }
 
-// CTAs per SM: six with one stage (80 registers each), three with two, two with three or four.
-__host__ __device__ constexpr int stc_ctas(int nst) { return nst == 1 ? 6 : (nst == 2 ? 3 : 2); }
-
-// A diagonal tile: its first variable and size, its rank rows of W (first, count), its column ranks (first, count).
-struct StcTile {
-  int t0, mt, krow0, kr, kcol0, kc, pad[2];
-};
 struct SweepTcLaunch {
   SweepTcArgs base;      // the arguments as of tile 0 at variable, rank row and column rank 0
   const StcTile* tiles;
   int i0, i1;            // the launch's tiles
   int m;                 // largest tile
+  int alo, blo, ulo, vlo;  // (StcOps)
   const uint64_t* D;
   int64_t ldD, sample0, N, C;
   const float* rs;
@@ -699,65 +856,57 @@ struct SweepTcLaunch {
 // allocate and load anew: n = 65,536, 20 x 5,000 samples, tiles of 512, bf16: 60.8 -> 57.4 ms a solve; n = 16,384,
 // 10 x 1,000, tiles of 256: 7.22 -> 6.78; 20 requests of n = 512 to 4,096 on four streams: 11.0 -> 8.8.  A queue of (tile, block) items over fewer CTAs, the same number on each
 // SM, was slower: 63 ms with four or five CTAs on each, for the CTAs then run out of step and their y out of L2.)
-template <int FLAGS, int MODE, int NST>
-__global__ void __launch_bounds__(STC_NS, stc_ctas(NST))
-    k_sweep_tc(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapB,
+template <int FLAGS, int MODE, bool OV>
+__global__ void __launch_bounds__(StcPlan<OV>::THREADS, stc_ctas(MODE, OV))
+    k_sweep_tc(const __grid_constant__ CUtensorMap mapY, const __grid_constant__ CUtensorMap mapYp, const __grid_constant__ CUtensorMap mapB,
                const __grid_constant__ CUtensorMap mapW, const __grid_constant__ CUtensorMap mapU,
-               const __grid_constant__ CUtensorMap mapY64, const __grid_constant__ CUtensorMap mapV,
-               const __grid_constant__ SweepTcLaunch d) {
+               const __grid_constant__ CUtensorMap mapV, const __grid_constant__ SweepTcLaunch d) {
   extern __shared__ __align__(1024) unsigned char stc_smem[];
-  const StcCta k = stc_cta_setup<MODE, NST>(stc_smem);
+  constexpr int NST = stc_stages(MODE, OV);
+  const StcCta k = stc_cta_setup<MODE, NST, OV>(stc_smem);
   const int tid = threadIdx.x;
   const int c0 = blockIdx.x * STC_NS;  // (a chunk holds fewer than 2^31 samples)
-  const bool act = c0 + tid < d.C;
-  const int cs = act ? c0 + tid : (int)d.C - 1;  // inactive lanes shadow a valid sample, write nothing
-  const int64_t g = d.sample0 + cs, sh = g / d.N;
-  const uint32_t ks = (uint32_t)(g - sh * d.N) + 1u;  // lattice point index k = 1..N (N < 2^31)
-  const float rs = d.rs ? d.rs[cs] : 1.0f;
   StcPlace pl;
   pl.wx = c0;
   pl.wy = 0;
   pl.yrow = c0;
-  pl.ysrow = d.Ys + (int64_t)cs * d.ldys;
-  pl.wcol = d.W + cs;
+  const StcOps o{&mapY, &mapYp, &mapB, &mapW, &mapU, &mapV, d.alo, d.blo, d.base.wlo, d.ulo, d.vlo, d.base.err};
+  StcRun run{0, 0, 0, 0, 0};
+  if (OV && tid >= STC_NS) {
+    if (tid == STC_NS) {
 #pragma unroll 1
-  for (int i = d.i0; i < d.i1; i++) {
-    if (tid == 0) {
-      const int4 t = __ldg(reinterpret_cast<const int4*>(d.tiles + i));
-      const int2 c = __ldg(reinterpret_cast<const int2*>(d.tiles + i) + 2);
-      SweepTcArgs& p = *k.args;
-      p = d.base;
-      p.rec += (int64_t)i * d.m * STC_REC;
-      p.BT += (int64_t)i * d.m * p.ldbt;
-      p.mt = t.y;
-      p.t0 = t.x;
-      p.a += t.x;
-      p.b += t.x;
-      p.brow0 = i * d.m;
-      p.urow0 = i * d.m;
-      p.krow0 = t.z;
-      p.kr = t.w;
-      p.kcol0 = c.x;
-      p.kc = c.y;
-      p.vmap += c.x;
-      p.wscale += c.x;
-      p.rscale += (int64_t)i * d.m;
+      for (int i = d.i0; i < d.i1; i++) {
+        const StcTile t = d.tiles[i];
+        if (!stc_produce<MODE, NST>(o, t, i * d.m, k, pl, run)) break;
+      }
     }
-    __syncthreads();
-    // log P of the tile = log(prod) + pe log 2 + lsum, prod kept in [1, 2)
-    float prod = 1.0f, lsum = 0.0f;
-    int pe = 0;
-    if (!stc_tile<FLAGS, MODE, NST>(&mapY, &mapB, &mapW, &mapU, &mapY64, &mapV, *k.args, k, pl, act,
-                                    d.D + sh * d.ldD + k.args->t0, ks, rs, prod, lsum, pe))
-      break;
-    if (act) {
-      const double lp = (double)(logf(prod) + lsum) + (double)pe * 0.69314718055994530942;
-      if (i == 0) d.logP[g] = lp;
-      else atomicAdd(d.logP + g, lp);  // (this thread's alone: an add that nothing waits for)
+  } else {
+    const bool act = c0 + tid < d.C;
+    const int cs = act ? c0 + tid : (int)d.C - 1;  // inactive lanes shadow a valid sample, write nothing
+    const int64_t g = d.sample0 + cs;
+    const int64_t sh = g / d.N;
+    const uint64_t* Ds = d.D + sh * d.ldD;
+    const uint32_t ks = (uint32_t)(g - sh * d.N) + 1u;  // lattice point index k = 1..N (N < 2^31)
+    const float rs = d.rs ? d.rs[cs] : 1.0f;
+    pl.ysrow = d.Ys + (int64_t)cs * d.ldys;
+    pl.wcol = d.W + cs;
+    uint32_t step = 0;
+#pragma unroll 1
+    for (int i = d.i0; i < d.i1; i++) {
+      stc_args<OV>(k, d.base, d.tiles, i, d.i1, d.m, i == d.i0);
+      // log P of the tile = log(prod) + pe log 2 + lsum, prod kept in [1, 2)
+      float prod = 1.0f, lsum = 0.0f;
+      int pe = 0;
+      if (!stc_tile<FLAGS, MODE, NST, OV>(*k.args, k, pl, step, o, run, i * d.m, act, Ds, ks, rs, prod, lsum, pe))
+        break;
+      if (act) {
+        const double lp = (double)(logf(prod) + lsum) + (double)pe * 0.69314718055994530942;
+        if (i == 0) d.logP[g] = lp;
+        else atomicAdd(d.logP + g, lp);  // (this thread's alone: an add that nothing waits for)
+      }
     }
-    __syncthreads();  // the arguments read by all
   }
-  stc_cta_release<MODE>(k);
+  stc_cta_release<MODE, OV>(k);
 }
 
 }  // namespace tlrmvn

@@ -1,6 +1,7 @@
-"""GPU: the whole-tile sweep's launches: more tiles than one launch takes (16,384 variables), and more samples than the
-SMs hold in one pass (equal passes).  Tolerance: the float32 path's 1e-4 relative per sample against the float64
-path; passes of another size give the same bits."""
+"""GPU: the whole-tile sweep's launches: more tiles than one launch takes (16,384 variables; also more column ranks
+than are staged at a time), more samples than the SMs hold in one pass (equal passes), and few samples, whose products
+overlap the sweep.  Tolerance: the float32 path's 1e-4 relative per sample against the float64
+path; passes of another size, overlapped or not, give the same bits."""
 import math
 
 import numpy as np
