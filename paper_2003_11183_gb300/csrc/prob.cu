@@ -28,6 +28,9 @@
 namespace tlrmvn {
 
 // ---- Student-t scale (Algorithm 7): chi_nu^-1(w0)/sqrt(nu) ------------------------
+// Float64 chains at one SM's 2 lanes a clock: one warp a block, so that few samples spread over all SMs (10,000
+// samples, nu = 7: 0.17 -> 0.16 ms; 100,000: 0.85 -> 0.78).
+constexpr int CHI_T = 32;
 __global__ void k_chi_scale(double* rs, float* rs32, const uint64_t* Q, const uint64_t* D, int64_t ldD,
                             int64_t coord, int64_t sample0, int64_t N, int64_t C, double nu, int periodize) {
   int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -834,12 +837,17 @@ int make_tensor_map_16(CUtensorMap* map, const void* base, uint64_t inner, uint6
 
 // splitmix64 (S. Vigna): output number t of the generator started at `seed`.
 uint64_t splitmix64_seed_at(uint64_t seed, uint64_t t);
-static uint64_t splitmix64_at(uint64_t seed, uint64_t t) { return splitmix64_seed_at(seed, t); }
-uint64_t splitmix64_seed_at(uint64_t seed, uint64_t t) {
+static __host__ __device__ __forceinline__ uint64_t splitmix64_at(uint64_t seed, uint64_t t) {
   uint64_t z = seed + (t + 1) * 0x9E3779B97F4A7C15ULL;
   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
   z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
   return z ^ (z >> 31);
+}
+uint64_t splitmix64_seed_at(uint64_t seed, uint64_t t) { return splitmix64_at(seed, t); }
+// The lattice shifts of a call that gives a seed (on the host they took 30 us and a copy that the stream waited for).
+static __global__ void k_lattice_shifts(uint64_t seed, int64_t count, uint64_t* D) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < count) D[t] = splitmix64_at(seed, (uint64_t)t);
 }
 
 // Freed scratch stays in the device's default memory pool between calls: a
@@ -1233,7 +1241,7 @@ static int run_chunks(Factor& F, const T* Bt, const T* Ut, const T* Vt, const Li
     const int64_t Cc = std::min(C, S - c0);
     if (mvt) {
       pf.begin(TLRMVN_KC_CHI);
-      k_chi_scale<<<blocks_for(Cc, 128), 128, 0, st>>>(rs, rs32, F.Q, dD, F.n + 1, F.n, c0, N, Cc, nu, o.periodize);
+      k_chi_scale<<<blocks_for(Cc, CHI_T), CHI_T, 0, st>>>(rs, rs32, F.Q, dD, F.n + 1, F.n, c0, N, Cc, nu, o.periodize);
       pf.end();
     }
     for (int i = 0; i < F.r; i++) {
@@ -1321,9 +1329,10 @@ static int run_chunks(Factor& F, const T* Bt, const T* Ut, const T* Vt, const Li
 //        float32 path: hi parts, then as many rows of lo parts
 //   Y16  C x 2 my16 16-bit, sample-major: the tile's y (hi) in columns [0, my16) and
 //        its lo part in [my16, 2 my16)
-// out_of_range (float32 path): set when a y or a projection left fp16's range, and the results are not to be used.
+// err_out: the device flags of SweepTcArgs::err, to be read once the stream has got there (err[1], float32 path: a y
+// or a projection left fp16's range, and the results are not to be used).
 static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts& o, const Tuning& tu,
-                         const uint64_t* dD, double* logP, Scratch& sc, cudaStream_t st, Prof& pf, bool* out_of_range) {
+                         const uint64_t* dD, double* logP, Scratch& sc, cudaStream_t st, Prof& pf, int** err_out) {
   const int64_t M = o.n_shifts, N = o.n_points, S = M * N;
   const int m = F.m;
   TcOperands tco;
@@ -1385,19 +1394,14 @@ static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts&
     const int64_t Cc = std::min(C, S - c0);
     if (mvt) {
       pf.begin(TLRMVN_KC_CHI);
-      k_chi_scale<<<blocks_for(Cc, 128), 128, 0, st>>>(nullptr, rs32, F.Q, dD, F.n + 1, F.n, c0, N, Cc, nu,
+      k_chi_scale<<<blocks_for(Cc, CHI_T), CHI_T, 0, st>>>(nullptr, rs32, F.Q, dD, F.n + 1, F.n, c0, N, Cc, nu,
                                                        o.periodize);
       pf.end();
     }
     sweep_tiles_tc(F, L, rs32, dD, c0, N, Cc, o.periodize, Y, ly, logP, tco, tu, st, pf);
     TLR_CUDA(cudaGetLastError());
   }
-  int herr[2] = {0, 0};
-  TLR_CUDA(cudaMemcpyAsync(herr, err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
-  TLR_CUDA(cudaStreamSynchronize(st));
-  if (herr[0])
-    return fail(TLRMVN_E_TIMEOUT, "tensor-core kernel gave up waiting (code " + std::to_string(herr[0]) + ")");
-  *out_of_range = herr[1] != 0;
+  *err_out = err;
   return TLRMVN_OK;
 }
 
@@ -1447,18 +1451,11 @@ int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, co
   TLR_CHECK(sc.get(&ell, M));
   if (per_sample_dev) logP = per_sample_dev;
   else TLR_CHECK(sc.get(&logP, S));
-  // lattice shifts
-  {
-    std::vector<uint64_t> hD;
-    const uint64_t* src = o.shifts;
-    if (!src) {
-      hD.resize((size_t)M * (n + 1));
-      for (size_t t = 0; t < hD.size(); t++) hD[t] = splitmix64_at(o.seed, t);
-      src = hD.data();
-    }
-    TLR_CUDA(cudaMemcpyAsync(dD, src, (size_t)M * (n + 1) * 8, cudaMemcpyHostToDevice, st));
-    if (!hD.empty()) TLR_CUDA(cudaStreamSynchronize(st));
-  }
+  const int64_t nd = M * (n + 1);
+  if (o.shifts)
+    TLR_CUDA(cudaMemcpyAsync(dD, o.shifts, (size_t)nd * 8, cudaMemcpyHostToDevice, st));
+  else
+    k_lattice_shifts<<<blocks_for(nd, 256), 256, 0, st>>>(o.seed, nd, dD);
   TLR_CUDA(cudaMemsetAsync(bad, 0, 2 * sizeof(int), st));
   Prof pf(st);
   pf.begin(TLRMVN_KC_PREP);
@@ -1472,31 +1469,40 @@ int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, co
     return fail(TLRMVN_E_INVAL, "limits must satisfy a_i <= b_i, a_i < +inf, b_i > -inf, no NaN");
   }
   TLR_CHECK(ensure_copies(F, o.precision, st));
-  int s;
   const Lims L{ap, bp, ap32, bp32, hbad[1] == 0};
   const Tuning tu = F.tuning(o.precision);
-  if (o.precision == TLRMVN_FP64)
-    s = run_chunks<double, double>(F, F.B, F.Ucat, F.Vcat, L, nu, o, tu, dD, logP, sc, st, pf);
-  else {
-    bool out_of_range = false;
+  // the estimate of the samples' logs
+  auto reduce = [&]() -> int {
+    pf.begin(TLRMVN_KC_REDUCE);
+    k_shift_reduce<<<(unsigned)M, 256, 0, st>>>(logP, N, ell);
+    pf.end();
+    pf.begin(TLRMVN_KC_REDUCE);
+    k_final<<<1, 256, 0, st>>>(ell, (int)M, logp_dev, err_dev);
+    pf.end();
+    if (ell_dev_out) TLR_CUDA(cudaMemcpyAsync(ell_dev_out, ell, M * 8, cudaMemcpyDeviceToDevice, st));
+    TLR_CUDA(cudaGetLastError());
+    return TLRMVN_OK;
+  };
+  if (o.precision != TLRMVN_FP64) {
+    int herr[2] = {0, 0};
     {
       Scratch own(st);
-      s = run_chunks_tc(F, L, nu, o, tu, dD, logP, own, st, pf, &out_of_range);
+      int* err = nullptr;
+      TLR_CHECK(run_chunks_tc(F, L, nu, o, tu, dD, logP, own, st, pf, &err));
+      TLR_CHECK(reduce());
+      TLR_CUDA(cudaMemcpyAsync(herr, err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
+      TLR_CUDA(cudaStreamSynchronize(st));
     }
-    if (s == TLRMVN_OK && out_of_range) {  // limits tens of thousands of standard deviations out
-      TLR_CHECK(ensure_copies(F, TLRMVN_FP32 + SIMT_COPIES, st));
-      s = run_chunks<float, float>(F, (const float*)nullptr, F.U32, F.V32, L, nu, o, tu, dD, logP, sc, st, pf);
-    }
+    if (herr[0])
+      return fail(TLRMVN_E_TIMEOUT, "tensor-core kernel gave up waiting (code " + std::to_string(herr[0]) + ")");
+    if (!herr[1]) return pf.collect();
+    // float32, limits tens of thousands of standard deviations out
+    TLR_CHECK(ensure_copies(F, TLRMVN_FP32 + SIMT_COPIES, st));
+    TLR_CHECK((run_chunks<float, float>(F, (const float*)nullptr, F.U32, F.V32, L, nu, o, tu, dD, logP, sc, st, pf)));
+  } else {
+    TLR_CHECK((run_chunks<double, double>(F, F.B, F.Ucat, F.Vcat, L, nu, o, tu, dD, logP, sc, st, pf)));
   }
-  TLR_CHECK(s);
-  pf.begin(TLRMVN_KC_REDUCE);
-  k_shift_reduce<<<(unsigned)M, 256, 0, st>>>(logP, N, ell);
-  pf.end();
-  pf.begin(TLRMVN_KC_REDUCE);
-  k_final<<<1, 256, 0, st>>>(ell, (int)M, logp_dev, err_dev);
-  pf.end();
-  if (ell_dev_out) TLR_CUDA(cudaMemcpyAsync(ell_dev_out, ell, M * 8, cudaMemcpyDeviceToDevice, st));
-  TLR_CUDA(cudaGetLastError());
+  TLR_CHECK(reduce());
   TLR_CUDA(cudaStreamSynchronize(st));
   return pf.collect();
 }
@@ -1530,6 +1536,31 @@ extern "C" int tlrmvn_prob_device(tlrmvn_factor_t f, const double* a, const doub
   return s;
 }
 
+// The host-array solve.  Its device copies are stream-ordered scratch: cudaMalloc and cudaFree of them took a sixth
+// of a solve of n = 1,024 and made other streams wait.
+static int prob_host(Factor& F, const double* a, const double* b, double nu, const tlrmvn_opts& o, double* logp,
+                     double* err, double* per_shift, double* per_sample, cudaStream_t st) {
+  const int64_t n = F.n, M = o.n_shifts, S = M * (int64_t)o.n_points;
+  Scratch sc(st);
+  double *da = nullptr, *db = nullptr, *out2 = nullptr, *dell = nullptr, *dps = nullptr;
+  TLR_CHECK(sc.get(&da, n));
+  TLR_CHECK(sc.get(&db, n));
+  TLR_CHECK(sc.get(&out2, 2));
+  if (per_shift) TLR_CHECK(sc.get(&dell, M));
+  if (per_sample) TLR_CHECK(sc.get(&dps, S));
+  TLR_CUDA(cudaMemcpyAsync(da, a, n * 8, cudaMemcpyHostToDevice, st));
+  TLR_CUDA(cudaMemcpyAsync(db, b, n * 8, cudaMemcpyHostToDevice, st));
+  TLR_CHECK(prob_impl(F, da, db, nu, o, out2, out2 + 1, dell, dps, st));
+  double h[2];
+  TLR_CUDA(cudaMemcpyAsync(h, out2, 16, cudaMemcpyDeviceToHost, st));
+  if (per_shift) TLR_CUDA(cudaMemcpyAsync(per_shift, dell, M * 8, cudaMemcpyDeviceToHost, st));
+  if (per_sample) TLR_CUDA(cudaMemcpyAsync(per_sample, dps, S * 8, cudaMemcpyDeviceToHost, st));
+  TLR_CUDA(cudaStreamSynchronize(st));
+  *logp = h[0];
+  *err = h[1];
+  return TLRMVN_OK;
+}
+
 extern "C" int tlrmvn_prob(tlrmvn_factor_t f, const double* a, const double* b, double nu, const tlrmvn_opts* opts,
                            double* logp, double* err, double* per_shift, double* per_sample) {
   if (!f || !a || !b || !logp || !err) return fail(TLRMVN_E_INVAL, "null argument");
@@ -1538,37 +1569,7 @@ extern "C" int tlrmvn_prob(tlrmvn_factor_t f, const double* a, const double* b, 
   int cur = 0;
   cudaGetDevice(&cur);
   TLR_CUDA(cudaSetDevice(F.device));
-  cudaStream_t st = pick_stream(opts->stream);
-  const int64_t n = F.n, M = opts->n_shifts, S = M * (int64_t)opts->n_points;
-  double *da = nullptr, *db = nullptr, *out2 = nullptr, *dell = nullptr, *dps = nullptr;
-  int s = dalloc(&da, n);
-  if (s == TLRMVN_OK) s = dalloc(&db, n);
-  if (s == TLRMVN_OK) s = dalloc(&out2, 2);
-  if (s == TLRMVN_OK && per_shift) s = dalloc(&dell, M);
-  if (s == TLRMVN_OK && per_sample) s = dalloc(&dps, S);
-  if (s == TLRMVN_OK) {
-    cudaError_t e = cudaMemcpyAsync(da, a, n * 8, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(db, b, n * 8, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) s = cuda_fail(e, "copy limits");
-  }
-  if (s == TLRMVN_OK) s = prob_impl(F, da, db, nu, *opts, out2, out2 + 1, dell, dps, st);
-  if (s == TLRMVN_OK) {
-    double h[2];
-    cudaError_t e = cudaMemcpyAsync(h, out2, 16, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && per_shift) e = cudaMemcpyAsync(per_shift, dell, M * 8, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && per_sample) e = cudaMemcpyAsync(per_sample, dps, S * 8, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) s = cuda_fail(e, "copy results");
-    else {
-      *logp = h[0];
-      *err = h[1];
-    }
-  }
-  dfree(da);
-  dfree(db);
-  dfree(out2);
-  dfree(dell);
-  dfree(dps);
+  const int s = prob_host(F, a, b, nu, *opts, logp, err, per_shift, per_sample, pick_stream(opts->stream));
   cudaSetDevice(cur);
   return s;
 }
