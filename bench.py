@@ -37,7 +37,7 @@ METRIC = "MVN/MVT QMC sample-dims/sec at n=65,536 vs FP64 path; p50/p99 solve la
 # those sources are unchanged (otherwise null); the summaries with the capture
 # commands are under profiles/.
 TRAFFIC = {
-    "k_sweep_tc": {"bytes_per_sample_dim": 20.7063,
+    "k_sweep_tc": {"bytes_per_sample_dim": 23.1201,
                    "capture": "profiles/k_sweep_tc_n16384.md",
                    "files": ["paper_2003_11183_gb300/csrc/sweep_tc.cuh",
                              "paper_2003_11183_gb300/csrc/sweep.cuh",
@@ -45,7 +45,7 @@ TRAFFIC = {
                              "paper_2003_11183_gb300/csrc/tcgen05.cuh",
                              "paper_2003_11183_gb300/csrc/common.cuh",
                              "include/tlrmvn.h"],
-                   "sources": "2091dce6350b70d328d34a085ab1b5bd34780cc9845b0990a2bf7b7e42bc9294"},
+                   "sources": "006e64bb546b2d4b313fc26f36d6c11fadb27b3dfdeae34b832172181ae6583b"},
 }
 
 
@@ -539,7 +539,7 @@ def run_ours(args):
                      peak_measured_source="tlrmvn_measure_fp32_peak: 8 independent FMA chains per thread, "
                                           "8 x 256 threads per SM, CUDA events",
                      flops_per_sample_dim=work["sweep"], sample_dims_per_launch=units,
-                     kernel={0: "k_diag<double>", 1: "k_diag_f32"}.get(prec, "k_sweep_tc"))
+                     kernel={0: "k_diag64", 1: "k_sweep_tc (split fp16 products)"}.get(prec, "k_sweep_tc"))
             if prec >= 2:
                 tach = work["tensor"] * units / (d["avg_launch_ms"] / 1e3) / 1e12
                 d["tensor_share"] = {"bound": "tensor", "unit": "TFLOP/s", "achieved": tach, "peak": bf16_peak,

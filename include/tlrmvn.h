@@ -55,7 +55,9 @@ extern "C" {
 /* ---- option values --------------------------------------------------- */
 /* Arithmetic of the integrand (tlrmvn_opts.precision). */
 #define TLRMVN_FP64        0  /* everything in float64 */
-#define TLRMVN_FP32        1  /* diagonal-tile sweep and low-rank shifts in float32 */
+#define TLRMVN_FP32        1  /* float32: the sweep, and its products on tcgen05 tensor cores with every operand
+                                 split into fp16 parts (errors no larger than float32 FMAs'); limits tens of
+                                 thousands of standard deviations out take float32 FMA kernels instead */
 #define TLRMVN_BF16_SHIFT  2  /* float32 sweep; low-rank shifts on tcgen05 tensor cores, bf16 in, fp32 accumulate */
 #define TLRMVN_FP16_SHIFT  3  /* as BF16_SHIFT with fp16 operands: U and V scaled per off-diagonal tile by
                                  powers of two into fp16's range, the inverse applied to each projection
@@ -200,16 +202,15 @@ int tlrmvn_prob_device(tlrmvn_factor_t f, const double* a, const double* b, doub
 
 /* Launch choices of the integrand for one factor and precision (no counterpart
  * in the paper; they change how the work is launched, not what is computed):
- *   sub       variables per sub-tile of the float32 sweep (64 or 128) or of the
- *             float64 sweep (32 or 64); the coupling between sub-tiles of a
- *             diagonal tile is a dense product
- *   threads   threads per block of the float32 sweep; 0 = the occupancy rule
+ *   sub       variables per sub-tile of the float64 sweep (32 or 64) or of the general
+ *             float32 one (64 or 128: limits beyond the tensor-core path's range); the
+ *             coupling between sub-tiles of a diagonal tile is a dense product
+ *   threads   threads per block of the general float32 sweep; 0 = the occupancy rule
  *   chunk     samples in flight per pass; 0 = as many as fit the memory rule
  *             (opts->sample_chunk, when set, still takes precedence)
- *   tc_ctas   whole-tile sweeps of the BF16-/FP16-shift paths sharing an SM (1..6; with spt 2
- *             at most 4 take effect)
- *   spt       samples per thread of the whole-tile sweep: 1 or 2 (two independent chains
- *             per thread, 256 samples per block)
+ *   tc_ctas   whole-tile sweeps of the BF16-/FP16-shift paths sharing an SM (1..6), where the
+ *             samples fill more than two a SM
+ *   spt       1 or 2, without effect (accepted for callers and caches that set it)
  *   ms        tlrmvn_autotune: device milliseconds per solve of the choice (-1
  *             when it came from the cache); candidates: how many were timed */
 typedef struct {
@@ -248,10 +249,9 @@ int tlrmvn_set_tuning(tlrmvn_factor_t f, int precision, const tlrmvn_tuning* t);
  * integrand, estimator) is captured once in a CUDA graph; tlrmvn_batch_run
  * replays it for new limits.  Needed by likelihood fitting, where the same
  * covariances meet new limits at every step (Section 5 of the paper).
- *   opts: precision TLRMVN_FP32 (float sweep, float SIMT shifts and
- *         projections) or TLRMVN_BF16_SHIFT (every tile through the same
- *         whole-tile tcgen05 sweep as tlrmvn_prob's BF16-shift path, with the
- *         chunk's projections and y in block-private bf16 buffers; results equal
+ *   opts: precision TLRMVN_FP32 or TLRMVN_BF16_SHIFT (every tile through the same
+ *         whole-tile tcgen05 sweep as tlrmvn_prob in that precision, with the
+ *         chunk's projections and y in block-private 16-bit buffers; results equal
  *         that path's on the same shifts up to the order of its float sums);
  *         opts->shifts must be NULL: problem p draws its shifts from seed
  *         opts->seed + p exactly as tlrmvn_prob does with that seed; n_shifts /
@@ -395,10 +395,10 @@ int tlrmvn_selftest_ndtri(const float* p, const float* lp, int n, float* out);
  * a device error. */
 int tlrmvn_measure_fp32_peak(void* stream, double* tflops);
 
-/* Kernel classes of the integrand, for tlrmvn_profile_get.  On the BF16-shift
- * path with tiles of more than 64 variables the shifts, the coupling and the
- * projections are computed inside the diagonal-tile sweep's kernel and are
- * timed as TLRMVN_KC_DIAG. */
+/* Kernel classes of the integrand, for tlrmvn_profile_get.  On the float32, BF16- and
+ * FP16-shift paths the shifts, the coupling and the projections are computed inside
+ * the diagonal tiles' sweep kernel, one launch for about 16,384 variables, and
+ * are timed as TLRMVN_KC_DIAG. */
 #define TLRMVN_KC_SHIFT   0  /* low-rank limit shifts  Delta_i = U_i W_i           */
 #define TLRMVN_KC_DIAG    1  /* diagonal-tile SOV sweep (eq. 2 on B_i)              */
 #define TLRMVN_KC_VPROJ   2  /* projections  W_col_i = V_i^T y_i                    */

@@ -55,15 +55,14 @@ void dfree(T*& p) {
 // ---- launch choices ----------------------------------------------------------
 // Launch choices of the integrand for one factor and precision, made by the
 // autotuner (tlrmvn_autotune) or left at these defaults:
-//   sub      variables per sub-tile of the float32 and float64 sweeps (64 or 128;
-//            the in-tile coupling between sub-tiles is a dense product)
-//   threads  threads per block of the float32 sweep (0: the occupancy rule)
+//   sub      variables per sub-tile of the float64 sweep (32 or 64) and of the general float32 one (64 or 128), which
+//            serves limits beyond the tensor-core path's range (the in-tile coupling between sub-tiles is a dense product)
+//   threads  threads per block of the general float32 sweep (0: the occupancy rule)
 //   chunk    samples in flight per pass (0: as many as the memory rule allows)
-//   tc_ctas  whole-tile sweeps (BF16-/FP16-shift paths) sharing an SM: 6 (all that
-//            fit: 80 registers, 28 KB of shared memory and 64 TMEM columns each), or
+//   tc_ctas  whole-tile sweeps of more than two CTAs an SM (BF16-/FP16-shift paths) sharing an SM: 6 (all that
+//            fit: 80 registers, 37 KB of shared memory and 64 TMEM columns each), or
 //            fewer by reserving shared memory
-//   spt      samples per thread of the whole-tile sweep: 1, or 2 (256 samples per
-//            CTA, two independent chains per thread, 128 TMEM columns, four CTAs per SM)
+//   spt      1 or 2: kept for callers and caches that set it, without effect
 struct Tuning {
   int sub = 64;
   int threads = 0;

@@ -1,7 +1,7 @@
 // tcgen05 / TMA building blocks of the tensor-core products (sm_103a): stage
 // shapes and instruction descriptors, shared-memory matrix descriptors, bounded
 // mbarrier waits, 2-D TMA loads, the 16-bit (bf16 or fp16) MMA and its commit.  Used by the
-// whole-tile sweep of the BF16-shift integrand (sweep_tc.cuh), whose products are
+// whole-tile sweep (sweep_tc.cuh), whose products are
 //
 //   D (M x N) += A (M x K) * B (N x K)^T     bf16 or fp16 operands (both the same type):
 //                                             B K-major; A K-major,

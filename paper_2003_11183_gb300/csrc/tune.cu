@@ -1,7 +1,7 @@
 // Autotuner of the integrand's launch choices (tlrmvn_autotune).
 //
 // For one factor, precision and solve size it times a small set of candidate
-// launch choices (Tuning: sweep sub-tile, sweep block size, samples per pass,
+// launch choices (Tuning: float64 sweep's sub-tile, samples per pass,
 // whole-tile sweeps per SM) with CUDA events on real solves of the caller's own
 // problem, keeps the fastest on the factor (every later tlrmvn_prob on that
 // factor and precision uses it) and records it in a cache file, so that the next
@@ -52,13 +52,11 @@ static std::vector<Tuning> candidates(const Factor& F, int precision, int64_t S)
         c.push_back(t);
       }
   } else if (precision == TLRMVN_FP32) {
-    for (int sub : {64, 128})
-      for (int threads : {0, 64, 128, 256}) {
-        Tuning t;
-        t.sub = sub;
-        t.threads = threads;
-        c.push_back(t);
-      }
+    for (int64_t chunk : {(int64_t)0, (S / 2 + 255) / 256 * 256}) {
+      Tuning t;
+      t.chunk = chunk;
+      c.push_back(t);
+    }
   } else {
     for (int sub : {32, 64}) {
       Tuning t;
