@@ -423,6 +423,7 @@ struct Batch {
   BatchTcProblem* dtprobs = nullptr;
   CUtensorMap* dmaps = nullptr;
   unsigned short *W16 = nullptr, *Y16 = nullptr;
+  size_t nw = 0, ny = 0;  // their elements
   CUtensorMap mapW{}, mapY{}, mapYp{};
   int* derr = nullptr;
   double *logP = nullptr, *ell = nullptr, *out = nullptr, *a_st = nullptr, *b_st = nullptr;
@@ -486,6 +487,12 @@ static int resident_ctas(const void* kernel, int threads, size_t dyn_smem, int d
   const size_t smem = (dyn_smem + fa.sharedSizeBytes + 127) / 128 * 128 + (size_t)res_blk;
   n = std::min<int>(n, (int)((size_t)smem_sm / smem));
   *out = std::max(n, 1);
+  return TLRMVN_OK;
+}
+
+static int zero_buffers(Batch& B) {
+  TLR_CUDA(cudaMemsetAsync(B.W16, 0, B.nw * 2, B.st));
+  TLR_CUDA(cudaMemsetAsync(B.Y16, 0, B.ny * 2, B.st));
   return TLRMVN_OK;
 }
 
@@ -671,18 +678,17 @@ static int batch_build(Batch& B, int count, const tlrmvn_factor_t* factors, cons
   B.grid_max = std::max(1, std::min(B.per_sm_max * B.sms, B.n_items));
   {
     // CTA-private W (kwmax rank rows x 128 samples; float32: twice, hi and lo) and sample-major y (128 rows of
-    // hi / lo columns), zeroed once: padding rows and columns meet zero
-    // operand entries and must stay finite
+    // hi / lo columns), zeroed: padding rows and columns meet zero operand entries and must stay finite
     B.kwmax = std::max<int64_t>(B.kwmax, 64);
     const int64_t wrows = B.kwmax * (B.f32 ? 2 : 1);
     if ((int64_t)B.grid_max * wrows >= ((int64_t)1 << 31))
       return fail(TLRMVN_E_NOTSUP, "batched projections exceed the tensor map's coordinate range");
-    const size_t nw = (size_t)B.grid_max * wrows * STC_NS, ny = (size_t)B.grid_max * STC_NS * 2 * B.my;
-    TLR_CHECK(dalloc(&B.W16, nw));
-    TLR_CHECK(dalloc(&B.Y16, ny));
+    B.nw = (size_t)B.grid_max * wrows * STC_NS;
+    B.ny = (size_t)B.grid_max * STC_NS * 2 * B.my;
+    TLR_CHECK(dalloc(&B.W16, B.nw));
+    TLR_CHECK(dalloc(&B.Y16, B.ny));
     TLR_CHECK(dalloc(&B.derr, 2));
-    TLR_CUDA(cudaMemsetAsync(B.W16, 0, nw * 2, st));
-    TLR_CUDA(cudaMemsetAsync(B.Y16, 0, ny * 2, st));
+    TLR_CHECK(zero_buffers(B));
     TLR_CUDA(cudaMemsetAsync(B.derr, 0, 2 * sizeof(int), st));
     const uint32_t deep = B.f32 ? 32 : 64;
     TLR_CHECK(make_tensor_map_16(&B.mapYp, B.Y16, 2 * B.my, (uint64_t)B.grid_max * STC_NS, 2 * B.my * 2, STC_NS,
@@ -770,6 +776,13 @@ static int batch_run(Batch& B, const double* const* a, const double* const* b, d
   int bad = 0, terr[2] = {0, 0};
   memcpy(&bad, B.h_out + 2 * B.count, sizeof(int));
   memcpy(terr, B.h_out + 2 * B.count + 1, 2 * sizeof(int));
+  if (bad || terr[0] || terr[1]) {  // (values of this run may not be finite, and a later run's padding would read them)
+    const int s = zero_buffers(B);
+    if (s != TLRMVN_OK) {
+      cudaSetDevice(cur);
+      return s;
+    }
+  }
   if (!bad && !terr[0] && terr[1]) {  // (float32) a y left fp16's range
     const int s = simt_prepare(B);
     if (s != TLRMVN_OK) {

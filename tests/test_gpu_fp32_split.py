@@ -70,3 +70,25 @@ def test_y_beyond_fp16_range(tl):
         one = [tl.tlrmvn_prob(F, w.a, w.b, math.inf, tl.FP32, 2, 130, seed=7 + p)[0] for p in range(2)]
         assert rel(near, one) < 1e-6
         plan.close()
+
+
+def test_batch_after_values_beyond_range(tl):
+    # a plan whose blocks serve a problem of larger tiles with y beyond fp16's range in one run and one of smaller tiles in
+    # the next: what the first left in the blocks' buffers (the smaller one's padding) must not reach it, nor what
+    # invalid limits left.  (About as many items as blocks, so that blocks change problems from run to run.)
+    M, N = 2, 12800
+    ws = [synth.small_workload(0, m, 330 + m, ragged_n=n) for n, m in ((300, 100), (280, 70))]
+    Fs = [tl.tlrmvn_factor_kernel(w.xy, w.kernel, w.params, w.nugget, w.a, w.b, w.m, w.tol, 0, 0) for w in ws]
+    plan = tl.BatchPlan(Fs, math.inf, M, N, seed=9)
+    a, b = [w.a for w in ws], [w.b for w in ws]
+    first = plan.run(a, b)[0]
+    far, nan = b[0].copy(), b[0].copy()
+    far[::3] = -2.0e6
+    nan[::7] = np.nan
+    for _ in range(8):
+        plan.run(a, [far, b[1]])
+        assert rel(plan.run(a, b)[0], first) < 1e-6
+        with pytest.raises(tl.TlrmvnError):
+            plan.run(a, [nan, b[1]])
+        assert rel(plan.run(a, b)[0], first) < 1e-6
+    plan.close()
