@@ -228,11 +228,6 @@ __global__ void k_final_batch(const double* ell, int M, double* out) {
   final_estimate(ell + (int64_t)blockIdx.x * M, M, out + 2 * blockIdx.x, out + 2 * blockIdx.x + 1);
 }
 
-template <typename S, typename D>
-__global__ void k_convert(const S* src, D* dst, int64_t count) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < count) dst[i] = (D)src[i];
-}
 // U16[(i*m + v) * kmax + k] = Ucat_i[v][k] for k < Krow_i, else 0
 __global__ void k_pad_u16(const double* Ucat, const int64_t* krow_off, int m, int64_t kmax, int64_t count,
                           __nv_bfloat16* U16) {
