@@ -295,6 +295,12 @@ __device__ __forceinline__ float rcp_ftz(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// The smaller of two, NaN if either is (fminf drops a NaN; the same one instruction).
+__device__ __forceinline__ float min_nan(float x, float y) {
+  float z;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(z) : "f"(x), "f"(y));
+  return z;
+}
 
 // float32 normal quantile, lower half.  Two regions:
 //  * p > 8.4e-5 (L = log2(4 p (1 - p)) > -11.54; all but about 1 in 6,000 calls):

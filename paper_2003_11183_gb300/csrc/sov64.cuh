@@ -275,7 +275,7 @@ __device__ __forceinline__ double sov_step_f64(const double* T, double at, doubl
     uc = fma(wc, f, nb ? m : hb);
     c = hb;
     near1 = bt > 3.09;  // c < 1e-3
-    rare = bt < -13.0 || (bt > 13.0 && zero_so_far);
+    rare = !(bt >= -13.0) || (bt > 13.0 && zero_so_far);  // (a NaN too)
   } else {
     const double xa = fabs(at);
     const bool na = at < 0.0;
@@ -286,8 +286,8 @@ __device__ __forceinline__ double sov_step_f64(const double* T, double at, doubl
     uc = fma(wc, f, nb ? 1.0 - hb : hb);
     c = ha + hb;
     near1 = at < -3.3 && bt > 3.3;
-    // (both limits in one tail beyond the table, a zero-width interval, a NaN)
-    rare = !(f > 1e-37) || (near1 && c == 0.0 && zero_so_far);
+    // (both limits in one tail beyond the table, a zero-width interval; a NaN, which its side's zero hides from f)
+    rare = !(at <= bt) || !(f > 1e-37) || (near1 && c == 0.0 && zero_so_far);
   }
   const double p = fmin(u, uc);
   rare = rare || !(p >= 4.6e-13);  // 2^-41 = 4.547e-13

@@ -134,13 +134,13 @@ __device__ __forceinline__ void sov_step_f32(float at, float bt, float w, float 
   sov_step<float>(at, bt, w, wc, ld, y);
 }
 
-// Phi(-x) in float32 for x >= 0 (zero beyond 13, where it falls below the normal floats), straight-line:
+// Phi(-x) in float32 for x >= 0 (zero beyond 13, where it falls below the normal floats; NaN for a NaN), straight-line:
 // exp(-x^2/2) R(x), with R half the scaled complementary error function as a degree-9 polynomial in
 // 1 / (2.5 + x) (coefficients from csrc/fit_mills.py; its even and odd halves side by side), and the
 // exponential from x^2 in two parts, x^2 + er exactly: -(x^2 + er) log2(e)/2 = n + f with n the nearest
 // integer, 2^f by the hardware and 2^n added to the exponent.  Relative error about 3e-7 at most.
 __device__ __forceinline__ float phi_neg_f32(float x) {
-  x = fminf(x, 13.0f);
+  x = min_nan(x, 13.0f);
   const float x2 = x * x, er = fmaf(x, x, -x2);
   const float kf = fmaf(x2, -7.213475108e-01f, 12582912.0f);  // the integer n in the low bits
   float f = fmaf(x2, -7.213475108e-01f, 12582912.0f - kf);
@@ -169,7 +169,7 @@ __device__ __forceinline__ float phi_neg_f32(float x) {
 //
 // The fast path is straight-line code for every lane, and one branch follows for
 // the lanes it does not serve (limits in the deep tail; a quantile below 8.4e-5, a
-// lane in 6,000): the chain from a variable's sum to its y is what bounds the
+// lane in 6,000; a NaN, whose log must reach lsum, for the product's renormalisation drops it): the chain from a variable's sum to its y is what bounds the
 // sweeps, and branches cut it (the one-sided case, the quantile's tail when that
 // started at 0.0017 and one warp in ten took it, the underflow test) and keep the compiler from
 // filling its waits.  With u = Phi(at) + w (Phi(bt) - Phi(at)) and uc = 1 - u both accurate, the
@@ -195,9 +195,9 @@ __device__ __forceinline__ void sov_step_f32_upper(float bt, float w, float wc, 
   const float u = w * ph, uc = fmaf(wc, ph, pc);
   const float L = lg2_ftz(u * uc);  // log2(4 u uc) - 2
   y = ndtri_poly_f32(L + 5.0f) * (uc - u);
-  if (L < NDTRI_LMIN - 2.0f) {
-    // (a deep limit always comes here: u < Phi(-8.9) = 2.8e-19; above it pp > 3e-29)
-    const bool deep = bt < -8.9f;
+  if (!(L >= NDTRI_LMIN - 2.0f)) {
+    // (a deep limit always comes here: u < Phi(-8.9) = 2.8e-19; above it pp > 3e-29; and a NaN, as a deep one)
+    const bool deep = !(bt >= -8.9f);
     const float2 r = sov_step_rare_f32(-INFINITY, bt, w, wc, fminf(u, uc), deep);
     y = (deep || u <= uc) ? r.x : -r.x;
     f = deep ? 1.0f : f;
