@@ -128,10 +128,11 @@ __global__ void __launch_bounds__(192) k_diag64(DiagArgs64 p) {
     for (; u < v; u++) s0 = fma(__ldg(Brow + u), ys[u * ld + tid], s0);
     dl += (s0 + s1) + (s2 + s3);
     const double lvv = __ldg(Brow + v), iv = inv[v];
-    // (limit - shift) / l_vv to the last bit from the reciprocal: the quotient and its remainder
+    // (limit - shift) / l_vv to the last bit from the reciprocal: the quotient and its remainder, which is not finite
+    // where the limit or the quotient is infinite (a limit like DBL_MAX over a small l_vv) or l_vv is 0 or infinite
     auto quotient = [&](double lim) {
       const double num = fma(lim, rs, -dl), q = num * iv, r = fma(-q, lvv, num);
-      return (__double2hiint(num) & 0x7FF00000) == 0x7FF00000 ? q : fma(r, iv, q);
+      return (__double2hiint(r) & 0x7FF00000) == 0x7FF00000 ? q : fma(r, iv, q);
     };
     const double bt = quotient(p.b[v]), at = ONE ? 0.0 : quotient(p.a[v]);
     double w, wc;

@@ -254,6 +254,7 @@ static __device__ __noinline__ double2 sov_step_rare_f64(double at, double bt, d
     const double e = fma(bt, 0.70710678118654752440, -t) + bt * -4.833646656726456726e-17;
     ld = bt < 39.0 ? -0.5 * erfc(t) * (1.0 - (2.0 * t + 1.0 / t) * e) : 0.0;
   }
+  if (ld == -INFINITY && isnan(y)) y = 0.0;  // (an infinite limit: the sample counts as zero, whatever y is)
   return make_double2(y, ld);
 }
 

@@ -1,10 +1,12 @@
 """GPU: numbers that are not finite on their way through the integrand. A NaN in a factor reaches the log of every sample
 that meets it, in each precision, for one- and two-sided limits, single and batched, and never counts as probability
-1."""
+1; limits so large that dividing them overflows count as infinite ones; a sample of probability zero (an infinite
+standardised limit) counts as zero and spoils no other."""
 import math
 
 import numpy as np
 import pytest
+from scipy.special import log_ndtr
 
 pytestmark = pytest.mark.gpu
 
@@ -63,3 +65,33 @@ def test_nan_in_a_batched_factor(tl, precision, sides):
     lp, _ = plan.run([a], [b])
     assert not np.isfinite(lp[0])
     plan.close()
+
+
+@pytest.mark.parametrize("precision", PRECISIONS)
+@pytest.mark.parametrize("sides", [1, 2])
+def test_zero_probability_samples(tl, precision, sides):
+    # x2 = x1 and x3 = x1 / 5 + x2 / 2 + z3: with x1 below 0.5 and x2 below 0.2 a sample has x2's factor 0 or 1
+    B = [np.array([[1.0, 0.0, 0.0], [1.0, 0.0, 0.0], [0.2, 0.5, 1.0]])]
+    F = tl.tlrmvn_factor_import(tl.build_export(3, 3, np.array([0, 3]), np.arange(3), B, {}, {}))
+    a = np.full(3, -np.inf if sides == 1 else -9.0)
+    lp, _, _, pm = tl.tlrmvn_prob(F, a, [0.5, 0.2, 30.0], math.inf, getattr(tl, precision), 2, 500, seed=3,
+                                  per_sample=True)
+    pm = np.ravel(pm)
+    zero = np.isneginf(pm)
+    # the samples below 0.2 are Phi(0.2) / Phi(0.5) = 0.84 of them
+    assert abs(np.mean(~zero) - 0.84) < 0.02 and np.allclose(pm[~zero], log_ndtr(0.5), atol=1e-6)
+    assert abs(lp - log_ndtr(0.2)) < 0.02
+
+
+@pytest.mark.parametrize("precision", PRECISIONS)
+@pytest.mark.parametrize("lo,hi", [(-np.inf, 1.79e308), (-1.79e308, 0.5), (-1.79e308, 1.79e308), (-np.inf, -1.79e308),
+                                   (1.5e308, 1.79e308)])
+def test_huge_limits(tl, precision, lo, hi):
+    # a diagonal of 0.5: 1.79e308 / 0.5 is beyond float64
+    B = [np.array([[0.5, 0.0, 0.0], [0.1, 0.5, 0.0], [0.2, 0.1, 0.9]])]
+    F = tl.tlrmvn_factor_import(tl.build_export(3, 3, np.array([0, 3]), np.arange(3), B, {}, {}))
+    inf = [math.copysign(math.inf, x) if abs(x) > 1e300 else x for x in (lo, hi)]
+    got = [tl.tlrmvn_prob(F, [x, -np.inf, -9.0], [y, 0.3, 0.4], math.inf, getattr(tl, precision), 2, 100, seed=3)[0]
+           for x, y in ([(lo, hi)] if max(inf) == -math.inf or min(inf) == math.inf else [(lo, hi), inf])]
+    # the same as with infinite limits, which may not both lie at one end
+    assert got[0] == got[1] if len(got) == 2 else np.isneginf(got[0])
