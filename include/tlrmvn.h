@@ -61,7 +61,8 @@ extern "C" {
 #define TLRMVN_BF16_SHIFT  2  /* float32 sweep; low-rank shifts on tcgen05 tensor cores, bf16 in, fp32 accumulate */
 #define TLRMVN_FP16_SHIFT  3  /* as BF16_SHIFT with fp16 operands: U and V scaled per off-diagonal tile by
                                  powers of two into fp16's range, the inverse applied to each projection
-                                 before it is stored (TLRMVN_E_NOTSUP if a tile's range cannot be met) */
+                                 before it is stored (TLRMVN_E_NOTSUP if a tile's range cannot be met); limits tens
+                                 of thousands of standard deviations out take the float32 FMA kernels instead */
 
 /* Preconditioner (tlrmvn_factor_opts.reorder), Section 3.3. */
 #define TLRMVN_REORDER_NONE       0  /* geometric order only ("tlrmvn") */

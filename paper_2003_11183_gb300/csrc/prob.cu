@@ -891,6 +891,8 @@ struct Scratch {
   }
 };
 
+// Scratch of the general float32 path per sample in flight.
+static int64_t simt_sample_bytes(const Factor& F) { return (F.ktot + 2 * (int64_t)F.m) * 4 + 8; }
 // Samples per pass: opts.sample_chunk, else the factor's tuned chunk, else as
 // many as keep the projection buffer W within 8 GiB (SIMT paths) or 32 GiB (bf16
 // path); a multiple of 256.
@@ -1325,10 +1327,11 @@ static int run_chunks(Factor& F, const T* Bt, const T* Ut, const T* Vt, const Li
 //        float32 path: hi parts, then as many rows of lo parts
 //   Y16  C x 2 my16 16-bit, sample-major: the tile's y (hi) in columns [0, my16) and
 //        its lo part in [my16, 2 my16)
-// err_out: the device flags of SweepTcArgs::err, to be read once the stream has got there (err[1], float32 path: a y
-// or a projection left fp16's range, and the results are not to be used).
+// err_out: the device flags of SweepTcArgs::err, to be read once the stream has got there (err[1], float32 and
+// FP16-shift paths: a y or a projection left fp16's range, and the results are not to be used).
 static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts& o, const Tuning& tu,
-                         const uint64_t* dD, double* logP, Scratch& sc, cudaStream_t st, Prof& pf, int** err_out) {
+                         const uint64_t* dD, double* logP, Scratch& sc, cudaStream_t st, Prof& pf, int** err_out,
+                         int64_t* scratch) {
   const int64_t M = o.n_shifts, N = o.n_points, S = M * N;
   const int m = F.m;
   TcOperands tco;
@@ -1348,6 +1351,7 @@ static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts&
   TLR_CHECK(sc.get(&W, (size_t)wrows * ldw));
   TLR_CHECK(sc.get(&Y, (size_t)ly * C));
   TLR_CHECK(sc.get(&err, 2));
+  *scratch = C * (wrows * 2 + ly * 2);
   const bool mvt = std::isfinite(nu);
   if (mvt) TLR_CHECK(sc.get(&rs32, (size_t)C));
   // padding columns of W and Y must hold finite values: they meet zero operand columns
@@ -1424,6 +1428,8 @@ int64_t prob_scratch_bytes(const Factor& F, const tlrmvn_opts& o) {
     const int64_t es = o.precision == TLRMVN_FP64 ? 8 : 4;
     const int64_t C = chunk_simt(o, tu, S, F.ktot, m, es);
     simt = C * ((F.ktot + 2 * m) * es + 8);
+  } else if (o.precision == TLRMVN_FP16_SHIFT) {  // (the same, in passes that the scratch of the usual path holds)
+    simt = 256 * simt_sample_bytes(F);
   }
   return bytes + std::max(simt, tc);
 }
@@ -1481,10 +1487,11 @@ int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, co
   };
   if (o.precision != TLRMVN_FP64) {
     int herr[2] = {0, 0};
+    int64_t scratch = 0;
     {
       Scratch own(st);
       int* err = nullptr;
-      TLR_CHECK(run_chunks_tc(F, L, nu, o, tu, dD, logP, own, st, pf, &err));
+      TLR_CHECK(run_chunks_tc(F, L, nu, o, tu, dD, logP, own, st, pf, &err, &scratch));
       TLR_CHECK(reduce());
       TLR_CUDA(cudaMemcpyAsync(herr, err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
       TLR_CUDA(cudaStreamSynchronize(st));
@@ -1492,9 +1499,11 @@ int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, co
     if (herr[0])
       return fail(TLRMVN_E_TIMEOUT, "tensor-core kernel gave up waiting (code " + std::to_string(herr[0]) + ")");
     if (!herr[1]) return pf.collect();
-    // float32, limits tens of thousands of standard deviations out
+    // limits tens of thousands of standard deviations out: the general float32 path (FP16-shift: in the same scratch)
+    tlrmvn_opts og = o;
+    if (o.precision == TLRMVN_FP16_SHIFT) og.sample_chunk = std::max<int64_t>(256, scratch / simt_sample_bytes(F) / 256 * 256);
     TLR_CHECK(ensure_copies(F, TLRMVN_FP32 + SIMT_COPIES, st));
-    TLR_CHECK((run_chunks<float, float>(F, (const float*)nullptr, F.U32, F.V32, L, nu, o, tu, dD, logP, sc, st, pf)));
+    TLR_CHECK((run_chunks<float, float>(F, (const float*)nullptr, F.U32, F.V32, L, nu, og, tu, dD, logP, sc, st, pf)));
   } else {
     TLR_CHECK((run_chunks<double, double>(F, F.B, F.Ucat, F.Vcat, L, nu, o, tu, dD, logP, sc, st, pf)));
   }

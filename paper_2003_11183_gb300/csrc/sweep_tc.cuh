@@ -67,6 +67,8 @@ enum StcMode { STC_BF16 = 0, STC_FP16 = 1, STC_FP32 = 2 };
 constexpr int STC_SUB = 64;   // variables per sub-tile
 constexpr int STC_NS = 128;   // samples per CTA (TMEM lanes)
 constexpr int STC_KB = 32;    // K depth of a coupling k-block
+// The largest y and projection that the fp16 operands hold (STC_FP32: with a margin for the grid of its leading parts).
+__host__ __device__ constexpr float stc_range(int mode) { return mode == STC_FP32 ? 32768.0f : 65504.0f; }
 using StcCfg = tc::Cfg<64, true, false, STC_KB, 1>;
 using StcShiftCfg = tc::Cfg<64, false, true, 64, 1>;  // 16-bit shift k-block: W (MN-major) x U rows, 64 deep
 using StcProjCfg = tc::Cfg<64, false, false, 64, 1>;  // 16-bit projection k-block: y rows x V rows, 64 deep
@@ -136,7 +138,7 @@ struct SweepTcArgs {
   const float* rscale;    // STC_FP32: per variable of the tile, the inverse of its row's scale
   StcTile t;              // the tile (for the products)
   int wlo;                // STC_FP32: the lo parts' row offset in W
-  int* err;               // [0] a bounded wait's code; [1] (STC_FP32) a y or a projection beyond fp16's range
+  int* err;               // [0] a bounded wait's code; [1] (STC_FP32, STC_FP16) a y or a projection beyond fp16's range
 
   // from the arguments as of tile 0, variable 0 and column rank 0 to those of tile i of at most m variables
   __device__ void at(const StcTile& tile, int i, int m) {
@@ -676,14 +678,14 @@ __device__ __forceinline__ bool stc_tile(const SweepTcArgs& p, const StcCta& k, 
             const float y0 = __uint_as_float(r[j]), y1 = __uint_as_float(r[j + 1]);
             if constexpr (SPLIT) {
               split_f32(y0, y1, hi2[j / 2], lo2[j / 2]);
-              top = fmaxf(top, j < nb ? fmaxf(fabsf(y0), fabsf(y1)) : 0.0f);
             } else {
               float h0, h1, l0, l1;
               hi2[j / 2] = Op::pack(y0, y1, h0, h1);
               lo2[j / 2] = Op::pack(y0 - h0, y1 - h1, l0, l1);
             }
+            if (F16) top = max_nan(top, j < nb ? max_nan(fabsf(y0), fabsf(y1)) : 0.0f);
           }
-          if (SPLIT && top > 32768.0f) p.err[1] = 1;
+          if (F16 && !(top <= stc_range(MODE))) p.err[1] = 1;
           if (nb == DIAG_VB) {
             uint4* dh = reinterpret_cast<uint4*>(row);
             uint4* dlo = reinterpret_cast<uint4*>(row + p.ys_lo);
@@ -752,7 +754,7 @@ __device__ __forceinline__ bool stc_tile(const SweepTcArgs& p, const StcCta& k, 
               const float w1 = (__uint_as_float(r[j + 1]) + __uint_as_float(l[j + 1])) * ws[r1 - rb];
               uint32_t hi, lo;
               split_f32(w0, w1, hi, lo);
-              top = fmaxf(top, fmaxf(fabsf(w0), two ? fabsf(w1) : 0.0f));
+              top = max_nan(top, max_nan(fabsf(w0), two ? fabsf(w1) : 0.0f));
               unsigned short* d0 = pl.wcol + (int64_t)vm[rr - rb] * p.ldw;
               d0[0] = (unsigned short)hi;
               d0[(int64_t)p.wlo * p.ldw] = (unsigned short)lo;
@@ -762,14 +764,18 @@ __device__ __forceinline__ bool stc_tile(const SweepTcArgs& p, const StcCta& k, 
                 d1[(int64_t)p.wlo * p.ldw] = (unsigned short)(lo >> 16);
               }
             }
-          if (top > 32768.0f) p.err[1] = 1;
+          if (!(top <= stc_range(MODE))) p.err[1] = 1;
         }
       } else if (act) {
+        float top = 0.0f;
 #pragma unroll
         for (int j = 0; j < 16; j++)
-          if (r0 + h + j < p.kc)
-            pl.wcol[(int64_t)vm[r0 - rb + h + j] * p.ldw] =
-                Op::one(F16 ? __uint_as_float(r[j]) * ws[r0 - rb + h + j] : __uint_as_float(r[j]));
+          if (r0 + h + j < p.kc) {
+            const float w = F16 ? __uint_as_float(r[j]) * ws[r0 - rb + h + j] : __uint_as_float(r[j]);
+            pl.wcol[(int64_t)vm[r0 - rb + h + j] * p.ldw] = Op::one(w);
+            if (F16) top = max_nan(top, fabsf(w));
+          }
+        if (F16 && !(top <= stc_range(MODE))) p.err[1] = 1;
       }
     }
     if (OV) stc_done<OV>(k, 0);
