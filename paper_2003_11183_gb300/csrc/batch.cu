@@ -776,7 +776,7 @@ static int batch_run(Batch& B, const double* const* a, const double* const* b, d
   int bad = 0, terr[2] = {0, 0};
   memcpy(&bad, B.h_out + 2 * B.count, sizeof(int));
   memcpy(terr, B.h_out + 2 * B.count + 1, 2 * sizeof(int));
-  if (bad || terr[0] || terr[1]) {  // (values of this run may not be finite, and a later run's padding would read them)
+  if (bad || terr[0] || terr[1]) {  // (fp16 values of this run may not be finite, and a later run's padding would read them)
     const int s = zero_buffers(B);
     if (s != TLRMVN_OK) {
       cudaSetDevice(cur);

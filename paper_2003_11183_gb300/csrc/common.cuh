@@ -331,6 +331,7 @@ __device__ __forceinline__ float ndtri_tail_f32(float lp) {
     const float den = fmaf(fmaf(1.2021132975e-01f, s, 7.3700164250e-01f), s, 1.0f);
     return -num / den;
   }
+  if (t > 1e6f) return -1.41421356f * t;  // (to 1e-11; the cubic below would overflow at 1e13)
   const float s = t - 5.0f;
   const float num =
       fmaf(fmaf(fmaf(1.7337203997e-02f, s, 4.2868294337e-01f), s, 3.0812263860e+00f), s, 6.6579051150e+00f);

@@ -67,8 +67,10 @@ enum StcMode { STC_BF16 = 0, STC_FP16 = 1, STC_FP32 = 2 };
 constexpr int STC_SUB = 64;   // variables per sub-tile
 constexpr int STC_NS = 128;   // samples per CTA (TMEM lanes)
 constexpr int STC_KB = 32;    // K depth of a coupling k-block
-// The largest y and projection that the fp16 operands hold (STC_FP32: with a margin for the grid of its leading parts).
-__host__ __device__ constexpr float stc_range(int mode) { return mode == STC_FP32 ? 32768.0f : 65504.0f; }
+// The largest y and projection that the operands hold (STC_FP32: with a margin for the grid of its leading parts).
+__host__ __device__ constexpr float stc_range(int mode) {
+  return mode == STC_FP32 ? 32768.0f : (mode == STC_FP16 ? 65504.0f : 3.38e38f);
+}
 using StcCfg = tc::Cfg<64, true, false, STC_KB, 1>;
 using StcShiftCfg = tc::Cfg<64, false, true, 64, 1>;  // 16-bit shift k-block: W (MN-major) x U rows, 64 deep
 using StcProjCfg = tc::Cfg<64, false, false, 64, 1>;  // 16-bit projection k-block: y rows x V rows, 64 deep
@@ -773,9 +775,19 @@ __device__ __forceinline__ bool stc_tile(const SweepTcArgs& p, const StcCta& k, 
           if (r0 + h + j < p.kc) {
             const float w = F16 ? __uint_as_float(r[j]) * ws[r0 - rb + h + j] : __uint_as_float(r[j]);
             pl.wcol[(int64_t)vm[r0 - rb + h + j] * p.ldw] = Op::one(w);
-            if (F16) top = max_nan(top, fabsf(w));
+            top = max_nan(top, fabsf(w));
           }
         if (F16 && !(top <= stc_range(MODE))) p.err[1] = 1;
+        if (!F16 && !(top <= stc_range(MODE))) {
+          // bf16: a NaN or an overflow makes the sample's log NaN, and W keeps finite values, for its padding rows
+          // meet zeros (a plan's blocks go from problem to problem: y is finite by itself, ndtri_tail_f32)
+          lsum = NAN;
+#pragma unroll 1
+          for (int j = 0; j < 16 && r0 + h + j < p.kc; j++) {
+            unsigned short* const w = pl.wcol + (int64_t)vm[r0 - rb + h + j] * p.ldw;
+            if ((*w & 0x7F80) == 0x7F80) *w = 0;
+          }
+        }
       }
     }
     if (OV) stc_done<OV>(k, 0);
