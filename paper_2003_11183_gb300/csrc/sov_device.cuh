@@ -7,28 +7,31 @@ namespace tlrmvn {
 
 // ---- Student-t scale (Algorithm 7): chi_nu^-1(w0)/sqrt(nu) ------------------------
 // Regularised incomplete gamma P(a,x) and Q(a,x) = 1 - P: power series below
-// x = a + 1, Legendre continued fraction (modified Lentz) above.
-__device__ inline void gamma_pq(double a, double x, double& P, double& Q) {
-  if (!(x > 0.0)) {
-    P = 0.0;
-    Q = 1.0;
-    return;
-  }
-  double lpref = a * log(x) - x - lgamma(a);
+// x = a + 1, Legendre continued fraction (modified Lentz) above; lga = log Gamma(a), x > 0.
+// Both need some 8.5 sqrt(a) terms near x = a.  f1: the derivative of P.
+__device__ inline void gamma_pq(double a, double lga, double x, double& P, double& Q, double& f1) {
+  // log of x^a e^-x / Gamma(a); for large a by Stirling's series around x = a, where the logs' rounding would count
+  const double u = (x - a) / a;
+  const double lpref = a > 1000.0 ? 0.5 * log(a * 0.15915494309189535) - (1.0 - 1.0 / (30.0 * a * a)) / (12.0 * a) -
+                                        a * (u - log1p(u))
+                                  : a * log(x) - x - lga;
+  const double pref = exp(lpref);
+  f1 = pref / x;
+  const int terms = 2000 + (int)fmin(10.0 * sqrt(a), 200000.0);
   if (x < a + 1.0) {
     double ap = a, term = 1.0 / a, sum = term;
-    for (int it = 0; it < 2000; it++) {
+    for (int it = 0; it < terms; it++) {
       ap += 1.0;
       term *= x / ap;
       sum += term;
       if (fabs(term) <= fabs(sum) * 1.2e-16) break;
     }
-    P = sum * exp(lpref);
+    P = sum * pref;
     Q = 1.0 - P;
   } else {
     const double tiny = 1e-300;
     double bq = x + 1.0 - a, c = 1.0 / tiny, d = 1.0 / bq, h = d;
-    for (int i = 1; i < 2000; i++) {
+    for (int i = 1; i < terms; i++) {
       double an = -i * (i - a);
       bq += 2.0;
       d = an * d + bq;
@@ -40,34 +43,38 @@ __device__ inline void gamma_pq(double a, double x, double& P, double& Q) {
       h *= del;
       if (fabs(del - 1.0) <= 4.5e-16) break;  // a few ulp: exact equality may never occur
     }
-    Q = exp(lpref) * h;
+    Q = pref * h;
     P = 1.0 - Q;
   }
 }
 
-// x with P(a, x) = p (q = 1 - p exactly): Wilson-Hilferty start, Halley steps.
+// x with P(a, x) = p (q = 1 - p exactly): Halley steps, kept between the points known to lie on either side of it.
+// Start: Wilson-Hilferty's cube, or, where its base is small and it lies far too low or is negative, the leading term of
+// the series, p = x^a / Gamma(a + 1), which never lies above x.
 __device__ inline double gamma_p_inv(double a, double p, double q) {
-  double z = ndtri2(p, q, log(p));
-  double t = 1.0 / (9.0 * a);
-  double base = 1.0 - t + z * sqrt(t);
-  double x = a * base * base * base;
-  if (!(x > 0.0)) x = exp((log(p) + lgamma(a + 1.0)) / a);
-  const double lga = lgamma(a);
+  const double z = ndtri2(p, q, log(p)), t = 1.0 / (9.0 * a), lga = lgamma(a);
+  const double base = 1.0 - t + z * sqrt(t);
+  double x = a * base * base * base, lo = 0.0, hi = INFINITY;
+  if (base < 0.5) {
+    const double x0 = exp((log(p) + lga + log(a)) / a);
+    x = fmax(x, x0);
+    lo = 0.999999 * x0;
+  }
+  if (!(x > 0.0)) return x;  // (below the smallest double)
   for (int it = 0; it < 100; it++) {
-    double P, Q;
-    gamma_pq(a, x, P, Q);
-    double f = (p < 0.5) ? (P - p) : (q - Q);
-    double f1 = exp((a - 1.0) * log(x) - x - lga);
-    if (!(f1 > 0.0)) break;
-    double dx = f / f1;
-    double h2 = (a - 1.0) / x - 1.0;
-    double corr = 0.5 * dx * h2;
-    double step = (fabs(corr) < 0.5) ? dx / (1.0 - corr) : dx;
+    double P, Q, f1;
+    gamma_pq(a, lga, x, P, Q, f1);
+    const double f = (p < 0.5) ? (P - p) : (q - Q);
+    if (f < 0.0) lo = x;
+    else hi = x;
+    const double dx = f / f1;
+    const double corr = 0.5 * dx * ((a - 1.0) / x - 1.0);
+    const double step = (fabs(corr) < 0.5) ? dx / (1.0 - corr) : dx;
     double xn = x - step;
-    if (!(xn > 0.0)) xn = 0.5 * x;
     // Halley converges cubically: once a step is below 1e-12 x the next iterate
     // is exact to rounding, so stop there instead of chasing the last ulp
     const bool done = fabs(xn - x) <= 1e-12 * x;
+    if (!done && !(xn > lo && xn < hi)) xn = hi < INFINITY ? 0.5 * (lo + hi) : 2.0 * x;  // (also where f1 underflows)
     x = xn;
     if (done) break;
   }
