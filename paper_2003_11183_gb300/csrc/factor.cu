@@ -445,7 +445,8 @@ __global__ void __launch_bounds__(256) k_potrf_inv64(double* A, int nb, int ld, 
   for (int k = 0; k < nb; k++) {
     if (tid < 32) {
       const double d = L[k * P64_LD + k];
-      const double rs = rsqrt(d), l0 = d * rs, l = fma(fma(-l0, l0, d), 0.5 * rs, l0);
+      // (an infinite pivot has an infinite root and, divided by it, a column of zeros)
+      const double rs = rsqrt(d), l0 = d * rs, l = d < INFINITY ? fma(fma(-l0, l0, d), 0.5 * rs, l0) : d;
       if (tid == 0) {
         if (!(d > 0.0)) atomicExch(status, TLRMVN_E_NOT_SPD);
         diag[0] = l;
@@ -454,11 +455,11 @@ __global__ void __launch_bounds__(256) k_potrf_inv64(double* A, int nb, int ld, 
     }
     __syncthreads();
     const double l = diag[0], rs = diag[1];
-    if (!(rs > 0.0)) return;
+    if (!(rs >= 0.0)) return;
     const int rows = nb - 1 - k;  // below the pivot
     if (tid < rows) {
       const double x = L[(k + 1 + tid) * P64_LD + k], q = x * rs;
-      L[(k + 1 + tid) * P64_LD + k] = fma(fma(-q, l, x), rs, q);
+      L[(k + 1 + tid) * P64_LD + k] = rs > 0.0 ? fma(fma(-q, l, x), rs, q) : q;
     }
     if (tid == 128) {
       L[k * P64_LD + k] = l;
