@@ -146,7 +146,8 @@ __global__ void k_cov_tiles(const TileJob* jobs, CovSrc src, int m) {
 
 // ---- univariate conditioning (Trinh & Genz) of diagonal blocks --------------------------
 // One block per CTA; right-looking pivoted Cholesky of a copy of the block (its lower triangle packed in shared memory
-// when it fits there, SH, else in `work`).  Writes log of the estimate; with emit, also the pivot order and the
+// when it fits there, SH, else in `work`; TS: the tables in shared memory too, which tiles past 3,100 variables leave no
+// room for).  Writes log of the estimate; with emit, also the pivot order and the
 // truncated expectations in the new order.
 //
 // A step is a chain (probabilities of all remaining variables, their least, a square root, the column, the update), and
@@ -155,13 +156,13 @@ __global__ void k_cov_tiles(const TileJob* jobs, CovSrc src, int m) {
 // no log), the pivot's owner passes on its square root and probability, and while one warp works out the truncated
 // mean, which only the next step needs, the others update the triangle; the logs come at the end.  All conditionings of
 // n = 1,024 in tiles of 128: 15.6 -> 5.1 ms.
-template <bool SH>
+template <bool SH, bool TS>
 __global__ void __launch_bounds__(512) k_uc(const int* blist, const double* diagS, const int* bsize, int m,
                                             const double* acur, const double* bcur, double* work, double* logp_out,
                                             int emit, int* order_out, double* y_out, int* status, const double* tables) {
   extern __shared__ __align__(16) double shm[];
-  double* T = shm;
-  double* sa = T + T64_A * T64_W;
+  const double* T = TS ? shm : tables;
+  double* sa = shm + (TS ? T64_A * T64_W : 0);
   double* sb = sa + m;
   double* ss = sb + m;
   double* lcol = ss + m;
@@ -179,8 +180,9 @@ __global__ void __launch_bounds__(512) k_uc(const int* blist, const double* diag
   double* A = work + (SH ? (size_t)0 : (size_t)blockIdx.x * m * m);
   const double* S = diagS + (size_t)b * m * m;
   auto at_ = [&](int i, int j) -> double& { return SH ? tri[i * (i + 1) / 2 + j] : A[(size_t)i * m + j]; };
-  for (int t = tid; t < T64_A * T64_W / 2; t += blockDim.x)
-    reinterpret_cast<double2*>(T)[t] = reinterpret_cast<const double2*>(tables)[t];
+  if (TS)
+    for (int t = tid; t < T64_A * T64_W / 2; t += blockDim.x)
+      reinterpret_cast<double2*>(shm)[t] = reinterpret_cast<const double2*>(tables)[t];
   for (int i = wid; i < mb; i += nw)
     for (int j = lane; j <= i; j += 32) at_(i, j) = S[(size_t)i * m + j];
   for (int t = tid; t < mb; t += blockDim.x) {
@@ -332,16 +334,14 @@ static int launch_uc(int blocks, int m, cudaStream_t st, const int* blist, const
                      const double* a, const double* b, double* work, double* logp, int* order, double* y, int* status) {
   const double* tables = nullptr;
   TLR_CHECK(tables64(&tables, st));
-  const size_t base = ((size_t)T64_A * T64_W + 6 * (size_t)m) * sizeof(double) + (size_t)m * sizeof(int);
-  const size_t full = base + (size_t)m * (m + 1) / 2 * sizeof(double);
+  const size_t own = 6 * (size_t)m * sizeof(double) + (size_t)m * sizeof(int);
+  const size_t base = (size_t)T64_A * T64_W * sizeof(double) + own, full = base + (size_t)m * (m + 1) / 2 * sizeof(double);
   const int threads = m >= 256 ? 512 : 256;
-  if (full <= 200 * 1024) {
-    TLR_CHECK(raise_smem_limit((const void*)k_uc<true>, full));
-    k_uc<true><<<blocks, threads, full, st>>>(blist, diagS, bsize, m, a, b, work, logp, 1, order, y, status, tables);
-  } else {
-    TLR_CHECK(raise_smem_limit((const void*)k_uc<false>, base));
-    k_uc<false><<<blocks, threads, base, st>>>(blist, diagS, bsize, m, a, b, work, logp, 1, order, y, status, tables);
-  }
+  const size_t most = 200 * 1024;
+  const auto kernel = full <= most ? k_uc<true, true> : (base <= most ? k_uc<false, true> : k_uc<false, false>);
+  const size_t smem = full <= most ? full : (base <= most ? base : own);
+  TLR_CHECK(raise_smem_limit((const void*)kernel, smem));
+  kernel<<<blocks, threads, smem, st>>>(blist, diagS, bsize, m, a, b, work, logp, 1, order, y, status, tables);
   TLR_CUDA(cudaGetLastError());
   return TLRMVN_OK;
 }
