@@ -365,10 +365,11 @@ const char* tlrmvn_last_error(void);   /* thread-local detail of the last failur
 /* Exercises the bounded-wait path of the tensor-core kernels (no counterpart in
  * the paper): one thread waits `polls` times (1 .. 2^20) on an mbarrier that
  * nothing arrives at, then gives up and records a code, as those kernels do
- * when a copy or MMA never completes.  Returns TLRMVN_E_TIMEOUT when the wait
+ * when a copy or MMA never completes, and an estimate over a solve with that code
+ * must leave its outputs as they are.  Returns TLRMVN_E_TIMEOUT when the wait
  * gave up (the expected outcome; the CUDA context stays usable), TLRMVN_OK if
  * the barrier unexpectedly completed, TLRMVN_E_INVAL for polls out of range,
- * TLRMVN_E_CUDA on a launch failure.  stream: cudaStream_t or NULL. */
+ * TLRMVN_E_CUDA on a launch failure or when the outputs changed.  stream: cudaStream_t or NULL. */
 int tlrmvn_selftest_wait_timeout(int polls, void* stream);
 
 /* Evaluates, on the GPU, the float32 Phi(-x) that the float sweep uses for

@@ -223,7 +223,14 @@ __device__ void final_estimate(const double* ell, int M, double* logp, double* e
     *errp = (M > 1 && mx > -INFINITY) ? sqrt(sq / (M - 1) / M) / mean : NAN;
   }
 }
-__global__ void k_final(const double* ell, int M, double* logp, double* errp) { final_estimate(ell, M, logp, errp); }
+// err: flags of the integrand (SweepTcArgs::err) or null; where one is set the outputs stay as they are.  ell_out: null, or
+// where the per-shift logs go too.
+__global__ void k_final(const double* ell, int M, double* logp, double* errp, const int* err, double* ell_out) {
+  if (err && (err[0] || err[1])) return;
+  final_estimate(ell, M, logp, errp);
+  if (ell_out)
+    for (int s = threadIdx.x; s < M; s += blockDim.x) ell_out[s] = ell[s];
+}
 // one problem per block: ell + blockIdx.x * M -> out[2 * blockIdx.x], out[2 * blockIdx.x + 1]
 __global__ void k_final_batch(const double* ell, int M, double* out) {
   final_estimate(ell + (int64_t)blockIdx.x * M, M, out + 2 * blockIdx.x, out + 2 * blockIdx.x + 1);
@@ -1473,15 +1480,14 @@ int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, co
   TLR_CHECK(ensure_copies(F, o.precision, st));
   const Lims L{ap, bp, ap32, bp32, hbad[1] == 0};
   const Tuning tu = F.tuning(o.precision);
-  // the estimate of the samples' logs
-  auto reduce = [&]() -> int {
+  // the estimate of the samples' logs, unless a flag of err is set
+  auto reduce = [&](const int* err) -> int {
     pf.begin(TLRMVN_KC_REDUCE);
     k_shift_reduce<<<(unsigned)M, 256, 0, st>>>(logP, N, ell);
     pf.end();
     pf.begin(TLRMVN_KC_REDUCE);
-    k_final<<<1, 256, 0, st>>>(ell, (int)M, logp_dev, err_dev);
+    k_final<<<1, 256, 0, st>>>(ell, (int)M, logp_dev, err_dev, err, ell_dev_out);
     pf.end();
-    if (ell_dev_out) TLR_CUDA(cudaMemcpyAsync(ell_dev_out, ell, M * 8, cudaMemcpyDeviceToDevice, st));
     TLR_CUDA(cudaGetLastError());
     return TLRMVN_OK;
   };
@@ -1492,7 +1498,7 @@ int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, co
       Scratch own(st);
       int* err = nullptr;
       TLR_CHECK(run_chunks_tc(F, L, nu, o, tu, dD, logP, own, st, pf, &err, &scratch));
-      TLR_CHECK(reduce());
+      TLR_CHECK(reduce(err));
       TLR_CUDA(cudaMemcpyAsync(herr, err, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
       TLR_CUDA(cudaStreamSynchronize(st));
     }
@@ -1507,7 +1513,7 @@ int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, co
   } else {
     TLR_CHECK((run_chunks<double, double>(F, F.B, F.Ucat, F.Vcat, L, nu, o, tu, dD, logP, sc, st, pf)));
   }
-  TLR_CHECK(reduce());
+  TLR_CHECK(reduce(nullptr));
   TLR_CUDA(cudaStreamSynchronize(st));
   return pf.collect();
 }
@@ -1582,18 +1588,28 @@ extern "C" int tlrmvn_prob(tlrmvn_factor_t f, const double* a, const double* b, 
 extern "C" int tlrmvn_selftest_wait_timeout(int polls, void* stream) {
   if (polls < 1 || polls > (1 << 20)) return fail(TLRMVN_E_INVAL, "polls must be in [1, 2^20]");
   cudaStream_t st = pick_stream(stream);
+  // err[2], then a log mean and the three outputs of an estimate over it, as bytes 0xA5
+  constexpr size_t bytes = 2 * sizeof(int) + 4 * sizeof(double);
   int* err = nullptr;
-  TLR_CUDA(cudaMallocAsync((void**)&err, sizeof(int), st));
-  int herr = 0;
-  cudaError_t e = cudaMemsetAsync(err, 0, sizeof(int), st);
+  TLR_CUDA(cudaMallocAsync((void**)&err, bytes, st));
+  double* const out = reinterpret_cast<double*>(err + 2);
+  unsigned char h[bytes];
+  cudaError_t e = cudaMemsetAsync(out, 0xA5, 4 * sizeof(double), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, 2 * sizeof(int), st);
   if (e == cudaSuccess) {
     k_wait_selftest<<<1, 32, 0, st>>>(err, (uint32_t)polls);
+    k_final<<<1, 256, 0, st>>>(out, 1, out + 1, out + 2, err, out + 3);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(h, err, bytes, cudaMemcpyDeviceToHost, st);
   cudaFreeAsync(err, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e, "wait self-test");
+  int herr = 0;
+  memcpy(&herr, h, sizeof(int));
+  if (herr)
+    for (size_t i = 2 * sizeof(int); i < bytes; i++)
+      if (h[i] != 0xA5) return fail(TLRMVN_E_CUDA, "an estimate was written after a wait gave up");
   if (herr) return fail(TLRMVN_E_TIMEOUT, "wait self-test gave up after " + std::to_string(polls) + " polls (code " +
                                               std::to_string(herr) + ")");
   return TLRMVN_OK;
