@@ -439,9 +439,9 @@ __global__ void __launch_bounds__(256) k_scale_rows(const double* B, const doubl
     rscale[row] = (float)(1.0 / s);
   }
 }
-// hi (a multiple of 2^-10), lo or third fp16 part of x, |x| <= 1
+// hi (a multiple of 2^-7), lo or third fp16 part of x, |x| <= 1
 __device__ __forceinline__ __half split_part(double x, int h) {
-  const __half hi = __double2half(rint(x * 1024.0) * 0.0009765625);
+  const __half hi = __double2half(rint(x * 128.0) * 0.0078125);
   if (h == 0) return hi;
   const double r = x - (double)__half2float(hi);
   const __half lo = __double2half(r);

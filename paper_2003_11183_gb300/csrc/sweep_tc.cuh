@@ -54,13 +54,19 @@ namespace tlrmvn {
 //                       itself, always towards zero (ten times the error of float32 FMAs).  So the factor's operands
 //                       are scaled by powers of two into [-1, 1] (each row of U and of the tile's part left of the
 //                       sub-tile, each row of V) and the projections to order 1, and hi parts are rounded to multiples
-//                       of 2^-10: the products hi*hi are multiples of 2^-20 and their sums, below 16, exact; the
-//                       other products (hi*lo, lo*hi, lo*lo), 2^-10 of those, have an accumulator of their own (128
-//                       TMEM columns).  The factor's operands have a third part, and hi*third is added there: their
-//                       rounding to two parts, the same for all samples, was the largest error left.  Errors of
-//                       the samples' logs against 64 bits (rms; float32 FMAs before in brackets): n = 8,192, tiles
-//                       of 256: 1.9e-5 (2.7e-5); n = 1,024, tiles of 128, nu = 7: 4.5e-6 (6.3e-6); n = 2,048, tiles
-//                       of 512: 1.0e-5 (1.3e-5).  Times against the float32 FMA products and sweeps: n = 16,384, 20
+//                       of 2^-7 (the factor's) and 2^-11 (y, projections): the products hi*hi are multiples of 2^-18
+//                       and their sums, below 64, exact; the other products (hi*lo, lo*hi, lo*lo), 2^-7 of those,
+//                       have an accumulator of their own (128 TMEM columns).  The factor's operands have a third
+//                       part, and hi*third is added there: their rounding to two parts, the same for all samples, was
+//                       the largest error left, and the third part lets their grid be coarse.  With 2^-10 for
+//                       both, sums were exact below 16 only, and rows of many equal entries pass that: the mean error of
+//                       the samples' logs, as a share of them, 1.8e-7 at n = 512, b = -1, all entries 0.05 (now
+//                       7e-9; float32 FMAs 4.5e-8), 1.8e-7 at n = 2,048, b = -3, positive random entries (6e-9; 5e-9).
+//                       Errors of the samples' logs against 64 bits (rms; float32 FMAs in brackets): n = 2,000 points,
+//                       tiles of 256, exponential kernel of range 0.1, b = -2: 9.8e-6 (1.5e-5), b = 1: 2.3e-6 (3.8e-6);
+//                       range 0.5, b = 0: 5.9e-6 (6.2e-6); range 3, b = 0: 1.0e-5 (7.9e-6), b = 3: 1.3e-6 (2.4e-6).
+//                       y is held to 23 bits, so sums that a few y tens of standard deviations out make up are
+//                       less exact: all entries 0.05, b = -20: 1.8e-3 of 4,320 (4.6e-4).  Times against the float32 FMA products and sweeps: n = 16,384, 20
 //                       x 5,000 samples: 55.0 -> 25.9 ms a solve; n = 4,096, nu = 7, 10 x 1,000: 4.41 -> 2.35 ms; 64
 //                       batched problems, 10 x 2,000: 87.9 -> 18.8 ms.
 enum StcMode { STC_BF16 = 0, STC_FP16 = 1, STC_FP32 = 2 };
@@ -103,10 +109,10 @@ struct Op16<true> {
   static __device__ __forceinline__ unsigned short one(float a) { return __half_as_ushort(__float2half_rn(a)); }
 };
 
-// hi and lo fp16 parts of two floats for STC_FP32, packed low word first: hi a multiple of 2^-10 (of more above 2)
+// hi and lo fp16 parts of two floats for STC_FP32, packed low word first: hi a multiple of 2^-11 (of more above 1)
 __device__ __forceinline__ void split_f32(float a, float b, uint32_t& hi, uint32_t& lo) {
   float ha, hb, la, lb;
-  hi = Op16<true>::pack((a + 12288.0f) - 12288.0f, (b + 12288.0f) - 12288.0f, ha, hb);
+  hi = Op16<true>::pack((a + 6144.0f) - 6144.0f, (b + 6144.0f) - 6144.0f, ha, hb);
   lo = Op16<true>::pack(a - ha, b - hb, la, lb);
 }
 
