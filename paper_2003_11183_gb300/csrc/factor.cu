@@ -273,8 +273,9 @@ __global__ void __launch_bounds__(512) k_uc(const int* blist, const double* diag
         const double at = sha, bt = shb, p = shp;
         double y = 0.0;
         if (p > 0.0) {
-          const double ea = fabs(at) <= 13.0 ? t64_density(T, fabs(at)) : 0.0;
-          const double eb = fabs(bt) <= 13.0 ? t64_density(T, fabs(bt)) : 0.0;
+          // (densities to the last bits, and one exp for a one-sided limit)
+          const double ea = fabs(at) < INFINITY ? exp(-0.5 * at * at - TLR_LOG_SQRT2PI) : 0.0;
+          const double eb = fabs(bt) < INFINITY ? exp(-0.5 * bt * bt - TLR_LOG_SQRT2PI) : 0.0;
           // (1 / p by Newton from float32: p >= 1e-37; fewer dependent steps than a division)
           double ri = (double)(1.0f / (float)p);
           ri = fma(fma(-p, ri, 1.0), ri, ri);

@@ -209,16 +209,6 @@ __device__ __forceinline__ double t64_phi_wide(const double* T, double x) {
   const double hi = fma(e[8], d4, fma(f, d2, c));
   return fma(hi, d4, fma(b, d2, a));
 }
-// phi(x) for 0 <= x <= 13: minus the derivative of the same polynomial (to about 1e-13)
-__device__ __forceinline__ double t64_density(const double* T, double x) {
-  const double big = 105553116266496.0;
-  const double s = x + big, d = x - (s - big);
-  const double* e = T + (__double2loint(s) & 1023) * T64_W;
-  const double d2 = d * d, d4 = d2 * d2;
-  const double a = fma(2.0 * e[2], d, e[1]), b = fma(4.0 * e[4], d, 3.0 * e[3]);
-  const double c = fma(6.0 * e[6], d, 5.0 * e[5]), f = fma(8.0 * e[8], d, 7.0 * e[7]);
-  return -fma(fma(f, d2, c), d4, fma(b, d2, a));
-}
 // Phi^-1(p) for 2^-41 <= p <= 1/2
 __device__ __forceinline__ double t64_ndtri(const double* T, double p) {
   const int hi = min(__double2hiint(p), 0x3FDFFFFF);  // (1/2 itself: the end of the last interval)
