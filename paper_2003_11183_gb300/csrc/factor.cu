@@ -990,9 +990,12 @@ static void kd_order(const double* xy, int64_t n, int m, std::vector<int64_t>& p
   split(0, n);
 }
 
-// Device buffers of one factorisation; freed on every exit path.
+// Device buffers of one factorisation; freed on every exit path.  kept: the host lists of copies that the stream may not
+// have got to yet, until a status is read (a copy from pageable memory need not be staged before the call returns where
+// the GPU reads host memory through the host's page tables).
 struct Build {
   std::vector<void*> ptrs;
+  std::vector<std::vector<char>> kept;
   template <typename T>
   int get(T** p, size_t count) {
     TLR_CHECK(dalloc(p, std::max<size_t>(count, 1)));
@@ -1005,16 +1008,19 @@ struct Build {
 };
 
 template <typename T>
-static int upload(T* dst, const std::vector<T>& src, cudaStream_t st) {
+static int upload(T* dst, const std::vector<T>& src, Build& bd, cudaStream_t st) {
   if (src.empty()) return TLRMVN_OK;
-  TLR_CUDA(cudaMemcpyAsync(dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, st));
+  const char* p = reinterpret_cast<const char*>(src.data());
+  bd.kept.emplace_back(p, p + src.size() * sizeof(T));
+  TLR_CUDA(cudaMemcpyAsync(dst, bd.kept.back().data(), src.size() * sizeof(T), cudaMemcpyHostToDevice, st));
   return TLRMVN_OK;
 }
 
-static int check_status(int* d_status, cudaStream_t st, const char* what) {
+static int check_status(int* d_status, Build& bd, cudaStream_t st, const char* what) {
   int h = 0;
   TLR_CUDA(cudaMemcpyAsync(&h, d_status, sizeof(int), cudaMemcpyDeviceToHost, st));
   TLR_CUDA(cudaStreamSynchronize(st));
+  bd.kept.clear();
   if (h) return fail(h, std::string(what) + ": covariance block is not positive definite");
   return TLRMVN_OK;
 }
@@ -1048,7 +1054,7 @@ static int gemm_batched_groups(const std::vector<GemmEntry>& ent) {
 }
 template <bool TA, bool TB>
 static int run_batched(std::vector<GemmEntry>& ent, std::vector<GemmSeg>& seg, GemmEntry* d_ent, GemmSeg* d_seg,
-                       size_t ent_cap, size_t seg_cap, cudaStream_t st) {
+                       size_t ent_cap, size_t seg_cap, Build& bd, cudaStream_t st) {
   if (ent.empty()) return TLRMVN_OK;
   if (ent.size() > ent_cap || seg.size() > seg_cap) return fail(TLRMVN_E_CUDA, "internal: gemm job list overflow");
   int maxM = 0, maxN = 0;
@@ -1056,8 +1062,8 @@ static int run_batched(std::vector<GemmEntry>& ent, std::vector<GemmSeg>& seg, G
     maxM = std::max(maxM, e.M);
     maxN = std::max(maxN, e.N);
   }
-  TLR_CHECK(upload(d_ent, ent, st));
-  TLR_CHECK(upload(d_seg, seg, st));
+  TLR_CHECK(upload(d_ent, ent, bd, st));
+  TLR_CHECK(upload(d_seg, seg, bd, st));
   const int g = gemm_batched_groups(ent), bt = 16 * g;
   auto* k = g == 4 ? k_gemm_batched<TA, TB, 4> : (g == 2 ? k_gemm_batched<TA, TB, 2> : k_gemm_batched<TA, TB, 1>);
   for (size_t z0 = 0; z0 < ent.size(); z0 += 65535) {
@@ -1066,8 +1072,7 @@ static int run_batched(std::vector<GemmEntry>& ent, std::vector<GemmSeg>& seg, G
     k<<<grid, 256, 0, st>>>(d_ent + z0, d_seg);
   }
   TLR_CUDA(cudaGetLastError());
-  // (the host vectors may be reused: a copy from pageable memory returns once it has been staged; the device lists
-  // are overwritten by later uploads of the same stream only)
+  // (the device lists are overwritten by later uploads of the same stream only)
   return TLRMVN_OK;
 }
 
@@ -1078,7 +1083,7 @@ static int run_batched(std::vector<GemmEntry>& ent, std::vector<GemmSeg>& seg, G
 // block diagonal at a time, as GEMMs: X_ij = -X_ii sum_{j <= k < i} L_ik X_kj.  P (m x 64) is scratch.  (One CTA
 // for the whole block is bound by one SM's float64 rate: ~20 ms at m = 512.)
 static int chol_inverse(double* A, int mb, int m, double* Linv, double* P, GemmEntry* d_ent, GemmSeg* d_seg,
-                        size_t ent_cap, size_t seg_cap, int* d_status, cudaStream_t st, const char* what) {
+                        size_t ent_cap, size_t seg_cap, int* d_status, Build& bd, cudaStream_t st, const char* what) {
   std::vector<GemmEntry> ent;
   std::vector<GemmSeg> seg;
   TLR_CHECK(raise_smem_limit((const void*)k_potrf_inv64, P64_SMEM));
@@ -1095,12 +1100,12 @@ static int chol_inverse(double* A, int mb, int m, double* Linv, double* P, GemmE
     seg.clear();
     seg.push_back(GemmSeg{Apan, Xkk, m, m, nb});  // P = A_21 L_11^-T
     ent.push_back(GemmEntry{P, 64, rest, nb, 0, 1, 1.0, 0.0});
-    TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+    TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
     ent.clear();
     seg.clear();
     seg.push_back(GemmSeg{P, P, 64, 64, nb});  // A_22 -= P P^T (the lower triangle)
     ent.push_back(GemmEntry{A + (size_t)(k0 + nb) * m + k0 + nb, m, rest, rest, 0, 1, -1.0, 1.0, GEMM_LOWER});
-    TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+    TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
     TLR_CUDA(cudaMemcpy2DAsync(Apan, (size_t)m * sizeof(double), P, 64 * sizeof(double), (size_t)nb * sizeof(double),
                                (size_t)rest, cudaMemcpyDeviceToDevice, st));
   }
@@ -1115,7 +1120,7 @@ static int chol_inverse(double* A, int mb, int m, double* Linv, double* P, GemmE
       seg.push_back(GemmSeg{A + (size_t)64 * i * m + 64 * j, Linv + (size_t)64 * j * m + 64 * j, m, m, 64 * d});
       ent.push_back(GemmEntry{P + (size_t)64 * i * 64, 64, ni, 64, (int)seg.size() - 1, (int)seg.size(), 1.0, 0.0});
     }
-    TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+    TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
     ent.clear();
     seg.clear();
     for (int i = d; i < nblk; i++) {
@@ -1123,9 +1128,9 @@ static int chol_inverse(double* A, int mb, int m, double* Linv, double* P, GemmE
       seg.push_back(GemmSeg{Linv + (size_t)64 * i * m + 64 * i, P + (size_t)64 * i * 64, m, 64, ni});
       ent.push_back(GemmEntry{Linv + (size_t)64 * i * m + 64 * j, m, ni, 64, (int)seg.size() - 1, (int)seg.size(), -1.0, 0.0});
     }
-    TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+    TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
   }
-  return check_status(d_status, st, what);
+  return check_status(d_status, bd, st, what);
 }
 
 static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, std::vector<int> sizes,
@@ -1202,8 +1207,8 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
   TLR_CHECK(bd.get(&d_pmj, (size_t)r));
   TLR_CHECK(bd.get(&d_cj, (size_t)r));
   TLR_CHECK(bd.get(&d_pj, std::max<size_t>(npairs, 1)));
-  TLR_CHECK(upload(d_idx, idx_h, st));
-  TLR_CHECK(upload(d_bsize, sizes, st));
+  TLR_CHECK(upload(d_idx, idx_h, bd, st));
+  TLR_CHECK(upload(d_bsize, sizes, bd, st));
   TLR_CUDA(cudaMemsetAsync(d_status, 0, sizeof(int), st));
   TLR_CUDA(cudaMemsetAsync(d_capped, 0, sizeof(int), st));
   if (reorder) {
@@ -1213,15 +1218,15 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
         ah[(size_t)b * m + t] = a_ref[idx_h[(size_t)b * m + t]];
         bh[(size_t)b * m + t] = b_ref[idx_h[(size_t)b * m + t]];
       }
-    TLR_CHECK(upload(d_a, ah, st));
-    TLR_CHECK(upload(d_b, bh, st));
+    TLR_CHECK(upload(d_a, ah, bd, st));
+    TLR_CHECK(upload(d_b, bh, bd, st));
   }
   // diagonal blocks of Sigma
   {
     std::vector<TileJob> tj(r);
     for (int b = 0; b < r; b++)
       tj[b] = TileJob{diagS + (size_t)b * m * m, d_idx + (size_t)b * m, d_idx + (size_t)b * m, sizes[b], sizes[b]};
-    TLR_CHECK(upload(d_tj, tj, st));
+    TLR_CHECK(upload(d_tj, tj, bd, st));
     k_cov_tiles<<<dim3(std::max(1, (m * m + 255) / 256 / 4), r), 256, 0, st>>>(d_tj, src, m);
     TLR_CUDA(cudaGetLastError());
   }
@@ -1232,9 +1237,9 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
     // Algorithm 4: one UC estimate per original block, then a selection sort
     std::vector<int> bl(r);
     std::iota(bl.begin(), bl.end(), 0);
-    TLR_CHECK(upload(d_blist, bl, st));
+    TLR_CHECK(upload(d_blist, bl, bd, st));
     TLR_CHECK(launch_uc(r, m, st, d_blist, diagS, d_bsize, d_a, d_b, work, d_logp, d_order, d_y, d_status));
-    TLR_CHECK(check_status(d_status, st, "block reordering"));
+    TLR_CHECK(check_status(d_status, bd, st, "block reordering"));
     // within-block order: the UC pivot order of each original block
     for (int b = 0; b < r; b++) {
       TLR_CHECK(permute_block(diagS + (size_t)b * m * m, ptmp, d_idx + (size_t)b * m, d_a + (size_t)b * m,
@@ -1280,7 +1285,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
       std::vector<AcaJob> aj(jobs.size());
       for (size_t t = 0; t < jobs.size(); t++)
         aj[t] = AcaJob{Sij + t * m * m, Uslot((int)jobs[t].s), Vslot((int)jobs[t].s), jobs[t].mi, jobs[t].mj};
-      TLR_CHECK(upload(d_aj, aj, st));
+      TLR_CHECK(upload(d_aj, aj, bd, st));
       TLR_CHECK(launch_aca((int)aj.size(), m, cap, o.tol, st, d_aj, d_ranks, d_capped));
       std::vector<int> got(jobs.size());
       TLR_CUDA(cudaMemcpyAsync(got.data(), d_ranks, got.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1297,7 +1302,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
       std::vector<Trunc> jobs;
       auto flush = [&]() -> int {
         if (tj.empty()) return TLRMVN_OK;
-        TLR_CHECK(upload(d_tj, tj, st));
+        TLR_CHECK(upload(d_tj, tj, bd, st));
         k_cov_tiles<<<dim3(std::max(1, (m * m + 255) / 256 / 4), (unsigned)tj.size()), 256, 0, st>>>(d_tj, src, m);
         TLR_CUDA(cudaGetLastError());
         TLR_CHECK(truncate(jobs));
@@ -1318,10 +1323,10 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
       if (o.reorder == TLRMVN_REORDER_ITERATIVE) {
         // -- lines 4-8: UC of every remaining block; the smallest estimate takes position j
         std::vector<int> bl(pos2blk.begin() + j, pos2blk.end());
-        TLR_CHECK(upload(d_blist, bl, st));
+        TLR_CHECK(upload(d_blist, bl, bd, st));
         TLR_CHECK(launch_uc((int)bl.size(), m, st, d_blist, diagS, d_bsize, d_a, d_b, work, d_logp, d_order, d_y,
                             d_status));
-        TLR_CHECK(check_status(d_status, st, "iterative block reordering"));
+        TLR_CHECK(check_status(d_status, bd, st, "iterative block reordering"));
         std::vector<double> p(bl.size());
         TLR_CUDA(cudaMemcpyAsync(p.data(), d_logp, p.size() * 8, cudaMemcpyDeviceToHost, st));
         TLR_CUDA(cudaStreamSynchronize(st));
@@ -1343,7 +1348,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
           if (rk[s]) pj.push_back(PermJob{side(s, c), rk[s]});
         }
         if (!pj.empty()) {
-          TLR_CHECK(upload(d_pmj, pj, st));
+          TLR_CHECK(upload(d_pmj, pj, bd, st));
           k_permute_rows<<<(unsigned)pj.size(), 256, 0, st>>>(d_pmj, ord, sizes[c], cap);
           TLR_CUDA(cudaGetLastError());
         }
@@ -1352,7 +1357,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
       const int cj = pos2blk[j], mj = sizes[cj];
       double* Sjj = diagS + (size_t)cj * m * m;
       // -- line 10: L_jj and its inverse
-      TLR_CHECK(chol_inverse(Sjj, mj, m, Linv, Pch, d_ent, d_seg, ent_cap, seg_cap, d_status, st,
+      TLR_CHECK(chol_inverse(Sjj, mj, m, Linv, Pch, d_ent, d_seg, ent_cap, seg_cap, d_status, bd, st,
                              "diagonal Cholesky"));
       if (j == r - 1) break;
       // -- line 12: L_ij = Sigma_ij (.) Sigma_jj^-T = U (L_jj^-1 V)^T, truncated; in batches
@@ -1369,7 +1374,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             seg.push_back(GemmSeg{Linv, side(s, cj), m, cap, mj});
             ent.push_back(GemmEntry{Ys + t * m * cap, cap, mj, rk[s], (int)t, (int)t + 1, 1.0, 0.0});
           }
-          TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
           ent.clear();
           seg.clear();
           std::vector<Trunc> jobs;
@@ -1380,7 +1385,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             ent.push_back(GemmEntry{Sij + t * m * m, m, sizes[ci], mj, (int)t, (int)t + 1, 1.0, 0.0});
             jobs.push_back(Trunc{s, ci, sizes[ci], mj});
           }
-          TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
           TLR_CHECK(truncate(jobs));
         }
       }
@@ -1395,7 +1400,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
                                     mj, rk[s]});
         }
         if (!cj_jobs.empty()) {
-          TLR_CHECK(upload(d_cj, cj_jobs, st));
+          TLR_CHECK(upload(d_cj, cj_jobs, bd, st));
           k_condition<<<(unsigned)cj_jobs.size(), 256, 0, st>>>(d_cj, d_y + (size_t)chosen * m, cap);
           TLR_CUDA(cudaGetLastError());
           TLR_CUDA(cudaStreamSynchronize(st));
@@ -1414,7 +1419,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             seg.push_back(GemmSeg{Vslot((int)s), Vslot((int)s), cap, cap, mj});
             ent.push_back(GemmEntry{Xs + t * cap * cap, rk[s], rk[s], rk[s], (int)t, (int)t + 1, 1.0, 0.0});
           }
-          TLR_CHECK((run_batched<true, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<true, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
           ent.clear();
           seg.clear();
           for (size_t t = 0; t < is.size(); t++) {
@@ -1423,7 +1428,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             seg.push_back(GemmSeg{Xs + t * cap * cap, Uslot((int)s), rk[s], cap, rk[s]});
             ent.push_back(GemmEntry{Ys + t * m * cap, m, rk[s], sizes[ci], (int)t, (int)t + 1, 1.0, 0.0});
           }
-          TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
           ent.clear();
           seg.clear();
           for (size_t t = 0; t < is.size(); t++) {
@@ -1432,7 +1437,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             seg.push_back(GemmSeg{Uslot((int)s), Ys + t * m * cap, cap, m, rk[s]});
             ent.push_back(GemmEntry{diagS + (size_t)ci * m * m, m, sizes[ci], sizes[ci], (int)t, (int)t + 1, -1.0, 1.0});
           }
-          TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
         }
       }
       // -- lines 15-19, off-diagonal: Sigma_i1j1 (-) L_i1j L_j1j^T, truncated; in batches
@@ -1452,7 +1457,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             seg.push_back(GemmSeg{side(s1, cj), side(s2, cj), cap, cap, mj});
             ent.push_back(GemmEntry{Xs + t * cap * cap, rk[s2], rk[s1], rk[s2], (int)t, (int)t + 1, 1.0, 0.0});
           }
-          TLR_CHECK((run_batched<true, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<true, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
           ent.clear();
           seg.clear();
           for (size_t t = 0; t < nb; t++) {  // Z_t = -U_i1j X_t (mi1 x k2)
@@ -1461,7 +1466,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             seg.push_back(GemmSeg{side(s1, ci1), Xs + t * cap * cap, cap, rk[s2], rk[s1]});
             ent.push_back(GemmEntry{Ys + t * m * cap, cap, sizes[ci1], rk[s2], (int)t, (int)t + 1, -1.0, 0.0});
           }
-          TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
           ent.clear();
           seg.clear();
           std::vector<Trunc> jobs;
@@ -1474,7 +1479,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             ent.push_back(GemmEntry{Sij + t * m * m, m, sizes[ci1], sizes[cj1], g0, g0 + 2, 1.0, 0.0});
             jobs.push_back(Trunc{s, ci1, sizes[ci1], sizes[cj1]});
           }
-          TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
           TLR_CHECK(truncate(jobs));
         }
       }
@@ -1499,10 +1504,10 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
       int chosen = 0;
       if (o.reorder == TLRMVN_REORDER_ITERATIVE) {
         std::vector<int> bl(pos2blk.begin() + j, pos2blk.end());
-        TLR_CHECK(upload(d_blist, bl, st));
+        TLR_CHECK(upload(d_blist, bl, bd, st));
         TLR_CHECK(launch_uc((int)bl.size(), m, st, d_blist, diagS, d_bsize, d_a, d_b, work, d_logp, d_order, d_y,
                             d_status));
-        TLR_CHECK(check_status(d_status, st, "iterative block reordering"));
+        TLR_CHECK(check_status(d_status, bd, st, "iterative block reordering"));
         std::vector<double> p(bl.size());
         TLR_CUDA(cudaMemcpyAsync(p.data(), d_logp, p.size() * 8, cudaMemcpyDeviceToHost, st));
         TLR_CUDA(cudaStreamSynchronize(st));
@@ -1533,13 +1538,13 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
         for (int k = 0; k < j; k++)
           if (rank[(size_t)j * r + k] > 0) pj.push_back(PermJob{Uslot(slot[(size_t)j * r + k]), rank[(size_t)j * r + k]});
         if (!pj.empty()) {
-          TLR_CHECK(upload(d_pmj, pj, st));
+          TLR_CHECK(upload(d_pmj, pj, bd, st));
           k_permute_rows<<<(unsigned)pj.size(), 256, 0, st>>>(d_pmj, ord, mj, cap);
           TLR_CUDA(cudaGetLastError());
         }
       }
       // -- L_jj and its inverse
-      TLR_CHECK(chol_inverse(Sjj, mj, m, Linv, Pch, d_ent, d_seg, ent_cap, seg_cap, d_status, st,
+      TLR_CHECK(chol_inverse(Sjj, mj, m, Linv, Pch, d_ent, d_seg, ent_cap, seg_cap, d_status, bd, st,
                              "diagonal Cholesky"));
       const int nrem = r - 1 - j;
       if (nrem == 0) break;
@@ -1550,7 +1555,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
           int bi = pos2blk[j + 1 + q];
           tj[q] = TileJob{Sij + (size_t)q * m * m, d_idx + (size_t)bi * m, d_idx + (size_t)bj * m, sizes[bi], mj};
         }
-        TLR_CHECK(upload(d_tj, tj, st));
+        TLR_CHECK(upload(d_tj, tj, bd, st));
         k_cov_tiles<<<dim3(std::max(1, (m * m + 255) / 256 / 4), nrem), 256, 0, st>>>(d_tj, src, m);
         TLR_CUDA(cudaGetLastError());
         TLR_CUDA(cudaStreamSynchronize(st));
@@ -1585,7 +1590,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             seg.push_back(GemmSeg{Vslot(slot[(size_t)i * r + pr.k]), Vslot(slot[(size_t)j * r + pr.k]), cap, cap, mk});
             ent.push_back(GemmEntry{Xs + pr.xo, kjk, kik, kjk, (int)seg.size() - 1, (int)seg.size(), 1.0, 0.0});
           }
-          TLR_CHECK((run_batched<true, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<true, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
           ent.clear();
           seg.clear();
           for (auto& pr : pairs) {  // Y_ik = X_ik U_jk^T
@@ -1594,7 +1599,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             seg.push_back(GemmSeg{Xs + pr.xo, Uslot(slot[(size_t)j * r + pr.k]), kjk, cap, kjk});
             ent.push_back(GemmEntry{Ys + pr.yo, m, kik, mj, (int)seg.size() - 1, (int)seg.size(), 1.0, 0.0});
           }
-          TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
           ent.clear();
           seg.clear();
           size_t p0 = 0;
@@ -1609,7 +1614,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             if ((int)seg.size() > s0)
               ent.push_back(GemmEntry{Sij + (size_t)q * m * m, m, sizes[pos2blk[i]], mj, s0, (int)seg.size(), -1.0, 1.0});
           }
-          TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
         }
       }
       // -- L_ij = S_ij L_jj^-T
@@ -1620,7 +1625,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
         seg.push_back(GemmSeg{Sij + (size_t)q * m * m, Linv, m, m, mj});
         ent.push_back(GemmEntry{Lij + (size_t)q * m * m, m, mi, mj, q, q + 1, 1.0, 0.0, GEMM_KTRI});
       }
-      TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+      TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
       // -- ACA of every L_ij into fresh slots
       {
         std::vector<AcaJob> aj(nrem);
@@ -1630,7 +1635,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
           slot[(size_t)i * r + j] = s;
           aj[q] = AcaJob{Lij + (size_t)q * m * m, Uslot(s), Vslot(s), sizes[pos2blk[i]], mj};
         }
-        TLR_CHECK(upload(d_aj, aj, st));
+        TLR_CHECK(upload(d_aj, aj, bd, st));
         TLR_CHECK(launch_aca(nrem, m, cap, o.tol, st, d_aj, d_ranks, d_capped));
         std::vector<int> rk(nrem);
         TLR_CUDA(cudaMemcpyAsync(rk.data(), d_ranks, nrem * sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -1647,7 +1652,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
           cj.push_back(CondJob{Uslot(s), Vslot(s), d_a + (size_t)bi * m, d_b + (size_t)bi * m, sizes[bi], mj, k});
         }
         if (!cj.empty()) {
-          TLR_CHECK(upload(d_cj, cj, st));
+          TLR_CHECK(upload(d_cj, cj, bd, st));
           k_condition<<<(unsigned)cj.size(), 256, 0, st>>>(d_cj, yj, cap);
           TLR_CUDA(cudaGetLastError());
           TLR_CUDA(cudaStreamSynchronize(st));
@@ -1675,7 +1680,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             seg.push_back(GemmSeg{Vslot(s), Vslot(s), cap, cap, mj});
             ent.push_back(GemmEntry{Xs + xof[t], k, k, k, (int)t, (int)t + 1, 1.0, 0.0});
           }
-          TLR_CHECK((run_batched<true, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<true, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
           ent.clear();
           seg.clear();
           for (size_t t = 0; t < qs.size(); t++) {
@@ -1684,7 +1689,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             seg.push_back(GemmSeg{Xs + xof[t], Uslot(s), k, cap, k});
             ent.push_back(GemmEntry{Ys + yof[t], m, k, mi, (int)t, (int)t + 1, 1.0, 0.0});
           }
-          TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
           ent.clear();
           seg.clear();
           for (size_t t = 0; t < qs.size(); t++) {
@@ -1693,7 +1698,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
             seg.push_back(GemmSeg{Uslot(s), Ys + yof[t], cap, m, k});
             ent.push_back(GemmEntry{diagS + (size_t)bi * m * m, m, mi, mi, (int)t, (int)t + 1, -1.0, 1.0});
           }
-          TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, st)));
+          TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, ent_cap, seg_cap, bd, st)));
         }
       }
     }
@@ -1731,7 +1736,7 @@ static int factor_build(const CovSrc& src, int64_t n, std::vector<int64_t> geo, 
       }
     }
     if (!pj.empty()) {
-      TLR_CHECK(upload(d_pj, pj, st));
+      TLR_CHECK(upload(d_pj, pj, bd, st));
       k_pack<<<(unsigned)pj.size(), 256, 0, st>>>(d_pj, m, cap);
       TLR_CUDA(cudaGetLastError());
     }
@@ -1835,11 +1840,11 @@ static int reorder_tiles(Factor& F, const double* a, const double* b, cudaStream
       hb[(size_t)j * m + v] = b[orig];
     }
   }
-  TLR_CHECK(upload(d_bsize, sizes, st));
-  TLR_CHECK(upload(d_blist, bl, st));
-  TLR_CHECK(upload(d_a, ha, st));
-  TLR_CHECK(upload(d_b, hb, st));
-  TLR_CHECK(upload(d_kro, F.krow_off, st));
+  TLR_CHECK(upload(d_bsize, sizes, bd, st));
+  TLR_CHECK(upload(d_blist, bl, bd, st));
+  TLR_CHECK(upload(d_a, ha, bd, st));
+  TLR_CHECK(upload(d_b, hb, bd, st));
+  TLR_CHECK(upload(d_kro, F.krow_off, bd, st));
   TLR_CUDA(cudaMemsetAsync(d_status, 0, sizeof(int), st));
   std::vector<GemmEntry> ent;
   std::vector<GemmSeg> seg;
@@ -1849,11 +1854,11 @@ static int reorder_tiles(Factor& F, const double* a, const double* b, cudaStream
     ent.push_back(GemmEntry{S + j * mm, m, sizes[j], sizes[j], j, j + 1, 1.0, 0.0});
   }
   TLR_CUDA(cudaMemsetAsync(S, 0, r * mm * 8, st));
-  TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, (size_t)r, (size_t)r, st)));
+  TLR_CHECK((run_batched<false, true>(ent, seg, d_ent, d_seg, (size_t)r, (size_t)r, bd, st)));
   // P_j: the univariate-conditioning pivot order with the new limits
   TLR_CHECK(raise_smem_limit((const void*)k_potrf, m * sizeof(double)));
   TLR_CHECK(launch_uc(r, m, st, d_blist, S, d_bsize, d_a, d_b, work, d_logp, d_order, d_y, d_status));
-  TLR_CHECK(check_status(d_status, st, "within-tile reordering"));
+  TLR_CHECK(check_status(d_status, bd, st, "within-tile reordering"));
   // Lt_j = chol(P S_j P^T) (in work); X_j = P^T Lt_j; Binv_j = B_j^-1; Q_j = Binv_j X_j
   const unsigned gx = (unsigned)std::max<size_t>(1, std::min<size_t>(64, (mm + 255) / 256));
   k_gather_sym<<<dim3(gx, r), 256, 0, st>>>(S, d_order, d_bsize, m, work);
@@ -1863,7 +1868,7 @@ static int reorder_tiles(Factor& F, const double* a, const double* b, cudaStream
   k_trinv_cols<<<dim3((m + 7) / 8, r), 256, 8 * (size_t)m * sizeof(double), st>>>(F.B, m, mm, Binv, m, mm, 0, d_bsize,
                                                                                    m);
   TLR_CUDA(cudaGetLastError());
-  TLR_CHECK(check_status(d_status, st, "within-tile reordering (Cholesky)"));
+  TLR_CHECK(check_status(d_status, bd, st, "within-tile reordering (Cholesky)"));
   k_scatter_rows<<<dim3(gx, r), 256, 0, st>>>(work, d_order, d_bsize, m, X);
   ent.clear();
   seg.clear();
@@ -1872,7 +1877,7 @@ static int reorder_tiles(Factor& F, const double* a, const double* b, cudaStream
     ent.push_back(GemmEntry{Qm + j * mm, m, sizes[j], sizes[j], j, j + 1, 1.0, 0.0});
   }
   TLR_CUDA(cudaMemsetAsync(Qm, 0, r * mm * 8, st));
-  TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, (size_t)r, (size_t)r, st)));
+  TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, (size_t)r, (size_t)r, bd, st)));
   // the new factor: B_j = Lt_j; V^T rows of column block j times Q_j; rows of U permuted
   TLR_CUDA(cudaMemcpyAsync(G.B, work, r * mm * 8, cudaMemcpyDeviceToDevice, st));
   if (F.ktot > 0) {
@@ -1886,7 +1891,7 @@ static int reorder_tiles(Factor& F, const double* a, const double* b, cudaStream
       ent.push_back(GemmEntry{G.Vcat + (size_t)m * F.kcol_off[j], m, (int)kc, sizes[j], (int)seg.size() - 1,
                               (int)seg.size(), 1.0, 0.0});
     }
-    TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, (size_t)r, (size_t)r, st)));
+    TLR_CHECK((run_batched<false, false>(ent, seg, d_ent, d_seg, (size_t)r, (size_t)r, bd, st)));
     int64_t kmax = 0;
     for (int j = 0; j < r; j++) kmax = std::max(kmax, F.krow(j));
     const unsigned gu = (unsigned)std::max<int64_t>(1, std::min<int64_t>(256, ((int64_t)m * kmax + 255) / 256));
