@@ -44,8 +44,12 @@ static std::string tune_key(const Factor& F, int precision, int64_t S, bool mvt)
 static std::vector<Tuning> candidates(const Factor& F, int precision, int64_t S) {
   std::vector<Tuning> c;
   if (precision == TLRMVN_BF16_SHIFT || precision == TLRMVN_FP16_SHIFT) {
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, F.device);
     for (int ctas : {6, 4})
       for (int64_t chunk : {(int64_t)0, (S / 2 + 255) / 256 * 256}) {
+        // (a pass of at most two CTAs an SM takes the overlapped sweep, which the number does not reach)
+        if (ctas != 6 && ((chunk ? std::min(chunk, S) : S) + 127) / 128 <= 2 * (int64_t)sms) continue;
         Tuning t;
         t.tc_ctas = ctas;
         t.chunk = chunk;
