@@ -978,51 +978,44 @@ static int diag64_threads(int64_t C, int sms) {
   return 32 * best;
 }
 
-// Launch shape of the float sweep: samples per thread (spt) and per block (ns).
+// Threads per block of the general float sweep, a sample each.
 // Each sample's chain of special functions is latency-bound, so a launch takes
 // (waves) x (time of one block) and a second wave for a few leftover blocks
 // nearly doubles it.  Unless the factor's tuning fixes the block size, this
 // takes, among blocks of 2 to 8 warps, the fewest waves over C samples
 // (occupancy from the CUDA occupancy calculator, which accounts for registers
 // and shared memory), and among those the one nearest 128 samples per block.
-// One sample per thread (two per thread, k_diag_f32<2, .>, measured slower).
-struct SweepShape {
-  int spt, threads, ns;
-};
 typedef void (*SweepKernel)(DiagArgs32);
 static SweepKernel sweep_kernel(int flags) {
-  static const SweepKernel table[8] = {k_diag_f32<1, 0>, k_diag_f32<1, 1>, k_diag_f32<1, 2>, k_diag_f32<1, 3>,
-                                       k_diag_f32<1, 4>, k_diag_f32<1, 5>, k_diag_f32<1, 6>, k_diag_f32<1, 7>};
-  return table[flags & 7];
+  static const SweepKernel table[4] = {k_diag_f32<0>, k_diag_f32<1>, k_diag_f32<2>, k_diag_f32<3>};
+  return table[flags & 3];
 }
-static SweepShape sweep_shape(int64_t C, int mt, int forced) {
-  const int spt = 1;
-  if (forced >= 32 && forced <= 256 && forced % 32 == 0) return SweepShape{spt, forced, forced * spt};
+static int sweep_threads(int64_t C, int mt, int forced) {
+  if (forced >= 32 && forced <= 256 && forced % 32 == 0) return forced;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   // one-entry memo per thread: a solve asks for the same (C, mt) once per sub-tile
   thread_local int64_t memo_c = -1;
   thread_local int memo_mt = -1, memo_dev = -1;
-  thread_local SweepShape memo{1, 128, 128};
+  thread_local int memo = 128;
   if (memo_c == C && memo_mt == mt && memo_dev == dev) return memo;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  SweepShape best{spt, 128 / spt, 128};
+  int best = 128;
   int64_t best_waves = INT64_MAX;
-  for (int bd = 64 / spt; bd <= 256 / spt; bd += 32) {
-    const int ns = bd * spt;
+  for (int bd = 64; bd <= 256; bd += 32) {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_kernel(SWEEP_PERIODIZE | SWEEP_ONE_SIDED), bd,
-                                                      sweep_smem_bytes(mt, ns)) !=
+                                                      sweep_smem_bytes(mt, bd)) !=
             cudaSuccess ||
         per_sm < 1) {
       cudaGetLastError();
       continue;
     }
-    const int64_t blocks = (C + ns - 1) / ns, slots = (int64_t)per_sm * std::max(sms, 1);
+    const int64_t blocks = (C + bd - 1) / bd, slots = (int64_t)per_sm * std::max(sms, 1);
     const int64_t waves = (blocks + slots - 1) / slots;
-    if (waves < best_waves || (waves == best_waves && std::abs(ns - 128) < std::abs(best.ns - 128))) {
+    if (waves < best_waves || (waves == best_waves && std::abs(bd - 128) < std::abs(best - 128))) {
       best_waves = waves;
-      best = SweepShape{spt, bd, ns};
+      best = bd;
     }
   }
   memo_c = C;
@@ -1068,7 +1061,7 @@ static size_t sweep_tc_launch_smem(int ctas, int mode, bool ov) {
   return need;
 }
 static int set_sweep_smem(int sub) {
-  for (int flags = 0; flags < 8; flags++)
+  for (int flags = 0; flags < 4; flags++)
     TLR_CHECK(raise_smem_limit((const void*)sweep_kernel(flags), sweep_smem_bytes(sub, 256)));
   return TLRMVN_OK;
 }
@@ -1163,7 +1156,7 @@ static void sweep_tile_f32(const Factor& F, int i, bool has_shift, float* Dl, in
                            float* Yv, double* logP, const Tuning& tu, cudaStream_t st, Prof& pf) {
   const int m = F.m, mt = (int)F.tsize(i);
   const int sub = tu.sub;
-  const SweepShape sh = sweep_shape(Cc, std::min(mt, sub), tu.threads);
+  const int bd = sweep_threads(Cc, std::min(mt, sub), tu.threads);
   for (int q0 = 0; q0 < mt; q0 += sub) {
     const int mq = std::min(sub, mt - q0);
     if (q0 > 0) {
@@ -1195,14 +1188,10 @@ static void sweep_tile_f32(const Factor& F, int i, bool has_shift, float* Dl, in
     a.first = (i == 0 && q0 == 0);
     a.Yv = Yv + (size_t)q0 * C;
     a.ldyv = C;
-    a.Ys = nullptr;
-    a.ldys = 0;
-    a.ys_lo = 0;
     a.logP = logP;
     pf.begin(TLRMVN_KC_DIAG);
-    const int flags = (periodize ? SWEEP_PERIODIZE : 0) | SWEEP_YV | (L.one_sided ? SWEEP_ONE_SIDED : 0);
-    launch_pdl(sweep_kernel(flags), dim3((unsigned)blocks_for(Cc, sh.ns)), dim3(sh.threads), sweep_smem_bytes(mq, sh.ns), st,
-               a);
+    const int flags = (periodize ? SWEEP_PERIODIZE : 0) | (L.one_sided ? SWEEP_ONE_SIDED : 0);
+    launch_pdl(sweep_kernel(flags), dim3((unsigned)blocks_for(Cc, bd)), dim3(bd), sweep_smem_bytes(mq, bd), st, a);
     pf.end();
   }
 }

@@ -23,11 +23,8 @@ struct DiagArgs32 {
   const uint64_t* D;
   int64_t ldD, coord0, sample0, N, C;
   int periodize, first;
-  float* Yv;             // y variable-major, Yv[v * ldyv + c], or null
+  float* Yv;             // y variable-major, Yv[v * ldyv + c]
   int64_t ldyv;
-  __nv_bfloat16* Ys;     // y sample-major bf16, Ys[c * ldys + v], or null
-  int64_t ldys;
-  int64_t ys_lo;         // > 0: also the low part bf16(y - hi) at Ys[c * ldys + ys_lo + v]
   double* logP;
 };
 
@@ -61,29 +58,26 @@ __host__ __device__ inline size_t sweep_smem_bytes(int mt, int ns) {
 }
 
 // FLAGS, fixed for a launch: SWEEP_PERIODIZE (tent-periodised lattice),
-// SWEEP_YV (also write y as float to Yv), SWEEP_ONE_SIDED (every lower limit of
-// the problem is -inf: the one-sided step only).
-enum { SWEEP_PERIODIZE = 1, SWEEP_YV = 2, SWEEP_ONE_SIDED = 4 };
+// SWEEP_ONE_SIDED (every lower limit of the problem is -inf: the one-sided step only).
+enum { SWEEP_PERIODIZE = 1, SWEEP_ONE_SIDED = 2 };
 
-// SPT samples per thread (samples c0 + tid + s * blockDim.x): every broadcast
-// load of B and of the per-variable constants serves SPT chains, and the SPT
-// chains are independent instruction streams for the scheduler.  Each
-// variable's lattice offsets are loaded one variable ahead and its window
+// One sample per thread (two chains per thread measured slower).  Each
+// variable's lattice offset is loaded one variable ahead and its window
 // column before its special functions, and the block's limit shifts are added
 // after its sums over earlier variables, so that those loads are in flight
 // while other work runs.
-template <int SPT, int FLAGS>
+template <int FLAGS>
 __global__ void k_diag_f32(DiagArgs32 p) {
-  constexpr bool PER = FLAGS & SWEEP_PERIODIZE, YV = FLAGS & SWEEP_YV, ONE = FLAGS & SWEEP_ONE_SIDED;
+  constexpr bool PER = FLAGS & SWEEP_PERIODIZE, ONE = FLAGS & SWEEP_ONE_SIDED;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int bd = blockDim.x, tid = threadIdx.x, ns = SPT * bd, ld = ns + 1;
+  const int bd = blockDim.x, tid = threadIdx.x, ld = bd + 1;
   const int mt = p.mt;
   float* ys = reinterpret_cast<float*>(smem_raw);
   const int wbt = (mt + 15) & ~15;  // row length of the staged triangle
-  float* s_bt = reinterpret_cast<float*>(smem_raw + sweep_ys_bytes(mt, ns));
-  float4* s_abi = reinterpret_cast<float4*>(smem_raw + sweep_ys_bytes(mt, ns) + sweep_bt_bytes(mt));
+  float* s_bt = reinterpret_cast<float*>(smem_raw + sweep_ys_bytes(mt, bd));
+  float4* s_abi = reinterpret_cast<float4*>(smem_raw + sweep_ys_bytes(mt, bd) + sweep_bt_bytes(mt));
   uint64_t* s_q = reinterpret_cast<uint64_t*>(s_abi + mt);
-  const int64_t c0 = (int64_t)blockIdx.x * ns;
+  const int64_t c0 = (int64_t)blockIdx.x * bd;
   pdl_trigger();
   // limits, diagonal, triangle and generators are not written by the preceding kernels
   for (int t = tid; t < mt; t += bd) {
@@ -105,96 +99,68 @@ __global__ void k_diag_f32(DiagArgs32 p) {
   }
   __syncthreads();
   pdl_wait();  // the limit shifts, y and log P of the preceding kernels
-  bool act[SPT];
-  int64_t cs[SPT];
-  uint32_t ks[SPT];  // lattice point index k = 1..N (N < 2^31)
-  const uint64_t* Ds[SPT];
-  float rs[SPT];
   // log P of the sub-tile = log(prod) + pe log 2 + lsum: prod is kept in [1, 2)
   // with its binary exponent in pe, so it neither underflows nor needs a log per variable
-  float prod[SPT], lsum[SPT];
-  int pe[SPT];
-#pragma unroll
-  for (int s = 0; s < SPT; s++) {
-    act[s] = c0 + tid + s * bd < p.C;
-    cs[s] = act[s] ? c0 + tid + s * bd : p.C - 1;  // inactive lanes shadow a valid sample, write nothing
-    const int64_t g = p.sample0 + cs[s];
-    const int64_t sh = g / p.N;
-    ks[s] = (uint32_t)(g - sh * p.N) + 1u;
-    Ds[s] = p.D + sh * p.ldD + p.coord0;
-    rs[s] = p.rs ? p.rs[cs[s]] : 1.0f;
-    prod[s] = 1.0f;
-    lsum[s] = 0.0f;
-    pe[s] = 0;
-  }
+  float prod = 1.0f, lsum = 0.0f;
+  int pe = 0;
+  const bool act = c0 + tid < p.C;
+  const int64_t cs = act ? c0 + tid : p.C - 1;  // inactive lanes shadow a valid sample, write nothing
+  const int64_t g = p.sample0 + cs, sh = g / p.N;
+  const uint32_t ks = (uint32_t)(g - sh * p.N) + 1u;  // lattice point index k = 1..N (N < 2^31)
+  const uint64_t* const Ds = p.D + sh * p.ldD + p.coord0;
+  const float rs = p.rs ? p.rs[cs] : 1.0f;
   for (int v0 = 0; v0 < mt; v0 += DIAG_VB) {
     const int nb = min(DIAG_VB, mt - v0);
-    // acc[s][i] = sums of the block's variables 2i (x) and 2i + 1 (y), as pairs for the
+    // acc[i] = sums of the block's variables 2i (x) and 2i + 1 (y), as pairs for the
     // paired float32 FMAs (each pair FMA rounds as two fmaf)
-    float2 acc[SPT][DIAG_VB / 2], dl[SPT][DIAG_VB / 2];
+    float2 acc[DIAG_VB / 2], dl[DIAG_VB / 2];
 #pragma unroll
-    for (int s = 0; s < SPT; s++)
-#pragma unroll
-      for (int j = 0; j < DIAG_VB / 2; j++) {
-        dl[s][j].x = (p.Delta && 2 * j < nb) ? p.Delta[(int64_t)(v0 + 2 * j) * p.ldd + cs[s]] : 0.0f;
-        dl[s][j].y = (p.Delta && 2 * j + 1 < nb) ? p.Delta[(int64_t)(v0 + 2 * j + 1) * p.ldd + cs[s]] : 0.0f;
-        acc[s][j] = make_float2(0.0f, 0.0f);
-      }
-    // lattice offsets of the block's first variable
-    uint64_t dnext[SPT];
-#pragma unroll
-    for (int s = 0; s < SPT; s++) dnext[s] = Ds[s][v0];
+    for (int j = 0; j < DIAG_VB / 2; j++) {
+      dl[j].x = (p.Delta && 2 * j < nb) ? p.Delta[(int64_t)(v0 + 2 * j) * p.ldd + cs] : 0.0f;
+      dl[j].y = (p.Delta && 2 * j + 1 < nb) ? p.Delta[(int64_t)(v0 + 2 * j + 1) * p.ldd + cs] : 0.0f;
+      acc[j] = make_float2(0.0f, 0.0f);
+    }
+    uint64_t dnext = Ds[v0];  // lattice offset of the block's first variable
     // sums over the sub-tile's earlier variables for the block's 16 variables
     const float* bcol = s_bt + v0;
 #pragma unroll 2
     for (int u = 0; u < v0; u++) {
-      float yu[SPT];
-#pragma unroll
-      for (int s = 0; s < SPT; s++) yu[s] = ys[u * ld + tid + s * bd];
+      const float yu = ys[u * ld + tid];
       const float4* b4 = reinterpret_cast<const float4*>(bcol + u * wbt);
       const float4 q[4] = {b4[0], b4[1], b4[2], b4[3]};
+      const float2 yy = make_float2(yu, yu);
 #pragma unroll
-      for (int s = 0; s < SPT; s++) {
-        const float2 yy = make_float2(yu[s], yu[s]);
-#pragma unroll
-        for (int h = 0; h < 4; h++) {
-          acc[s][2 * h] = __ffma2_rn(make_float2(q[h].x, q[h].y), yy, acc[s][2 * h]);
-          acc[s][2 * h + 1] = __ffma2_rn(make_float2(q[h].z, q[h].w), yy, acc[s][2 * h + 1]);
-        }
+      for (int h = 0; h < 4; h++) {
+        acc[2 * h] = __ffma2_rn(make_float2(q[h].x, q[h].y), yy, acc[2 * h]);
+        acc[2 * h + 1] = __ffma2_rn(make_float2(q[h].z, q[h].w), yy, acc[2 * h + 1]);
       }
     }
 #pragma unroll
-    for (int s = 0; s < SPT; s++)
-#pragma unroll
-      for (int j = 0; j < DIAG_VB / 2; j++) acc[s][j] = __fadd2_rn(acc[s][j], dl[s][j]);
-    // one variable of eq. 2 for each slot: sum[s] = its sum over the earlier variables
-    // and the shifts; returns its y (also stored for the later variables and blocks)
-    auto step = [&](int j, const float (&sum)[SPT], float (&y)[SPT]) {
+    for (int j = 0; j < DIAG_VB / 2; j++) acc[j] = __fadd2_rn(acc[j], dl[j]);
+    // one variable of eq. 2: sum = its sum over the earlier variables and the shifts; returns its y (also stored for
+    // the later variables and blocks)
+    auto step = [&](int j, float sum) -> float {
       const int v = v0 + j;
       const float4 abi = s_abi[v];
       const float av = abi.x, bv = abi.y, iv = abi.z;
-      const uint64_t qv = s_q[v];
-#pragma unroll
-      for (int s = 0; s < SPT; s++) {
-        const uint64_t dv = dnext[s];
-        dnext[s] = Ds[s][(j + 1 < nb) ? v + 1 : v];  // next variable's offset (the last one reloads its own)
-        const float bt = (bv * rs[s] - sum[s]) * iv;
-        float w, wc;
-        lattice_wf((uint64_t)ks[s] * qv + dv, PER ? 1 : 0, w, wc);
-        float f;
-        if (ONE) {
-          sov_step_f32_upper(bt, w, wc, f, lsum[s], y[s]);
-        } else {
-          const float at = (av * rs[s] - sum[s]) * iv;
-          sov_step_f32_prod(at, bt, w, wc, f, lsum[s], y[s]);
-        }
-        prod[s] *= f;  // prod in [1, 2) and f >= Phi(-12): a normal float
-        const int pb = __float_as_int(prod[s]);
-        pe[s] += (pb >> 23) - 127;
-        prod[s] = __int_as_float((pb & 0x007FFFFF) | 0x3F800000);
-        ys[v * ld + tid + s * bd] = y[s];
-        if (YV && act[s]) p.Yv[(int64_t)v * p.ldyv + cs[s]] = y[s];
+      const uint64_t qv = s_q[v], dv = dnext;
+      dnext = Ds[(j + 1 < nb) ? v + 1 : v];  // next variable's offset (the last one reloads its own)
+      const float bt = (bv * rs - sum) * iv;
+      float w, wc, f, y;
+      lattice_wf((uint64_t)ks * qv + dv, PER ? 1 : 0, w, wc);
+      if (ONE) {
+        sov_step_f32_upper(bt, w, wc, f, lsum, y);
+      } else {
+        const float at = (av * rs - sum) * iv;
+        sov_step_f32_prod(at, bt, w, wc, f, lsum, y);
       }
+      prod *= f;  // prod in [1, 2) and f >= 2.5e-19: a normal float
+      const int pb = __float_as_int(prod);
+      pe += (pb >> 23) - 127;
+      prod = __int_as_float((pb & 0x007FFFFF) | 0x3F800000);
+      ys[v * ld + tid] = y;
+      if (act) p.Yv[(int64_t)v * p.ldyv + cs] = y;
+      return y;
     };
     // the block's variables in pairs (v even, v + 1): after y_v the pair's second sum
     // takes B[v+1][v] y_v and the window moves two places, the later sums taking
@@ -207,61 +173,33 @@ __global__ void k_diag_f32(DiagArgs32 p) {
       const int v = v0 + j;
       const float4* b4 = reinterpret_cast<const float4*>(s_band + v * 16);
       const float4 q[4] = {b4[0], b4[1], b4[2], b4[3]};
-      float sum[SPT], y0[SPT];
-#pragma unroll
-      for (int s = 0; s < SPT; s++) sum[s] = acc[s][0].x;
-      step(j, sum, y0);
+      const float y0 = step(j, acc[0].x);
       if (j + 1 == nb) break;  // (a ragged block's last variable: the window is not needed)
       const float4* c4 = reinterpret_cast<const float4*>(s_band + (v + 1) * 16);
       const float4 r[4] = {c4[0], c4[1], c4[2], c4[3]};
+      const float sum = fmaf(q[3].z, y0, acc[0].y);
+      const float2 yy = make_float2(y0, y0);
 #pragma unroll
-      for (int s = 0; s < SPT; s++) {
-        sum[s] = fmaf(q[3].z, y0[s], acc[s][0].y);
-        const float2 yy = make_float2(y0[s], y0[s]);
-#pragma unroll
-        for (int h = 0; h < 3; h++) {
-          acc[s][2 * h] = __ffma2_rn(make_float2(q[h].x, q[h].y), yy, acc[s][2 * h + 1]);
-          acc[s][2 * h + 1] = __ffma2_rn(make_float2(q[h].z, q[h].w), yy, acc[s][2 * h + 2]);
-        }
-        acc[s][6] = __ffma2_rn(make_float2(q[3].x, q[3].y), yy, acc[s][7]);
-        acc[s][7] = make_float2(0.0f, 0.0f);
+      for (int h = 0; h < 3; h++) {
+        acc[2 * h] = __ffma2_rn(make_float2(q[h].x, q[h].y), yy, acc[2 * h + 1]);
+        acc[2 * h + 1] = __ffma2_rn(make_float2(q[h].z, q[h].w), yy, acc[2 * h + 2]);
       }
-      float y1[SPT];
-      step(j + 1, sum, y1);
+      acc[6] = __ffma2_rn(make_float2(q[3].x, q[3].y), yy, acc[7]);
+      acc[7] = make_float2(0.0f, 0.0f);
+      const float y1 = step(j + 1, sum);
+      const float2 zz = make_float2(y1, y1);
 #pragma unroll
-      for (int s = 0; s < SPT; s++) {
-        const float2 yy = make_float2(y1[s], y1[s]);
-#pragma unroll
-        for (int h = 0; h < 3; h++) {
-          acc[s][2 * h] = __ffma2_rn(make_float2(r[h].x, r[h].y), yy, acc[s][2 * h]);
-          acc[s][2 * h + 1] = __ffma2_rn(make_float2(r[h].z, r[h].w), yy, acc[s][2 * h + 1]);
-        }
-        acc[s][6] = __ffma2_rn(make_float2(r[3].x, r[3].y), yy, acc[s][6]);
+      for (int h = 0; h < 3; h++) {
+        acc[2 * h] = __ffma2_rn(make_float2(r[h].x, r[h].y), zz, acc[2 * h]);
+        acc[2 * h + 1] = __ffma2_rn(make_float2(r[h].z, r[h].w), zz, acc[2 * h + 1]);
       }
+      acc[6] = __ffma2_rn(make_float2(r[3].x, r[3].y), zz, acc[6]);
     }
   }
-#pragma unroll
-  for (int s = 0; s < SPT; s++) {
-    if (!act[s]) continue;
-    const int64_t g = p.sample0 + cs[s];
-    const double lp = (double)(logf(prod[s]) + lsum[s]) + (double)pe[s] * 0.69314718055994530942;
-    if (p.first) p.logP[g] = lp;
-    else p.logP[g] += lp;
-  }
-  if (p.Ys) {
-    __syncthreads();
-    const int nw = bd >> 5, warp = tid >> 5, lane = tid & 31;
-    for (int j = warp; j < ns; j += nw) {
-      if (c0 + j >= p.C) break;
-      __nv_bfloat16* row = p.Ys + (c0 + j) * p.ldys;
-      for (int v = lane; v < p.mt; v += 32) {
-        const float yv = ys[v * ld + j];
-        const __nv_bfloat16 hi = __float2bfloat16_rn(yv);
-        row[v] = hi;
-        if (p.ys_lo) row[p.ys_lo + v] = __float2bfloat16_rn(yv - __bfloat162float(hi));
-      }
-    }
-  }
+  if (!act) return;
+  const double lp = (double)(logf(prod) + lsum) + (double)pe * 0.69314718055994530942;
+  if (p.first) p.logP[g] = lp;
+  else p.logP[g] += lp;
 }
 
 }  // namespace tlrmvn
