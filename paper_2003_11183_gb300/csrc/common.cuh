@@ -313,7 +313,7 @@ __device__ __forceinline__ float max_nan(float x, float y) {
 //    polynomial in L + 3 (the variable of M. Giles, Approximating the erfinv
 //    function, GPU Computing Gems, 2011, in the base of the hardware logarithm;
 //    coefficients from the library's own fit, csrc/fit_ndtri.py, relative error at most
-//    1.4e-7 and 4e-8 rms in float32), its even and odd halves evaluated side by side:
+//    2.4e-7 and 5e-8 rms in float32 with an exact logarithm), its even and odd halves evaluated side by side:
 //    half the dependent steps of Horner's rule;
 //  * below: Wichura's tail forms in t = sqrt(-log p) (M. J. Wichura, Algorithm AS
 //    241, Applied Statistics 37 (1988) 477-484, PPND7, coefficients as

@@ -5,7 +5,7 @@ error function, "Approximating the erfinv function", GPU Computing Gems, 2011, i
 base of the hardware logarithm) and x = 1 - 2p, Phi^-1(p) = x S(L) with S a smooth
 function of L.  For p > 8.4e-5 (L > -8 / ln 2) S is fitted here as a degree-11
 polynomial in L + 3 with the smallest maximum relative error (1.4e-8 in float64).  In float32, its even and
-odd halves evaluated side by side, the relative error is 1.4e-7 at most and 4e-8 rms;
+odd halves evaluated side by side, the relative error is 2.4e-7 at most and 5e-8 rms (an exact logarithm);
 the shift 3 keeps the two halves from cancelling.  The reference values come from
 SciPy's float64 normal quantile through p = exp(-w) / (2 (1 + x)), w = -L ln 2, which has no
 cancellation.
