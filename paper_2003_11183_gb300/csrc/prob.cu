@@ -1403,7 +1403,8 @@ static int run_chunks_tc(Factor& F, const Lims& L, double nu, const tlrmvn_opts&
 
 // Bytes of stream-ordered scratch one tlrmvn_prob call takes (used for admission
 // by the serving loop); mirrors the buffers of prob_impl and the chunk loops.
-int64_t prob_scratch_bytes(const Factor& F, const tlrmvn_opts& o) {
+// general: as if the float32 path were the general one alone.
+int64_t prob_scratch_bytes(const Factor& F, const tlrmvn_opts& o, bool general) {
   const int64_t M = o.n_shifts, N = o.n_points, S = M * N, n = F.n, m = F.m;
   const Tuning tu = F.tuning(o.precision);
   int64_t bytes = n * (8 * 2 + 4 * 2) + (M * (n + 1) + STC_DPAD) * 8 + M * 8 + S * 8 + 256;
@@ -1427,7 +1428,7 @@ int64_t prob_scratch_bytes(const Factor& F, const tlrmvn_opts& o) {
   } else if (o.precision == TLRMVN_FP16_SHIFT) {  // (the same, in passes that the scratch of the usual path holds)
     simt = 256 * simt_sample_bytes(F);
   }
-  return bytes + std::max(simt, tc);
+  return bytes + (general && o.precision == TLRMVN_FP32 ? simt : std::max(simt, tc));
 }
 
 int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, const tlrmvn_opts& o,

@@ -22,7 +22,7 @@ namespace tlrmvn {
 
 int prob_impl(Factor& F, const double* a_dev, const double* b_dev, double nu, const tlrmvn_opts& o,
               double* logp_dev, double* err_dev, double* ell_dev_out, double* per_sample_dev, cudaStream_t st);
-int64_t prob_scratch_bytes(const Factor& F, const tlrmvn_opts& o);
+int64_t prob_scratch_bytes(const Factor& F, const tlrmvn_opts& o, bool general);
 
 using Clock = std::chrono::steady_clock;
 
@@ -178,7 +178,13 @@ extern "C" int tlrmvn_server_submit(tlrmvn_server_t srv, int factor, const doubl
   r->opts = *opts;
   if (opts->shifts) r->shifts.assign(opts->shifts, opts->shifts + (size_t)opts->n_shifts * (F.n + 1));
   r->opts.shifts = nullptr;
-  r->bytes = prob_scratch_bytes(F, r->opts) + (2 * F.n + 2) * 8;
+  auto scratch = [&](bool general) { return prob_scratch_bytes(F, r->opts, general) + (2 * F.n + 2) * 8; };
+  r->bytes = scratch(false);
+  // (the split float32 path's operands are padded, to half as much again on many small tiles: a request for which the
+  // general path's scratch fits runs in smaller passes instead of being refused)
+  if (r->bytes > S.budget && r->opts.sample_chunk <= 0 && scratch(true) <= S.budget)
+    for (int64_t c = (int64_t)r->opts.n_shifts * r->opts.n_points; r->bytes > S.budget && c > 256; r->bytes = scratch(false))
+      r->opts.sample_chunk = c = std::max<int64_t>(256, c / 2);
   if (r->bytes > S.budget) {
     const int64_t r_bytes = r->bytes;
     delete r;
@@ -235,7 +241,7 @@ extern "C" int tlrmvn_server_stats(tlrmvn_server_t srv, tlrmvn_server_stats_t* o
 extern "C" int tlrmvn_prob_scratch_bytes(tlrmvn_factor_t f, const tlrmvn_opts* opts, int64_t* bytes) {
   if (!f || !opts || !bytes) return fail(TLRMVN_E_INVAL, "null argument");
   const Factor& F = *reinterpret_cast<Factor*>(f);
-  *bytes = prob_scratch_bytes(F, *opts) + (2 * F.n + 2) * 8;
+  *bytes = prob_scratch_bytes(F, *opts, false) + (2 * F.n + 2) * 8;
   return TLRMVN_OK;
 }
 
