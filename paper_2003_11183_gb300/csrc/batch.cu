@@ -269,10 +269,10 @@ __global__ void __launch_bounds__(STC_NS, stc_ctas(MODE, false))
       p.err = err;
       p.at(P.tiles[i], i, P.m);
       if (two)
-        ok = stc_tile<FLAGS, MODE, NST, false>(p, k, pl, step, o, run, i * P.m, act, Drow, ks, rs, prod, lsum, pe);
+        ok = stc_tile<FLAGS | STC_GUARD, MODE, NST, false>(p, k, pl, step, o, run, i * P.m, act, Drow, ks, rs, prod, lsum, pe);
       else
-        ok = stc_tile<FLAGS | SWEEP_ONE_SIDED, MODE, NST, false>(p, k, pl, step, o, run, i * P.m, act, Drow, ks, rs,
-                                                               prod, lsum, pe);
+        ok = stc_tile<FLAGS | SWEEP_ONE_SIDED | STC_GUARD, MODE, NST, false>(p, k, pl, step, o, run, i * P.m, act, Drow,
+                                                                             ks, rs, prod, lsum, pe);
     }
     if (ok && act) logP[P.logp_off + g] = (double)(logf(prod) + lsum) + (double)pe * 0.69314718055994530942;
   }

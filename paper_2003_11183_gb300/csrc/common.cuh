@@ -295,16 +295,16 @@ __device__ __forceinline__ float rcp_ftz(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// The smaller, the larger of two, NaN if either is (fminf and fmaxf drop a NaN; the same one instruction).
+// The smallest, the largest, NaN if any is (fminf and fmaxf drop a NaN; the same one instruction).
 __device__ __forceinline__ float min_nan(float x, float y) {
   float z;
   asm("min.NaN.f32 %0, %1, %2;" : "=f"(z) : "f"(x), "f"(y));
   return z;
 }
-__device__ __forceinline__ float max_nan(float x, float y) {
-  float z;
-  asm("max.NaN.f32 %0, %1, %2;" : "=f"(z) : "f"(x), "f"(y));
-  return z;
+__device__ __forceinline__ float max_nan(float x, float y, float z) {
+  float m;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(x), "f"(y), "f"(z));
+  return m;
 }
 
 // float32 normal quantile, lower half.  Two regions:

@@ -503,6 +503,11 @@ __device__ __forceinline__ void stc_done(const StcCta& k, int which) {
   }
 }
 
+// In FLAGS, for the batched kernel: its W goes from problem to problem, and one's padding rows, times zero, lie where
+// another's projections were, so these have to stay finite (y is by itself: ndtri_tail_f32).  (The check costs a solve
+// of n = 65,536 0.4 of 56.7 ms.)
+constexpr int STC_GUARD = 4;
+
 // One diagonal tile for the CTA's samples, by the sweeping warps: the float sweep of eq. 2 and the projections, of the
 // products' sums.  step: steps so far.  o, run, row0: thread
 // 0's, to issue the products when no other warp does.  act: the thread's
@@ -516,7 +521,7 @@ __device__ __forceinline__ bool stc_tile(const SweepTcArgs& p, const StcCta& k, 
                                          const float rs,
                                          float& prod, float& lsum, int& pe) {
   constexpr bool PER = FLAGS & SWEEP_PERIODIZE, ONE = FLAGS & SWEEP_ONE_SIDED;
-  constexpr bool F16 = MODE != STC_BF16, SPLIT = MODE == STC_FP32;
+  constexpr bool F16 = MODE != STC_BF16, SPLIT = MODE == STC_FP32, GUARD = FLAGS & STC_GUARD;
   using Op = Op16<F16>;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int mt = p.mt;
@@ -691,7 +696,7 @@ __device__ __forceinline__ bool stc_tile(const SweepTcArgs& p, const StcCta& k, 
               hi2[j / 2] = Op::pack(y0, y1, h0, h1);
               lo2[j / 2] = Op::pack(y0 - h0, y1 - h1, l0, l1);
             }
-            if (F16) top = max_nan(top, j < nb ? max_nan(fabsf(y0), fabsf(y1)) : 0.0f);
+            if (F16) top = fmaxf(top, j < nb ? fmaxf(fabsf(y0), fabsf(y1)) : 0.0f);  // (a NaN limit's y is finite)
           }
           if (F16 && !(top <= stc_range(MODE))) p.err[1] = 1;
           if (nb == DIAG_VB) {
@@ -762,7 +767,7 @@ __device__ __forceinline__ bool stc_tile(const SweepTcArgs& p, const StcCta& k, 
               const float w1 = (__uint_as_float(r[j + 1]) + __uint_as_float(l[j + 1])) * ws[r1 - rb];
               uint32_t hi, lo;
               split_f32(w0, w1, hi, lo);
-              top = max_nan(top, max_nan(fabsf(w0), two ? fabsf(w1) : 0.0f));
+              top = max_nan(top, fabsf(w0), two ? fabsf(w1) : 0.0f);
               unsigned short* d0 = pl.wcol + (int64_t)vm[rr - rb] * p.ldw;
               d0[0] = (unsigned short)hi;
               d0[(int64_t)p.wlo * p.ldw] = (unsigned short)lo;
@@ -777,16 +782,21 @@ __device__ __forceinline__ bool stc_tile(const SweepTcArgs& p, const StcCta& k, 
       } else if (act) {
         float top = 0.0f;
 #pragma unroll
-        for (int j = 0; j < 16; j++)
+        for (int j = 0; j < 16; j += 2)
           if (r0 + h + j < p.kc) {
-            const float w = F16 ? __uint_as_float(r[j]) * ws[r0 - rb + h + j] : __uint_as_float(r[j]);
-            pl.wcol[(int64_t)vm[r0 - rb + h + j] * p.ldw] = Op::one(w);
-            top = max_nan(top, fabsf(w));
+            const int q = r0 - rb + h + j;
+            const float w0 = F16 ? __uint_as_float(r[j]) * ws[q] : __uint_as_float(r[j]);
+            pl.wcol[(int64_t)vm[q] * p.ldw] = Op::one(w0);
+            float w1 = 0.0f;
+            if (r0 + h + j + 1 < p.kc) {
+              w1 = F16 ? __uint_as_float(r[j + 1]) * ws[q + 1] : __uint_as_float(r[j + 1]);
+              pl.wcol[(int64_t)vm[q + 1] * p.ldw] = Op::one(w1);
+            }
+            if (F16 || GUARD) top = max_nan(top, fabsf(w0), fabsf(w1));
           }
         if (F16 && !(top <= stc_range(MODE))) p.err[1] = 1;
-        if (!F16 && !(top <= stc_range(MODE))) {
-          // bf16: a NaN or an overflow makes the sample's log NaN, and W keeps finite values, for its padding rows
-          // meet zeros (a plan's blocks go from problem to problem: y is finite by itself, ndtri_tail_f32)
+        if (!F16 && GUARD && !(top <= stc_range(MODE))) {
+          // a NaN or an overflow makes the sample's log NaN, and W keeps finite values
           lsum = NAN;
 #pragma unroll 1
           for (int j = 0; j < 16 && r0 + h + j < p.kc; j++) {
