@@ -37,7 +37,7 @@ METRIC = "MVN/MVT QMC sample-dims/sec at n=65,536 vs FP64 path; p50/p99 solve la
 # those sources are unchanged (otherwise null); the summaries with the capture
 # commands are under profiles/.
 TRAFFIC = {
-    "k_sweep_tc": {"bytes_per_sample_dim": 23.1201,
+    "k_sweep_tc": {"bytes_per_sample_dim": 22.5678,
                    "capture": "profiles/k_sweep_tc_n16384.md",
                    "files": ["paper_2003_11183_gb300/csrc/sweep_tc.cuh",
                              "paper_2003_11183_gb300/csrc/sweep.cuh",
@@ -45,7 +45,7 @@ TRAFFIC = {
                              "paper_2003_11183_gb300/csrc/tcgen05.cuh",
                              "paper_2003_11183_gb300/csrc/common.cuh",
                              "include/tlrmvn.h"],
-                   "sources": "006e64bb546b2d4b313fc26f36d6c11fadb27b3dfdeae34b832172181ae6583b"},
+                   "sources": "713fd8962e977858ebf5c09f358b12553ac2d4bd5e22f40a56393176e3cdef29"},
 }
 
 

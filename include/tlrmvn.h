@@ -56,10 +56,10 @@ extern "C" {
 /* Arithmetic of the integrand (tlrmvn_opts.precision). */
 #define TLRMVN_FP64        0  /* everything in float64 */
 #define TLRMVN_FP32        1  /* float32: the sweep, and its products on tcgen05 tensor cores with every operand
-                                 split into fp16 parts (errors of the size of float32 FMAs', sums without their
-                                 bias; y is held to 23 bits, which counts where limits lie tens of standard
-                                 deviations out); limits tens of
-                                 thousands of standard deviations out take float32 FMA kernels instead */
+                                 split into fp16 parts (errors of the size of float32 FMAs'; y is held to 23 bits,
+                                 which shows where limits lie five and more standard deviations out and most sums
+                                 consist of a few such y); limits tens of thousands of standard deviations out
+                                 take float32 FMA kernels instead */
 #define TLRMVN_BF16_SHIFT  2  /* float32 sweep; low-rank shifts on tcgen05 tensor cores, bf16 in, fp32 accumulate */
 #define TLRMVN_FP16_SHIFT  3  /* as BF16_SHIFT with fp16 operands: U and V scaled per off-diagonal tile by
                                  powers of two into fp16's range, the inverse applied to each projection

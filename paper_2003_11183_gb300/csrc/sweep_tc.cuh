@@ -65,8 +65,8 @@ namespace tlrmvn {
 //                       Errors of the samples' logs against 64 bits (rms; float32 FMAs in brackets): n = 2,000 points,
 //                       tiles of 256, exponential kernel of range 0.1, b = -2: 9.8e-6 (1.5e-5), b = 1: 2.3e-6 (3.8e-6);
 //                       range 0.5, b = 0: 5.9e-6 (6.2e-6); range 3, b = 0: 1.0e-5 (7.9e-6), b = 3: 1.3e-6 (2.4e-6).
-//                       y is held to 23 bits, so sums that a few y tens of standard deviations out make up are
-//                       less exact: all entries 0.05, b = -20: 1.8e-3 of 4,320 (4.6e-4).  Times against the float32 FMA products and sweeps: n = 16,384, 20
+//                       y is held to 23 bits, so sums that a few large y make up are less exact: all entries
+//                       0.05, b = -5: 4.2e-5 of 327 (2.7e-5), b = -20: 1.8e-3 of 4,320 (4.6e-4).  Times against the float32 FMA products and sweeps: n = 16,384, 20
 //                       x 5,000 samples: 55.0 -> 25.9 ms a solve; n = 4,096, nu = 7, 10 x 1,000: 4.41 -> 2.35 ms; 64
 //                       batched problems, 10 x 2,000: 87.9 -> 18.8 ms.
 enum StcMode { STC_BF16 = 0, STC_FP16 = 1, STC_FP32 = 2 };
