@@ -45,7 +45,7 @@ TRAFFIC = {
                              "paper_2003_11183_gb300/csrc/tcgen05.cuh",
                              "paper_2003_11183_gb300/csrc/common.cuh",
                              "include/tlrmvn.h"],
-                   "sources": "713fd8962e977858ebf5c09f358b12553ac2d4bd5e22f40a56393176e3cdef29"},
+                   "sources": "35a7e106a487363cef6cfbc61a6d3e7b37b65b3f9ece792e0ac8952c475e01da"},
 }
 
 

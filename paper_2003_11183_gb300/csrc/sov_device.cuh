@@ -184,15 +184,18 @@ __device__ __forceinline__ float phi_neg_f32(float x) {
 // quantile takes 4 p (1 - p) = 4 u uc and 1 - 2p = +-(uc - u) from them directly: no
 // minimum, comparison or select on the way to y.
 
-// (y, the step's log) of a lane off the fast path
+// (y, the step's log) of a lane off the fast path, the only one whose y may be large: cut to CAP in size (0: not)
+template <int CAP>
 static __device__ __noinline__ float2 sov_step_rare_f32(float at, float bt, float w, float wc, float pp, bool deep) {
   if (!deep) return make_float2(ndtri_tail_f32(__logf(pp)), 0.0f);
   float ld, y;
   sov_step_f32(at, bt, w, wc, ld, y);
+  if (CAP) y = fminf(fmaxf(y, (float)-CAP), (float)CAP);
   return make_float2(y, ld);
 }
 
 // The one-sided (at = -inf) case.
+template <int CAP = 0>
 __device__ __forceinline__ void sov_step_f32_upper(float bt, float w, float wc, float& f, float& lsum, float& y) {
   const float h = phi_neg_f32(fabsf(bt)), m = 1.0f - h;  // Phi(-|bt|), Phi(|bt|)
   const bool neg = bt < 0.0f, near1 = bt > 3.5f;
@@ -206,7 +209,7 @@ __device__ __forceinline__ void sov_step_f32_upper(float bt, float w, float wc, 
   if (!(L >= NDTRI_LMIN - 2.0f)) {
     // (a deep limit always comes here: u < Phi(-8.9) = 2.8e-19; above it pp > 3e-29; and a NaN, as a deep one)
     const bool deep = !(bt >= -8.9f);
-    const float2 r = sov_step_rare_f32(-INFINITY, bt, w, wc, fminf(u, uc), deep);
+    const float2 r = sov_step_rare_f32<CAP>(-INFINITY, bt, w, wc, fminf(u, uc), deep);
     y = (deep || u <= uc) ? r.x : -r.x;
     f = deep ? 1.0f : f;
     lsum += r.y;
@@ -214,6 +217,7 @@ __device__ __forceinline__ void sov_step_f32_upper(float bt, float w, float wc, 
 }
 
 // Any interval.  With both limits on one side of 0 the probability is the difference of the two smaller tails.
+template <int CAP = 0>
 __device__ __forceinline__ void sov_step_f32_prod(float at, float bt, float w, float wc, float& f, float& lsum,
                                                   float& y) {
   const float ha = phi_neg_f32(fabsf(at)), hb = phi_neg_f32(fabsf(bt)), ma = 1.0f - ha;
@@ -228,7 +232,7 @@ __device__ __forceinline__ void sov_step_f32_prod(float at, float bt, float w, f
   y = ndtri_poly_f32(L + 5.0f) * (uc - u);
   const bool deep = !(diff >= 2.5e-19f);  // (also a zero-width interval and, through the comparison, a NaN)
   if (deep || L < NDTRI_LMIN - 2.0f) {
-    const float2 r = sov_step_rare_f32(at, bt, w, wc, fminf(u, uc), deep);
+    const float2 r = sov_step_rare_f32<CAP>(at, bt, w, wc, fminf(u, uc), deep);
     y = (deep || u <= uc) ? r.x : -r.x;
     f = deep ? 1.0f : f;
     lsum += r.y;

@@ -618,10 +618,10 @@ __device__ __forceinline__ bool stc_tile(const SweepTcArgs& p, const StcCta& k, 
         float w, wc, f, y;
         lattice_wf((uint64_t)ks * qv + dv, PER ? 1 : 0, w, wc);
         if (ONE) {
-          sov_step_f32_upper(bt, w, wc, f, lsum, y);
+          sov_step_f32_upper<F16 ? (int)stc_range(MODE) : 0>(bt, w, wc, f, lsum, y);
         } else {
           const float at = fmaf(abi.x, rs, -sum) * abi.z;
-          sov_step_f32_prod(at, bt, w, wc, f, lsum, y);
+          sov_step_f32_prod<F16 ? (int)stc_range(MODE) : 0>(at, bt, w, wc, f, lsum, y);
         }
         prod *= f;
         return y;
@@ -696,9 +696,9 @@ __device__ __forceinline__ bool stc_tile(const SweepTcArgs& p, const StcCta& k, 
               hi2[j / 2] = Op::pack(y0, y1, h0, h1);
               lo2[j / 2] = Op::pack(y0 - h0, y1 - h1, l0, l1);
             }
-            if (F16) top = fmaxf(top, j < nb ? fmaxf(fabsf(y0), fabsf(y1)) : 0.0f);  // (a NaN limit's y is finite)
+            if (F16) top = fmaxf(top, j < nb ? fmaxf(fabsf(y0), fabsf(y1)) : 0.0f);
           }
-          if (F16 && !(top <= stc_range(MODE))) p.err[1] = 1;
+          if (F16 && top >= stc_range(MODE)) p.err[1] = 1;  // (the step cuts y to it: what follows stays finite)
           if (nb == DIAG_VB) {
             uint4* dh = reinterpret_cast<uint4*>(row);
             uint4* dlo = reinterpret_cast<uint4*>(row + p.ys_lo);
